@@ -9,13 +9,11 @@
 //   to the lower index y W + x; the N strongest (R' descending, index ascending); BRIEF bits
 //   [S(x + p_k) > S(x + q_k)] of the binomial-smoothed image S for 256 given point pairs.
 //
-// Kernels: lorb_maps (gray and S over the areas' neighbourhood, S by separable passes),
-// lorb_response (FAST + Harris on 32 x 16 tiles staged in shared memory; FAST by a compass
-// pre-test and 16-bit run masks), lorb_nms (survivors appended with warp-aggregated atomics, their
-// order is irrelevant since the selection below is exact, and counted in a histogram of coarse
-// response bins), lorb_prune (the survivors in the bins that can hold the N strongest),
-// lorb_select (one block: radix selection of the N-th key, then a bitonic sort of the N winners),
-// lorb_brief (a warp per keypoint, bits packed by ballots).
+// Kernels: lorb_detect (gray, FAST, Harris and non-maximum suppression of a tile on chip; survivors
+// appended, their order being irrelevant since the selection below is exact, and counted in a
+// histogram of coarse response bins), lorb_prune (the survivors in the bins that can hold the N
+// strongest; when those are too many to rank, its last block selects the N strongest itself) and
+// lorb_rank_brief (rank by counting, then the BRIEF bits from the point's patch of the frame).
 #include "stitch_internal.cuh"
 
 namespace {
@@ -23,9 +21,6 @@ namespace {
 constexpr int LORB_MARGIN = 18;
 constexpr int LORB_MAX_AREAS = 64;
 constexpr int LORB_MAX_POINTS = 2048;
-constexpr int LT_X = 32, LT_Y = 16;           // response tile
-constexpr int LG_X = LT_X + 6, LG_Y = LT_Y + 6;  // gray with the radius-3 halo
-constexpr int LD_X = LT_X + 4, LD_Y = LT_Y + 4;  // gradients at the tensor window positions
 constexpr int SEL_THREADS = 1024;
 
 struct LorbAreas {
@@ -48,151 +43,7 @@ __device__ __forceinline__ bool in_areas(const LorbAreas& a, int x, int y) {
     return false;
 }
 
-// gray (uint8) and binomial-smoothed gray S (unnormalised, at most 255 * 256: uint16) on
-// [x0, x1) x [y0, y1) (x0 a multiple of 4); S by a horizontal then a vertical [1,4,6,4,1] pass (the
-// same integers as the 5 x 5 product weights).  The tile's gray, with a halo of 4 columns and 2
-// rows, is staged from groups of 4 pixels: three aligned 32-bit words where the group lies inside
-// the image and the frame's base and pitch are multiples of 4 bytes, clamped byte loads otherwise.
-__device__ __forceinline__ int gray_of(int r, int g, int b) { return (77 * r + 150 * g + 29 * b + 128) >> 8; }
-
-__global__ void __launch_bounds__(256) lorb_maps(const uint8_t* __restrict__ frame, long long pitch, int W, int H,
-                                                 int x0, int y0, int x1, int y1, uint8_t* __restrict__ gray,
-                                                 uint16_t* __restrict__ smooth) {
-    __shared__ int g[20][40];  // columns bx - 4 .. bx + 35, rows by - 2 .. by + 17
-    __shared__ int hs[20][32];
-    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;  // 32 x 8 threads
-    const int bx = x0 + blockIdx.x * 32, by = y0 + blockIdx.y * 16;
-    const bool words = ((reinterpret_cast<uintptr_t>(frame) | (uintptr_t)pitch) & 3) == 0;
-    for (int q = threadIdx.x; q < 20 * 10; q += 256) {
-        const int r = q / 10, j = q - r * 10;
-        const int y = min(max(by - 2 + r, 0), H - 1), gx0 = bx - 4 + 4 * j;
-        const uint8_t* row = frame + (long long)y * pitch;
-        if (words && gx0 >= 0 && gx0 + 3 < W) {
-            const uint32_t* w = reinterpret_cast<const uint32_t*>(row + 3LL * gx0);
-            const uint32_t a = __ldg(w), b = __ldg(w + 1), c = __ldg(w + 2);
-            // bytes R G B R | G B R G | B R G B
-            g[r][4 * j] = gray_of(a & 255, (a >> 8) & 255, (a >> 16) & 255);
-            g[r][4 * j + 1] = gray_of(a >> 24, b & 255, (b >> 8) & 255);
-            g[r][4 * j + 2] = gray_of((b >> 16) & 255, b >> 24, c & 255);
-            g[r][4 * j + 3] = gray_of((c >> 8) & 255, (c >> 16) & 255, c >> 24);
-        } else {
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                const int x = min(max(gx0 + k, 0), W - 1);
-                const uint8_t* p = row + 3LL * x;
-                g[r][4 * j + k] = gray_of(p[0], p[1], p[2]);
-            }
-        }
-    }
-    __syncthreads();
-    for (int q = threadIdx.x; q < 20 * 32; q += 256) {
-        const int r = q >> 5, c = q & 31;  // window columns c + 2 .. c + 6 (canvas x - 2 .. x + 2)
-        hs[r][c] = g[r][c + 2] + 4 * g[r][c + 3] + 6 * g[r][c + 4] + 4 * g[r][c + 5] + g[r][c + 6];
-    }
-    __syncthreads();
-    for (int rr = ty; rr < 16; rr += 8) {
-        const int x = bx + tx, y = by + rr;
-        if (x >= x1 || y >= y1) continue;
-        gray[(long long)y * W + x] = (uint8_t)g[rr + 2][tx + 4];
-        // S only where its 5 x 5 window is inside the image (BRIEF never reads it elsewhere)
-        if (x < 2 || y < 2 || x >= W - 2 || y >= H - 2) continue;
-        smooth[(long long)y * W + x] =
-            (uint16_t)(hs[rr][tx] + 4 * hs[rr + 1][tx] + 6 * hs[rr + 2][tx] + 4 * hs[rr + 3][tx] + hs[rr + 4][tx]);
-    }
-}
-
-// FAST-9 + Harris response R' (INT64_MIN where not a candidate) on [x0, x1) x [y0, y1)
-__global__ void __launch_bounds__(256) lorb_response(const uint8_t* __restrict__ gray, int W, int x0, int y0,
-                                                     int x1, int y1, const __grid_constant__ LorbAreas areas,
-                                                     int fast_t, long long harris_t, long long* __restrict__ resp) {
-    __shared__ int g[LG_Y][LG_X];
-    __shared__ int dxs[LD_Y][LD_X], dys[LD_Y][LD_X];
-    __shared__ int hxx[LD_Y][LT_X], hyy[LD_Y][LT_X], hxy[LD_Y][LT_X];
-    const int bx = x0 + blockIdx.x * LT_X, by = y0 + blockIdx.y * LT_Y;
-    const int t = threadIdx.x;
-    // gray of the tile and its radius-3 halo (inside the image: candidates keep a wider margin)
-    for (int q = t; q < LG_X * LG_Y; q += 256) {
-        const int r = q / LG_X, c = q - r * LG_X;
-        const int x = bx - 3 + c, y = by - 3 + r;
-        g[r][c] = (x >= 0 && y >= 0 && x < x1 + 3 && y < y1 + 3) ? gray[(long long)y * W + x] : 0;
-    }
-    __syncthreads();
-    for (int q = t; q < LD_X * LD_Y; q += 256) {
-        const int r = q / LD_X, c = q - r * LD_X;  // position (bx - 2 + c, by - 2 + r)
-        dxs[r][c] = g[r + 1][c + 2] - g[r + 1][c];
-        dys[r][c] = g[r + 2][c + 1] - g[r][c + 1];
-    }
-    __syncthreads();
-    const int b5[5] = {1, 4, 6, 4, 1};
-    for (int q = t; q < LT_X * LD_Y; q += 256) {
-        const int r = q / LT_X, c = q - r * LT_X;
-        int sxx = 0, syy = 0, sxy = 0;
-#pragma unroll
-        for (int k = 0; k < 5; ++k) {
-            const int ix = dxs[r][c + k], iy = dys[r][c + k];
-            sxx += b5[k] * ix * ix;
-            syy += b5[k] * iy * iy;
-            sxy += b5[k] * ix * iy;
-        }
-        hxx[r][c] = sxx;
-        hyy[r][c] = syy;
-        hxy[r][c] = sxy;
-    }
-    __syncthreads();
-    constexpr int fdx[16] = {0, 1, 2, 3, 3, 3, 2, 1, 0, -1, -2, -3, -3, -3, -2, -1};
-    constexpr int fdy[16] = {-3, -3, -2, -1, 0, 1, 2, 3, 3, 3, 2, 1, 0, -1, -2, -3};
-    for (int q = t; q < LT_X * LT_Y; q += 256) {
-        const int r = q / LT_X, c = q - r * LT_X;
-        const int x = bx + c, y = by + r;
-        if (x >= x1 || y >= y1) continue;
-        long long out = LLONG_MIN;
-        if (in_areas(areas, x, y)) {
-            // FAST-9: a run of >= 9 contiguous circle pixels all brighter than p + t, or all darker
-            // than p - t.  Such an arc holds at least 2 of the 4 compass pixels (0, 4, 8, 12), so a
-            // pixel with fewer than 2 brighter and fewer than 2 darker compass pixels is no corner;
-            // the others test the 16-bit masks, doubled so that a run may wrap around.
-            const int p = g[r + 3][c + 3], hi = p + fast_t, lo = p - fast_t;
-            int nb = 0, nd = 0;
-#pragma unroll
-            for (int k = 0; k < 16; k += 4) {
-                const int v = g[r + 3 + fdy[k]][c + 3 + fdx[k]];
-                nb += v > hi;
-                nd += v < lo;
-            }
-            bool corner = false;
-            if (nb >= 2 || nd >= 2) {
-                unsigned mb = 0, md = 0;
-#pragma unroll
-                for (int k = 0; k < 16; ++k) {
-                    const int v = g[r + 3 + fdy[k]][c + 3 + fdx[k]];
-                    mb |= (unsigned)(v > hi) << k;
-                    md |= (unsigned)(v < lo) << k;
-                }
-                mb |= mb << 16;
-                md |= md << 16;
-                unsigned rb = mb, rd = md;
-#pragma unroll
-                for (int k = 1; k < 9; ++k) {
-                    rb &= mb >> k;
-                    rd &= md >> k;
-                }
-                corner = (rb | rd) != 0;
-            }
-            if (corner) {
-                long long A = 0, B = 0, C = 0;
-#pragma unroll
-                for (int k = 0; k < 5; ++k) {
-                    A += (long long)b5[k] * hxx[r + k][c];
-                    B += (long long)b5[k] * hyy[r + k][c];
-                    C += (long long)b5[k] * hxy[r + k][c];
-                }
-                const long long rr = 25 * (A * B - C * C) - (A + B) * (A + B);
-                if (rr > harris_t) out = rr;
-            }
-        }
-        resp[(long long)y * W + x] = out;
-    }
-}
+__device__ __forceinline__ unsigned gray_of(unsigned r, unsigned g, unsigned b) { return (77u * r + 150u * g + 29u * b + 128u) >> 8; }
 
 // Coarse, monotone (non-decreasing in R') bin of a response: the position of its leading bit and
 // the 4 bits below it; R' <= 0 in bin 0.  The N strongest candidates all lie in the bins at or above
@@ -205,98 +56,227 @@ __device__ __forceinline__ int lorb_bin(long long r) {
     return 16 * e + m;
 }
 
-// non-maximum suppression: survivors appended to cand (ties to the lower index), and counted in
-// the bin histogram
-__global__ void __launch_bounds__(256) lorb_nms(const long long* __restrict__ resp, int W, int x0, int y0, int x1,
-                                                int y1, Cand* __restrict__ cand, int* __restrict__ ncand, int cap,
-                                                int* __restrict__ hist) {
-    const int x = x0 + blockIdx.x * 32 + (threadIdx.x & 31), y = y0 + blockIdx.y * 8 + (threadIdx.x >> 5);
-    bool keep = false;
-    long long r = LLONG_MIN;
-    int idx = 0;
-    if (x < x1 && y < y1) {
-        idx = y * W + x;
-        r = resp[idx];
-        keep = r != LLONG_MIN;
-        for (int dy = -1; dy <= 1 && keep; ++dy)
-            for (int dx = -1; dx <= 1 && keep; ++dx) {
-                if (!dx && !dy) continue;
-                const int xx = x + dx, yy = y + dy;
-                if (xx < x0 || yy < y0 || xx >= x1 || yy >= y1) continue;  // outside: never a candidate
-                const int q = yy * W + xx;
-                const long long o = resp[q];
-                if (o == LLONG_MIN) continue;
-                keep = r > o || (r == o && idx < q);
-            }
-    }
-    const unsigned m = __ballot_sync(0xffffffffu, keep);
-    if (!m) return;
-    int base = 0;
-    const int lane = threadIdx.x & 31, leader = __ffs(m) - 1;
-    if (lane == leader) base = atomicAdd(ncand, __popc(m));
-    base = __shfl_sync(0xffffffffu, base, leader);
-    if (keep) {
-        const int pos = base + __popc(m & ((1u << lane) - 1));
-        if (pos < cap) {
-            cand[pos] = Cand{r, idx, 0};
-            atomicAdd(&hist[lorb_bin(r)], 1);
-        }
-    }
+// Counters of a call, zero between calls but for n2 (lorb_prune's last block clears them): survivors,
+// finished lorb_prune blocks, pruned candidates, survivors per response bin.
+struct LorbCount {
+    int n, done, n2, pad;
+    int hist[LORB_BINS];
+};
+
+// lorb_detect: gray, FAST, Harris response and non-maximum suppression of one tile, appending the
+// survivors to cand (their order is irrelevant) and counting them in the bin histogram.
+//
+// A block of 256 threads evaluates 64 x 32 pixels and owns the inner 60 x 30: the ring around them
+// gives the suppression its neighbours, so no response ever leaves the chip.  What bounds it is
+// instruction issue: 8.3 MPix of a 4K view cost about 30 instructions each (reading the 25 MB takes
+// 4 us).  Hence:
+//  - the tile's gray is staged as words that hold a pixel and the one below it (16 bits each), so one
+//    32-bit load and one 16-bit-pair minimum or maximum serve two pixels, at any offset;
+//  - a pair is tested on its 4 compass pixels first (an arc of 9 of the 16 circle pixels holds two
+//    neighbouring ones).  The pairs that pass are gathered per warp, so the 16-pixel test and then
+//    the Harris response of the corners run with full warps instead of under a branch that nearly
+//    every warp takes for a few lanes.
+// One 3840 x 2160 view: 35 us against 134 us for gray and smoothed maps, response map (8 bytes per
+// pixel written and read back) and suppression as three kernels.
+constexpr int DT_EX = 64, DT_EY = 32;   // evaluated pixels
+constexpr int DT_OX = 60, DT_OY = 30;   // owned pixels: columns 2 .. 61, rows 1 .. 30
+constexpr int DT_PX = 72, DT_PY = 39;   // gray words: 18 groups of 4 columns, 13 strips of 3 rows
+constexpr int DT_WARPS = 8;
+
+// whether either of the two pixels p (16 bits each) has an arc value above it (mb: the largest of the
+// arcs' smallest values) or below it (md) by more than the threshold; lim = threshold + 256
+__device__ __forceinline__ unsigned fast_excess(unsigned p, unsigned mb, unsigned md) {
+    return __vmaxu2((mb + 0x01000100u) - p, (p + 0x01000100u) - md);
 }
 
-// The candidates in the bins at or above the threshold bin (where the count from the top reaches
-// N) appended to cand2: a superset of the N strongest, typically a small one.  Grid-stride; every
-// block finds the threshold bin from the histogram (a suffix sum over the bins).
-constexpr int PRUNE_THREADS = 1024, PRUNE_BLOCKS = 64;
-__global__ void __launch_bounds__(PRUNE_THREADS) lorb_prune(const Cand* __restrict__ cand, const int* __restrict__ ncand,
-                                                            int cap, int npts, const int* __restrict__ hist,
-                                                            Cand* __restrict__ cand2, int* __restrict__ n2,
-                                                            int* __restrict__ overflow) {
-    static_assert(PRUNE_THREADS == LORB_BINS, "one bin per thread");
-    __shared__ int wsum[32];
-    __shared__ int s_b;
+__global__ void __launch_bounds__(256, 5) lorb_detect(const uint8_t* __restrict__ frame, long long pitch, int W, int H,
+                                                      int ox, int oy, const __grid_constant__ LorbAreas areas, int lim,
+                                                      long long harris_t, Cand* __restrict__ cand, int* __restrict__ ncand,
+                                                      int cap, int* __restrict__ hist, int* __restrict__ n2) {
+    __shared__ __align__(16) unsigned P[DT_PX * DT_PY];
+    __shared__ long long R[DT_EX * DT_EY];
+    __shared__ unsigned mask[DT_EY][2];  // which pixels of a row have a response
+    __shared__ uint16_t pairs[DT_WARPS][128], corners[DT_WARPS][256];
+    __shared__ int s_n, s_base;
     const int t = threadIdx.x, lane = t & 31, w = t >> 5;
-    const int total = *ncand, n = min(total, cap), want = min(n, npts);
-    if (blockIdx.x == 0 && t == 0) *overflow = total > cap ? 1 : 0;
-    if (t == 0) s_b = LORB_BINS;  // want == 0: nothing
-    // suffix sums: thread t takes bin 1023 - t and an inclusive prefix sum over t
-    const int b = LORB_BINS - 1 - t;
-    int v = hist[b];
-    for (int off = 1; off < 32; off <<= 1) {
-        const int o = __shfl_up_sync(0xffffffffu, v, off);
-        if (lane >= off) v += o;
-    }
-    if (lane == 31) wsum[w] = v;
-    __syncthreads();
-    if (w == 0) {
-        int x = wsum[lane];
-        for (int off = 1; off < 32; off <<= 1) {
-            const int o = __shfl_up_sync(0xffffffffu, x, off);
-            if (lane >= off) x += o;
+    // owned pixels start at (bx, by); bx is 1 modulo 4, so the staged columns start at a multiple of 4
+    const int bx = ox + DT_OX * blockIdx.x, by = oy + DT_OY * blockIdx.y;
+    if (blockIdx.x == 0 && blockIdx.y == 0 && t == 0) *n2 = 0;
+    bool any = false;
+    for (int k = 0; k < areas.n; ++k)
+        any |= bx < areas.r[k][2] && bx + DT_OX > areas.r[k][0] && by < areas.r[k][3] && by + DT_OY > areas.r[k][1];
+    if (!any) return;
+    if (t < 2 * DT_EY) mask[t >> 1][t & 1] = 0u;
+    if (t == 0) s_n = 0;
+    if (t < 18 * 13) {
+        const int j = t % 18, st = t / 18, gx0 = bx - 5 + 4 * j;
+        const bool words = ((reinterpret_cast<uintptr_t>(frame) | (uintptr_t)pitch) & 3) == 0 && gx0 + 3 < W;
+        unsigned g[4][4];
+        if (words) {
+            unsigned v[4][3];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const int y = min(by - 4 + 3 * st + k, H - 1);
+                const unsigned* q = reinterpret_cast<const unsigned*>(frame + (long long)y * pitch + 3LL * gx0);
+                v[k][0] = __ldg(q);
+                v[k][1] = __ldg(q + 1);
+                v[k][2] = __ldg(q + 2);
+            }
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                // bytes R G B R | G B R G | B R G B
+                const unsigned a = v[k][0], b = v[k][1], c = v[k][2];
+                g[k][0] = __dp4a(a, 0x001D964Du, 128u) >> 8;
+                g[k][1] = __dp4a(b, 0x00001D96u, __dp4a(a, 0x4D000000u, 128u)) >> 8;
+                g[k][2] = __dp4a(c, 0x0000001Du, __dp4a(b, 0x964D0000u, 128u)) >> 8;
+                g[k][3] = __dp4a(c, 0x1D964D00u, 128u) >> 8;
+            }
+        } else {
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const uint8_t* row = frame + (long long)min(by - 4 + 3 * st + k, H - 1) * pitch;
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const uint8_t* q = row + 3LL * min(gx0 + i, W - 1);
+                    g[k][i] = gray_of(__ldg(q), __ldg(q + 1), __ldg(q + 2));
+                }
+            }
         }
-        wsum[lane] = x;
+#pragma unroll
+        for (int k = 0; k < 3; ++k)
+            *reinterpret_cast<uint4*>(P + (3 * st + k) * DT_PX + 4 * j) =
+                make_uint4(g[k][0] | g[k + 1][0] << 16, g[k][1] | g[k + 1][1] << 16, g[k][2] | g[k + 1][2] << 16,
+                           g[k][3] | g[k + 1][3] << 16);
     }
     __syncthreads();
-    const int S = v + (w > 0 ? wsum[w - 1] : 0);  // candidates in bins >= b
-    const int S_above = S - hist[b];             // in bins > b
-    if (want > 0 && S >= want && S_above < want) s_b = b;
+    // evaluated pixel (ex, ey) is image pixel (bx - 2 + ex, by - 1 + ey), staged at P[ey + 3][ex + 3];
+    // warp w takes rows 4 w .. 4 w + 3 through all phases
+    constexpr int fo[16] = {-3 * DT_PX,     -3 * DT_PX + 1, -2 * DT_PX + 2, -DT_PX + 3, 3,  DT_PX + 3,  2 * DT_PX + 2,  3 * DT_PX + 1,
+                            3 * DT_PX,      3 * DT_PX - 1,  2 * DT_PX - 2,  DT_PX - 3,  -3, -DT_PX - 3, -2 * DT_PX - 2, -3 * DT_PX - 1};
+    const unsigned below = (1u << lane) - 1u;
+    int np = 0;
+#pragma unroll
+    for (int it = 0; it < 4; ++it) {
+        const int ey = 4 * w + 2 * (it >> 1), ex = 32 * (it & 1) + lane;
+        const unsigned* c = P + (ey + 3) * DT_PX + ex + 3;
+        const unsigned p = c[0], n = c[fo[0]], e = c[fo[4]], s = c[fo[8]], o = c[fo[12]];
+        const unsigned x = fast_excess(p, __vminu2(__vmaxu2(n, s), __vmaxu2(e, o)), __vmaxu2(__vminu2(n, s), __vminu2(e, o)));
+        const bool pass = ((int)(x & 0xffffu) > lim || (int)(x >> 16) > lim) && ex >= 1 && ex <= 62;
+        const unsigned m = __ballot_sync(0xffffffffu, pass);
+        if (pass) pairs[w][np + __popc(m & below)] = (uint16_t)(ey * DT_EX + ex);
+        np += __popc(m);
+    }
+    __syncwarp();
+    int nc = 0;
+    for (int i0 = 0; i0 < np; i0 += 32) {
+        bool lo = false, hi = false;
+        int at = 0;
+        if (i0 + lane < np) {
+            at = pairs[w][i0 + lane];
+            const int ex = at & (DT_EX - 1), ey = at / DT_EX;
+            const unsigned* c = P + (ey + 3) * DT_PX + ex + 3;
+            unsigned v[16];
+#pragma unroll
+            for (int k = 0; k < 16; ++k) v[k] = c[fo[k]];
+            unsigned mb, md;
+            {
+                unsigned m3[16];
+#pragma unroll
+                for (int k = 0; k < 16; ++k) m3[k] = __vimin3_u16x2(v[k], v[(k + 1) & 15], v[(k + 2) & 15]);
+                mb = __vimin3_u16x2(m3[0], m3[3], m3[6]);
+#pragma unroll
+                for (int k = 1; k < 16; ++k) mb = __vmaxu2(mb, __vimin3_u16x2(m3[k], m3[(k + 3) & 15], m3[(k + 6) & 15]));
+            }
+            {
+                unsigned m3[16];
+#pragma unroll
+                for (int k = 0; k < 16; ++k) m3[k] = __vimax3_u16x2(v[k], v[(k + 1) & 15], v[(k + 2) & 15]);
+                md = __vimax3_u16x2(m3[0], m3[3], m3[6]);
+#pragma unroll
+                for (int k = 1; k < 16; ++k) md = __vminu2(md, __vimax3_u16x2(m3[k], m3[(k + 3) & 15], m3[(k + 6) & 15]));
+            }
+            const unsigned x = fast_excess(c[0], mb, md);
+            const int ix = bx - 2 + ex, iy = by - 1 + ey;
+            lo = (int)(x & 0xffffu) > lim && in_areas(areas, ix, iy);
+            hi = (int)(x >> 16) > lim && in_areas(areas, ix, iy + 1);
+        }
+        const unsigned ml = __ballot_sync(0xffffffffu, lo), mh = __ballot_sync(0xffffffffu, hi);
+        if (lo) corners[w][nc + __popc(ml & below)] = (uint16_t)at;
+        nc += __popc(ml);
+        if (hi) corners[w][nc + __popc(mh & below)] = (uint16_t)(at + DT_EX);
+        nc += __popc(mh);
+    }
+    __syncwarp();
+    for (int i = lane; i < nc; i += 32) {
+        const int at = corners[w][i], ex = at & (DT_EX - 1), ey = at / DT_EX;
+        const uint16_t* c = reinterpret_cast<const uint16_t*>(P + (ey + 3) * DT_PX + ex + 3);  // the pixel's own half
+        const int b5[5] = {1, 4, 6, 4, 1};
+        int A = 0, B = 0, C = 0;  // at most 256 * 255 * 255
+#pragma unroll
+        for (int r = -2; r <= 2; ++r) {
+            int sxx = 0, syy = 0, sxy = 0;
+#pragma unroll
+            for (int k = -2; k <= 2; ++k) {
+                const int ix = (int)c[2 * (r * DT_PX + k + 1)] - (int)c[2 * (r * DT_PX + k - 1)];
+                const int iy = (int)c[2 * ((r + 1) * DT_PX + k)] - (int)c[2 * ((r - 1) * DT_PX + k)];
+                sxx += b5[k + 2] * ix * ix;
+                syy += b5[k + 2] * iy * iy;
+                sxy += b5[k + 2] * ix * iy;
+            }
+            A += b5[r + 2] * sxx;
+            B += b5[r + 2] * syy;
+            C += b5[r + 2] * sxy;
+        }
+        const long long tr = (long long)A + B, rr = 25 * ((long long)A * B - (long long)C * C) - tr * tr;
+        if (rr > harris_t) {
+            R[at] = rr;
+            atomicOr(&mask[ey][ex >> 5], 1u << (ex & 31));
+        }
+    }
     __syncthreads();
-    const int bT = s_b;
-    for (int i0 = blockIdx.x * PRUNE_THREADS; i0 < n; i0 += gridDim.x * PRUNE_THREADS) {
-        const int i = i0 + t;
-        Cand cv{0, 0, 0};
+    // non-maximum suppression (ties to the lower index), survivors into the pair list's memory: no two
+    // are neighbours, so at most a quarter of the evaluated pixels
+    uint16_t* surv = &pairs[0][0];
+    static_assert(sizeof(pairs) / sizeof(uint16_t) >= (DT_OX / 2) * (DT_OY / 2), "room for the survivors");
+    for (int i0 = 0; i0 < nc; i0 += 32) {
         bool keep = false;
-        if (i < n) {
-            cv = cand[i];
-            keep = lorb_bin(cv.r) >= bT;
+        int at = 0;
+        if (i0 + lane < nc) {
+            at = corners[w][i0 + lane];
+            const int ex = at & (DT_EX - 1), ey = at / DT_EX;
+            if (ex >= 2 && ex < 2 + DT_OX && ey >= 1 && ey < 1 + DT_OY && (mask[ey][ex >> 5] >> (ex & 31) & 1u)) {
+                const long long r = R[at];
+                keep = true;
+#pragma unroll
+                for (int dy = -1; dy <= 1; ++dy) {
+                    const unsigned long long m = mask[ey + dy][0] | (unsigned long long)mask[ey + dy][1] << 32;
+                    const unsigned nb = (unsigned)(m >> (ex - 1)) & 7u;
+#pragma unroll
+                    for (int dx = -1; dx <= 1; ++dx) {
+                        if ((dx || dy) && (nb >> (dx + 1) & 1u)) {
+                            const long long o = R[at + dy * DT_EX + dx];
+                            keep &= r > o || (r == o && (dy > 0 || (dy == 0 && dx > 0)));
+                        }
+                    }
+                }
+            }
         }
         const unsigned m = __ballot_sync(0xffffffffu, keep);
-        if (!m) continue;
         int base = 0;
-        const int leader = __ffs(m) - 1;
-        if (lane == leader) base = atomicAdd(n2, __popc(m));
-        base = __shfl_sync(0xffffffffu, base, leader);
-        if (keep) cand2[base + __popc(m & ((1u << lane) - 1))] = cv;
+        if (lane == 0 && m) base = atomicAdd(&s_n, __popc(m));
+        base = __shfl_sync(0xffffffffu, base, 0);
+        if (keep) surv[base + __popc(m & below)] = (uint16_t)at;
+    }
+    __syncthreads();
+    if (t == 0) s_base = s_n ? atomicAdd(ncand, s_n) : 0;
+    __syncthreads();
+    for (int i = t; i < s_n; i += 256) {
+        const int at = surv[i], pos = s_base + i;
+        const long long r = R[at];
+        if (pos < cap) {
+            cand[pos] = Cand{r, (by - 1 + at / DT_EX) * W + bx - 2 + (at & (DT_EX - 1)), 0};
+            atomicAdd(&hist[lorb_bin(r)], 1);
+        }
     }
 }
 
@@ -342,24 +322,25 @@ __device__ __forceinline__ int select_digit(const int* hist, int* wsum, int& nee
     return r;
 }
 
-// One block: the N strongest survivors, sorted.  Radix selection (8-bit digits, most
-// significant first) of the N-th largest u; survivors above it are taken, and among those equal
-// to it the lowest indices (a second radix selection on the index); then a bitonic sort.
-__global__ void __launch_bounds__(SEL_THREADS) lorb_select(const Cand* __restrict__ cand,
-                                                           const int* __restrict__ ncand, int cap, int npts,
-                                                           int W, int* __restrict__ out_xy,
-                                                           long long* __restrict__ out_resp, int* __restrict__ count,
-                                                           int* __restrict__ overflow) {
-    __shared__ int hist[256];
-    __shared__ unsigned long long s_prefix;
-    __shared__ int s_need;
-    __shared__ Cand win[LORB_MAX_POINTS];
-    __shared__ int s_nwin;
-    __shared__ int s_wsum[32], s_pick[2];
+// The N strongest of a crowded candidate set, sorted, by one block of SEL_THREADS threads: radix
+// selection (8-bit digits, most significant first) of the N-th largest u; survivors above it are
+// taken, and among those equal to it the lowest indices (a second radix selection on the index);
+// then a bitonic sort.
+struct SelectSmem {
+    Cand win[LORB_MAX_POINTS];
+    int hist[256], wsum[32], pick[2];
+    unsigned long long prefix;
+    int need, nwin;
+};
+
+__device__ void lorb_select(const Cand* __restrict__ cand, int n, int npts, int W, int* __restrict__ out_xy,
+                            long long* __restrict__ out_resp, SelectSmem& sm) {
+    int* hist = sm.hist;
+    Cand* win = sm.win;
+    unsigned long long& s_prefix = sm.prefix;
+    int &s_need = sm.need, &s_nwin = sm.nwin;
+    int *s_wsum = sm.wsum, *s_pick = sm.pick;
     const int t = threadIdx.x;
-    const int total = *ncand;
-    if (t == 0 && overflow) *overflow = total > cap ? 1 : 0;
-    const int n = min(total, cap);
     const int want = min(n, npts);
     if (t == 0) {
         s_prefix = 0;
@@ -374,7 +355,7 @@ __global__ void __launch_bounds__(SEL_THREADS) lorb_select(const Cand* __restric
         __syncthreads();
         const unsigned long long prefix = s_prefix;
         for (int i = t; i < n; i += SEL_THREADS) {
-            const unsigned long long u = ukey(cand[i].r);
+            const unsigned long long u = ukey(__ldcg(&cand[i].r));
             if ((u & mask) == prefix) atomicAdd(&hist[(u >> (8 * d)) & 255], 1);
         }
         __syncthreads();
@@ -399,8 +380,8 @@ __global__ void __launch_bounds__(SEL_THREADS) lorb_select(const Cand* __restric
             for (int k = t; k < 256; k += SEL_THREADS) hist[k] = 0;
             __syncthreads();
             for (int i = t; i < n; i += SEL_THREADS) {
-                if (ukey(cand[i].r) != uT) continue;
-                const unsigned ix = (unsigned)cand[i].idx;
+                if (ukey(__ldcg(&cand[i].r)) != uT) continue;
+                const unsigned ix = (unsigned)__ldcg(&cand[i].idx);
                 if ((ix & imask) == prefix) atomicAdd(&hist[(ix >> (8 * d)) & 255], 1);
             }
             __syncthreads();
@@ -418,7 +399,7 @@ __global__ void __launch_bounds__(SEL_THREADS) lorb_select(const Cand* __restric
     }
     // gather the winners: u > uT, or u == uT with index <= iT
     for (int i = t; i < n && want > 0; i += SEL_THREADS) {
-        const Cand c = cand[i];
+        const Cand c{__ldcg(&cand[i].r), __ldcg(&cand[i].idx), 0};
         const unsigned long long u = ukey(c.r);
         if (u > uT || (u == uT && c.idx <= iT)) {
             const int pos = atomicAdd(&s_nwin, 1);
@@ -452,24 +433,155 @@ __global__ void __launch_bounds__(SEL_THREADS) lorb_select(const Cand* __restric
         out_xy[2 * i + 1] = win[i].idx / W;
         out_resp[i] = win[i].r;
     }
-    if (t == 0) *count = want;
 }
 
-// BRIEF: a warp per keypoint, lane l computes bits l, l + 32, ..., packed by ballots
-__global__ void __launch_bounds__(256) lorb_brief(const uint16_t* __restrict__ smooth, int W,
-                                                  const __grid_constant__ LorbPattern pat,
-                                                  const int* __restrict__ xy, const int* __restrict__ count,
-                                                  unsigned* __restrict__ desc) {
-    const int k = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-    if (k >= *count) return;
-    const int x = xy[2 * k], y = xy[2 * k + 1];
+// The candidates in the bins at or above the threshold bin (where the count from the top reaches
+// N) appended to cand2: a superset of the N strongest, typically a small one.  Grid-stride; every
+// block finds the threshold bin from the histogram (a suffix sum over the bins).  The last block to
+// finish (a ticket; no block waits) writes the number of points, clears the counters for the next
+// call, and selects the points itself when cand2 is too crowded to be ranked by counting.
+constexpr int PRUNE_THREADS = 1024, PRUNE_BLOCKS = 64;
+constexpr int RANK_MAX = 8192;  // candidates that lorb_rank_brief ranks by counting
+__global__ void __launch_bounds__(PRUNE_THREADS) lorb_prune(const Cand* __restrict__ cand, LorbCount* __restrict__ cnt, int cap,
+                                                            int npts, Cand* __restrict__ cand2, int W,
+                                                            int* __restrict__ out_xy, long long* __restrict__ out_resp,
+                                                            int* __restrict__ count) {
+    static_assert(PRUNE_THREADS == LORB_BINS && PRUNE_THREADS == SEL_THREADS, "one bin per thread; the block also selects");
+    __shared__ SelectSmem sm;
+    __shared__ int wsum[32];
+    __shared__ int s_b, s_last;
+    const int t = threadIdx.x, lane = t & 31, w = t >> 5;
+    const int n = min(cnt->n, cap), want = min(n, npts);
+    const int* hist = cnt->hist;
+    if (t == 0) s_b = LORB_BINS;  // want == 0: nothing
+    // suffix sums: thread t takes bin 1023 - t and an inclusive prefix sum over t
+    const int b = LORB_BINS - 1 - t;
+    int v = hist[b];
+    for (int off = 1; off < 32; off <<= 1) {
+        const int o = __shfl_up_sync(0xffffffffu, v, off);
+        if (lane >= off) v += o;
+    }
+    if (lane == 31) wsum[w] = v;
+    __syncthreads();
+    if (w == 0) {
+        int x = wsum[lane];
+        for (int off = 1; off < 32; off <<= 1) {
+            const int o = __shfl_up_sync(0xffffffffu, x, off);
+            if (lane >= off) x += o;
+        }
+        wsum[lane] = x;
+    }
+    __syncthreads();
+    const int S = v + (w > 0 ? wsum[w - 1] : 0);  // candidates in bins >= b
+    const int S_above = S - hist[b];             // in bins > b
+    if (want > 0 && S >= want && S_above < want) s_b = b;
+    __syncthreads();
+    const int bT = s_b;
+    for (int i0 = blockIdx.x * PRUNE_THREADS; i0 < n; i0 += gridDim.x * PRUNE_THREADS) {
+        const int i = i0 + t;
+        Cand cv{0, 0, 0};
+        bool keep = false;
+        if (i < n) {
+            cv = cand[i];
+            keep = lorb_bin(cv.r) >= bT;
+        }
+        const unsigned m = __ballot_sync(0xffffffffu, keep);
+        if (!m) continue;
+        int base = 0;
+        const int leader = __ffs(m) - 1;
+        if (lane == leader) base = atomicAdd(&cnt->n2, __popc(m));
+        base = __shfl_sync(0xffffffffu, base, leader);
+        if (keep) cand2[base + __popc(m & ((1u << lane) - 1))] = cv;
+    }
+    __threadfence();
+    __syncthreads();
+    if (t == 0) s_last = atomicAdd(&cnt->done, 1) == (int)gridDim.x - 1;
+    __syncthreads();
+    if (!s_last) return;
+    // every block has read n and the histogram, and appended to cand2
+    cnt->hist[t] = 0;
+    if (t == 0) {
+        *count = want;
+        cnt->n = 0;
+        cnt->done = 0;
+    }
+    const int n2 = __ldcg(&cnt->n2);
+    if (n2 > RANK_MAX) lorb_select(cand2, n2, npts, W, out_xy, out_resp, sm);
+}
+
+// A block per candidate: its rank among the pruned candidates (how many are stronger, or as strong
+// with a lower index) is its place among the points; a candidate ranked below N is dropped.  Then the
+// point's BRIEF bits from a 35 x 35 patch of the frame: gray, the separable [1,4,6,4,1] sums (the
+// unnormalised S, at most 255 * 256), and one comparison per thread, packed by ballots.  A few
+// hundred points need 0.4 MB of patches, so no smoothed map of the image is ever formed; the kernel
+// is a chain of latencies (14 us for 500 points of a 4K view, against 19 us for a one-block selection
+// and 11 us for BRIEF on the map, whose pattern was read from parameter space lane by lane).
+constexpr int RB_P = 35, RB_S = 31;  // patch, positions of S
+__global__ void __launch_bounds__(256) lorb_rank_brief(const uint8_t* __restrict__ frame, long long pitch, int W,
+                                                       const __grid_constant__ LorbPattern pat,
+                                                       const Cand* __restrict__ cand2, const LorbCount* __restrict__ cnt,
+                                                       const int* __restrict__ count, int* __restrict__ xy,
+                                                       long long* __restrict__ resp, unsigned* __restrict__ desc) {
+    __shared__ uint8_t g[RB_P * RB_P];
+    __shared__ uint16_t hs[RB_P][RB_S + 1], S[RB_S][RB_S + 1];
+    __shared__ int s_w[8];
+    const int t = threadIdx.x, lane = t & 31, w = t >> 5;
+    const int n2 = cnt->n2, want = *count;
+    const bool selected = n2 > RANK_MAX;  // lorb_prune has written xy and resp
+    const char4 pr = make_char4(pat.p[t][0], pat.p[t][1], pat.p[t][2], pat.p[t][3]);
+    for (int i = blockIdx.x; i < (selected ? want : n2); i += gridDim.x) {
+        int k = i, x, y;
+        if (selected) {
+            x = xy[2 * k];
+            y = xy[2 * k + 1];
+        } else {
+            const Cand c = cand2[i];
+            int c0 = 0;
+            for (int j = t; j < n2; j += 256) {
+                const Cand o = cand2[j];
+                c0 += o.r > c.r || (o.r == c.r && o.idx < c.idx);
+            }
+            c0 = __reduce_add_sync(0xffffffffu, c0);
+            if (lane == 0) s_w[w] = c0;
+            __syncthreads();
+            k = 0;
 #pragma unroll
-    for (int j = 0; j < 8; ++j) {
-        const int b = 32 * j + lane;
-        const int sp = smooth[(long long)(y + pat.p[b][1]) * W + x + pat.p[b][0]];
-        const int sq = smooth[(long long)(y + pat.p[b][3]) * W + x + pat.p[b][2]];  // uint16 -> int
-        const unsigned bits = __ballot_sync(0xffffffffu, sp > sq);
-        if (lane == 0) desc[8 * k + j] = bits;  // bit b of the descriptor: byte b/8, bit b%8 (little endian)
+            for (int q = 0; q < 8; ++q) k += s_w[q];
+            x = c.idx % W;
+            y = c.idx / W;
+            if (t == 0 && k < want) {
+                xy[2 * k] = x;
+                xy[2 * k + 1] = y;
+                resp[k] = c.r;
+            }
+        }
+        if (k < want) {  // the whole block
+            const uint8_t* p0 = frame + (long long)(y - 17) * pitch + 3LL * (x - 17);  // points keep 18 px from the border
+#pragma unroll
+            for (int q0 = 0; q0 < RB_P * RB_P; q0 += 256) {
+                const int q = q0 + t;
+                if (q < RB_P * RB_P) {
+                    const int r = q / RB_P;
+                    const uint8_t* p = p0 + (long long)r * pitch + 3 * (q - r * RB_P);
+                    g[q] = (uint8_t)gray_of(__ldg(p), __ldg(p + 1), __ldg(p + 2));
+                }
+            }
+            __syncthreads();
+            for (int q = t; q < RB_P * RB_S; q += 256) {
+                const int r = q / RB_S, c = q - r * RB_S;
+                const uint8_t* p = g + r * RB_P + c;
+                hs[r][c] = (uint16_t)(p[0] + 4 * p[1] + 6 * p[2] + 4 * p[3] + p[4]);
+            }
+            __syncthreads();
+            for (int q = t; q < RB_S * RB_S; q += 256) {
+                const int r = q / RB_S, c = q - r * RB_S;
+                S[r][c] = (uint16_t)(hs[r][c] + 4 * hs[r + 1][c] + 6 * hs[r + 2][c] + 4 * hs[r + 3][c] + hs[r + 4][c]);
+            }
+            __syncthreads();
+            const unsigned bits = __ballot_sync(0xffffffffu, S[15 + pr.y][15 + pr.x] > S[15 + pr.w][15 + pr.z]);
+            if (lane == 0) desc[8 * k + w] = bits;  // bit b of the descriptor: byte b/8, bit b%8 (little endian)
+        }
+        __syncthreads();
     }
 }
 
@@ -478,22 +590,16 @@ __global__ void __launch_bounds__(256) lorb_brief(const uint16_t* __restrict__ s
 struct stitch_lorb {
     int device = 0;
     int max_w = 0, max_h = 0, max_points = 0, cap = 0;
-    uint8_t* gray = nullptr;
-    uint16_t* smooth = nullptr;
-    long long* resp = nullptr;
     Cand* cand = nullptr;
     Cand* cand2 = nullptr;  // the pruned candidates
-    int* ncand = nullptr;   // [0] survivors, [1] overflow flag, [2] pruned count, then the bin histogram
+    LorbCount* cnt = nullptr;
 };
 
 static void lorb_free(stitch_lorb* c) {
     if (!c) return;
-    cudaFree(c->gray);
-    cudaFree(c->smooth);
-    cudaFree(c->resp);
     cudaFree(c->cand);
     cudaFree(c->cand2);
-    cudaFree(c->ncand);
+    cudaFree(c->cnt);
     delete c;
 }
 
@@ -519,18 +625,15 @@ extern "C" stitch_status stitch_lorb_create(int32_t max_width, int32_t max_heigh
     c->max_w = max_width;
     c->max_h = max_height;
     c->max_points = max_points;
-    const size_t N = (size_t)max_width * max_height;
     c->cap = (int)(((size_t)max_width + 1) / 2 * (((size_t)max_height + 1) / 2));  // NMS survivors are never adjacent
     stitch_status st = STITCH_OK;
-    if (cudaMalloc(&c->gray, N) != cudaSuccess || cudaMalloc(&c->smooth, N * sizeof(uint16_t)) != cudaSuccess ||
-        cudaMalloc(&c->resp, N * sizeof(long long)) != cudaSuccess ||
-        cudaMalloc(&c->cand, (size_t)c->cap * sizeof(Cand)) != cudaSuccess ||
+    if (cudaMalloc(&c->cand, (size_t)c->cap * sizeof(Cand)) != cudaSuccess ||
         cudaMalloc(&c->cand2, (size_t)c->cap * sizeof(Cand)) != cudaSuccess ||
-        cudaMalloc(&c->ncand, (4 + LORB_BINS) * sizeof(int)) != cudaSuccess) {
+        cudaMalloc(&c->cnt, sizeof(LorbCount)) != cudaSuccess) {
         cudaGetLastError();
         st = STITCH_ENOMEM;
     }
-    if (st == STITCH_OK && cudaMemset(c->ncand, 0, (4 + LORB_BINS) * sizeof(int)) != cudaSuccess) st = STITCH_ECUDA;
+    if (st == STITCH_OK && cudaMemset(c->cnt, 0, sizeof(LorbCount)) != cudaSuccess) st = STITCH_ECUDA;
     if (prev >= 0) cudaSetDevice(prev);
     if (st != STITCH_OK) {
         lorb_free(c);
@@ -591,26 +694,21 @@ extern "C" stitch_status stitch_lorb_detect(stitch_lorb* c, const uint8_t* frame
     auto ok = [&](cudaError_t e) {
         if (e != cudaSuccess && st == STITCH_OK) st = STITCH_ECUDA;
     };
-    int* hist = c->ncand + 4;
-    ok(cudaMemsetAsync(c->ncand, 0, (4 + LORB_BINS) * sizeof(int), s));
     if (ar.n > 0) {
-        // gray and S on the candidates' box grown by the BRIEF reach (15 + 2) and the FAST / tensor
-        // halo, inside the image
-        const int mx0 = std::max(bx0 - 17, 0) & ~3, my0 = std::max(by0 - 17, 0);  // x0 on a 4-pixel group
-        const int mx1 = std::min(bx1 + 17, (int)width), my1 = std::min(by1 + 17, (int)height);
-        lorb_maps<<<dim3((mx1 - mx0 + 31) / 32, (my1 - my0 + 15) / 16), 256, 0, s>>>(
-            frame, pitch, width, height, mx0, my0, mx1, my1, c->gray, c->smooth);
-        lorb_response<<<dim3((bx1 - bx0 + LT_X - 1) / LT_X, (by1 - by0 + LT_Y - 1) / LT_Y), 256, 0, s>>>(
-            c->gray, width, bx0, by0, bx1, by1, ar, params->fast_t, (long long)params->harris_t, c->resp);
-        lorb_nms<<<dim3((bx1 - bx0 + 31) / 32, (by1 - by0 + 7) / 8), 256, 0, s>>>(c->resp, width, bx0, by0, bx1, by1,
-                                                                               c->cand, c->ncand, c->cap, hist);
+        // tiles over the candidates' box, owned pixels starting at a column 1 modulo 4
+        const int ox = 1 + ((bx0 - 1) & ~3), oy = by0;
+        lorb_detect<<<dim3((bx1 - ox + DT_OX - 1) / DT_OX, (by1 - oy + DT_OY - 1) / DT_OY), 256, 0, s>>>(
+            frame, pitch, width, height, ox, oy, ar, std::min(params->fast_t, 255) + 256, (long long)params->harris_t,
+            c->cand, &c->cnt->n, c->cap, c->cnt->hist, &c->cnt->n2);
+    } else {
+        ok(cudaMemsetAsync(&c->cnt->n2, 0, sizeof(int), s));
     }
-    lorb_prune<<<PRUNE_BLOCKS, PRUNE_THREADS, 0, s>>>(c->cand, c->ncand, c->cap, params->max_points, hist, c->cand2,
-                                                      c->ncand + 2, c->ncand + 1);
-    lorb_select<<<1, SEL_THREADS, 0, s>>>(c->cand2, c->ncand + 2, c->cap, params->max_points, width, xy,
-                                          reinterpret_cast<long long*>(resp), count, nullptr);
-    lorb_brief<<<(params->max_points + 7) / 8 + 1, 256, 0, s>>>(c->smooth, width, pat, xy, count,
-                                                                reinterpret_cast<unsigned*>(desc));
+    lorb_prune<<<PRUNE_BLOCKS, PRUNE_THREADS, 0, s>>>(c->cand, c->cnt, c->cap, params->max_points, c->cand2, width, xy,
+                                                      reinterpret_cast<long long*>(resp), count);
+    // the pruned candidates are a few more than the points: a block each, or a few passes
+    lorb_rank_brief<<<std::min(2 * params->max_points + 64, 1216), 256, 0, s>>>(
+        frame, pitch, width, pat, c->cand2, c->cnt, count, xy, reinterpret_cast<long long*>(resp),
+        reinterpret_cast<unsigned*>(desc));
     ok(cudaGetLastError());
     if (prev >= 0 && prev != c->device) cudaSetDevice(prev);
     return st;
