@@ -14,9 +14,12 @@
 // Sums run in local coordinates x' = x - c_i (c_i a fixed point of camera i's footprint) so the
 // single-precision terms stay small: with S(f) = sum f, d/da11 = S(gu x'/w) + c_x S(gu/w) etc.,
 // applied in double precision at the end.  Per pixel and camera the 10 terms are reduced by warp
-// shuffles and a block tree to one partial per (tile, camera slot); a second kernel sums each
+// shuffles and a block tree to one partial per (tile, camera slot); a last kernel sums each
 // camera's partials with compensated (TwoSum) single-precision arithmetic and applies the chain
 // rule to canvas coordinates in double precision.
+//
+// Launches: k_backward_maps (every slot's tile map, in double precision), k_backward for the tiles of
+// at most 2 and at most 4 candidate cameras, k_backward_many for the others, k_backward_final.
 #include "stitch_internal.cuh"
 
 namespace {
@@ -30,23 +33,40 @@ constexpr int BW_MARGIN = 64;                        // px: how far params may m
 
 struct BwTile {
     int x0, y0, first, count;  // canvas origin, candidate cameras (range in the camera list)
+    int id;                    // position of the tile's loss partial
 };
 
-// One camera's sample at a pixel: bilinear value and its derivatives (before gain, in [0,1]
-// units), source position and w.
+// A (tile, candidate camera) slot: the camera's map anchored in the tile, from the call's parameters.
+struct __align__(16) BwMap {
+    TileMap tm;
+    int ax, ay;   // anchor: dx, dy are taken from it
+    float gain;
+    int cam, W, H;
+    int cx, cy;   // local origin
+    int pos;      // position of the slot's partials: the slots of a camera in a row, in tile order
+};
+static_assert(sizeof(BwMap) == 80, "read as five 16-byte words");
+
+// One camera's sample at a pixel: bilinear value and its derivatives (before gain, in [0,1] units).
 struct GSample {
     float b[3], bu[3], bv[3];
-    float u, v, w;
-    bool valid;
 };
 
-__device__ __forceinline__ void gsample(const uint8_t* __restrict__ px, long long pitch, int W, int H,
-                                        const TileMap& t, float dx, float dy, GSample& s) {
-    const Pos p = map_pos(t, (float)t.U0, (float)t.V0, dx, dy);
-    s.u = p.u;
-    s.v = p.v;
-    s.w = p.den;
-    s.valid = (p.den > 0.f) & (p.u >= -0.5f) & (p.u < (float)W - 0.5f) & (p.v >= -0.5f) & (p.v < (float)H - 0.5f);
+// The source position lies in the camera's image (and in front of the camera).
+__device__ __forceinline__ bool gvalid(const Pos& p, int W, int H) {
+    return (p.den > 0.f) & (p.u >= -0.5f) & (p.u < (float)W - 0.5f) & (p.v >= -0.5f) & (p.v < (float)H - 0.5f);
+}
+
+// Byte j of w as a float (exact).
+__device__ __forceinline__ float byte_f(unsigned w, unsigned j) {
+    return __uint_as_float(__byte_perm(w, 0x4B000000u, 0x7440u | j)) - 8388608.0f;
+}
+
+// The sample at p.  Two neighbouring RGB texels are 6 bytes at any offset: where base and pitch allow
+// it and the 12 bytes from the first one's word on lie in the row, they are two or three aligned
+// 32-bit loads per row and a funnel shift instead of six byte loads.
+__device__ __forceinline__ void gsample(const uint8_t* __restrict__ px, long long pitch, int W, int H, const Pos& p,
+                                        bool words, GSample& s) {
     int i0, j0;
     float fx, fy;
     bool cu = false, cv = false;
@@ -57,15 +77,36 @@ __device__ __forceinline__ void gsample(const uint8_t* __restrict__ px, long lon
     else if (p.iv >= H - 1) { j0 = H - 1; fy = 0.f; cv = true; }
     else { j0 = p.iv; fy = p.fv; }
     // an exact integer u = W-1 sits on the last texel: one-sided derivative there is 0 as well
-    const int di = (i0 + 1 < W) ? 3 : 0;
     const long long dj = (j0 + 1 < H) ? pitch : 0;
     const uint8_t* a = px + (long long)j0 * pitch + 3 * i0;
     const uint8_t* b = a + dj;
+    unsigned ta, tb, ua, ub;  // the first four bytes (R G B R) and the last two (G B) of both rows
+    const int off = (3 * i0) & 3;
+    if (words && 3 * i0 - off + 12 <= 3 * W) {
+        const unsigned* wa = reinterpret_cast<const unsigned*>(a - off);
+        const unsigned* wb = reinterpret_cast<const unsigned*>(b - off);
+        const unsigned a0 = __ldg(wa), a1 = __ldg(wa + 1), b0 = __ldg(wb), b1 = __ldg(wb + 1);
+        unsigned a2 = 0u, b2 = 0u;
+        if (off == 3) {
+            a2 = __ldg(wa + 2);
+            b2 = __ldg(wb + 2);
+        }
+        ta = __funnelshift_r(a0, a1, 8 * off);
+        ua = __funnelshift_r(a1, a2, 8 * off);
+        tb = __funnelshift_r(b0, b1, 8 * off);
+        ub = __funnelshift_r(b1, b2, 8 * off);
+    } else {
+        const int di = (i0 + 1 < W) ? 3 : 0;
+        ta = (unsigned)__ldg(a) | (unsigned)__ldg(a + 1) << 8 | (unsigned)__ldg(a + 2) << 16 | (unsigned)__ldg(a + di) << 24;
+        ua = (unsigned)__ldg(a + di + 1) | (unsigned)__ldg(a + di + 2) << 8;
+        tb = (unsigned)__ldg(b) | (unsigned)__ldg(b + 1) << 8 | (unsigned)__ldg(b + 2) << 16 | (unsigned)__ldg(b + di) << 24;
+        ub = (unsigned)__ldg(b + di + 1) | (unsigned)__ldg(b + di + 2) << 8;
+    }
     const float k255 = 1.0f / 255.0f;
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-        const float p00 = u8_to_f(__ldg(a + c)), p01 = u8_to_f(__ldg(a + di + c));
-        const float p10 = u8_to_f(__ldg(b + c)), p11 = u8_to_f(__ldg(b + di + c));
+        const float p00 = byte_f(ta, c), p01 = c == 0 ? byte_f(ta, 3) : byte_f(ua, c - 1);
+        const float p10 = byte_f(tb, c), p11 = c == 0 ? byte_f(tb, 3) : byte_f(ub, c - 1);
         const float top = fmaf(fx, p01 - p00, p00), bot = fmaf(fx, p11 - p10, p10);
         s.b[c] = fmaf(fy, bot - top, top) * k255;
         s.bu[c] = cu ? 0.f : fmaf(fy, (p11 - p10) - (p01 - p00), p01 - p00) * k255;
@@ -79,61 +120,218 @@ __device__ __forceinline__ float warp_sum(float v) {
     return v;
 }
 
-// Canvas->camera parameters of one camera as doubles: a11..a32, gain (a33 comes from the rig).
-struct BwCam {
-    double a[9];  // a11 a12 a13 a21 a22 a23 a31 a32 a33
-    float gain;
-    int cx, cy;   // local origin
-    int W, H;
+// The tile map of every slot, one thread each.  FP64 runs at two lanes per clock and SM whether a
+// warp has one lane active or 32, so this work in the first threads of every tile's block (60 double
+// operations in 2 to 4 lanes) cost the 8150 tiles of 4 x 1080p about 50 us of the FP64 pipe; with full warps
+// it is 7 us for all of them.
+__global__ void __launch_bounds__(64) k_backward_maps(const CamDev* __restrict__ cams, const double* __restrict__ params,
+                                                      const int4* __restrict__ slots, int nslots,
+                                                      const int* __restrict__ centers, int canvas_w, int canvas_h,
+                                                      BwMap* __restrict__ maps) {
+    const int q = blockIdx.x * 64 + threadIdx.x;
+    if (q >= nslots) return;
+    const int4 sl = slots[q];  // tile origin, camera, position of the partials
+    const int c = sl.z;
+    const double* p = params + 9 * c;
+    const double A[9] = {p[0], p[1], p[2], p[3], p[4], p[5], p[6], p[7], cams[c].A[8]};
+    // anchor at the tile origin clamped into the canvas; w > 0 there for every candidate is
+    // not guaranteed, so anchor where w is largest among the tile corners
+    BwMap m;
+    m.ax = sl.x;
+    m.ay = sl.y;
+    double best = -1e300;
+    for (int k = 0; k < 4; ++k) {
+        const int x = min(sl.x + (k & 1) * (BW_TX - 1), canvas_w - 1);
+        const int y = min(sl.y + (k >> 1) * (BW_TY - 1), canvas_h - 1);
+        const double w = A[6] * x + A[7] * y + A[8];
+        if (w > best) {
+            best = w;
+            m.ax = x;
+            m.ay = y;
+        }
+    }
+    m.tm = make_tile_map(A, m.ax, m.ay);
+    m.gain = (float)p[8];
+    m.cam = c;
+    m.W = cams[c].W;
+    m.H = cams[c].H;
+    m.cx = centers[2 * c];
+    m.cy = centers[2 * c + 1];
+    m.pos = sl.w;
+    maps[q] = m;
+}
+
+// The 10 gradient terms of a camera's sample at a pixel added to acc; r is the residual of the pixel.
+__device__ __forceinline__ void grad_terms(const GSample& s, const Pos& p, const float r[3], float g, float xl, float yl,
+                                           float acc[BW_NV]) {
+    const float gu = 2.f * g * (r[0] * s.bu[0] + r[1] * s.bu[1] + r[2] * s.bu[2]);
+    const float gv = 2.f * g * (r[0] * s.bv[0] + r[1] * s.bv[1] + r[2] * s.bv[2]);
+    const float gg = 2.f * (r[0] * s.b[0] + r[1] * s.b[1] + r[2] * s.b[2]);
+    const float iw = 1.0f / p.den;
+    const float q = -(gu * p.u + gv * p.v) * iw;
+    const float guw = gu * iw, gvw = gv * iw;
+    acc[0] = fmaf(guw, xl, acc[0]);
+    acc[1] = fmaf(guw, yl, acc[1]);
+    acc[2] += guw;
+    acc[3] = fmaf(gvw, xl, acc[3]);
+    acc[4] = fmaf(gvw, yl, acc[4]);
+    acc[5] += gvw;
+    acc[6] = fmaf(q, xl, acc[6]);
+    acc[7] = fmaf(q, yl, acc[7]);
+    acc[8] += q;
+    acc[9] += gg;
+}
+
+// Sums over the warp of M values per lane, M halved at each step: in step xor k a lane keeps one half
+// of the values and gets its partner's sums of them for its own of the other half.  Every sum adds
+// the same pairs as warp_sum (the lanes 16, 8, 4, 2, 1 apart), so the results are bit-identical, with
+// about M instead of 5 M shuffles.  Value index(i) of lane l's results v[0 .. left) is sum index(i).
+template <int M, int K, int BASE = 0>
+struct WarpSums {
+    static constexpr int HALF = (M + 1) / 2;
+    static constexpr int LEFT = WarpSums<HALF, K / 2>::LEFT;
+    __device__ __forceinline__ static void run(float* v, int lane) {
+        const bool up = lane & K;
+#pragma unroll
+        for (int i = 0; i < HALF; ++i) {
+            const float hi = i + HALF < M ? v[i + HALF] : 0.f;
+            const float keep = up ? hi : v[i], send = up ? v[i] : hi;
+            v[i] = keep + __shfl_xor_sync(0xffffffffu, send, K);
+        }
+        WarpSums<HALF, K / 2>::run(v, lane);
+    }
+    // which of the M sums lane's result i is, or -1
+    __device__ __forceinline__ static int index(int i, int lane) {
+        const int q = WarpSums<HALF, K / 2>::index(i, lane);
+        if (q < 0) return -1;
+        const int r = q + (lane & K ? HALF : 0);
+        return r < M ? r : -1;
+    }
+};
+template <int M, int BASE>
+struct WarpSums<M, 0, BASE> {
+    static constexpr int LEFT = M;
+    __device__ __forceinline__ static void run(float*, int) {}
+    __device__ __forceinline__ static int index(int i, int) { return i; }
 };
 
-__global__ void __launch_bounds__(BW_THREADS) k_backward(const CamDev* __restrict__ cams, FramePtrs fp,
-                                                          const double* __restrict__ params,
-                                                          const BwTile* __restrict__ tiles,
-                                                          const int* __restrict__ camlist,
-                                                          const int* __restrict__ centers, int canvas_w,
-                                                          int canvas_h, float* __restrict__ partials,
-                                                          float* __restrict__ loss_partials) {
-    __shared__ TileMap tm[MAXC];
-    __shared__ int cw[MAXC], chh[MAXC];
-    __shared__ float cgain[MAXC];
-    __shared__ int ccx[MAXC], ccy[MAXC], cid[MAXC];
-    __shared__ float red[BW_THREADS / 32][BW_SLOTS * BW_NV + 1];
+// A tile with at most N candidate cameras: validity from the positions first, then one sample per
+// valid camera of the pixels that at least two see, kept in registers for both the sum and the
+// gradient.  Bound by instruction issue: 57 + 80 us for the 4727 + 3423 tiles of 4 x 1080p, against 227 us when
+// every candidate was sampled twice at every pixel, from byte loads, with 5 shuffles for each of 40 sums.
+template <int N>
+__global__ void __launch_bounds__(BW_THREADS, N == 2 ? 4 : 2) k_backward(const FramePtrs fp, const BwMap* __restrict__ maps,
+                                                                        const BwTile* __restrict__ tiles, int canvas_w,
+                                                                        int canvas_h, float* __restrict__ partials, int nslots,
+                                                                        float* __restrict__ loss_partials) {
+    __shared__ __align__(16) BwMap m[N];
+    __shared__ float red[BW_THREADS / 32][N * BW_NV + 1];
+    const BwTile tl = tiles[blockIdx.x];
+    const int n = tl.count, t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    if (t < 5 * n) reinterpret_cast<int4*>(m)[t] = reinterpret_cast<const int4*>(maps + tl.first)[t];
+    __syncthreads();
+    float loss = 0.f;
+    float acc[N * BW_NV];
+#pragma unroll
+    for (int v = 0; v < N * BW_NV; ++v) acc[v] = 0.f;
+    bool some = false;
+#pragma unroll 1
+    for (int k = 0; k < BW_PPT; ++k) {
+        const int q = t + k * BW_THREADS;
+        const int x = tl.x0 + q % BW_TX, y = tl.y0 + q / BW_TX;
+        Pos p[N];
+        bool ok[N];
+        int kv = 0;
+#pragma unroll
+        for (int a = 0; a < N; ++a) {
+            ok[a] = false;
+            if (a < n) {
+                p[a] = map_pos(m[a].tm, (float)m[a].tm.U0, (float)m[a].tm.V0, (float)(x - m[a].ax), (float)(y - m[a].ay));
+                ok[a] = gvalid(p[a], m[a].W, m[a].H);
+            }
+            kv += ok[a];
+        }
+        if (kv < 2 || x >= canvas_w || y >= canvas_h) continue;
+        some = true;
+        GSample s[N];
+        float S[3] = {0.f, 0.f, 0.f};
+#pragma unroll
+        for (int a = 0; a < N; ++a) {
+            if (!ok[a]) continue;
+            const int c = m[a].cam;
+            const uint8_t* px = fp.p[c];
+            const long long pitch = fp.pitch[c];
+            gsample(px, pitch, m[a].W, m[a].H, p[a], ((reinterpret_cast<uintptr_t>(px) | (uintptr_t)pitch) & 3) == 0, s[a]);
+#pragma unroll
+            for (int ch = 0; ch < 3; ++ch) S[ch] = fmaf(m[a].gain, s[a].b[ch], S[ch]);
+        }
+#pragma unroll
+        for (int a = 0; a < N; ++a) {
+            if (!ok[a]) continue;
+            const float g = m[a].gain;
+            float r[3];
+#pragma unroll
+            for (int ch = 0; ch < 3; ++ch) r[ch] = (float)kv * (g * s[a].b[ch]) - S[ch];
+            // with the mean m = S/k, sum_{i<j} |I_i - I_j|^2 = k sum_i |I_i - m|^2
+            // = sum_i |r_i|^2 / k; r_i is small and accurate, so no cancellation
+            loss += (r[0] * r[0] + r[1] * r[1] + r[2] * r[2]) / (float)kv;
+            grad_terms(s[a], p[a], r, g, (float)(x - m[a].cx), (float)(y - m[a].cy), acc + a * BW_NV);
+        }
+    }
+    // block reduction: warp sums, then a tree over warps; a tile (or warp) that no two cameras see has
+    // only zeros
+    if (!__syncthreads_or(some)) {
+        if (t < n * BW_NV) partials[(long long)(t % BW_NV) * nslots + m[t / BW_NV].pos] = 0.f;
+        if (t == 0) loss_partials[tl.id] = 0.f;
+        return;
+    }
+    using Sums = WarpSums<N * BW_NV, 16>;
+    if (__any_sync(0xffffffffu, some)) {
+        Sums::run(acc, lane);
+#pragma unroll
+        for (int i = 0; i < Sums::LEFT; ++i) {
+            const int v = Sums::index(i, lane);
+            if (v >= 0) red[warp][v] = acc[i];
+        }
+        const float lw = warp_sum(loss);
+        if (lane == 0) red[warp][N * BW_NV] = lw;
+    } else {
+        for (int v = lane; v <= N * BW_NV; v += 32) red[warp][v] = 0.f;
+    }
+    __syncthreads();
+    if (t <= N * BW_NV) {
+        float sum = 0.f;
+#pragma unroll
+        for (int w = 0; w < BW_THREADS / 32; ++w) sum += red[w][t];
+        if (t == N * BW_NV) loss_partials[tl.id] = sum;
+        else if (t < n * BW_NV) partials[(long long)(t % BW_NV) * nslots + m[t / BW_NV].pos] = sum;
+    }
+}
 
+// Tiles with more candidates (up to MAXC), in groups of BW_SLOTS cameras: samples are taken again for
+// the gradient, as registers do not hold them all.
+__global__ void __launch_bounds__(BW_THREADS) k_backward_many(const FramePtrs fp, const BwMap* __restrict__ maps,
+                                                              const BwTile* __restrict__ tiles, int canvas_w, int canvas_h,
+                                                              float* __restrict__ partials, int nslots,
+                                                              float* __restrict__ loss_partials) {
+    __shared__ __align__(16) BwMap m[MAXC];
+    __shared__ float red[BW_THREADS / 32][BW_SLOTS * BW_NV + 1];
     const BwTile tl = tiles[blockIdx.x];
     const int n = tl.count;  // <= MAXC
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
-    if (t < n) {
-        const int c = camlist[tl.first + t];
-        const double* p = params + 9 * c;
-        double A[9] = {p[0], p[1], p[2], p[3], p[4], p[5], p[6], p[7], cams[c].A[8]};
-        // anchor at the tile origin clamped into the canvas; w > 0 there for every candidate is
-        // not guaranteed, so anchor where w is largest among the tile corners
-        int ax = tl.x0, ay = tl.y0;
-        double best = -1e300;
-        for (int k = 0; k < 4; ++k) {
-            const int x = min(tl.x0 + (k & 1) * (BW_TX - 1), canvas_w - 1);
-            const int y = min(tl.y0 + (k >> 1) * (BW_TY - 1), canvas_h - 1);
-            const double w = A[6] * x + A[7] * y + A[8];
-            if (w > best) {
-                best = w;
-                ax = x;
-                ay = y;
-            }
-        }
-        tm[t] = make_tile_map(A, ax, ay);
-        // store the anchor in the tile map's frame: dx, dy are taken from (ax, ay)
-        ccx[t] = ax;
-        ccy[t] = ay;
-        cid[t] = c;
-        cw[t] = cams[c].W;
-        chh[t] = cams[c].H;
-        cgain[t] = (float)p[8];
-    }
+    static_assert(5 * MAXC <= BW_THREADS, "one 16-byte word per thread");
+    if (t < 5 * n) reinterpret_cast<int4*>(m)[t] = reinterpret_cast<const int4*>(maps + tl.first)[t];
     __syncthreads();
-
+    auto pos_of = [&](int a, int x, int y) {
+        return map_pos(m[a].tm, (float)m[a].tm.U0, (float)m[a].tm.V0, (float)(x - m[a].ax), (float)(y - m[a].ay));
+    };
+    auto sample = [&](int a, const Pos& p, GSample& s) {
+        const uint8_t* px = fp.p[m[a].cam];
+        const long long pitch = fp.pitch[m[a].cam];
+        gsample(px, pitch, m[a].W, m[a].H, p, ((reinterpret_cast<uintptr_t>(px) | (uintptr_t)pitch) & 3) == 0, s);
+    };
     float loss = 0.f;
-    for (int g0 = 0; g0 < max(n, 1); g0 += BW_SLOTS) {
+    for (int g0 = 0; g0 < n; g0 += BW_SLOTS) {
         float acc[BW_SLOTS][BW_NV];
 #pragma unroll
         for (int s = 0; s < BW_SLOTS; ++s)
@@ -148,71 +346,49 @@ __global__ void __launch_bounds__(BW_THREADS) k_backward(const CamDev* __restric
             int kv = 0;
             float S[3] = {0.f, 0.f, 0.f};
             for (int a = 0; a < n; ++a) {
+                const Pos p = pos_of(a, x, y);
+                if (!gvalid(p, m[a].W, m[a].H)) continue;
                 GSample s;
-                gsample(fp.p[cid[a]], fp.pitch[cid[a]], cw[a], chh[a], tm[a], (float)(x - ccx[a]),
-                        (float)(y - ccy[a]), s);
-                if (!s.valid) continue;
+                sample(a, p, s);
                 ++kv;
 #pragma unroll
-                for (int c = 0; c < 3; ++c) S[c] = fmaf(cgain[a], s.b[c], S[c]);
+                for (int c = 0; c < 3; ++c) S[c] = fmaf(m[a].gain, s.b[c], S[c]);
             }
             if (kv < 2) continue;
             // pass 2: loss (first group only) and gradient terms of this group's cameras
             for (int a = 0; a < n; ++a) {
+                const int slot = a - g0;
+                if (g0 > 0 && (slot < 0 || slot >= BW_SLOTS)) continue;
+                const Pos p = pos_of(a, x, y);
+                if (!gvalid(p, m[a].W, m[a].H)) continue;
                 GSample s;
-                gsample(fp.p[cid[a]], fp.pitch[cid[a]], cw[a], chh[a], tm[a], (float)(x - ccx[a]),
-                        (float)(y - ccy[a]), s);
-                if (!s.valid) continue;
-                const float g = cgain[a];
+                sample(a, p, s);
+                const float g = m[a].gain;
                 float r[3];
 #pragma unroll
                 for (int c = 0; c < 3; ++c) r[c] = (float)kv * (g * s.b[c]) - S[c];
-                if (g0 == 0) {
-                    // with the mean m = S/k, sum_{i<j} |I_i - I_j|^2 = k sum_i |I_i - m|^2
-                    // = sum_i |r_i|^2 / k; r_i is small and accurate, so no cancellation
-                    loss += (r[0] * r[0] + r[1] * r[1] + r[2] * r[2]) / (float)kv;
-                }
-                const int slot = a - g0;
-                if (slot < 0 || slot >= BW_SLOTS) continue;
-                const float gu = 2.f * g * (r[0] * s.bu[0] + r[1] * s.bu[1] + r[2] * s.bu[2]);
-                const float gv = 2.f * g * (r[0] * s.bv[0] + r[1] * s.bv[1] + r[2] * s.bv[2]);
-                const float gg = 2.f * (r[0] * s.b[0] + r[1] * s.b[1] + r[2] * s.b[2]);
-                const float iw = 1.0f / s.w;
-                const float xl = (float)(x - centers[2 * cid[a]]), yl = (float)(y - centers[2 * cid[a] + 1]);
-                const float q = -(gu * s.u + gv * s.v) * iw;
-                const float guw = gu * iw, gvw = gv * iw;
+                if (g0 == 0) loss += (r[0] * r[0] + r[1] * r[1] + r[2] * r[2]) / (float)kv;
                 // unrolled slot selection keeps the accumulators in registers
 #pragma unroll
-                for (int ss = 0; ss < BW_SLOTS; ++ss) {
-                    if (ss != slot) continue;
-                    acc[ss][0] = fmaf(guw, xl, acc[ss][0]);
-                    acc[ss][1] = fmaf(guw, yl, acc[ss][1]);
-                    acc[ss][2] += guw;
-                    acc[ss][3] = fmaf(gvw, xl, acc[ss][3]);
-                    acc[ss][4] = fmaf(gvw, yl, acc[ss][4]);
-                    acc[ss][5] += gvw;
-                    acc[ss][6] = fmaf(q, xl, acc[ss][6]);
-                    acc[ss][7] = fmaf(q, yl, acc[ss][7]);
-                    acc[ss][8] += q;
-                    acc[ss][9] += gg;
-                }
+                for (int ss = 0; ss < BW_SLOTS; ++ss)
+                    if (ss == slot) grad_terms(s, p, r, g, (float)(x - m[a].cx), (float)(y - m[a].cy), acc[ss]);
             }
         }
-        // block reduction of this group's slots: warp shuffles, then a tree over warps
+        // block reduction of this group's slots: warp sums, then a tree over warps
+        using Sums = WarpSums<BW_SLOTS * BW_NV, 16>;
+        Sums::run(&acc[0][0], lane);
 #pragma unroll
-        for (int s = 0; s < BW_SLOTS; ++s)
-#pragma unroll
-            for (int v = 0; v < BW_NV; ++v) {
-                const float w = warp_sum(acc[s][v]);
-                if (lane == 0) red[warp][s * BW_NV + v] = w;
-            }
+        for (int i = 0; i < Sums::LEFT; ++i) {
+            const int v = Sums::index(i, lane);
+            if (v >= 0) red[warp][v] = acc[0][i];
+        }
         __syncthreads();
         if (t < BW_SLOTS * BW_NV) {
             float sum = 0.f;
 #pragma unroll
             for (int w = 0; w < BW_THREADS / 32; ++w) sum += red[w][t];
-            const int s = t / BW_NV, v = t - s * BW_NV;
-            if (g0 + s < n) partials[(long long)(tl.first + g0 + s) * BW_NV + v] = sum;
+            const int a = g0 + t / BW_NV;
+            if (a < n) partials[(long long)(t % BW_NV) * nslots + m[a].pos] = sum;
         }
         __syncthreads();
     }
@@ -222,7 +398,7 @@ __global__ void __launch_bounds__(BW_THREADS) k_backward(const CamDev* __restric
     if (t == 0) {
         float sum = 0.f;
         for (int w = 0; w < BW_THREADS / 32; ++w) sum += red[w][BW_SLOTS * BW_NV];
-        loss_partials[blockIdx.x] = sum;
+        loss_partials[tl.id] = sum;
     }
 }
 
@@ -233,118 +409,101 @@ __device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
     e = (a - (s - bb)) + (b - bb);
 }
 
-// Compensated sum of (sum, compensation) pairs across a block.
-__device__ __forceinline__ void block_csum(float& s, float& c, float* sh_s, float* sh_c) {
-    sh_s[threadIdx.x] = s;
-    sh_c[threadIdx.x] = c;
-    __syncthreads();
-    for (int stride = blockDim.x / 2; stride > 0; stride >>= 1) {
-        if ((int)threadIdx.x < stride) {
-            float ns, ne;
-            two_sum(sh_s[threadIdx.x], sh_s[threadIdx.x + stride], ns, ne);
-            sh_s[threadIdx.x] = ns;
-            sh_c[threadIdx.x] += sh_c[threadIdx.x + stride] + ne;
-        }
-        __syncthreads();
-    }
-    s = sh_s[0];
-    c = sh_c[0];
-}
-
-// One block per camera (blockIdx.x < ncam) and one for the loss (blockIdx.x == ncam).
-__global__ void __launch_bounds__(256) k_backward_final(const CamDev* __restrict__ cams, int ncam,
-                                                         const float* __restrict__ partials,
-                                                         const float* __restrict__ loss_partials, int ntiles,
-                                                         const int* __restrict__ cam_slots,
-                                                         const int* __restrict__ cam_slot_start,
-                                                         const int* __restrict__ centers, double* __restrict__ loss,
-                                                         double* __restrict__ grad) {
-    __shared__ float sh_s[256], sh_c[256];
-    const int b = blockIdx.x;
-    if (b == ncam) {
-        float s = 0.f, c = 0.f;
-        for (int k = threadIdx.x; k < ntiles; k += blockDim.x) {
-            float ns, ne;
-            two_sum(s, loss_partials[k], ns, ne);
-            s = ns;
-            c += ne;
-        }
-        block_csum(s, c, sh_s, sh_c);
-        if (threadIdx.x == 0) *loss = (double)s + (double)c;
-        return;
-    }
-    // the camera's BW_NV sums at once: each slot's values are read together (one index load, five
-    // 8-byte loads); per value the order of the additions, and the tree, are those of block_csum
-    __shared__ float ss[BW_NV][256], sc[BW_NV][256];
-    double S[BW_NV];
-    const int lo = cam_slot_start[b], hi = cam_slot_start[b + 1];
-    float s[BW_NV], c[BW_NV];
-#pragma unroll
-    for (int v = 0; v < BW_NV; ++v) s[v] = c[v] = 0.f;
-    static_assert(BW_NV % 2 == 0, "pairs of values per load");
-#pragma unroll 2
-    for (int k = lo + threadIdx.x; k < hi; k += blockDim.x) {
-        const float2* p = reinterpret_cast<const float2*>(partials + (long long)cam_slots[k] * BW_NV);
-        float x[BW_NV];
-#pragma unroll
-        for (int v = 0; v < BW_NV / 2; ++v) {
-            const float2 q = p[v];
-            x[2 * v] = q.x;
-            x[2 * v + 1] = q.y;
-        }
-#pragma unroll
-        for (int v = 0; v < BW_NV; ++v) {
-            float ns, ne;
-            two_sum(s[v], x[v], ns, ne);
-            s[v] = ns;
-            c[v] += ne;
-        }
-    }
+// Compensated sums of NS runs x[v * stride + lo .. v * stride + hi) by a block of 256 threads: thread t
+// adds every 256th value from lo + t on, a tree adds the threads' pairs.  The loads of 8 values per
+// run are in flight before their additions.
+template <int NS>
+__device__ __forceinline__ void block_csums(const float* __restrict__ x, long long stride, int lo, int hi, double S[NS]) {
+    __shared__ float sh_s[NS][256], sh_c[NS][256];
+    constexpr int D = 8;
     const int t = threadIdx.x;
+    float s[NS], c[NS];
 #pragma unroll
-    for (int v = 0; v < BW_NV; ++v) {
-        ss[v][t] = s[v];
-        sc[v][t] = c[v];
+    for (int v = 0; v < NS; ++v) s[v] = c[v] = 0.f;
+    for (int k0 = lo + t; k0 < hi; k0 += D * 256) {
+        float r[NS][D];
+#pragma unroll
+        for (int d = 0; d < D; ++d)
+#pragma unroll
+            for (int v = 0; v < NS; ++v) r[v][d] = k0 + d * 256 < hi ? __ldg(x + v * stride + k0 + d * 256) : 0.f;
+#pragma unroll
+        for (int d = 0; d < D; ++d) {
+            if (k0 + d * 256 >= hi) break;
+#pragma unroll
+            for (int v = 0; v < NS; ++v) {
+                float ns, ne;
+                two_sum(s[v], r[v][d], ns, ne);
+                s[v] = ns;
+                c[v] += ne;
+            }
+        }
+    }
+#pragma unroll
+    for (int v = 0; v < NS; ++v) {
+        sh_s[v][t] = s[v];
+        sh_c[v][t] = c[v];
     }
     __syncthreads();
-    for (int stride = blockDim.x / 2; stride > 0; stride >>= 1) {
-        if (t < stride) {
+    for (int h = 128; h > 0; h >>= 1) {
+        if (t < h) {
 #pragma unroll
-            for (int v = 0; v < BW_NV; ++v) {
+            for (int v = 0; v < NS; ++v) {
                 float ns, ne;
-                two_sum(ss[v][t], ss[v][t + stride], ns, ne);
-                ss[v][t] = ns;
-                sc[v][t] += sc[v][t + stride] + ne;
+                two_sum(sh_s[v][t], sh_s[v][t + h], ns, ne);
+                sh_s[v][t] = ns;
+                sh_c[v][t] += sh_c[v][t + h] + ne;
             }
         }
         __syncthreads();
     }
 #pragma unroll
-    for (int v = 0; v < BW_NV; ++v) S[v] = (double)ss[v][0] + (double)sc[v][0];
-    if (threadIdx.x == 0 && grad) {
-        const double cx = centers[2 * b], cy = centers[2 * b + 1];
-        double* gr = grad + 9 * b;
-        gr[0] = S[0] + cx * S[2];
-        gr[1] = S[1] + cy * S[2];
-        gr[2] = S[2];
-        gr[3] = S[3] + cx * S[5];
-        gr[4] = S[4] + cy * S[5];
-        gr[5] = S[5];
-        gr[6] = S[6] + cx * S[8];
-        gr[7] = S[7] + cy * S[8];
-        gr[8] = S[9];
-    }
-    (void)cams;
+    for (int v = 0; v < NS; ++v) S[v] = (double)sh_s[v][0] + (double)sh_c[v][0];
 }
 
+// Blocks (group, camera): the terms 3 g .. 3 g + 2 of the camera (group 3: the gain's term), so that four
+// blocks share its walk over the partials; a further block (0, ncam) sums the loss.  A chain of
+// latencies: 8 us for the 8150 tiles of 4 x 1080p, against 29 us with a block per camera that
+// reached each slot's terms through an index.
+__global__ void __launch_bounds__(256) k_backward_final(int ncam, const float* __restrict__ partials, int nslots,
+                                                         const float* __restrict__ loss_partials, int ntiles,
+                                                         const int* __restrict__ cam_slot_start,
+                                                         const int* __restrict__ centers, double* __restrict__ loss,
+                                                         double* __restrict__ grad) {
+    const int b = blockIdx.y, g = blockIdx.x;
+    double S[3];
+    if (b == ncam) {
+        if (g != 0) return;
+        block_csums<1>(loss_partials, 0, 0, ntiles, S);
+        if (threadIdx.x == 0) *loss = S[0];
+        return;
+    }
+    if (!grad) return;
+    const int lo = cam_slot_start[b], hi = cam_slot_start[b + 1];
+    double* gr = grad + 9 * b;
+    if (g == 3) {
+        block_csums<1>(partials + 9LL * nslots, 0, lo, hi, S);
+        if (threadIdx.x == 0) gr[8] = S[0];
+        return;
+    }
+    block_csums<3>(partials + 3LL * g * nslots, nslots, lo, hi, S);
+    if (threadIdx.x == 0) {
+        gr[3 * g] = S[0] + centers[2 * b] * S[2];
+        gr[3 * g + 1] = S[1] + centers[2 * b + 1] * S[2];
+        if (g < 2) gr[3 * g + 2] = S[2];
+    }
+}
+
+// tiles by candidate count: at most 2, at most 4, more
+constexpr int BW_CLASSES = 3;
+
 struct BwState {
-    BwTile* tiles = nullptr;
-    int ntiles = 0;
-    int* camlist = nullptr;
+    BwTile* tiles = nullptr;  // class by class
+    int ntiles = 0, nclass[BW_CLASSES] = {}, nslots = 0;
+    int4* slots = nullptr;    // per slot: tile origin, camera, position of its partials
+    BwMap* maps = nullptr;
     int* centers = nullptr;
-    int* cam_slots = nullptr;
     int* cam_slot_start = nullptr;
-    float* partials = nullptr;
+    float* partials = nullptr;  // [BW_NV][nslots]
     float* loss_partials = nullptr;
 };
 
@@ -367,8 +526,9 @@ stitch_status backward_plan(stitch_rig* r) {
     BwState* bs = new (std::nothrow) BwState();
     if (!bs) return STITCH_ENOMEM;
     r->bw = bs;
-    std::vector<BwTile> tiles;
+    std::vector<BwTile> tiles[BW_CLASSES];
     std::vector<int> camlist, centers(2 * g.ncam, 0);
+    std::vector<int4> sl;
     std::vector<std::vector<int>> slots(g.ncam);
     for (int i = 0; i < g.ncam; ++i) {
         const Rect v = r->hcam[i].V;
@@ -379,7 +539,7 @@ stitch_status backward_plan(stitch_rig* r) {
     for (int y0 = 0; y0 < Hc; y0 += BW_TY)
         for (int x0 = 0; x0 < Wc; x0 += BW_TX) {
             const int x1 = std::min(x0 + BW_TX, Wc), y1 = std::min(y0 + BW_TY, Hc);
-            BwTile t{x0, y0, (int)camlist.size(), 0};
+            BwTile t{x0, y0, (int)camlist.size(), 0, bs->ntiles};
             for (int i = 0; i < g.ncam; ++i) {
                 const CamDev& c = r->hcam[i];
                 if (!c.visible) continue;
@@ -393,25 +553,34 @@ stitch_status backward_plan(stitch_rig* r) {
                 camlist.resize(t.first);
                 continue;
             }
-            for (int k = 0; k < t.count; ++k) slots[camlist[t.first + k]].push_back(t.first + k);
-            tiles.push_back(t);
+            for (int k = 0; k < t.count; ++k) {
+                slots[camlist[t.first + k]].push_back(t.first + k);
+                sl.push_back(make_int4(x0, y0, camlist[t.first + k], 0));
+            }
+            tiles[t.count <= 2 ? 0 : t.count <= 4 ? 1 : 2].push_back(t);
+            ++bs->ntiles;
         }
-    std::vector<int> cam_slots, start(g.ncam + 1, 0);
+    // a camera's partials lie in a row, in tile order
+    std::vector<int> start(g.ncam + 1, 0);
     for (int i = 0; i < g.ncam; ++i) {
-        start[i] = (int)cam_slots.size();
-        cam_slots.insert(cam_slots.end(), slots[i].begin(), slots[i].end());
+        start[i + 1] = start[i] + (int)slots[i].size();
+        for (size_t k = 0; k < slots[i].size(); ++k) sl[slots[i][k]].w = start[i] + (int)k;
     }
-    start[g.ncam] = (int)cam_slots.size();
+    std::vector<BwTile> all;
+    for (int k = 0; k < BW_CLASSES; ++k) {
+        bs->nclass[k] = (int)tiles[k].size();
+        all.insert(all.end(), tiles[k].begin(), tiles[k].end());
+    }
+    bs->nslots = (int)sl.size();
     stitch_status st;
-    if ((st = upload_bw(r, tiles, &bs->tiles)) != STITCH_OK) return st;
-    if ((st = upload_bw(r, camlist, &bs->camlist)) != STITCH_OK) return st;
+    if ((st = upload_bw(r, all, &bs->tiles)) != STITCH_OK) return st;
+    if ((st = upload_bw(r, sl, &bs->slots)) != STITCH_OK) return st;
     if ((st = upload_bw(r, centers, &bs->centers)) != STITCH_OK) return st;
-    if ((st = upload_bw(r, cam_slots, &bs->cam_slots)) != STITCH_OK) return st;
     if ((st = upload_bw(r, start, &bs->cam_slot_start)) != STITCH_OK) return st;
-    bs->ntiles = (int)tiles.size();
-    bs->partials = (float*)rig_alloc(r, sizeof(float) * BW_NV * std::max<size_t>(camlist.size(), 1));
+    bs->maps = (BwMap*)rig_alloc(r, sizeof(BwMap) * std::max(bs->nslots, 1));
+    bs->partials = (float*)rig_alloc(r, sizeof(float) * BW_NV * std::max(bs->nslots, 1));
     bs->loss_partials = (float*)rig_alloc(r, sizeof(float) * std::max(bs->ntiles, 1));
-    if (!bs->partials || !bs->loss_partials) return STITCH_ENOMEM;
+    if (!bs->maps || !bs->partials || !bs->loss_partials) return STITCH_ENOMEM;
     return STITCH_OK;
 }
 
@@ -421,13 +590,21 @@ stitch_status backward_run(stitch_rig* r, const FramePtrs& fp, const double* par
     if (!bs) return STITCH_EINVAL;
     const RigGeom& g = r->geom;
     if (bs->ntiles > 0) {
-        prof_mark(r, "backward", s);
-        k_backward<<<bs->ntiles, BW_THREADS, 0, s>>>(r->dcam, fp, params, bs->tiles, bs->camlist, bs->centers, g.nx[0],
-                                                    g.ny[0], bs->partials, bs->loss_partials);
+        prof_mark(r, "backward_maps", s);
+        k_backward_maps<<<(bs->nslots + 63) / 64, 64, 0, s>>>(r->dcam, params, bs->slots, bs->nslots, bs->centers, g.nx[0],
+                                                              g.ny[0], bs->maps);
+        const BwTile* tl = bs->tiles;
+        for (int k = 0; k < BW_CLASSES; tl += bs->nclass[k++]) {
+            if (bs->nclass[k] == 0) continue;
+            prof_mark(r, "backward", s);
+            auto fn = k == 0 ? k_backward<2> : k == 1 ? k_backward<4> : k_backward_many;
+            fn<<<bs->nclass[k], BW_THREADS, 0, s>>>(fp, bs->maps, tl, g.nx[0], g.ny[0], bs->partials, bs->nslots,
+                                                    bs->loss_partials);
+        }
     }
     prof_mark(r, "backward_final", s);
-    k_backward_final<<<g.ncam + 1, 256, 0, s>>>(r->dcam, g.ncam, bs->partials, bs->loss_partials, bs->ntiles,
-                                                bs->cam_slots, bs->cam_slot_start, bs->centers, loss, grad);
+    k_backward_final<<<dim3(4, g.ncam + 1), 256, 0, s>>>(g.ncam, bs->partials, bs->nslots, bs->loss_partials, bs->ntiles,
+                                                         bs->cam_slot_start, bs->centers, loss, grad);
     return launch_status();
 }
 
