@@ -17,12 +17,13 @@
 //      inliers: w > 0 and squared transfer error < (inlier_px scaled)^2; best: most inliers,
 //      ties to the earlier iteration; least squares on its inliers; returned in pixels.
 //
-// Kernels, in launch order: mt_build (a block per table: sorted keys and a radix directory),
-// mt_query (a warp per query), mt_order (quality order, bounding boxes), mt_prep (normalised
-// coordinates, growth schedule by a block scan), mt_hypotheses_b (a block per iteration: sample and
-// 8x8 solve with a thread per matrix entry), mt_score (a block per hypothesis), mt_best (arg-max,
-// inlier flags), mt_sums (a warp per normal-equation entry, ordered sums), mt_solve (refit and
-// back to pixels).
+// Kernels, in launch order: mt_keys (hash keys of both images), mt_match (a warp per query against every
+// descriptor of image B), mt_rank (quality order by counting, normalised coordinates, growth
+// schedule), mt_hypotheses (four iterations per block: samples, 4-point solves, inlier counts, the
+// best by an atomic maximum) and mt_final (inlier flags, ordered normal-equation sums, refit, back to
+// pixels).  What bounds them is FP64: this part issues one double-precision instruction per warp
+// and scheduler about every 64 cycles, with no gain from independent ones, so a chain costs its
+// number of instructions times 64 cycles, and lanes left idle are lost.
 #include <climits>
 
 #include "stitch_internal.cuh"
@@ -31,8 +32,7 @@ namespace {
 
 constexpr int MT_MAX_POINTS = 2048;
 constexpr int MT_MAX_TABLES = 32, MT_MAX_BITS = 20;
-constexpr int MT_DIR_BITS = 11;                        // radix directory of each sorted table
-constexpr int MT_DIR = (1 << MT_DIR_BITS) + 1;
+constexpr int MT_MAX_WORDS = 32;  // key words of a descriptor
 
 struct LshBits {
     int L, k;
@@ -48,13 +48,64 @@ __device__ __forceinline__ double dS(double a, double b) { return __dsub_rn(a, b
 __device__ __forceinline__ double dM(double a, double b) { return __dmul_rn(a, b); }
 __device__ __forceinline__ double dD(double a, double b) { return __ddiv_rn(a, b); }
 
-__device__ __forceinline__ unsigned lsh_key(const unsigned* d, const LshBits& lb, int l) {
-    unsigned key = 0;
-    for (int j = 0; j < lb.k; ++j) {
-        const int bit = lb.b[l][j];
-        key |= ((d[bit >> 5] >> (bit & 31)) & 1u) << j;
+// State of one call, set up by mt_keys.
+struct MtState {
+    int mn[4], mx[4];         // bounding boxes of the matched points: x, y in image A, x, y in image B
+    int n;                    // matches
+    int pad;
+    unsigned long long best;  // (inliers + 1) << 32 | (2^32 - 1 - iteration) of the best hypothesis, 0 when none
+    Norm norm;
+    double t2;                // squared inlier threshold in normalised coordinates,
+    float t_in, t_out;        // and a little below and above it (FastInlier)
+};
+
+constexpr float MT_EPS = 9.5367431640625e-7f;  // 2^-20, see FastInlier
+
+// Hash keys as words whose difference is tested at once: with k <= 16 two tables share a word (an
+// unused upper half differs in every bit), otherwise a table has a word of its own.
+__host__ __device__ __forceinline__ bool mt_packed(const LshBits& lb) { return lb.k <= 16; }
+__host__ __device__ __forceinline__ int mt_words(const LshBits& lb) { return mt_packed(lb) ? (lb.L + 1) / 2 : lb.L; }
+
+// One key word (blockIdx.y) of 128 descriptors of image A (blockIdx.z 0) or B; the first block also
+// sets up the call's state.  The bit positions are the same for the whole block, so they come from the
+// parameter space as uniform loads; the descriptors' words from shared memory.
+__global__ void __launch_bounds__(128) mt_keys(const unsigned* __restrict__ desc_a, const int* __restrict__ count_a,
+                                               const unsigned* __restrict__ desc_b, const int* __restrict__ count_b,
+                                               const __grid_constant__ LshBits lb, int cap, unsigned* __restrict__ keys_a,
+                                               unsigned* __restrict__ keys_b, MtState* __restrict__ st) {
+    __shared__ unsigned d[8][128];
+    const int t = threadIdx.x, i = blockIdx.x * 128 + t, w = blockIdx.y;
+    const bool isb = blockIdx.z != 0;
+    if (blockIdx.x == 0 && w == 0 && !isb && t < 4) {
+        st->mn[t] = INT_MAX;
+        st->mx[t] = INT_MIN;
+        if (t == 0) {
+            st->n = 0;
+            st->best = 0ull;
+        }
     }
-    return key;
+    const int n = min(isb ? *count_b : *count_a, cap);
+    if (i >= n) return;
+    const unsigned* src = (isb ? desc_b : desc_a) + 8 * (size_t)i;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) d[k][t] = __ldg(src + k);
+    auto key_of = [&](int l) {
+        unsigned key = 0;
+#pragma unroll 4
+        for (int j = 0; j < lb.k; ++j) {
+            const int bit = lb.b[l][j];
+            key |= ((d[bit >> 5][t] >> (bit & 31)) & 1u) << j;
+        }
+        return key;
+    };
+    unsigned key;
+    if (mt_packed(lb)) {
+        key = key_of(2 * w);
+        key |= 2 * w + 1 < lb.L ? key_of(2 * w + 1) << 16 : isb ? 0u : 0xffff0000u;
+    } else {
+        key = key_of(w);
+    }
+    (isb ? keys_b : keys_a)[(size_t)w * cap + i] = key;
 }
 
 __device__ __forceinline__ int hamming(const unsigned* a, const unsigned* b) {
@@ -62,48 +113,6 @@ __device__ __forceinline__ int hamming(const unsigned* a, const unsigned* b) {
 #pragma unroll
     for (int k = 0; k < 8; ++k) d += __popc(a[k] ^ b[k]);
     return d;
-}
-
-// one block per table: keys of image B's descriptors, sorted by (key, index)
-__global__ void __launch_bounds__(1024) mt_build(const unsigned* __restrict__ desc_b, const int* __restrict__ count_b,
-                                                 const __grid_constant__ LshBits lb, unsigned* __restrict__ keys,
-                                                 int* __restrict__ ord, int* __restrict__ dir, int cap) {
-    __shared__ unsigned long long e[MT_MAX_POINTS];
-    const int l = blockIdx.x, nb = min(*count_b, cap);
-    int m = 1;
-    while (m < nb) m <<= 1;
-    for (int i = threadIdx.x; i < m; i += blockDim.x)
-        e[i] = i < nb ? ((unsigned long long)lsh_key(desc_b + 8 * i, lb, l) << 32) | (unsigned)i : ~0ull;
-    __syncthreads();
-    for (int k = 2; k <= m; k <<= 1)
-        for (int j = k >> 1; j > 0; j >>= 1) {
-            for (int i = threadIdx.x; i < m; i += blockDim.x) {
-                const int o = i ^ j;
-                if (o <= i) continue;
-                const unsigned long long a = e[i], b = e[o];
-                if (((i & k) == 0) == (a > b)) {
-                    e[i] = b;
-                    e[o] = a;
-                }
-            }
-            __syncthreads();
-        }
-    for (int i = threadIdx.x; i < nb; i += blockDim.x) {
-        keys[(size_t)l * cap + i] = (unsigned)(e[i] >> 32);
-        ord[(size_t)l * cap + i] = (int)(unsigned)e[i];
-    }
-    // directory: dir[v] = first sorted position whose key's top bits are >= v (v = 0..2^D)
-    const int D = lb.k < MT_DIR_BITS ? lb.k : MT_DIR_BITS, shift = lb.k - D;
-    for (int v = threadIdx.x; v <= (1 << D); v += blockDim.x) {
-        const unsigned long long bound = (unsigned long long)v << shift;
-        int lo = 0, hi = nb;
-        while (lo < hi) {
-            const int mid = (lo + hi) >> 1;
-            if ((e[mid] >> 32) < bound) lo = mid + 1;
-            else hi = mid;
-        }
-        dir[(size_t)l * MT_DIR + v] = lo;
-    }
 }
 
 struct Top2 {
@@ -124,127 +133,194 @@ __device__ __forceinline__ void top2_add(Top2& t, int d, int b) {
     }
 }
 
-// a warp per query: lanes take the (table, probe) pairs; (nearest, second nearest other index)
-// merged across lanes.  A bucket is located through the table's directory (the range of sorted
-// positions whose key has given top bits), then by binary search inside that range.
-__global__ void __launch_bounds__(256) mt_query(const unsigned* __restrict__ desc_a, const int* __restrict__ count_a,
+// Whether a query meets a descriptor of image B in some table: the keys differ in at most one bit.
+// x & (x - 1) clears the lowest bit of x; on packed halves a borrow leaves the lower half only when
+// that half is 0, that is, when it has already met.
+template <bool PACKED>
+__device__ __forceinline__ bool mt_meets(const unsigned* __restrict__ keys_b, const unsigned* __restrict__ ka, int nw, int cap,
+                                         int b) {
+    unsigned acc = 0xffffffffu;
+#pragma unroll 4
+    for (int w = 0; w < nw; ++w) {
+        const unsigned x = ka[w] ^ __ldg(keys_b + (size_t)w * cap + b);
+        const unsigned z = x & (x - (PACKED ? 0x00010001u : 1u));
+        acc = PACKED ? __vminu2(acc, z) : min(acc, z);
+    }
+    return PACKED ? (acc & 0xffffu) == 0u || (acc >> 16) == 0u : acc == 0u;
+}
+
+// A warp per query, its lanes over every descriptor of image B: those that the query meets in a table
+// are gathered and their distances taken 32 at a time.  Testing all pairs costs some 20 instructions
+// each, 38 us for 1000 x 1000 points and 8 tables, nearly all of it load latency; hashing into sorted buckets and probing them took
+// 32 us (a bitonic sort per table, then a chain of dependent loads per probe).
+template <bool PACKED>
+__global__ void __launch_bounds__(256) mt_match(const unsigned* __restrict__ desc_a, const int* __restrict__ count_a,
                                                 const unsigned* __restrict__ desc_b, const int* __restrict__ count_b,
-                                                const __grid_constant__ LshBits lb, const unsigned* __restrict__ keys,
-                                                const int* __restrict__ ord, const int* __restrict__ dir, int cap,
-                                                int max_dist, int rnum, int rden, int* __restrict__ best) {
-    const int a = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+                                                const unsigned* __restrict__ keys_a, const unsigned* __restrict__ keys_b,
+                                                int nw, int cap, const int* __restrict__ xy_a, const int* __restrict__ xy_b,
+                                                int max_dist, int rnum, int rden, int2* __restrict__ best,
+                                                MtState* __restrict__ st) {
+    __shared__ unsigned s_ka[8][MT_MAX_WORDS];
+    __shared__ uint16_t s_hit[8][64];
+    __shared__ int s_mn[4], s_mx[4], s_n;
+    const int t = threadIdx.x, w = t >> 5, lane = t & 31, a = blockIdx.x * 8 + w;
     const int na = min(*count_a, cap), nb = min(*count_b, cap);
-    const int shift = lb.k > MT_DIR_BITS ? lb.k - MT_DIR_BITS : 0;
-    if (a >= na) return;
-    unsigned da[8];
+    if (blockIdx.x * 8 >= na) return;
+    if (t < 4) {
+        s_mn[t] = INT_MAX;
+        s_mx[t] = INT_MIN;
+        if (t == 0) s_n = 0;
+    }
+    __syncthreads();
+    if (a < na) {
+        if (lane < nw) s_ka[w][lane] = keys_a[(size_t)lane * cap + a];
+        unsigned da[8];
 #pragma unroll
-    for (int k = 0; k < 8; ++k) da[k] = desc_a[8 * a + k];
-    constexpr int INF = 1 << 30;
-    Top2 t{INF, -1, INF, -1};
-    const int per = lb.k + 1;
-    for (int pp = lane; pp < lb.L * per; pp += 32) {
-        const int l = pp / per, p = pp - l * per - 1;
-        const unsigned q0 = lsh_key(da, lb, l);
-        const unsigned q = p < 0 ? q0 : (q0 ^ (1u << p));
-        const unsigned* kl = keys + (size_t)l * cap;
-        const int* dl = dir + (size_t)l * MT_DIR;
-        int lo = dl[q >> shift], hi = dl[(q >> shift) + 1];
-        while (lo < hi) {
-            const int mid = (lo + hi) >> 1;
-            if (kl[mid] < q) lo = mid + 1;
-            else hi = mid;
+        for (int k = 0; k < 8; ++k) da[k] = desc_a[8 * (size_t)a + k];
+        __syncwarp();
+        constexpr int INF = 1 << 30;
+        Top2 best2{INF, -1, INF, -1};
+        int nh = 0;
+        auto take = [&](int n) {  // the first n gathered descriptors
+            if (lane < n) {
+                const int b = s_hit[w][lane];
+                top2_add(best2, hamming(da, desc_b + 8 * (size_t)b), b);
+            }
+            __syncwarp();
+        };
+        for (int b0 = 0; b0 < nb; b0 += 32) {
+            const int b = b0 + lane;
+            const bool hit = b < nb && mt_meets<PACKED>(keys_b, s_ka[w], nw, cap, b);
+            const unsigned m = __ballot_sync(0xffffffffu, hit);
+            if (hit) s_hit[w][nh + __popc(m & ((1u << lane) - 1u))] = (uint16_t)b;
+            nh += __popc(m);
+            __syncwarp();
+            if (nh >= 32) {
+                take(32);
+                nh -= 32;
+                const uint16_t rest = s_hit[w][32 + lane];
+                __syncwarp();
+                if (lane < nh) s_hit[w][lane] = rest;
+                __syncwarp();
+            }
         }
-        for (int i = lo; i < nb && kl[i] == q; ++i) {
-            const int b = ord[(size_t)l * cap + i];
-            top2_add(t, hamming(da, desc_b + 8 * b), b);
+        take(nh);
+        // merge: the union's two nearest distinct indices are among the lanes' two nearest
+        for (int off = 16; off > 0; off >>= 1) {
+            Top2 o;
+            o.d1 = __shfl_down_sync(0xffffffffu, best2.d1, off);
+            o.b1 = __shfl_down_sync(0xffffffffu, best2.b1, off);
+            o.d2 = __shfl_down_sync(0xffffffffu, best2.d2, off);
+            o.b2 = __shfl_down_sync(0xffffffffu, best2.b2, off);
+            if (o.b1 >= 0) top2_add(best2, o.d1, o.b1);
+            if (o.b2 >= 0) top2_add(best2, o.d2, o.b2);
+        }
+        if (lane == 0) {
+            const bool ok = best2.b1 >= 0 && best2.d1 <= max_dist &&
+                            (best2.d2 == INF || (long long)rden * best2.d1 < (long long)rnum * best2.d2);
+            best[a] = make_int2(ok ? best2.b1 : -1, best2.d1);
+            if (ok) {
+                const int v[4] = {xy_a[2 * a], xy_a[2 * a + 1], xy_b[2 * best2.b1], xy_b[2 * best2.b1 + 1]};
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    atomicMin(&s_mn[k], v[k]);
+                    atomicMax(&s_mx[k], v[k]);
+                }
+                atomicAdd(&s_n, 1);
+            }
         }
     }
-    // merge: the union's two nearest distinct indices are among the lanes' two nearest
-    for (int off = 16; off > 0; off >>= 1) {
-        Top2 o;
-        o.d1 = __shfl_down_sync(0xffffffffu, t.d1, off);
-        o.b1 = __shfl_down_sync(0xffffffffu, t.b1, off);
-        o.d2 = __shfl_down_sync(0xffffffffu, t.d2, off);
-        o.b2 = __shfl_down_sync(0xffffffffu, t.b2, off);
-        if (o.b1 >= 0) top2_add(t, o.d1, o.b1);
-        if (o.b2 >= 0) top2_add(t, o.d2, o.b2);
-    }
-    if (lane == 0) {
-        const bool ok = t.b1 >= 0 && t.d1 <= max_dist &&
-                        (t.d2 == INF || (long long)rden * t.d1 < (long long)rnum * t.d2);
-        best[2 * a] = ok ? t.b1 : -1;
-        best[2 * a + 1] = t.d1;
+    __syncthreads();
+    if (t < 4 && s_n > 0) {
+        atomicMin(&st->mn[t], s_mn[t]);
+        atomicMax(&st->mx[t], s_mx[t]);
+        if (t == 0) atomicAdd(&st->n, s_n);
     }
 }
 
-// one block: accepted matches in quality order, and the per-image normalisation
-__global__ void __launch_bounds__(1024) mt_order(const int* __restrict__ best, const int* __restrict__ count_a, int cap,
-                                                 const int* __restrict__ xy_a, const int* __restrict__ xy_b,
-                                                 int* __restrict__ matches, int* __restrict__ n_matches,
-                                                 Norm* __restrict__ norm) {
-    __shared__ unsigned long long e[MT_MAX_POINTS];
-    __shared__ int s_n;
-    __shared__ int mn[4], mx[4];
-    const int na = min(*count_a, cap), t = threadIdx.x;
-    if (t == 0) s_n = 0;
-    if (t < 4) {
-        mn[t] = INT_MAX;
-        mx[t] = INT_MIN;
+// The growth schedule by one block of 256 threads.  The top n grows to n + 1 at iteration E_j
+// (j = n - 4), E_0 = 1 and E_{j+1} = E_j + ceil(T_N m n (n-1) (n-2) / (N (N-1) (N-2) (N-3))) (m = 4,
+// T_N = 200000: the exact increment T_{n+1} - T_n of T_n = T_N C(n, m) / C(N, m)), up to n = N.
+__device__ __forceinline__ void mt_schedule(int N, long long* __restrict__ E) {
+    __shared__ long long wsum[8];
+    constexpr int PT = MT_MAX_POINTS / 256;
+    const int t = threadIdx.x, lane = t & 31, w = t >> 5;
+    if (N < 4) return;
+    const int K = N - 4;  // growth events j = 0 .. K-1 (n = 4 + j)
+    const long long Q = (long long)N * (N - 1) * (N - 2) * (N - 3);
+    long long d[PT], v = 0;
+#pragma unroll
+    for (int e = 0; e < PT; ++e) {
+        const long long n = 4 + PT * t + e;
+        d[e] = PT * t + e < K ? (800000LL * n * (n - 1) * (n - 2) + Q - 1) / Q : 0;
+        v += d[e];
     }
-    __syncthreads();
-    for (int a = t; a < na; a += blockDim.x)
-        if (best[2 * a] >= 0) {
-            const int pos = atomicAdd(&s_n, 1);
-            e[pos] = ((unsigned long long)best[2 * a + 1] << 32) | (unsigned)a;
-        }
-    __syncthreads();
-    const int n = s_n;
-    int m = 1;
-    while (m < n) m <<= 1;
-    for (int i = n + t; i < m; i += blockDim.x) e[i] = ~0ull;
-    __syncthreads();
-    for (int k = 2; k <= m; k <<= 1)
-        for (int j = k >> 1; j > 0; j >>= 1) {
-            for (int i = t; i < m; i += blockDim.x) {
-                const int o = i ^ j;
-                if (o <= i) continue;
-                const unsigned long long a = e[i], b = e[o];
-                if (((i & k) == 0) == (a > b)) {
-                    e[i] = b;
-                    e[o] = a;
-                }
-            }
-            __syncthreads();
-        }
-    for (int i = t; i < n; i += blockDim.x) {
-        const int a = (int)(unsigned)e[i];
-        const int b = best[2 * a];
-        matches[3 * i] = a;
-        matches[3 * i + 1] = b;
-        matches[3 * i + 2] = (int)(e[i] >> 32);
-        atomicMin(&mn[0], xy_a[2 * a]);
-        atomicMax(&mx[0], xy_a[2 * a]);
-        atomicMin(&mn[1], xy_a[2 * a + 1]);
-        atomicMax(&mx[1], xy_a[2 * a + 1]);
-        atomicMin(&mn[2], xy_b[2 * b]);
-        atomicMax(&mx[2], xy_b[2 * b]);
-        atomicMin(&mn[3], xy_b[2 * b + 1]);
-        atomicMax(&mx[3], xy_b[2 * b + 1]);
+    long long s = v;  // inclusive sums over the threads
+    for (int off = 1; off < 32; off <<= 1) {
+        const long long o = __shfl_up_sync(0xffffffffu, s, off);
+        if (lane >= off) s += o;
     }
+    if (lane == 31) wsum[w] = s;
     __syncthreads();
-    if (t == 0) {
-        *n_matches = n;
-        Norm z{0.0, 0.0, 0.0, 0.0, 1.0, 1.0};
-        if (n > 0) {
-            z.ca0 = dM(0.5, dA((double)mn[0], (double)mx[0]));
-            z.ca1 = dM(0.5, dA((double)mn[1], (double)mx[1]));
-            z.cb0 = dM(0.5, dA((double)mn[2], (double)mx[2]));
-            z.cb1 = dM(0.5, dA((double)mn[3], (double)mx[3]));
-            const int ra = max(mx[0] - mn[0], mx[1] - mn[1]), rb = max(mx[2] - mn[2], mx[3] - mn[3]);
-            z.sa = dD(2.0, (double)(ra > 1 ? ra : 1));
-            z.sb = dD(2.0, (double)(rb > 1 ? rb : 1));
+    for (int k = 0; k < w; ++k) s += wsum[k];
+    long long x = 1 + s - v;
+#pragma unroll
+    for (int e = 0; e < PT; ++e) {
+        if (PT * t + e <= K) E[PT * t + e] = x;
+        x += d[e];
+    }
+}
+
+// A warp per query: an accepted match's place in quality order is the number of accepted matches
+// before it.  It writes the match and its normalised coordinates (x, y, u, v), the latter also in
+// single precision for mt_count.  The last block computes the growth schedule.
+__global__ void __launch_bounds__(256) mt_rank(const int2* __restrict__ best, const int* __restrict__ count_a, int cap,
+                                               const int* __restrict__ xy_a, const int* __restrict__ xy_b,
+                                               MtState* __restrict__ st, int* __restrict__ matches,
+                                               int* __restrict__ n_matches, double* __restrict__ xyuv,
+                                               float* __restrict__ xyuvf, long long* __restrict__ E, double inlier_px) {
+    const int t = threadIdx.x, lane = t & 31, N = st->n;
+    if (blockIdx.x == gridDim.x - 1) {
+        mt_schedule(N, E);
+        return;
+    }
+    const int a = blockIdx.x * 8 + (t >> 5), na = min(*count_a, cap);
+    const bool first = blockIdx.x == 0 && t < 32;  // writes the call's results
+    if (first && lane == 0) *n_matches = N;
+    const int2 m = a < na ? best[a] : make_int2(-1, 0);
+    if (m.x < 0 && !first) return;
+    // normalisation: lane 0 .. 3 takes x, y of image A, x, y of image B
+    const int l = lane & 3, q = l & 2;
+    double c = 0.0, sc = 1.0;
+    if (N > 0) {
+        c = dM(0.5, dA((double)st->mn[l], (double)st->mx[l]));
+        const int r = max(st->mx[q] - st->mn[q], st->mx[q + 1] - st->mn[q + 1]);
+        sc = dD(2.0, (double)(r > 1 ? r : 1));
+    }
+    if (first && lane < 4) {
+        double* z = &st->norm.ca0;
+        z[l] = c;
+        if (l == 0) st->norm.sa = sc;
+        if (l == 2) {
+            const double tn = dM(inlier_px, sc), t2 = dM(tn, tn);
+            st->norm.sb = sc;
+            st->t2 = t2;
+            st->t_in = __double2float_rd(t2) * (1.0f - MT_EPS);
+            st->t_out = __double2float_ru(t2) * (1.0f + MT_EPS);
         }
-        *norm = z;
+    }
+    if (m.x < 0) return;
+    int r = 0;
+    for (int i = lane; i < na; i += 32) {
+        const int2 o = best[i];
+        r += o.x >= 0 && (o.y < m.y || (o.y == m.y && i < a));
+    }
+    r = __reduce_add_sync(0xffffffffu, r);
+    if (lane < 3) matches[3 * r + lane] = lane == 0 ? a : lane == 1 ? m.x : m.y;
+    if (lane < 4) {
+        const double v = dM(dS((double)(l < 2 ? xy_a[2 * a + l] : xy_b[2 * m.x + l - 2]), c), sc);
+        xyuv[4 * r + l] = v;
+        xyuvf[4 * r + l] = (float)v;
     }
 }
 
@@ -257,72 +333,6 @@ __device__ __forceinline__ bool inlier(const double h[8], double x, double y, do
     const double pu = dS(dD(dA(dA(dM(h[0], x), dM(h[1], y)), h[2]), w), u);
     const double pv = dS(dD(dA(dA(dM(h[3], x), dM(h[4], y)), h[5]), w), v);
     return dA(dM(pu, pu), dM(pv, pv)) < t2;
-}
-
-// one block: the normalised coordinates (x, y, u, v) of every match, and the PROSAC growth
-// schedule.  The top n grows to n + 1 at iteration E_j (j = n - 4), E_0 = 1 and E_{j+1} = E_j +
-// ceil(T_N m n (n-1) (n-2) / (N (N-1) (N-2) (N-3))) (m = 4, T_N = 200000: the exact increment
-// T_{n+1} - T_n of T_n = T_N C(n, m) / C(N, m)), up to n = N; E by a block scan.  For iteration t:
-// c = #{j < N - 4 : E_j <= t}, n(t) = 4 + c, uniform sampling when E_c < t.
-__global__ void __launch_bounds__(1024) mt_prep(const int* __restrict__ n_matches, const int* __restrict__ mt,
-                                                const int* __restrict__ xy_a, const int* __restrict__ xy_b,
-                                                const Norm* __restrict__ norm, int iters, double* __restrict__ xyuv,
-                                                int* __restrict__ nt, unsigned char* __restrict__ uni) {
-    __shared__ long long E[MT_MAX_POINTS];
-    __shared__ long long wsum[32];
-    const int N = *n_matches, tid = threadIdx.x;
-    const Norm z = *norm;
-    for (int i = tid; i < N; i += blockDim.x) {
-        const int a = mt[3 * i], b = mt[3 * i + 1];
-        xyuv[4 * i] = dM(dS((double)xy_a[2 * a], z.ca0), z.sa);
-        xyuv[4 * i + 1] = dM(dS((double)xy_a[2 * a + 1], z.ca1), z.sa);
-        xyuv[4 * i + 2] = dM(dS((double)xy_b[2 * b], z.cb0), z.sb);
-        xyuv[4 * i + 3] = dM(dS((double)xy_b[2 * b + 1], z.cb1), z.sb);
-    }
-    if (N < 4 || iters == 0) return;
-    const int K = N - 4;  // growth events j = 0..K-1 (n = 4 + j)
-    const long long Q = (long long)N * (N - 1) * (N - 2) * (N - 3);
-    long long d[2] = {0, 0};
-    for (int e = 0; e < 2; ++e) {
-        const int j = 2 * tid + e;
-        if (j < K) {
-            const long long n = 4 + j;
-            d[e] = (800000LL * n * (n - 1) * (n - 2) + Q - 1) / Q;
-        }
-    }
-    // inclusive scan of the pair sums over the block
-    long long v = d[0] + d[1];
-    const int lane = tid & 31, w = tid >> 5;
-    for (int off = 1; off < 32; off <<= 1) {
-        const long long o = __shfl_up_sync(0xffffffffu, v, off);
-        if (lane >= off) v += o;
-    }
-    if (lane == 31) wsum[w] = v;
-    __syncthreads();
-    if (w == 0) {
-        long long x = lane < (int)(blockDim.x >> 5) ? wsum[lane] : 0;
-        for (int off = 1; off < 32; off <<= 1) {
-            const long long o = __shfl_up_sync(0xffffffffu, x, off);
-            if (lane >= off) x += o;
-        }
-        wsum[lane] = x;
-    }
-    __syncthreads();
-    const long long excl = v - (d[0] + d[1]) + (w > 0 ? wsum[w - 1] : 0);
-    // E_j = 1 + sum_{i<j} d_i for j = 0..K
-    if (2 * tid <= K) E[2 * tid] = 1 + excl;
-    if (2 * tid + 1 <= K) E[2 * tid + 1] = 1 + excl + d[0];
-    __syncthreads();
-    for (int t = tid + 1; t <= iters; t += blockDim.x) {
-        int lo = 0, hi = K;  // c = first j in [0, K) with E_j > t, else K
-        while (lo < hi) {
-            const int mid = (lo + hi) >> 1;
-            if (E[mid] <= t) lo = mid + 1;
-            else hi = mid;
-        }
-        nt[t - 1] = 4 + lo;
-        uni[t - 1] = E[lo] < t ? 1 : 0;
-    }
 }
 
 __device__ __forceinline__ int nth_free(int j, const int* chosen, int c) {
@@ -339,321 +349,359 @@ __device__ __forceinline__ int nth_free(int j, const int* chosen, int c) {
     return j;
 }
 
-// M h = r on one block (at least 72 threads; every thread calls it): thread (i, j) of the first 72
-// holds entry j of row i of A = [M | r] in shared memory and receives the operations of the
-// sequential elimination (solve8) in the same order, so h is bit-identical; the pivot search and
-// the ordered subtractions of the back substitution run on one thread.  Returns false (on every
-// thread) when a pivot is below 1e-12 in magnitude or NaN; h in hs.
-struct BlockSolve {
-    double A[8][9];
-    double hs[8], fv[8], prod[8];
-    int piv, sing;
+// M h = r by 8 lanes (a lane per row of A = [M | r], four systems per warp): every entry receives the
+// operations of the sequential elimination with partial pivoting in the same order, so h is bit-identical.
+// Rows stay in their lanes; a lane keeps its row's place in the current order, and the pivot is the
+// largest magnitude, ties to the first row in that order.  240 double-precision instructions for four
+// systems, 8 us; a block per system with a thread per entry kept three schedulers busy for each.  False
+// when a pivot is below 1e-12 in magnitude or NaN.  All 32 lanes call it; h is complete in each.
+__device__ bool solve8(double A[9], double h[8]) {
+    constexpr unsigned FULL = 0xffffffffu;
+    const int lane = threadIdx.x & 31, group = lane & 24;
+    int place = lane & 7;
+    bool ok = true;
+#pragma unroll
+    for (int c = 0; c < 8; ++c) {
+        long long v = place >= c ? abs_bits(A[c]) : -1;
+        int p = place;
+#pragma unroll
+        for (int off = 4; off > 0; off >>= 1) {
+            const long long ov = __shfl_xor_sync(FULL, v, off);
+            const int op = __shfl_xor_sync(FULL, p, off);
+            if (ov > v || (ov == v && op < p)) {
+                v = ov;
+                p = op;
+            }
+        }
+        ok &= v >= __double_as_longlong(1e-12) && v <= 0x7ff0000000000000ll;
+        place = place == p ? c : place == c ? p : place;  // the pivot row and row c change places
+        const int src = group + __ffs(__ballot_sync(FULL, place == c) >> group) - 1;
+        const double f = dD(A[c], __shfl_sync(FULL, A[c], src));
+#pragma unroll
+        for (int j = c + 1; j < 9; ++j) {
+            const double x = __shfl_sync(FULL, A[j], src);
+            if (place > c) A[j] = dS(A[j], dM(f, x));
+        }
+    }
+    double prod[8];
+#pragma unroll
+    for (int c = 7; c >= 0; --c) {
+        double s = A[8];
+#pragma unroll
+        for (int k = c + 1; k < 8; ++k) s = dS(s, prod[k]);
+        const int src = group + __ffs(__ballot_sync(FULL, place == c) >> group) - 1;
+        h[c] = __shfl_sync(FULL, dD(s, A[c]), src);
+        prod[c] = dM(A[c], h[c]);
+    }
+    return ok;
+}
+
+// The inlier test of a hypothesis with its decision taken in single precision wherever that is
+// certain.  With (a, b) = (num_u - u w, num_v - v w), the test is w > 0 and a^2 + b^2 < t2 w^2.  All
+// coordinates lie in [-1, 1], so with Mu = |h0| + |h1| + |h2|, Mv likewise and Mw = |h6| + |h7| + 1,
+// rounding the inputs and evaluating in single precision moves w by less than 5 2^-24 Mw and a by less
+// than 8 2^-24 (Mu + Mw); the bounds used are 2^-20 of those sums, which also covers the rounding
+// of the double-precision test (2^-50 of them) and the final squares.  Between the bounds (and for
+// anything not finite) the double-precision test decides, so the flags are always its own: for 1000
+// hypotheses and 374 matches it runs for a few dozen warps, not 12 000.
+struct FastInlier {
+    float h[8], eu, ev, ew, t_in, t_out;
+    // hf: the hypothesis rounded to single precision
+    __device__ __forceinline__ FastInlier(const float* hf, const MtState* st) : t_in(st->t_in), t_out(st->t_out) {
+#pragma unroll
+        for (int k = 0; k < 8; ++k) h[k] = hf[k];
+        const float E = MT_EPS;
+        const float mw = fabsf(h[6]) + fabsf(h[7]) + 1.0f;
+        eu = E * (fabsf(h[0]) + fabsf(h[1]) + fabsf(h[2]) + mw) + 1e-30f;
+        ev = E * (fabsf(h[3]) + fabsf(h[4]) + fabsf(h[5]) + mw) + 1e-30f;
+        ew = E * mw;
+    }
+    // 1 inlier, 0 outlier, -1 undecided
+    __device__ __forceinline__ int operator()(float4 p) const {
+        const float w = fmaf(h[6], p.x, fmaf(h[7], p.y, 1.0f));
+        const float a = fabsf(fmaf(-p.z, w, fmaf(h[0], p.x, fmaf(h[1], p.y, h[2]))));
+        const float b = fabsf(fmaf(-p.w, w, fmaf(h[3], p.x, fmaf(h[4], p.y, h[5]))));
+        const float wl = w - ew, wh = fabsf(w) + ew, ah = a + eu, bh = b + ev, al = fmaxf(a - eu, 0.0f), bl = fmaxf(b - ev, 0.0f);
+        if (wl > 0.0f && fmaf(ah, ah, bh * bh) < t_in * (wl * wl)) return 1;
+        if (w + ew < 0.0f || fmaf(al, al, bl * bl) > fmaf(t_out, wh * wh, 1e-37f)) return 0;
+        return -1;
+    }
 };
 
-__device__ bool solve8_block(BlockSolve& b) {
-    const int t = threadIdx.x, i = t / 9, j = t - 9 * (t / 9);
-    const bool own = t < 72;
-    if (t == 0) b.sing = 0;
-    __syncthreads();
-    for (int c = 0; c < 8; ++c) {
-        if (t == 0) {
-            long long bst = abs_bits(b.A[c][c]);
-            int p = c;
-            for (int k = c + 1; k < 8; ++k) {
-                const long long v = abs_bits(b.A[k][c]);
-                if (v > bst) {
-                    bst = v;
-                    p = k;
+__device__ __forceinline__ bool mt_inlier(const FastInlier& fast, const double* h, const double* __restrict__ xyuv,
+                                          const float* __restrict__ xyuvf, int i, double t2) {
+    const int d = fast(reinterpret_cast<const float4*>(xyuvf)[i]);
+    if (d >= 0) return d != 0;
+    return inlier(h, xyuv[4 * i], xyuv[4 * i + 1], xyuv[4 * i + 2], xyuv[4 * i + 3], t2);
+}
+
+// Four iterations per block of 4 warps.  Each warp draws the sample of one (its place in the growth
+// schedule c = #{j < N - 4 : E_j <= t}, n(t) = 4 + c, uniform sampling when E_c < t), one warp solves the
+// four 4-point systems, then each warp counts the inliers of one.  The solving warp is another one
+// from each wave of `sms` blocks to the next, so that the blocks of an SM solve on different
+// schedulers.  30 us for 1000 iterations on 374 matches, against 61 us for the two kernels with a
+// block per iteration (FP64 inlier tests alone: 30 us at two lanes per clock and SM).
+__global__ void __launch_bounds__(128) mt_hypotheses(int iters, const long long* __restrict__ E,
+                                                     const unsigned* __restrict__ rnd, const double* __restrict__ xyuv,
+                                                     const float* __restrict__ xyuvf, int sms,
+                                                     double* __restrict__ hyp, MtState* __restrict__ st) {
+    __shared__ int sidx[4][4];
+    __shared__ double sh[4][8];
+    __shared__ float shf[4][8];
+    __shared__ int s_ok[4];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, it = 4 * blockIdx.x + w;
+    const int N = st->n;
+    if (N < 4) return;
+    {
+        const long long t = min(it, iters - 1) + 1;
+        const int K = N - 4;
+        // E does not decrease: whole segments of 64 events first, then the events of the next one
+        const int s = __popc(__ballot_sync(0xffffffffu, 64 * lane + 63 < K && E[min(64 * lane + 63, K)] <= t));
+        const int j = 64 * s + lane;
+        const int c = 64 * s + __popc(__ballot_sync(0xffffffffu, j < K && E[min(j, K)] <= t)) +
+                      __popc(__ballot_sync(0xffffffffu, j + 32 < K && E[min(j + 32, K)] <= t));
+        if (lane == 0) {
+            const int n = 4 + c;
+            const unsigned* rw = rnd + 4 * (size_t)(t - 1);
+            int idx[4];
+            if (E[c] < t) {
+                for (int k = 0; k < 4; ++k) idx[k] = nth_free((int)(rw[k] % (unsigned)(n - k)), idx, k);
+            } else {
+                idx[0] = n - 1;
+                int chosen[3];
+                for (int k = 0; k < 3; ++k) {
+                    chosen[k] = nth_free((int)(rw[k] % (unsigned)(n - 1 - k)), chosen, k);
+                    idx[k + 1] = chosen[k];
                 }
             }
-            b.piv = p;
-            if (bst < __double_as_longlong(1e-12) || bst > 0x7ff0000000000000ll) b.sing = 1;
+            for (int k = 0; k < 4; ++k) sidx[w][k] = idx[k];
         }
-        __syncthreads();
-        if (b.sing) return false;
-        const int p = b.piv;
-        if (p != c && own && i == c && j >= c) {  // columns left of c are never read again
-            const double x = b.A[c][j];
-            b.A[c][j] = b.A[p][j];
-            b.A[p][j] = x;
-        }
-        __syncthreads();
-        if (own && i > c && j == c) b.fv[i] = dD(b.A[i][c], b.A[c][c]);
-        __syncthreads();
-        if (own && i > c && j >= c) b.A[i][j] = dS(b.A[i][j], dM(b.fv[i], b.A[c][j]));
-        __syncthreads();
-    }
-    for (int c = 7; c >= 0; --c) {
-        if (t > c && t < 8) b.prod[t] = dM(b.A[c][t], b.hs[t]);
-        __syncthreads();
-        if (t == 0) {
-            double sacc = b.A[c][8];
-            for (int k = c + 1; k < 8; ++k) sacc = dS(sacc, b.prod[k]);
-            b.hs[c] = dD(sacc, b.A[c][c]);
-        }
-        __syncthreads();
-    }
-    return true;
-}
-
-// one block of 96 threads per iteration: its sample and 4-point hypothesis (valid flag 0 when
-// singular)
-__global__ void __launch_bounds__(96) mt_hypotheses_b(const int* __restrict__ n_matches, int iters,
-                                                      const int* __restrict__ nt,
-                                                      const unsigned char* __restrict__ uni,
-                                                      const unsigned* __restrict__ rnd,
-                                                      const double* __restrict__ xyuv, double* __restrict__ hyp,
-                                                      int* __restrict__ valid) {
-    __shared__ BlockSolve b;
-    __shared__ int sidx[4];
-    const int it = blockIdx.x, t = threadIdx.x;
-    if (*n_matches < 4) {
-        if (t == 0) valid[it] = 0;
-        return;
-    }
-    if (t == 0) {
-        const int n = nt[it];
-        const unsigned* rw = rnd + 4 * (size_t)it;
-        int idx[4];
-        if (uni[it]) {
-            for (int k = 0; k < 4; ++k) idx[k] = nth_free((int)(rw[k] % (unsigned)(n - k)), idx, k);
-        } else {
-            idx[0] = n - 1;
-            int chosen[3];
-            for (int k = 0; k < 3; ++k) {
-                chosen[k] = nth_free((int)(rw[k] % (unsigned)(n - 1 - k)), chosen, k);
-                idx[k + 1] = chosen[k];
-            }
-        }
-        for (int k = 0; k < 4; ++k) sidx[k] = idx[k];
     }
     __syncthreads();
-    if (t < 72) {
+    if (w == (int)((blockIdx.x / (unsigned)sms) & 3u)) {
         // rows 2k, 2k+1 of pair k: (x, y, 1, 0, 0, 0, -ux, -uy | u), (0, 0, 0, x, y, 1, -vx, -vy | v)
-        const int i = t / 9, j = t - 9 * (t / 9), k = i >> 1, m = sidx[k];
-        const double x = xyuv[4 * m], y = xyuv[4 * m + 1], u = xyuv[4 * m + 2], v = xyuv[4 * m + 3];
-        const double w = (i & 1) ? v : u;
-        double e;
-        if (j == 8) e = w;
-        else if (j == 6) e = -dM(w, x);
-        else if (j == 7) e = -dM(w, y);
-        else {
-            const int jj = (i & 1) ? j - 3 : j;  // position within the row's (x, y, 1) block
-            e = jj == 0 ? x : jj == 1 ? y : jj == 2 ? 1.0 : 0.0;
-        }
-        b.A[i][j] = e;
+        const int g = lane >> 3, r = lane & 7, m = sidx[g][r >> 1];
+        const bool odd = r & 1;
+        const double x = xyuv[4 * m], y = xyuv[4 * m + 1], u = xyuv[4 * m + 2 + odd];
+        double A[9] = {odd ? 0.0 : x, odd ? 0.0 : y, odd ? 0.0 : 1.0, odd ? x : 0.0, odd ? y : 0.0, odd ? 1.0 : 0.0,
+                       -dM(u, x), -dM(u, y), u};
+        double h[8];
+        const bool ok = solve8(A, h);
+        if (r == 0) s_ok[g] = ok;
+        double mine = h[0];
+#pragma unroll
+        for (int k = 1; k < 8; ++k) mine = r == k ? h[k] : mine;
+        sh[g][r] = mine;
+        shf[g][r] = (float)mine;
+        if (4 * (int)blockIdx.x + g < iters) hyp[8 * (size_t)(4 * blockIdx.x + g) + r] = mine;
     }
     __syncthreads();
-    const bool ok = solve8_block(b);
-    if (t == 0) valid[it] = ok ? 1 : 0;
-    if (ok && t < 8) hyp[8 * (size_t)it + t] = b.hs[t];
-}
-
-__device__ __forceinline__ double inlier_t2(double inlier_px, const Norm& z) {
-    const double tn = dM(inlier_px, z.sb);
-    return dM(tn, tn);
-}
-
-// one block per hypothesis: its inlier count (-1 when not valid)
-__global__ void __launch_bounds__(256) mt_score(const int* __restrict__ n_matches, const double* __restrict__ hyp,
-                                                const int* __restrict__ valid, const double* __restrict__ xyuv,
-                                                const Norm* __restrict__ norm, double inlier_px,
-                                                int* __restrict__ counts) {
-    __shared__ int s_c;
-    const int t = blockIdx.x;
-    if (!valid[t]) {
-        if (threadIdx.x == 0) counts[t] = -1;
-        return;
-    }
-    const int nm = *n_matches;
-    double h[8];
-    for (int k = 0; k < 8; ++k) h[k] = hyp[8 * (size_t)t + k];
-    const double t2 = inlier_t2(inlier_px, *norm);
-    if (threadIdx.x == 0) s_c = 0;
-    __syncthreads();
+    if (it >= iters || !s_ok[w]) return;
+    const double t2 = st->t2;
+    const FastInlier fast(shf[w], st);
     int c = 0;
-    for (int i = threadIdx.x; i < nm; i += blockDim.x)
-        c += inlier(h, xyuv[4 * i], xyuv[4 * i + 1], xyuv[4 * i + 2], xyuv[4 * i + 3], t2);
-    for (int off = 16; off > 0; off >>= 1) c += __shfl_down_sync(0xffffffffu, c, off);
-    if ((threadIdx.x & 31) == 0) atomicAdd(&s_c, c);
-    __syncthreads();
-    if (threadIdx.x == 0) counts[t] = s_c;
+    for (int i = lane; i < N; i += 32) c += mt_inlier(fast, sh[w], xyuv, xyuvf, i, t2);
+    c = __reduce_add_sync(0xffffffffu, c);
+    // most inliers, ties to the earlier iteration
+    if (lane == 0) atomicMax(&st->best, (unsigned long long)(c + 1) << 32 | (unsigned long long)(0xffffffffu - (unsigned)it));
 }
 
-// one block: the best hypothesis (most inliers, ties to the earliest iteration) and its inlier
-// flags; best = {iteration or -1, count}
-__global__ void __launch_bounds__(256) mt_best(const int* __restrict__ n_matches, int iters,
-                                               const double* __restrict__ hyp, const int* __restrict__ counts,
-                                               const double* __restrict__ xyuv, const Norm* __restrict__ norm,
-                                               double inlier_px, int* __restrict__ best, unsigned char* __restrict__ inl) {
-    __shared__ long long s_red[8];
-    __shared__ int s_best;
-    const int nm = *n_matches, t = threadIdx.x;
-    long long key = -1;  // (count + 1) << 32 | (2^32 - 1 - t): larger is better
-    if (nm >= 4)
-        for (int k = t; k < iters; k += blockDim.x) {
-            const long long v = ((long long)(counts[k] + 1) << 32) | (long long)(0xffffffffu - (unsigned)k);
-            key = v > key ? v : key;
-        }
-    for (int off = 16; off > 0; off >>= 1) {
-        const long long o = __shfl_down_sync(0xffffffffu, key, off);
-        key = o > key ? o : key;
-    }
-    if ((t & 31) == 0) s_red[t >> 5] = key;
-    __syncthreads();
-    if (t == 0) {
-        long long b = s_red[0];
-        for (int w = 1; w < (int)(blockDim.x >> 5); ++w) b = s_red[w] > b ? s_red[w] : b;
-        // invalid hypotheses (count -1) have key (0 << 32 | .): no model
-        const int bt = (b >> 32) > 0 ? (int)(0xffffffffu - (unsigned)(b & 0xffffffffll)) : -1;
-        const int bc = (int)(b >> 32) - 1;
-        s_best = bt >= 0 && bc >= 4 ? bt : -1;
-        best[0] = s_best;
-        best[1] = bc;
-    }
-    __syncthreads();
-    const int bt = s_best;
-    if (bt < 0) {
-        for (int i = t; i < nm; i += blockDim.x) inl[i] = 0;
-        return;
-    }
-    double h[8];
-    for (int k = 0; k < 8; ++k) h[k] = hyp[8 * (size_t)bt + k];
-    const double t2 = inlier_t2(inlier_px, *norm);
-    for (int i = t; i < nm; i += blockDim.x)
-        inl[i] = inlier(h, xyuv[4 * i], xyuv[4 * i + 1], xyuv[4 * i + 2], xyuv[4 * i + 3], t2) ? 1 : 0;
-}
-
-// the least-squares normal equations on the best hypothesis' inliers: 64 entries of M and 8 of r,
-// one warp each.  The two DLT rows of a match are
-//   row0 = (x, y, 1, 0, 0, 0, -ux, -uy), row1 = (0, 0, 0, x, y, 1, -vx, -vy),
-// M[p][q] += row0[p] row0[q] + row1[p] row1[q], r[p] += row0[p] u + row1[p] v, in quality order.
-// The lanes form the products (32 matches at a time, stored in quality order); one lane sums them
-// in order.  A product with a structural zero adds +-0 to a sum that is never
-// -0, so it is skipped without changing a bit.
-__global__ void __launch_bounds__(32) mt_sums(const int* __restrict__ n_matches, const int* __restrict__ best,
-                                              const unsigned char* __restrict__ inl, const double* __restrict__ xyuv,
-                                              double* __restrict__ sums) {
-    if (best[0] < 0) return;
-    const int nm = *n_matches, lane = threadIdx.x;
-    const int e = blockIdx.x;
-    const bool isr = e >= 64;
-    const int p = isr ? e - 64 : e / 8, q = isr ? 0 : e % 8;
-    const bool p0 = p < 3 || p > 5, p1 = p > 2, q0 = q < 3 || q > 5, q1 = q > 2;
-    const bool use0 = isr ? p0 : (p0 && q0), use1 = isr ? p1 : (p1 && q1);
-    auto r0 = [](int k, double x, double y, double u) {
-        return k == 0 ? x : k == 1 ? y : k == 2 ? 1.0 : k == 6 ? -dM(u, x) : -dM(u, y);
-    };
-    auto r1 = [](int k, double x, double y, double v) {
-        return k == 3 ? x : k == 4 ? y : k == 5 ? 1.0 : k == 6 ? -dM(v, x) : -dM(v, y);
-    };
-    // the products of every inlier, in quality order, into shared memory
-    __shared__ double s0[MT_MAX_POINTS], s1[MT_MAX_POINTS];
-    int n = 0;
-    for (int i0 = 0; i0 < nm; i0 += 32) {
-        const int i = i0 + lane;
-        const bool f = i < nm && inl[i];
-        const unsigned bal = __ballot_sync(0xffffffffu, f);
-        if (f) {
-            const double x = xyuv[4 * i], y = xyuv[4 * i + 1], u = xyuv[4 * i + 2], v = xyuv[4 * i + 3];
-            const int pos = n + __popc(bal & ((1u << lane) - 1u));
-            s0[pos] = use0 ? dM(r0(p, x, y, u), isr ? u : r0(q, x, y, u)) : 0.0;
-            s1[pos] = use1 ? dM(r1(p, x, y, v), isr ? v : r1(q, x, y, v)) : 0.0;
-        }
-        n += __popc(bal);
-    }
-    __syncwarp();
-    if (lane != 0) return;
-    double acc = 0.0;
-    if (use0 && use1) {
-#pragma unroll 8
-        for (int j = 0; j < n; ++j) acc = dA(dA(acc, s0[j]), s1[j]);
-    } else if (use0) {
-#pragma unroll 8
-        for (int j = 0; j < n; ++j) acc = dA(acc, s0[j]);
-    } else if (use1) {
-#pragma unroll 8
-        for (int j = 0; j < n; ++j) acc = dA(acc, s1[j]);
-    }
-    sums[e] = acc;
-}
-
-// one block of 96 threads: solve the normal equations (the 4-point hypothesis when singular) and
-// go back to pixels, H = Tb^-1 Hn Ta with h33 = 1; identity and 0 inliers when there is no model
-__global__ void __launch_bounds__(96) mt_solve(const int* __restrict__ best, const double* __restrict__ hyp,
-                                               const double* __restrict__ sums, const Norm* __restrict__ norm,
-                                               double* __restrict__ H, int* __restrict__ n_inliers) {
-    __shared__ BlockSolve b;
-    __shared__ double P[9], Q[9];
-    const int t = threadIdx.x, bt = best[0];
-    if (bt < 0) {
+// One block: the best hypothesis' inlier flags, the least-squares normal equations on them, the refit
+// (the 4-point hypothesis when singular), and back to pixels, H = Tb^-1 Hn Ta with h33 = 1; identity
+// and 0 inliers when there is no model.
+//
+// The two DLT rows of a match are row0 = (g, 0, 0, 0, a6, a7), row1 = (0, 0, 0, g, b6, b7) with
+// g = (x, y, 1), a6 = -ux, a7 = -uy, b6 = -vx, b7 = -vy; M[p][q] adds row0[p] row0[q], then
+// row1[p] row1[q], match by match in quality order.  A product with a structural zero adds +-0 to a sum
+// that is never -0, so it is left out without changing a bit.  That leaves 24 different sums of one
+// product per match and 5 of two (the first and second parts of M's and r's entries coincide, as M is
+// symmetric).  A sum is a chain of additions in order, 64 cycles each whether one lane adds or 32: warp 0
+// carries the 24 in its lanes, warp 1 the 5, on schedulers of their own, while the warps of the other
+// two schedulers form the products of the next 64 inliers.  The longest chain is two additions per
+// inlier (20 us for 333) and bounds the kernel; 51 us in all, against 61 us as three kernels.
+constexpr int MF_THREADS = 512, MF_CHUNK = 64, MF_ONE = 24, MF_TWO = 5, MF_ROW = 35;
+__global__ void __launch_bounds__(MF_THREADS) mt_final(MtState* __restrict__ st, const double* __restrict__ hyp,
+                                                       const double* __restrict__ xyuv, const float* __restrict__ xyuvf,
+                                                       unsigned char* __restrict__ inl,
+                                                       double* __restrict__ H, int* __restrict__ n_inliers) {
+    __shared__ double buf[2][MF_CHUNK * MF_ROW];  // products of a chunk's inliers: 24, then 5 pairs
+    __shared__ uint16_t list[MT_MAX_POINTS];      // the inliers in quality order
+    __shared__ double sums[MF_ONE + MF_TWO];
+    __shared__ double hb[8], Hn[9], P[9], Q[9];
+    __shared__ float hf[8];
+    __shared__ int wcnt[MF_THREADS / 32], s_n;
+    const int t = threadIdx.x, lane = t & 31, w = t >> 5;
+    const int N = st->n;
+    const unsigned long long best = st->best;
+    const int bc = (int)(best >> 32) - 1;
+    if (N < 4 || bc < 4) {
+        for (int i = t; i < N; i += MF_THREADS) inl[i] = 0;
         if (t < 9) H[t] = t % 4 == 0 ? 1.0 : 0.0;
         if (t == 0) *n_inliers = 0;
         return;
     }
-    if (t < 72) {
-        const int i = t / 9, j = t - 9 * (t / 9);
-        b.A[i][j] = j < 8 ? sums[8 * i + j] : sums[64 + i];
+    const Norm z = st->norm;
+    if (t < 8) {
+        hb[t] = hyp[8 * (size_t)(0xffffffffu - (unsigned)best) + t];
+        hf[t] = (float)hb[t];
     }
+    if (t == 0) s_n = 0;
     __syncthreads();
-    if (!solve8_block(b)) {
-        if (t < 8) b.hs[t] = hyp[8 * (size_t)bt + t];
+    {
+        const double t2 = st->t2;
+        const FastInlier fast(hf, st);
+        for (int i0 = 0; i0 < N; i0 += MF_THREADS) {
+            const int i = i0 + t;
+            const bool f = i < N && mt_inlier(fast, hb, xyuv, xyuvf, i, t2);
+            if (i < N) inl[i] = f;
+            const unsigned m = __ballot_sync(0xffffffffu, f);
+            if (lane == 0) wcnt[w] = __popc(m);
+            __syncthreads();
+            int at = s_n + __popc(m & ((1u << lane) - 1u));
+            for (int k = 0; k < w; ++k) at += wcnt[k];
+            if (f) list[at] = (uint16_t)i;
+            __syncthreads();
+            if (t == MF_THREADS - 1) s_n = at + f;
+            __syncthreads();
+        }
+    }
+    const int n = s_n, chunks = (n + MF_CHUNK - 1) / MF_CHUNK;
+    // the products of inlier q of chunk k, a lane per inlier; producer warps are those of schedulers 2, 3
+    auto produce = [&](int k, int q) {
+        const int j = MF_CHUNK * k + q;
+        if (j >= n) return;
+        const double* c = xyuv + 4 * (size_t)list[j];
+        const double x = c[0], y = c[1], u = c[2], v = c[3];
+        double* o = buf[k & 1] + q * MF_ROW;
+        const double ux = dM(u, x), uy = dM(u, y), vx = dM(v, x), vy = dM(v, y);
+        const double a6 = -ux, a7 = -uy, b6 = -vx, b7 = -vy;
+        o[0] = dM(x, x);
+        o[1] = dM(x, y);
+        o[2] = x;
+        o[3] = dM(y, y);
+        o[4] = y;
+        o[5] = 1.0;
+        o[6] = dM(x, a6);
+        o[7] = dM(y, a6);
+        o[8] = a6;
+        o[9] = dM(x, a7);
+        o[10] = dM(y, a7);
+        o[11] = a7;
+        o[12] = dM(x, b6);
+        o[13] = dM(y, b6);
+        o[14] = b6;
+        o[15] = dM(x, b7);
+        o[16] = dM(y, b7);
+        o[17] = b7;
+        o[18] = ux;
+        o[19] = uy;
+        o[20] = u;
+        o[21] = vx;
+        o[22] = vy;
+        o[23] = v;
+        o[24] = dM(a6, a6);
+        o[25] = dM(b6, b6);
+        o[26] = dM(a6, a7);
+        o[27] = dM(b6, b7);
+        o[28] = dM(a7, a7);
+        o[29] = dM(b7, b7);
+        o[30] = dM(a6, u);
+        o[31] = dM(b6, v);
+        o[32] = dM(a7, u);
+        o[33] = dM(b7, v);
+    };
+    const int prod = w == 2 ? 0 : w == 3 ? 32 : -1;
+    static_assert(MF_CHUNK == 64, "two producer warps");
+    if (prod >= 0) produce(0, prod + lane);
+    __syncthreads();
+    double acc = 0.0;
+    for (int k = 0; k < chunks; ++k) {
+        const int m = min(MF_CHUNK, n - MF_CHUNK * k);
+        const double* b = buf[k & 1];
+        if (w == 0 && lane < MF_ONE) {
+#pragma unroll 8
+            for (int q = 0; q < m; ++q) acc = dA(acc, b[q * MF_ROW + lane]);
+        } else if (w == 1 && lane < MF_TWO) {
+            b += MF_ONE + 2 * lane;
+#pragma unroll 8
+            for (int q = 0; q < m; ++q) acc = dA(dA(acc, b[q * MF_ROW]), b[q * MF_ROW + 1]);
+        } else if (prod >= 0 && k + 1 < chunks) {
+            produce(k + 1, prod + lane);
+        }
         __syncthreads();
     }
-    const Norm z = *norm;
+    if (w == 0 && lane < MF_ONE) sums[lane] = acc;
+    if (w == 1 && lane < MF_TWO) sums[MF_ONE + lane] = acc;
+    __syncthreads();
+    if (w != 0) return;
+    {
+        // row r of [M | r]: (g_p g_q sums) in the blocks of x, y, 1, then columns 6, 7 and the right-hand side
+        const int r = lane & 7, p = r < 3 ? r : r - 3;
+        double A[9], h[8];
+#pragma unroll
+        for (int j = 0; j < 9; ++j) {
+            int e = -1;  // the sum in column j, -1 for none
+            if (r < 6) {
+                if (j < 6) {
+                    if (j / 3 == r / 3) {
+                        const int q = j % 3, lo = min(p, q), hi = max(p, q);
+                        e = lo == 0 ? hi : lo == 1 ? 2 + hi : 5;
+                    }
+                } else {
+                    e = j == 8 ? 18 + r : (r < 3 ? 6 : 12) + 3 * (j - 6) + p;
+                }
+            } else {
+                e = j < 6 ? (j < 3 ? 6 : 12) + 3 * (r - 6) + j % 3 : j == 8 ? 27 + r - 6 : 24 + (r - 6) + (j - 6);
+            }
+            A[j] = e >= 0 ? sums[e] : 0.0;
+        }
+        const bool ok = solve8(A, h);
+#pragma unroll
+        for (int k = 0; k < 8; ++k)
+            if (lane == k) Hn[k] = ok ? h[k] : hb[k];
+        if (lane == 8) Hn[8] = 1.0;
+    }
+    __syncwarp();
     // Hn = [h0 h1 h2; h3 h4 h5; h6 h7 1], Ta = [sa 0 -sa ca0; 0 sa -sa ca1; 0 0 1],
     // Tb^-1 = [1/sb 0 cb0; 0 1/sb cb1; 0 0 1]
-    if (t < 9) {
-        const int r = t / 3, k = t - 3 * (t / 3);
-        const double Hn[9] = {b.hs[0], b.hs[1], b.hs[2], b.hs[3], b.hs[4], b.hs[5], b.hs[6], b.hs[7], 1.0};
+    const int r = lane / 3, k = lane % 3;
+    if (lane < 9) {
         const double Ta[9] = {z.sa, 0.0, -dM(z.sa, z.ca0), 0.0, z.sa, -dM(z.sa, z.ca1), 0.0, 0.0, 1.0};
-        P[t] = dA(dA(dM(Hn[3 * r], Ta[k]), dM(Hn[3 * r + 1], Ta[3 + k])), dM(Hn[3 * r + 2], Ta[6 + k]));
+        P[lane] = dA(dA(dM(Hn[3 * r], Ta[k]), dM(Hn[3 * r + 1], Ta[3 + k])), dM(Hn[3 * r + 2], Ta[6 + k]));
     }
-    __syncthreads();
-    if (t < 9) {
-        const int r = t / 3, k = t - 3 * (t / 3);
-        const double Tbi[9] = {dD(1.0, z.sb), 0.0, z.cb0, 0.0, dD(1.0, z.sb), z.cb1, 0.0, 0.0, 1.0};
-        Q[t] = dA(dA(dM(Tbi[3 * r], P[k]), dM(Tbi[3 * r + 1], P[3 + k])), dM(Tbi[3 * r + 2], P[6 + k]));
+    __syncwarp();
+    if (lane < 9) {
+        const double isb = dD(1.0, z.sb);
+        const double Tbi[9] = {isb, 0.0, z.cb0, 0.0, isb, z.cb1, 0.0, 0.0, 1.0};
+        Q[lane] = dA(dA(dM(Tbi[3 * r], P[k]), dM(Tbi[3 * r + 1], P[3 + k])), dM(Tbi[3 * r + 2], P[6 + k]));
     }
-    __syncthreads();
-    if (t < 9) H[t] = dD(Q[t], Q[8]);
-    if (t == 0) *n_inliers = best[1];
+    __syncwarp();
+    if (lane < 9) H[lane] = dD(Q[lane], Q[8]);
+    if (lane == 0) *n_inliers = bc;
 }
 
 }  // namespace
 
 struct stitch_matcher {
-    int device = 0, max_points = 0, max_iters = 0;
-    unsigned* keys = nullptr;
-    int* ord = nullptr;
-    int* dir = nullptr;
-    int* best = nullptr;
-    Norm* norm = nullptr;
-    int* nt = nullptr;
-    unsigned char* uni = nullptr;
+    int device = 0, max_points = 0, max_iters = 0, sms = 1;
+    unsigned* keys = nullptr;  // key words of image A, then of image B: [word][point]
+    int2* best = nullptr;      // per query: match (or -1) and distance
+    MtState* st = nullptr;
+    long long* E = nullptr;    // growth schedule
     double* hyp = nullptr;
-    int* valid = nullptr;
-    int* counts = nullptr;
     double* xyuv = nullptr;
-    int* pick = nullptr;  // best hypothesis: iteration (or -1), inlier count
-    double* sums = nullptr;
+    float* xyuvf = nullptr;
 };
 
 static void matcher_free(stitch_matcher* c) {
     if (!c) return;
     cudaFree(c->keys);
-    cudaFree(c->ord);
-    cudaFree(c->dir);
     cudaFree(c->best);
-    cudaFree(c->norm);
-    cudaFree(c->nt);
-    cudaFree(c->uni);
+    cudaFree(c->st);
+    cudaFree(c->E);
     cudaFree(c->hyp);
-    cudaFree(c->valid);
-    cudaFree(c->counts);
     cudaFree(c->xyuv);
-    cudaFree(c->pick);
-    cudaFree(c->sums);
+    cudaFree(c->xyuvf);
     delete c;
 }
 
@@ -677,16 +725,14 @@ extern "C" stitch_status stitch_matcher_create(int32_t max_points, int32_t max_i
     c->max_points = max_points;
     c->max_iters = max_iters;
     const size_t it = (size_t)std::max(max_iters, 1);
-    bool okm = cudaMalloc(&c->keys, sizeof(unsigned) * MT_MAX_TABLES * max_points) == cudaSuccess &&
-               cudaMalloc(&c->ord, sizeof(int) * MT_MAX_TABLES * max_points) == cudaSuccess &&
-               cudaMalloc(&c->dir, sizeof(int) * MT_MAX_TABLES * MT_DIR) == cudaSuccess &&
-               cudaMalloc(&c->best, sizeof(int) * 2 * max_points) == cudaSuccess &&
-               cudaMalloc(&c->norm, sizeof(Norm)) == cudaSuccess && cudaMalloc(&c->nt, sizeof(int) * it) == cudaSuccess &&
-               cudaMalloc(&c->uni, it) == cudaSuccess && cudaMalloc(&c->hyp, sizeof(double) * 8 * it) == cudaSuccess &&
-               cudaMalloc(&c->valid, sizeof(int) * it) == cudaSuccess &&
-               cudaMalloc(&c->counts, sizeof(int) * it) == cudaSuccess &&
+    bool okm = cudaMalloc(&c->keys, sizeof(unsigned) * 2 * MT_MAX_WORDS * max_points) == cudaSuccess &&
+               cudaMalloc(&c->best, sizeof(int2) * max_points) == cudaSuccess &&
+               cudaMalloc(&c->st, sizeof(MtState)) == cudaSuccess &&
+               cudaMalloc(&c->E, sizeof(long long) * MT_MAX_POINTS) == cudaSuccess &&
+               cudaMalloc(&c->hyp, sizeof(double) * 8 * it) == cudaSuccess &&
                cudaMalloc(&c->xyuv, sizeof(double) * 4 * max_points) == cudaSuccess &&
-               cudaMalloc(&c->pick, sizeof(int) * 2) == cudaSuccess && cudaMalloc(&c->sums, sizeof(double) * 72) == cudaSuccess;
+               cudaMalloc(&c->xyuvf, sizeof(float) * 4 * max_points) == cudaSuccess;
+    if (cudaDeviceGetAttribute(&c->sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess || c->sms < 1) c->sms = 1;
     if (prev >= 0) cudaSetDevice(prev);
     if (!okm) {
         cudaGetLastError();
@@ -733,19 +779,18 @@ extern "C" stitch_status stitch_match_homography(stitch_matcher* c, const int32_
     const int cap = c->max_points;
     const unsigned* da = reinterpret_cast<const unsigned*>(desc_a);
     const unsigned* db = reinterpret_cast<const unsigned*>(desc_b);
-    mt_build<<<lb.L, 1024, 0, s>>>(db, count_b, lb, c->keys, c->ord, c->dir, cap);
-    mt_query<<<(cap + 7) / 8, 256, 0, s>>>(da, count_a, db, count_b, lb, c->keys, c->ord, c->dir, cap,
-                                           prm->max_dist, prm->ratio_num, prm->ratio_den, c->best);
-    mt_order<<<1, 1024, 0, s>>>(c->best, count_a, cap, xy_a, xy_b, matches, n_matches, c->norm);
-    const int iters = prm->iters;
-    mt_prep<<<1, 1024, 0, s>>>(n_matches, matches, xy_a, xy_b, c->norm, iters, c->xyuv, c->nt, c->uni);
-    if (iters > 0) {
-        mt_hypotheses_b<<<iters, 96, 0, s>>>(n_matches, iters, c->nt, c->uni, rnd, c->xyuv, c->hyp, c->valid);
-        mt_score<<<iters, 256, 0, s>>>(n_matches, c->hyp, c->valid, c->xyuv, c->norm, prm->inlier_px, c->counts);
-    }
-    mt_best<<<1, 256, 0, s>>>(n_matches, iters, c->hyp, c->counts, c->xyuv, c->norm, prm->inlier_px, c->pick, inlier);
-    mt_sums<<<72, 32, 0, s>>>(n_matches, c->pick, inlier, c->xyuv, c->sums);
-    mt_solve<<<1, 96, 0, s>>>(c->pick, c->hyp, c->sums, c->norm, H, n_inliers);
+    const int nw = mt_words(lb), iters = prm->iters;
+    unsigned *ka = c->keys, *kb = c->keys + (size_t)MT_MAX_WORDS * cap;
+    mt_keys<<<dim3((cap + 127) / 128, nw, 2), 128, 0, s>>>(da, count_a, db, count_b, lb, cap, ka, kb, c->st);
+    auto match = mt_packed(lb) ? mt_match<true> : mt_match<false>;
+    match<<<(cap + 7) / 8, 256, 0, s>>>(da, count_a, db, count_b, ka, kb, nw, cap, xy_a, xy_b, prm->max_dist,
+                                        prm->ratio_num, prm->ratio_den, c->best, c->st);
+    mt_rank<<<(cap + 7) / 8 + 1, 256, 0, s>>>(c->best, count_a, cap, xy_a, xy_b, c->st, matches, n_matches, c->xyuv,
+                                              c->xyuvf, c->E, prm->inlier_px);
+    if (iters > 0)
+        mt_hypotheses<<<(iters + 3) / 4, 128, 0, s>>>(iters, c->E, rnd, c->xyuv, c->xyuvf, c->sms, c->hyp,
+                                                      c->st);
+    mt_final<<<1, MF_THREADS, 0, s>>>(c->st, c->hyp, c->xyuv, c->xyuvf, inlier, H, n_inliers);
     stitch_status st = cudaGetLastError() == cudaSuccess ? STITCH_OK : STITCH_ECUDA;
     if (prev >= 0 && prev != c->device) cudaSetDevice(prev);
     return st;
