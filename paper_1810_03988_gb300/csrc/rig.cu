@@ -320,6 +320,10 @@ stitch_status stitch_rig_create(const stitch_rig_desc* desc, int device, stitch_
     stitch_rig* r = new (std::nothrow) stitch_rig();
     if (!r) return STITCH_ENOMEM;
     r->device = device;
+    if (cudaDeviceGetAttribute(&r->sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess) {
+        cudaGetLastError();
+        r->sms = 1;
+    }
     r->desc = *desc;
     r->cams.assign(desc->cameras, desc->cameras + desc->num_cameras);
     r->desc.cameras = nullptr;

@@ -145,10 +145,9 @@ extern "C" stitch_status stitch_frames_static(const stitch_rig_desc* desc, const
             for (int l = 0; l < g.levels; ++l) {
                 if (!cv.take(sizeof(float4) * (size_t)c.Om[l].area(), &p)) return STITCH_ETOOLARGE;
                 c.G[l] = (float4*)p;
-                if (l + 1 < g.levels) {
-                    if (!cv.take(sizeof(float4) * (size_t)c.Z[l].area(), &p)) return STITCH_ETOOLARGE;
-                    c.Lp[l] = (float4*)p;
-                }
+                // room for the camera's Laplacian bands, which the kernels no longer store: what fits
+                // the array stays what it was
+                if (l + 1 < g.levels && !cv.take(sizeof(float4) * (size_t)c.Z[l].area(), &p)) return STITCH_ETOOLARGE;
             }
         }
         for (int l = 0; l < g.levels; ++l) {
@@ -162,6 +161,10 @@ extern "C" stitch_status stitch_frames_static(const stitch_rig_desc* desc, const
     static_assert(sizeof(r.hcam) == sizeof(CamPack), "descriptor pack layout");
     k_put_cams<<<1, 256, 0, s>>>(*reinterpret_cast<const CamPack*>(r.hcam), g.ncam, r.dcam);
     if (cudaGetLastError() != cudaSuccess) return STITCH_ECUDA;
+    int dev = -1;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&r.sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+        return STITCH_ECUDA;
     OutDesc od{out, out_pitch, desc->out_float};
     return plain_frames(&r, fp, od, s);
 }

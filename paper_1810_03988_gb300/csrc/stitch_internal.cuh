@@ -35,7 +35,6 @@ struct CamDev {
     Rect Z[MAXL];    // Z^l: region where the camera's weight pyramid can be non-zero
     // plain path buffers
     float4* G[MAXL];   // Gaussian pyramid (r, g, b, weight) on Om[l], row pitch Om[l].w()
-    float4* Lp[MAXL];  // (Laplacian r, g, b, weight) on Z[l] for l < L-1, row pitch Z[l].w()
     // fused path buffers
     void* FG[MAXL];    // Gaussian pyramid (r, g, b, weight) on Om[l] for l >= 1 (FP32 or FP16)
 };
@@ -501,12 +500,13 @@ struct ProfMark {
 
 struct stitch_rig {
     int device = 0;
+    int sms = 0;  // of the device (plain path)
     stitch_rig_desc desc{};
     std::vector<stitch_camera> cams;
     RigGeom geom{};
     CamDev hcam[MAXC]{};
     CamDev* dcam = nullptr;
-    float4* Bl[MAXL]{};  // plain path: blended band / collapse buffer per level (full level grid)
+    float4* Bl[MAXL]{};  // plain path: collapsed R^l of level l >= 1 (full level grid)
     std::vector<void*> allocs;
     std::vector<std::pair<uint32_t*, size_t>> guards;  // debug build: guard bands (words)
     long long scratch_bytes = 0;
