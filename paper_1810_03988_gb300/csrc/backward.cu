@@ -39,13 +39,18 @@ struct BwTile {
 // A (tile, candidate camera) slot: the camera's map anchored in the tile, from the call's parameters.
 struct __align__(16) BwMap {
     TileMap tm;
-    int ax, ay;   // anchor: dx, dy are taken from it
+    float fu0, fv0;  // U0, V0
+    float ox, oy;    // tile origin minus anchor: dx, dy are taken from the anchor
     float gain;
     int cam, W, H;
-    int cx, cy;   // local origin
-    int pos;      // position of the slot's partials: the slots of a camera in a row, in tile order
+    float wm, hm;    // W - 0.5, H - 0.5
+    int cx, cy;      // tile origin minus the camera's local origin
+    int pos;         // position of the slot's partials: the slots of a camera in a row, in tile order
+    int active;      // 0: no pixel of the tile can lie in the camera's image
+    int pad[3];
 };
-static_assert(sizeof(BwMap) == 80, "read as five 16-byte words");
+constexpr int BW_MAP_WORDS = sizeof(BwMap) / 16;
+static_assert(sizeof(BwMap) == 112, "read as 16-byte words");
 
 // One camera's sample at a pixel: bilinear value and its derivatives (before gain, in [0,1] units).
 struct GSample {
@@ -53,65 +58,48 @@ struct GSample {
 };
 
 // The source position lies in the camera's image (and in front of the camera).
-__device__ __forceinline__ bool gvalid(const Pos& p, int W, int H) {
-    return (p.den > 0.f) & (p.u >= -0.5f) & (p.u < (float)W - 0.5f) & (p.v >= -0.5f) & (p.v < (float)H - 0.5f);
+__device__ __forceinline__ bool gvalid(const Pos& p, const BwMap& m) {
+    return (p.den > 0.f) & (p.u >= -0.5f) & (p.u < m.wm) & (p.v >= -0.5f) & (p.v < m.hm);
 }
 
-// Byte j of w as a float (exact).
-__device__ __forceinline__ float byte_f(unsigned w, unsigned j) {
-    return __uint_as_float(__byte_perm(w, 0x4B000000u, 0x7440u | j)) - 8388608.0f;
-}
-
-// The sample at p.  Two neighbouring RGB texels are 6 bytes at any offset: where base and pitch allow
-// it and the 12 bytes from the first one's word on lie in the row, they are two or three aligned
-// 32-bit loads per row and a funnel shift instead of six byte loads.
-__device__ __forceinline__ void gsample(const uint8_t* __restrict__ px, long long pitch, int W, int H, const Pos& p,
-                                        bool words, GSample& s) {
+// The sample at p.  The texel values enter as 2^23 + byte, whose differences are those of the bytes,
+// R and G as one pair.
+__device__ __forceinline__ void gsample(const uint8_t* __restrict__ px, long long pitch, const BwMap& m, const Pos& p,
+                                        GSample& s) {
     int i0, j0;
     float fx, fy;
     bool cu = false, cv = false;
     if (p.iu < 0) { i0 = 0; fx = 0.f; cu = true; }
-    else if (p.iu >= W - 1) { i0 = W - 1; fx = 0.f; cu = true; }
+    else if (p.iu >= m.W - 1) { i0 = m.W - 1; fx = 0.f; cu = true; }
     else { i0 = p.iu; fx = p.fu; }
     if (p.iv < 0) { j0 = 0; fy = 0.f; cv = true; }
-    else if (p.iv >= H - 1) { j0 = H - 1; fy = 0.f; cv = true; }
+    else if (p.iv >= m.H - 1) { j0 = m.H - 1; fy = 0.f; cv = true; }
     else { j0 = p.iv; fy = p.fv; }
     // an exact integer u = W-1 sits on the last texel: one-sided derivative there is 0 as well
-    const long long dj = (j0 + 1 < H) ? pitch : 0;
     const uint8_t* a = px + (long long)j0 * pitch + 3 * i0;
-    const uint8_t* b = a + dj;
-    unsigned ta, tb, ua, ub;  // the first four bytes (R G B R) and the last two (G B) of both rows
-    const int off = (3 * i0) & 3;
-    if (words && 3 * i0 - off + 12 <= 3 * W) {
-        const unsigned* wa = reinterpret_cast<const unsigned*>(a - off);
-        const unsigned* wb = reinterpret_cast<const unsigned*>(b - off);
-        const unsigned a0 = __ldg(wa), a1 = __ldg(wa + 1), b0 = __ldg(wb), b1 = __ldg(wb + 1);
-        unsigned a2 = 0u, b2 = 0u;
-        if (off == 3) {
-            a2 = __ldg(wa + 2);
-            b2 = __ldg(wb + 2);
-        }
-        ta = __funnelshift_r(a0, a1, 8 * off);
-        ua = __funnelshift_r(a1, a2, 8 * off);
-        tb = __funnelshift_r(b0, b1, 8 * off);
-        ub = __funnelshift_r(b1, b2, 8 * off);
-    } else {
-        const int di = (i0 + 1 < W) ? 3 : 0;
-        ta = (unsigned)__ldg(a) | (unsigned)__ldg(a + 1) << 8 | (unsigned)__ldg(a + 2) << 16 | (unsigned)__ldg(a + di) << 24;
-        ua = (unsigned)__ldg(a + di + 1) | (unsigned)__ldg(a + di + 2) << 8;
-        tb = (unsigned)__ldg(b) | (unsigned)__ldg(b + 1) << 8 | (unsigned)__ldg(b + 2) << 16 | (unsigned)__ldg(b + di) << 24;
-        ub = (unsigned)__ldg(b + di + 1) | (unsigned)__ldg(b + di + 2) << 8;
+    const Texels q = load_texels(a, a + (j0 + 1 < m.H ? pitch : 0), i0, m.W, word_aligned(px, pitch));
+    constexpr float K23 = 8388608.0f, k255 = 1.0f / 255.0f;
+    {
+        const float2 a00 = make_float2(byte_f23(q.t00, 0), byte_f23(q.t00, 1)), a01 = make_float2(byte_f23(q.t01, 0), byte_f23(q.t01, 1));
+        const float2 a10 = make_float2(byte_f23(q.t10, 0), byte_f23(q.t10, 1)), a11 = make_float2(byte_f23(q.t11, 0), byte_f23(q.t11, 1));
+        const float2 d0 = f2sub(a01, a00), d1 = f2sub(a11, a10);
+        const float2 top = f2fma(f2(fx), d0, f2sub(a00, f2(K23))), bot = f2fma(f2(fx), d1, f2sub(a10, f2(K23)));
+        const float2 dv = f2sub(bot, top);
+        const float2 b = f2mul(f2fma(f2(fy), dv, top), f2(k255)), bu = f2mul(f2fma(f2(fy), f2sub(d1, d0), d0), f2(k255)),
+                     bv = f2mul(dv, f2(k255));
+        s.b[0] = b.x;
+        s.b[1] = b.y;
+        s.bu[0] = cu ? 0.f : bu.x;
+        s.bu[1] = cu ? 0.f : bu.y;
+        s.bv[0] = cv ? 0.f : bv.x;
+        s.bv[1] = cv ? 0.f : bv.y;
     }
-    const float k255 = 1.0f / 255.0f;
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-        const float p00 = byte_f(ta, c), p01 = c == 0 ? byte_f(ta, 3) : byte_f(ua, c - 1);
-        const float p10 = byte_f(tb, c), p11 = c == 0 ? byte_f(tb, 3) : byte_f(ub, c - 1);
-        const float top = fmaf(fx, p01 - p00, p00), bot = fmaf(fx, p11 - p10, p10);
-        s.b[c] = fmaf(fy, bot - top, top) * k255;
-        s.bu[c] = cu ? 0.f : fmaf(fy, (p11 - p10) - (p01 - p00), p01 - p00) * k255;
-        s.bv[c] = cv ? 0.f : (bot - top) * k255;
-    }
+    const float b00 = byte_f23(q.t00, 2), b01 = byte_f23(q.t01, 2), b10 = byte_f23(q.t10, 2), b11 = byte_f23(q.t11, 2);
+    const float d0 = b01 - b00, d1 = b11 - b10;
+    const float top = fmaf(fx, d0, b00 - K23), bot = fmaf(fx, d1, b10 - K23);
+    s.b[2] = fmaf(fy, bot - top, top) * k255;
+    s.bu[2] = cu ? 0.f : fmaf(fy, d1 - d0, d0) * k255;
+    s.bv[2] = cv ? 0.f : (bot - top) * k255;
 }
 
 __device__ __forceinline__ float warp_sum(float v) {
@@ -124,10 +112,12 @@ __device__ __forceinline__ float warp_sum(float v) {
 // warp has one lane active or 32, so this work in the first threads of every tile's block (60 double
 // operations in 2 to 4 lanes) cost the 8150 tiles of 4 x 1080p about 50 us of the FP64 pipe; with full warps
 // it is 7 us for all of them.
-__global__ void __launch_bounds__(64) k_backward_maps(const CamDev* __restrict__ cams, const double* __restrict__ params,
+__global__ void __launch_bounds__(64) k_backward_maps(const CamDev* __restrict__ cams, const double* params,
                                                       const int4* __restrict__ slots, int nslots,
                                                       const int* __restrict__ centers, int canvas_w, int canvas_h,
-                                                      BwMap* __restrict__ maps) {
+                                                      BwMap* maps) {
+    pdl_trigger();
+    pdl_wait();
     const int q = blockIdx.x * 64 + threadIdx.x;
     if (q >= nslots) return;
     const int4 sl = slots[q];  // tile origin, camera, position of the partials
@@ -137,8 +127,7 @@ __global__ void __launch_bounds__(64) k_backward_maps(const CamDev* __restrict__
     // anchor at the tile origin clamped into the canvas; w > 0 there for every candidate is
     // not guaranteed, so anchor where w is largest among the tile corners
     BwMap m;
-    m.ax = sl.x;
-    m.ay = sl.y;
+    int ax = sl.x, ay = sl.y;
     double best = -1e300;
     for (int k = 0; k < 4; ++k) {
         const int x = min(sl.x + (k & 1) * (BW_TX - 1), canvas_w - 1);
@@ -146,18 +135,39 @@ __global__ void __launch_bounds__(64) k_backward_maps(const CamDev* __restrict__
         const double w = A[6] * x + A[7] * y + A[8];
         if (w > best) {
             best = w;
-            m.ax = x;
-            m.ay = y;
+            ax = x;
+            ay = y;
         }
     }
-    m.tm = make_tile_map(A, m.ax, m.ay);
+    m.tm = make_tile_map(A, ax, ay);
+    m.fu0 = (float)m.tm.U0;
+    m.fv0 = (float)m.tm.V0;
+    m.ox = (float)(sl.x - ax);
+    m.oy = (float)(sl.y - ay);
     m.gain = (float)p[8];
     m.cam = c;
     m.W = cams[c].W;
     m.H = cams[c].H;
-    m.cx = centers[2 * c];
-    m.cy = centers[2 * c + 1];
+    m.wm = (float)m.W - 0.5f;
+    m.hm = (float)m.H - 0.5f;
+    m.cx = sl.x - centers[2 * c];
+    m.cy = sl.y - centers[2 * c + 1];
     m.pos = sl.w;
+    // the tile maps to the hull of its corners' images where w stays well away from 0: beyond one side
+    // of the image by half a pixel more than validity asks, none of its pixels is valid
+    float wlo = 3e38f, whi = 0.f, ulo = 3e38f, uhi = -3e38f, vlo = 3e38f, vhi = -3e38f;
+    for (int k = 0; k < 4; ++k) {
+        const Pos c4 = map_pos(m.tm, m.fu0, m.fv0, m.ox + (float)((k & 1) * (BW_TX - 1)), m.oy + (float)((k >> 1) * (BW_TY - 1)));
+        wlo = fminf(wlo, c4.den);
+        whi = fmaxf(whi, c4.den);
+        ulo = fminf(ulo, c4.u);
+        uhi = fmaxf(uhi, c4.u);
+        vlo = fminf(vlo, c4.v);
+        vhi = fmaxf(vhi, c4.v);
+    }
+    const bool out = wlo > 0.25f * whi && (uhi < -1.f || ulo > m.wm + 0.5f || vhi < -1.f || vlo > m.hm + 0.5f);
+    m.active = out ? 0 : 1;
+    m.pad[0] = m.pad[1] = m.pad[2] = 0;
     maps[q] = m;
 }
 
@@ -217,19 +227,32 @@ struct WarpSums<M, 0, BASE> {
 
 // A tile with at most N candidate cameras: validity from the positions first, then one sample per
 // valid camera of the pixels that at least two see, kept in registers for both the sum and the
-// gradient.  Bound by instruction issue: 57 + 80 us for the 4727 + 3423 tiles of 4 x 1080p, against 227 us when
+// gradient.  Bound by instruction issue: 56 + 75 us for the 4727 + 3423 tiles of 4 x 1080p, against 227 us when
 // every candidate was sampled twice at every pixel, from byte loads, with 5 shuffles for each of 40 sums.
 template <int N>
-__global__ void __launch_bounds__(BW_THREADS, N == 2 ? 4 : 2) k_backward(const FramePtrs fp, const BwMap* __restrict__ maps,
+__global__ void __launch_bounds__(BW_THREADS, N == 2 ? 4 : 2) k_backward(const FramePtrs fp, const BwMap* maps,
                                                                         const BwTile* __restrict__ tiles, int canvas_w,
-                                                                        int canvas_h, float* __restrict__ partials, int nslots,
-                                                                        float* __restrict__ loss_partials) {
+                                                                        int canvas_h, float* partials, int nslots,
+                                                                        float* loss_partials) {
     __shared__ __align__(16) BwMap m[N];
     __shared__ float red[BW_THREADS / 32][N * BW_NV + 1];
     const BwTile tl = tiles[blockIdx.x];
     const int n = tl.count, t = threadIdx.x, lane = t & 31, warp = t >> 5;
-    if (t < 5 * n) reinterpret_cast<int4*>(m)[t] = reinterpret_cast<const int4*>(maps + tl.first)[t];
+    pdl_trigger();
+    pdl_wait();
+    if (t < BW_MAP_WORDS * n) reinterpret_cast<int4*>(m)[t] = reinterpret_cast<const int4*>(maps + tl.first)[t];
     __syncthreads();
+    auto no_overlap = [&]() {  // only zeros: no two cameras see a pixel of the tile
+        if (t < n * BW_NV) partials[(long long)(t % BW_NV) * nslots + m[t / BW_NV].pos] = 0.f;
+        if (t == 0) loss_partials[tl.id] = 0.f;
+    };
+    int seen = 0;
+#pragma unroll
+    for (int a = 0; a < N; ++a) seen += a < n && m[a].active;
+    if (seen < 2) {
+        no_overlap();
+        return;
+    }
     float loss = 0.f;
     float acc[N * BW_NV];
 #pragma unroll
@@ -237,17 +260,17 @@ __global__ void __launch_bounds__(BW_THREADS, N == 2 ? 4 : 2) k_backward(const F
     bool some = false;
 #pragma unroll 1
     for (int k = 0; k < BW_PPT; ++k) {
-        const int q = t + k * BW_THREADS;
-        const int x = tl.x0 + q % BW_TX, y = tl.y0 + q / BW_TX;
+        const int dx = t % BW_TX, dy = t / BW_TX + k * (BW_THREADS / BW_TX), x = tl.x0 + dx, y = tl.y0 + dy;
+        const float fdx = (float)dx, fdy = (float)dy;
         Pos p[N];
         bool ok[N];
         int kv = 0;
 #pragma unroll
         for (int a = 0; a < N; ++a) {
             ok[a] = false;
-            if (a < n) {
-                p[a] = map_pos(m[a].tm, (float)m[a].tm.U0, (float)m[a].tm.V0, (float)(x - m[a].ax), (float)(y - m[a].ay));
-                ok[a] = gvalid(p[a], m[a].W, m[a].H);
+            if (a < n && m[a].active) {
+                p[a] = map_pos(m[a].tm, m[a].fu0, m[a].fv0, m[a].ox + fdx, m[a].oy + fdy);
+                ok[a] = gvalid(p[a], m[a]);
             }
             kv += ok[a];
         }
@@ -261,7 +284,7 @@ __global__ void __launch_bounds__(BW_THREADS, N == 2 ? 4 : 2) k_backward(const F
             const int c = m[a].cam;
             const uint8_t* px = fp.p[c];
             const long long pitch = fp.pitch[c];
-            gsample(px, pitch, m[a].W, m[a].H, p[a], ((reinterpret_cast<uintptr_t>(px) | (uintptr_t)pitch) & 3) == 0, s[a]);
+            gsample(px, pitch, m[a], p[a], s[a]);
 #pragma unroll
             for (int ch = 0; ch < 3; ++ch) S[ch] = fmaf(m[a].gain, s[a].b[ch], S[ch]);
         }
@@ -275,14 +298,13 @@ __global__ void __launch_bounds__(BW_THREADS, N == 2 ? 4 : 2) k_backward(const F
             // with the mean m = S/k, sum_{i<j} |I_i - I_j|^2 = k sum_i |I_i - m|^2
             // = sum_i |r_i|^2 / k; r_i is small and accurate, so no cancellation
             loss += (r[0] * r[0] + r[1] * r[1] + r[2] * r[2]) / (float)kv;
-            grad_terms(s[a], p[a], r, g, (float)(x - m[a].cx), (float)(y - m[a].cy), acc + a * BW_NV);
+            grad_terms(s[a], p[a], r, g, (float)(m[a].cx + dx), (float)(m[a].cy + dy), acc + a * BW_NV);
         }
     }
     // block reduction: warp sums, then a tree over warps; a tile (or warp) that no two cameras see has
     // only zeros
     if (!__syncthreads_or(some)) {
-        if (t < n * BW_NV) partials[(long long)(t % BW_NV) * nslots + m[t / BW_NV].pos] = 0.f;
-        if (t == 0) loss_partials[tl.id] = 0.f;
+        no_overlap();
         return;
     }
     using Sums = WarpSums<N * BW_NV, 16>;
@@ -310,25 +332,27 @@ __global__ void __launch_bounds__(BW_THREADS, N == 2 ? 4 : 2) k_backward(const F
 
 // Tiles with more candidates (up to MAXC), in groups of BW_SLOTS cameras: samples are taken again for
 // the gradient, as registers do not hold them all.
-__global__ void __launch_bounds__(BW_THREADS) k_backward_many(const FramePtrs fp, const BwMap* __restrict__ maps,
+__global__ void __launch_bounds__(BW_THREADS) k_backward_many(const FramePtrs fp, const BwMap* maps,
                                                               const BwTile* __restrict__ tiles, int canvas_w, int canvas_h,
-                                                              float* __restrict__ partials, int nslots,
-                                                              float* __restrict__ loss_partials) {
+                                                              float* partials, int nslots,
+                                                              float* loss_partials) {
     __shared__ __align__(16) BwMap m[MAXC];
     __shared__ float red[BW_THREADS / 32][BW_SLOTS * BW_NV + 1];
     const BwTile tl = tiles[blockIdx.x];
     const int n = tl.count;  // <= MAXC
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
-    static_assert(5 * MAXC <= BW_THREADS, "one 16-byte word per thread");
-    if (t < 5 * n) reinterpret_cast<int4*>(m)[t] = reinterpret_cast<const int4*>(maps + tl.first)[t];
+    pdl_trigger();
+    pdl_wait();
+    static_assert(BW_MAP_WORDS * MAXC <= BW_THREADS, "one 16-byte word per thread");
+    if (t < BW_MAP_WORDS * n) reinterpret_cast<int4*>(m)[t] = reinterpret_cast<const int4*>(maps + tl.first)[t];
     __syncthreads();
-    auto pos_of = [&](int a, int x, int y) {
-        return map_pos(m[a].tm, (float)m[a].tm.U0, (float)m[a].tm.V0, (float)(x - m[a].ax), (float)(y - m[a].ay));
+    auto pos_of = [&](int a, int dx, int dy) {
+        return map_pos(m[a].tm, m[a].fu0, m[a].fv0, m[a].ox + (float)dx, m[a].oy + (float)dy);
     };
     auto sample = [&](int a, const Pos& p, GSample& s) {
         const uint8_t* px = fp.p[m[a].cam];
         const long long pitch = fp.pitch[m[a].cam];
-        gsample(px, pitch, m[a].W, m[a].H, p, ((reinterpret_cast<uintptr_t>(px) | (uintptr_t)pitch) & 3) == 0, s);
+        gsample(px, pitch, m[a], p, s);
     };
     float loss = 0.f;
     for (int g0 = 0; g0 < n; g0 += BW_SLOTS) {
@@ -339,15 +363,15 @@ __global__ void __launch_bounds__(BW_THREADS) k_backward_many(const FramePtrs fp
             for (int v = 0; v < BW_NV; ++v) acc[s][v] = 0.f;
 #pragma unroll
         for (int k = 0; k < BW_PPT; ++k) {
-            const int q = t + k * BW_THREADS;
-            const int x = tl.x0 + q % BW_TX, y = tl.y0 + q / BW_TX;
-            if (x >= canvas_w || y >= canvas_h) continue;
+            const int dx = t % BW_TX, dy = t / BW_TX + k * (BW_THREADS / BW_TX);
+            if (tl.x0 + dx >= canvas_w || tl.y0 + dy >= canvas_h) continue;
             // pass 1: number of valid cameras and the sum of their intensities
             int kv = 0;
             float S[3] = {0.f, 0.f, 0.f};
             for (int a = 0; a < n; ++a) {
-                const Pos p = pos_of(a, x, y);
-                if (!gvalid(p, m[a].W, m[a].H)) continue;
+                if (!m[a].active) continue;
+                const Pos p = pos_of(a, dx, dy);
+                if (!gvalid(p, m[a])) continue;
                 GSample s;
                 sample(a, p, s);
                 ++kv;
@@ -359,8 +383,9 @@ __global__ void __launch_bounds__(BW_THREADS) k_backward_many(const FramePtrs fp
             for (int a = 0; a < n; ++a) {
                 const int slot = a - g0;
                 if (g0 > 0 && (slot < 0 || slot >= BW_SLOTS)) continue;
-                const Pos p = pos_of(a, x, y);
-                if (!gvalid(p, m[a].W, m[a].H)) continue;
+                if (!m[a].active) continue;
+                const Pos p = pos_of(a, dx, dy);
+                if (!gvalid(p, m[a])) continue;
                 GSample s;
                 sample(a, p, s);
                 const float g = m[a].gain;
@@ -371,7 +396,7 @@ __global__ void __launch_bounds__(BW_THREADS) k_backward_many(const FramePtrs fp
                 // unrolled slot selection keeps the accumulators in registers
 #pragma unroll
                 for (int ss = 0; ss < BW_SLOTS; ++ss)
-                    if (ss == slot) grad_terms(s, p, r, g, (float)(x - m[a].cx), (float)(y - m[a].cy), acc[ss]);
+                    if (ss == slot) grad_terms(s, p, r, g, (float)(m[a].cx + dx), (float)(m[a].cy + dy), acc[ss]);
             }
         }
         // block reduction of this group's slots: warp sums, then a tree over warps
@@ -413,7 +438,7 @@ __device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
 // adds every 256th value from lo + t on, a tree adds the threads' pairs.  The loads of 8 values per
 // run are in flight before their additions.
 template <int NS>
-__device__ __forceinline__ void block_csums(const float* __restrict__ x, long long stride, int lo, int hi, double S[NS]) {
+__device__ __forceinline__ void block_csums(const float* x, long long stride, int lo, int hi, double S[NS]) {
     __shared__ float sh_s[NS][256], sh_c[NS][256];
     constexpr int D = 8;
     const int t = threadIdx.x;
@@ -425,7 +450,7 @@ __device__ __forceinline__ void block_csums(const float* __restrict__ x, long lo
 #pragma unroll
         for (int d = 0; d < D; ++d)
 #pragma unroll
-            for (int v = 0; v < NS; ++v) r[v][d] = k0 + d * 256 < hi ? __ldg(x + v * stride + k0 + d * 256) : 0.f;
+            for (int v = 0; v < NS; ++v) r[v][d] = k0 + d * 256 < hi ? __ldcg(x + v * stride + k0 + d * 256) : 0.f;
 #pragma unroll
         for (int d = 0; d < D; ++d) {
             if (k0 + d * 256 >= hi) break;
@@ -464,11 +489,13 @@ __device__ __forceinline__ void block_csums(const float* __restrict__ x, long lo
 // blocks share its walk over the partials; a further block (0, ncam) sums the loss.  A chain of
 // latencies: 8 us for the 8150 tiles of 4 x 1080p, against 29 us with a block per camera that
 // reached each slot's terms through an index.
-__global__ void __launch_bounds__(256) k_backward_final(int ncam, const float* __restrict__ partials, int nslots,
-                                                         const float* __restrict__ loss_partials, int ntiles,
+__global__ void __launch_bounds__(256) k_backward_final(int ncam, const float* partials, int nslots,
+                                                         const float* loss_partials, int ntiles,
                                                          const int* __restrict__ cam_slot_start,
                                                          const int* __restrict__ centers, double* __restrict__ loss,
                                                          double* __restrict__ grad) {
+    pdl_trigger();
+    pdl_wait();
     const int b = blockIdx.y, g = blockIdx.x;
     double S[3];
     if (b == ncam) {
@@ -591,20 +618,20 @@ stitch_status backward_run(stitch_rig* r, const FramePtrs& fp, const double* par
     const RigGeom& g = r->geom;
     if (bs->ntiles > 0) {
         prof_mark(r, "backward_maps", s);
-        k_backward_maps<<<(bs->nslots + 63) / 64, 64, 0, s>>>(r->dcam, params, bs->slots, bs->nslots, bs->centers, g.nx[0],
-                                                              g.ny[0], bs->maps);
+        pdl_launch(k_backward_maps, (bs->nslots + 63) / 64, 64, 0, s, r->dcam, params, bs->slots, bs->nslots, bs->centers,
+                   g.nx[0], g.ny[0], bs->maps);
         const BwTile* tl = bs->tiles;
         for (int k = 0; k < BW_CLASSES; tl += bs->nclass[k++]) {
             if (bs->nclass[k] == 0) continue;
             prof_mark(r, "backward", s);
             auto fn = k == 0 ? k_backward<2> : k == 1 ? k_backward<4> : k_backward_many;
-            fn<<<bs->nclass[k], BW_THREADS, 0, s>>>(fp, bs->maps, tl, g.nx[0], g.ny[0], bs->partials, bs->nslots,
-                                                    bs->loss_partials);
+            pdl_launch(fn, bs->nclass[k], BW_THREADS, 0, s, fp, bs->maps, tl, g.nx[0], g.ny[0], bs->partials, bs->nslots,
+                       bs->loss_partials);
         }
     }
     prof_mark(r, "backward_final", s);
-    k_backward_final<<<dim3(4, g.ncam + 1), 256, 0, s>>>(g.ncam, bs->partials, bs->nslots, bs->loss_partials, bs->ntiles,
-                                                         bs->cam_slot_start, bs->centers, loss, grad);
+    pdl_launch(k_backward_final, dim3(4, g.ncam + 1), 256, 0, s, g.ncam, bs->partials, bs->nslots, bs->loss_partials,
+               bs->ntiles, bs->cam_slot_start, bs->centers, loss, grad);
     return launch_status();
 }
 

@@ -149,18 +149,6 @@ struct UpTile {
 };
 
 // ------------------------------------------------------------------------------------------------
-// packed single-precision pairs (f32x2: two IEEE binary32 lanes, each rounded exactly as the
-// scalar operation), used where the path computes on pairs of channels
-
-__device__ __forceinline__ float2 f2fma(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
-__device__ __forceinline__ float2 f2add(float2 a, float2 b) { return __fadd2_rn(a, b); }
-// a - b as a + (-1) b: the product is exact, so this is the rounded difference, bit for bit
-__device__ __forceinline__ float2 f2sub(float2 a, float2 b) { return __ffma2_rn(b, make_float2(-1.0f, -1.0f), a); }
-__device__ __forceinline__ float2 f2mul(float2 a, float2 b) { return __fmul2_rn(a, b); }
-__device__ __forceinline__ float2 f2add_rm(float2 a, float2 b) { return __fadd2_rd(a, b); }  // toward -infinity
-
-__device__ __forceinline__ float2 f2(float v) { return make_float2(v, v); }
-
 // (r, g, b, weight) as two pairs
 struct V4 {
     float2 a, b;
@@ -310,13 +298,16 @@ __device__ __forceinline__ void stage_footprint(uint32_t* __restrict__ foot, con
         return;
     }
     constexpr int SG = D1Cap<CAP>::SG;
+    // q / gpr as (q m) >> 20: m is above 2^20 / gpr by less than 3, and 3 gpr q < 2^20
+    static_assert(3 * (CAP / 4) * (SG * D1_THREADS - 1) < 1 << 20, "exact quotients");
+    const int m = (int)__fdividef(1048576.0f, (float)gpr) + 2;
     uint32_t w[SG][3];
 #pragma unroll
     for (int k = 0; k < SG; ++k) {
         const int q = t + k * D1_THREADS;
         w[k][0] = w[k][1] = w[k][2] = 0u;
         if (q < ng) {
-            const int rr = q / gpr, gx = q - rr * gpr;
+            const int rr = (q * m) >> 20, gx = q - rr * gpr;
             const int u0 = fx0 + 4 * gx;
             const uint8_t* src = px + (long long)(fy0 + rr) * pitch + 3 * u0;
             if (u0 + 4 <= W) {
@@ -345,9 +336,6 @@ __device__ __forceinline__ void stage_footprint(uint32_t* __restrict__ foot, con
     }
 }
 
-// 2^23 + byte j of w, as a float (exact)
-__device__ __forceinline__ float d1_bf(uint32_t w, uint32_t j) { return __uint_as_float(__byte_perm(w, 0x4B000000u, 0x7440u | j)); }
-
 // Bilinear RGB of four texel words with fractions (fx, fy), times `scale`.  The arithmetic is that
 // of sample_rgb (top = p00 + fx (p01 - p00), bot likewise, value = top + fy (bot - top), then the
 // scale), on exact 2^23-offset values whose differences are the byte differences, so the result
@@ -355,13 +343,13 @@ __device__ __forceinline__ float d1_bf(uint32_t w, uint32_t j) { return __uint_a
 __device__ __forceinline__ void d1_bilerp(uint32_t w00, uint32_t w01, uint32_t w10, uint32_t w11, float fx, float fy,
                                           float scale, V4& s) {
     constexpr float K23 = 8388608.0f;
-    const float2 a00 = make_float2(d1_bf(w00, 0), d1_bf(w00, 1)), a01 = make_float2(d1_bf(w01, 0), d1_bf(w01, 1));
-    const float2 a10 = make_float2(d1_bf(w10, 0), d1_bf(w10, 1)), a11 = make_float2(d1_bf(w11, 0), d1_bf(w11, 1));
+    const float2 a00 = make_float2(byte_f23(w00, 0), byte_f23(w00, 1)), a01 = make_float2(byte_f23(w01, 0), byte_f23(w01, 1));
+    const float2 a10 = make_float2(byte_f23(w10, 0), byte_f23(w10, 1)), a11 = make_float2(byte_f23(w11, 0), byte_f23(w11, 1));
     const float2 fxx = f2(fx), fyy = f2(fy);
     const float2 top = f2fma(fxx, f2sub(a01, a00), f2sub(a00, f2(K23)));
     const float2 bot = f2fma(fxx, f2sub(a11, a10), f2sub(a10, f2(K23)));
     s.a = f2mul(f2fma(fyy, f2sub(bot, top), top), f2(scale));
-    const float b00 = d1_bf(w00, 2), b01 = d1_bf(w01, 2), b10 = d1_bf(w10, 2), b11 = d1_bf(w11, 2);
+    const float b00 = byte_f23(w00, 2), b01 = byte_f23(w01, 2), b10 = byte_f23(w10, 2), b11 = byte_f23(w11, 2);
     const float btop = fmaf(fx, b01 - b00, b00 - K23), bbot = fmaf(fx, b11 - b10, b10 - K23);
     s.b.x = fmaf(fy, bbot - btop, btop) * scale;
 }
@@ -390,6 +378,21 @@ enum D1Mode { D1M_STAGED = 0, D1M_CLAMP = 1, D1M_FRAME = 2 };
 constexpr float D1_FLOOR_M = 12582912.0f;       // 1.5 * 2^23
 constexpr unsigned D1_FLOOR_BITS = 0x4B400000u;  // its bit pattern
 
+// The bilinear sample at p with its taps read from the frame.
+__device__ __forceinline__ void d1_frame_sample(const D1Ctx& x, const Pos& p, V4& s) {
+    int i0, j0;
+    float fx, fy;
+    if (p.iu < 0) { i0 = 0; fx = 0.0f; }
+    else if (p.iu >= x.W - 1) { i0 = x.W - 1; fx = 0.0f; }
+    else { i0 = p.iu; fx = p.fu; }
+    if (p.iv < 0) { j0 = 0; fy = 0.0f; }
+    else if (p.iv >= x.H - 1) { j0 = x.H - 1; fy = 0.0f; }
+    else { j0 = p.iv; fy = p.fv; }
+    const uint8_t* a = x.px + (long long)j0 * x.pitch + 3 * i0;
+    const Texels q = load_texels(a, a + (j0 + 1 < x.H ? x.pitch : 0), i0, x.W, word_aligned(x.px, x.pitch));
+    d1_bilerp(q.t00, q.t01, q.t10, q.t11, fx, fy, x.scale, s);
+}
+
 // Level-0 sample of virtual row r at the column whose anchored numerators and denominator at the
 // anchor row are (nuv, dqc): (r, g, b, normalised weight a), weight 0 outside Omega^0 (a < 0).
 // The colour there is whatever the taps give: Omega^0 holds the 5 x 5 support of every stored G^1
@@ -416,9 +419,7 @@ __device__ __forceinline__ V4 d1_sample(const D1Ctx& x, float2 nuv, float dqc, i
         p.iv = x.tm.V0 + (int)flv;
         p.fu = ru - flu;
         p.fv = rv - flv;
-        const float3 v = sample_rgb(x.px, x.pitch, p, x.W, x.H, x.scale);
-        s.a = make_float2(v.x, v.y);
-        s.b.x = v.z;
+        d1_frame_sample(x, p, s);
     } else {
         const float2 ruv = f2mul(n, f2(rden));
         const float2 tt = f2add_rm(ruv, f2(D1_FLOOR_M));
@@ -431,7 +432,7 @@ __device__ __forceinline__ V4 d1_sample(const D1Ctx& x, float2 nuv, float dqc, i
             // (the planner's footprint holds every tap; the debug build records one that it misses)
             const int raw = (int)(tv * (unsigned)x.S + tu + x.ibase);
             (void)STITCH_DCHECK(raw >= 0 && raw <= x.maxidx, 1, raw);
-            const int idx = min(max(raw, 0), x.maxidx);
+            const unsigned idx = min((unsigned)raw, (unsigned)x.maxidx);
             const uint32_t* p = x.foot + idx;
             w00 = p[0];
             w01 = p[1];
@@ -742,7 +743,10 @@ __global__ void __launch_bounds__(D1_THREADS, D1Cap<CAP>::BLOCKS) k_down1(const 
                                                                         const float4* __restrict__ d1cols,
                                                                         Slot* __restrict__ g0buf) {
     extern __shared__ float4 smem[];
-    down1_tile<T, CAP>(cams, g, fp, od, tiles[blockIdx.x], refs, d1w, d1cols, g0buf, smem);
+    pdl_trigger();
+    const D1Tile tl = tiles[blockIdx.x];
+    pdl_wait();
+    down1_tile<T, CAP>(cams, g, fp, od, tl, refs, d1w, d1cols, g0buf, smem);
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -963,7 +967,10 @@ __global__ void __launch_bounds__(RC_THREADS, 8) k_reduce_t(const CamDev* __rest
                                                            int l, const Tile* __restrict__ tiles, int n, int wave) {
     extern __shared__ float4 smem[];
     const int nb = blockIdx.x + wave;
-    reduce_col_tile<T>(cams, g, l, tiles[blockIdx.x], smem, nb < n ? tiles + nb : nullptr);
+    pdl_trigger();
+    const Tile tl = tiles[blockIdx.x];
+    pdl_wait();
+    reduce_col_tile<T>(cams, g, l, tl, smem, nb < n ? tiles + nb : nullptr);
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -1142,7 +1149,10 @@ __global__ void __launch_bounds__(256, 3) k_coarse_t(const CamDev* __restrict__ 
                                                    const LevelTile* __restrict__ tiles,
                                                    const int* __restrict__ camlist) {
     extern __shared__ float4 smem[];
-    coarse_tile<T, CSRig>(cams, g, l, Rl, Rc, tiles[blockIdx.x], camlist, smem);
+    pdl_trigger();
+    const LevelTile tl = tiles[blockIdx.x];
+    pdl_wait();
+    coarse_tile<T, CSRig>(cams, g, l, Rl, Rc, tl, camlist, smem);
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -1234,6 +1244,8 @@ __global__ void __launch_bounds__(U_THREADS) k_up_simple(const CamDev* __restric
                                                           OutDesc od, const UpTile* __restrict__ tiles,
                                                           const CamRef* __restrict__ refs) {
     __shared__ __align__(16) unsigned char stage[3 * U_TX * U_TY];
+    pdl_trigger();
+    pdl_wait();
     up_simple_tile(cams, g, fp, od, tiles[blockIdx.x], refs, stage);
 }
 
@@ -1304,6 +1316,7 @@ __device__ __forceinline__ void up_full_tile(const CamDev* __restrict__ cams, co
         ucs.fg2[t] = c.FG[2];
         ucs.dsc[t] = c.gain * (1.0f / 255.0f) * (1.0f / SLOT_RGB);
     }
+    pdl_wait();
     __syncthreads();
     // loads of level 1 and 2 data, all of a thread's loads in flight before the stores
     if (L >= 2) {
@@ -1504,41 +1517,56 @@ __device__ __forceinline__ void up_full_tile(const CamDev* __restrict__ cams, co
     }
 }
 
-// Blocks n .. n + n_simple - 1 take the ZERO (and fallback SOLO) canvas tiles `simple`, so that they
-// need no launch of their own.
-template <typename T, int NC, int NB>
+// The tiles of an up launch: n4 tiles with 3 or 4 cameras, then n2 with at most 2, then the ZERO (and
+// fallback SOLO) tiles, so that none of them needs a launch (and a tail) of its own; wave2, wave4:
+// resident blocks on the device (the distance of the L2 prefetch, see k_reduce_t).
+struct UpLaunch {
+    const UpTile *t4, *t2, *simple;
+    int n4, n2, wave;
+};
+
+// NCMAX: the most cameras a tile of this launch has (2 or 4)
+template <typename T, int NCMAX, int NB>
 __device__ __forceinline__ void up_full_block(const CamDev* __restrict__ cams, const RigGeom& g, const FramePtrs& fp,
-                                              const OutDesc& od, const T* __restrict__ R2, const UpTile* __restrict__ tiles,
-                                              const CamRef* __restrict__ refs, const Slot* __restrict__ g0buf, int n,
-                                              int wave, const UpTile* __restrict__ simple, float4* usm) {
-    if ((int)blockIdx.x >= n) {
-        up_simple_tile(cams, g, fp, od, simple[blockIdx.x - n], refs, reinterpret_cast<unsigned char*>(usm));
+                                              const OutDesc& od, const T* __restrict__ R2, const UpLaunch& ul,
+                                              const CamRef* __restrict__ refs, const Slot* __restrict__ g0buf, float4* usm) {
+    int b = blockIdx.x;
+    pdl_trigger();
+    if (NCMAX > 2) {
+        if (b < ul.n4) {
+            const int nb = b + ul.wave;
+            up_full_tile<T, NCMAX, NB>(cams, g, fp, od, R2, ul.t4[b], refs, g0buf, usm, nb < ul.n4 ? ul.t4 + nb : nullptr);
+            return;
+        }
+        b -= ul.n4;
+    }
+    if (b < ul.n2) {
+        const int nb = b + ul.wave;
+        up_full_tile<T, 2, NB>(cams, g, fp, od, R2, ul.t2[b], refs, g0buf, usm, nb < ul.n2 ? ul.t2 + nb : nullptr);
         return;
     }
-    const int nb = blockIdx.x + wave;  // prefetched: the tile one resident wave later (see k_reduce_t)
-    up_full_tile<T, NC, NB>(cams, g, fp, od, R2, tiles[blockIdx.x], refs, g0buf, usm, nb < n ? tiles + nb : nullptr);
+    pdl_wait();
+    up_simple_tile(cams, g, fp, od, ul.simple[b - ul.n2], refs, reinterpret_cast<unsigned char*>(usm));
 }
 // Two occupancies: k_up_full_b4 holds four resident blocks per SM (64 registers, a few spilled in
 // the level-1 phase, one camera's slot loads at a time), for rigs with many waves of canvas tiles;
 // k_up_full three, with two cameras' slot loads in flight, which wins when the launch is a few waves.
-template <typename T, int NC>
-__global__ void __launch_bounds__(U_THREADS) k_up_full(const CamDev* __restrict__ cams, RigGeom g, FramePtrs fp,
-                                                        OutDesc od, const T* __restrict__ R2,
-                                                        const UpTile* __restrict__ tiles,
-                                                        const CamRef* __restrict__ refs, const Slot* __restrict__ g0buf,
-                                                        int n, int wave, const UpTile* __restrict__ simple) {
+// Tiles with up to 4 cameras take 72 KB of shared memory, so three blocks fit whatever the mix.
+template <typename T, int NCMAX>
+__global__ void __launch_bounds__(U_THREADS, 3) k_up_full(const CamDev* __restrict__ cams, const __grid_constant__ RigGeom g,
+                                                           const __grid_constant__ FramePtrs fp, OutDesc od,
+                                                           const T* __restrict__ R2, const __grid_constant__ UpLaunch ul,
+                                                           const CamRef* __restrict__ refs, const Slot* __restrict__ g0buf) {
     extern __shared__ float4 usm[];
-    up_full_block<T, NC, (NC < 2 ? NC : 2)>(cams, g, fp, od, R2, tiles, refs, g0buf, n, wave, simple, usm);
+    up_full_block<T, NCMAX, 2>(cams, g, fp, od, R2, ul, refs, g0buf, usm);
 }
-template <typename T, int NC>
-__global__ void __launch_bounds__(U_THREADS, 4) k_up_full_b4(const CamDev* __restrict__ cams, RigGeom g, FramePtrs fp,
-                                                              OutDesc od, const T* __restrict__ R2,
-                                                              const UpTile* __restrict__ tiles,
-                                                              const CamRef* __restrict__ refs,
-                                                              const Slot* __restrict__ g0buf, int n, int wave,
-                                                              const UpTile* __restrict__ simple) {
+template <typename T>
+__global__ void __launch_bounds__(U_THREADS, 4) k_up_full_b4(const CamDev* __restrict__ cams, const __grid_constant__ RigGeom g,
+                                                              const __grid_constant__ FramePtrs fp, OutDesc od,
+                                                              const T* __restrict__ R2, const __grid_constant__ UpLaunch ul,
+                                                              const CamRef* __restrict__ refs, const Slot* __restrict__ g0buf) {
     extern __shared__ float4 usm[];
-    up_full_block<T, NC, 1>(cams, g, fp, od, R2, tiles, refs, g0buf, n, wave, simple, usm);
+    up_full_block<T, 2, 1>(cams, g, fp, od, R2, ul, refs, g0buf, usm);
 }
 
 template <int NC>
@@ -1690,7 +1718,7 @@ __device__ __forceinline__ void up_general_tile(const CamDev* __restrict__ cams,
             const float w = g.seam ? (own[k] == a ? 1.f : 0.f) : feather_weight(sp, c.W, c.H);
             if (!(w > 0.f)) continue;
             const float what = w / ws[k];
-            float3 v = bilinear_rgb(fp.p[i], fp.pitch[i], clamp_tap(sp, c.W, c.H), scale);
+            float3 v = bilinear_rgb(fp.p[i], fp.pitch[i], c.W, clamp_tap(sp, c.W, c.H), scale);
             if (L >= 2) {
                 const float3 e = expand_smem(g1, UG1_X, dx, dy);
                 v.x -= e.x;
@@ -1781,6 +1809,8 @@ __global__ void __launch_bounds__(U_THREADS) k_up_general(const CamDev* __restri
                                                            const UpTile* __restrict__ tiles,
                                                            const CamRef* __restrict__ refs) {
     __shared__ float4 smem[UG_SMEM_F4];
+    pdl_trigger();
+    pdl_wait();
     up_general_tile<T>(cams, g, fp, od, R2, tiles[blockIdx.x], refs, smem);
 }
 
@@ -1808,7 +1838,7 @@ struct FusedState {
     int n_staged = 0;            // down1 tiles with a staged source footprint
     bool d1_small = false;       // down1 with the smaller footprint capacity (13 blocks per SM)
     bool up_four = false;        // up_full with four resident blocks per SM
-    int wave_red = 0, wave_up2 = 0, wave_up4 = 0;  // resident blocks on the device (L2 prefetch distance)
+    int wave_red = 0, wave_up = 0;  // resident blocks on the device (L2 prefetch distance)
     void* R[MAXL] = {};          // R^l on the canvas grid, l >= 2
     CamRef* refs = nullptr;
     UpTile* up_tiles[UP_KINDS] = {};
@@ -2051,51 +2081,51 @@ stitch_status launch_all(stitch_rig* r, FusedState* fs, const FramePtrs& fp, con
     if (L >= 2 && fs->n_d1 > 0) {
         prof_mark(r, "fused_down1", s);
         if (fs->d1_small)
-            k_down1<T, D1_FOOT_SMALL><<<fs->n_d1, D1_THREADS, D1Cap<D1_FOOT_SMALL>::SMEM, s>>>(
-                r->dcam, g, fp, od, fs->d1_tiles, fs->refs, fs->d1w, fs->d1cols, (Slot*)fs->g0buf);
+            pdl_launch(k_down1<T, D1_FOOT_SMALL>, fs->n_d1, D1_THREADS, D1Cap<D1_FOOT_SMALL>::SMEM, s, r->dcam, g, fp, od,
+                       fs->d1_tiles, fs->refs, fs->d1w, fs->d1cols, (Slot*)fs->g0buf);
         else
-            k_down1<T, D1_FOOT><<<fs->n_d1, D1_THREADS, D1_SMEM, s>>>(r->dcam, g, fp, od, fs->d1_tiles, fs->refs, fs->d1w,
-                                                                     fs->d1cols, (Slot*)fs->g0buf);
+            pdl_launch(k_down1<T, D1_FOOT>, fs->n_d1, D1_THREADS, D1_SMEM, s, r->dcam, g, fp, od, fs->d1_tiles, fs->refs,
+                       fs->d1w, fs->d1cols, (Slot*)fs->g0buf);
     }
     for (int l = 1; l + 1 < L; ++l) {
         if (fs->n_rc[l + 1] == 0) continue;
         prof_mark(r, "fused_reduce", s);
-        k_reduce_t<T><<<fs->n_rc[l + 1], RC_THREADS, RC_SMEM, s>>>(r->dcam, g, l, fs->rc_tiles[l + 1], fs->n_rc[l + 1],
-                                                                   fs->wave_red);
+        pdl_launch(k_reduce_t<T>, fs->n_rc[l + 1], RC_THREADS, RC_SMEM, s, r->dcam, g, l, fs->rc_tiles[l + 1],
+                   fs->n_rc[l + 1], fs->wave_red);
     }
     for (int l = L - 1; l >= 2; --l) {
         if (fs->n_co[l] == 0) continue;
         prof_mark(r, "fused_coarse", s);
-        k_coarse_t<T><<<fs->n_co[l], 256, sizeof(float4) * CT_SMEM_F4, s>>>(r->dcam, g, l, (T*)fs->R[l],
-                                                   l + 1 < L ? (const T*)fs->R[l + 1] : nullptr, fs->co_tiles[l],
-                                                   fs->camlist);
+        pdl_launch(k_coarse_t<T>, fs->n_co[l], 256, sizeof(float4) * CT_SMEM_F4, s, r->dcam, g, l, (T*)fs->R[l],
+                   l + 1 < L ? (const T*)fs->R[l + 1] : nullptr, fs->co_tiles[l], fs->camlist);
     }
     const T* R2 = L >= 3 ? (const T*)fs->R[2] : nullptr;
-    // the ZERO canvas tiles ride along with the first up_full launch (or get their own)
-    const int ns = fs->n_up[UP_SIMPLE];
-    if (ns && !fs->n_up[UP_FULL2] && !fs->n_up[UP_FULL4]) {
-        prof_mark(r, "fused_up_simple", s);
-        k_up_simple<<<ns, U_THREADS, 0, s>>>(r->dcam, g, fp, od, fs->up_tiles[UP_SIMPLE], fs->refs);
-    }
-    if (fs->n_up[UP_FULL2]) {
+    const Slot* g0 = (const Slot*)fs->g0buf;
+    const int n2 = fs->n_up[UP_FULL2], n4 = fs->n_up[UP_FULL4], ns = fs->n_up[UP_SIMPLE];
+    UpLaunch ul{fs->up_tiles[UP_FULL4], fs->up_tiles[UP_FULL2], fs->up_tiles[UP_SIMPLE], n4, n2, fs->wave_up};
+    if (fs->up_four) {
+        // many waves of tiles with at most 2 cameras, four blocks per SM; the others three
         prof_mark(r, "fused_up_full", s);
-        auto k = fs->up_four ? k_up_full_b4<T, 2> : k_up_full<T, 2>;
-        k<<<fs->n_up[UP_FULL2] + ns, U_THREADS, up_full_smem<2>(), s>>>(
-            r->dcam, g, fp, od, R2, fs->up_tiles[UP_FULL2], fs->refs, (const Slot*)fs->g0buf, fs->n_up[UP_FULL2],
-            fs->wave_up2, fs->up_tiles[UP_SIMPLE]);
-    }
-    if (fs->n_up[UP_FULL4]) {
-        const int extra = fs->n_up[UP_FULL2] ? 0 : ns;
-        prof_mark(r, "fused_up_full4", s);
-        auto k = fs->up_four ? k_up_full_b4<T, 4> : k_up_full<T, 4>;
-        k<<<fs->n_up[UP_FULL4] + extra, U_THREADS, up_full_smem<4>(), s>>>(
-            r->dcam, g, fp, od, R2, fs->up_tiles[UP_FULL4], fs->refs, (const Slot*)fs->g0buf, fs->n_up[UP_FULL4],
-            fs->wave_up4, fs->up_tiles[UP_SIMPLE]);
+        ul.n4 = 0;
+        pdl_launch(k_up_full_b4<T>, n2 + ns, U_THREADS, up_full_smem<2>(), s, r->dcam, g, fp, od, R2, ul, fs->refs, g0);
+        if (n4) {
+            prof_mark(r, "fused_up_full4", s);
+            ul.n4 = n4;
+            ul.n2 = 0;
+            pdl_launch(k_up_full<T, 4>, n4, U_THREADS, up_full_smem<4>(), s, r->dcam, g, fp, od, R2, ul, fs->refs, g0);
+        }
+    } else if (n2 + n4) {
+        prof_mark(r, "fused_up_full", s);
+        if (n4) pdl_launch(k_up_full<T, 4>, n4 + n2 + ns, U_THREADS, up_full_smem<4>(), s, r->dcam, g, fp, od, R2, ul, fs->refs, g0);
+        else pdl_launch(k_up_full<T, 2>, n2 + ns, U_THREADS, up_full_smem<2>(), s, r->dcam, g, fp, od, R2, ul, fs->refs, g0);
+    } else if (ns) {
+        prof_mark(r, "fused_up_simple", s);
+        pdl_launch(k_up_simple, ns, U_THREADS, 0, s, r->dcam, g, fp, od, fs->up_tiles[UP_SIMPLE], fs->refs);
     }
     if (fs->n_up[UP_GENERAL]) {
         prof_mark(r, "fused_up_general", s);
-        k_up_general<T><<<fs->n_up[UP_GENERAL], U_THREADS, 0, s>>>(r->dcam, g, fp, od, R2,
-                                                                    fs->up_tiles[UP_GENERAL], fs->refs);
+        pdl_launch(k_up_general<T>, fs->n_up[UP_GENERAL], U_THREADS, 0, s, r->dcam, g, fp, od, R2, fs->up_tiles[UP_GENERAL],
+                   fs->refs);
     }
     return launch_status();
 }
@@ -2110,10 +2140,8 @@ stitch_status set_smem_attrs() {
                                          (int)up_full_smem<2>()));
     STITCH_CUDA_TRY(cudaFuncSetAttribute(k_up_full<T, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)up_full_smem<4>()));
-    STITCH_CUDA_TRY(cudaFuncSetAttribute(k_up_full_b4<T, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    STITCH_CUDA_TRY(cudaFuncSetAttribute(k_up_full_b4<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)up_full_smem<2>()));
-    STITCH_CUDA_TRY(cudaFuncSetAttribute(k_up_full_b4<T, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)up_full_smem<4>()));
     STITCH_CUDA_TRY(cudaFuncSetAttribute(k_coarse_t<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)(sizeof(float4) * CT_SMEM_F4)));
     return STITCH_OK;
@@ -2123,21 +2151,17 @@ stitch_status set_smem_attrs() {
 // prefetch chains.
 template <typename T>
 stitch_status set_waves(stitch_rig* r, FusedState* fs) {
-    int sms = 0, pr = 0, p2 = 0, p4 = 0;
+    int sms = 0, pr = 0, pu = 0;
     STITCH_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, r->device));
     STITCH_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&pr, k_reduce_t<T>, RC_THREADS, RC_SMEM));
     // four resident up_full blocks per SM when the blended canvas tiles make many waves of them
-    fs->up_four = fs->n_up[UP_FULL2] + fs->n_up[UP_FULL4] >= 8 * 4 * std::max(sms, 1);
-    if (fs->up_four) {
-        STITCH_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&p2, k_up_full_b4<T, 2>, U_THREADS, up_full_smem<2>()));
-        STITCH_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&p4, k_up_full_b4<T, 4>, U_THREADS, up_full_smem<4>()));
-    } else {
-        STITCH_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&p2, k_up_full<T, 2>, U_THREADS, up_full_smem<2>()));
-        STITCH_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&p4, k_up_full<T, 4>, U_THREADS, up_full_smem<4>()));
-    }
+    const int n2 = fs->n_up[UP_FULL2], n4 = fs->n_up[UP_FULL4];
+    fs->up_four = n2 > 0 && n2 + n4 >= 8 * 4 * std::max(sms, 1);
+    if (fs->up_four) STITCH_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&pu, k_up_full_b4<T>, U_THREADS, up_full_smem<2>()));
+    else if (n4) STITCH_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&pu, k_up_full<T, 4>, U_THREADS, up_full_smem<4>()));
+    else STITCH_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&pu, k_up_full<T, 2>, U_THREADS, up_full_smem<2>()));
     fs->wave_red = std::max(pr, 1) * sms;
-    fs->wave_up2 = std::max(p2, 1) * sms;
-    fs->wave_up4 = std::max(p4, 1) * sms;
+    fs->wave_up = std::max(pu, 1) * sms;
     return STITCH_OK;
 }
 
@@ -2540,12 +2564,15 @@ stitch_status fused_plan(stitch_rig* r) {
     int kernels = 0;
     if (L >= 2 && fs->n_d1 > 0) kernels += 1;
     for (int l = 2; l < L; ++l) kernels += (fs->n_rc[l] > 0) + (fs->n_co[l] > 0);
-    for (int k = 0; k < UP_KINDS; ++k) kernels += fs->n_up[k] > 0;
-    if (fs->n_up[UP_SIMPLE] && (fs->n_up[UP_FULL2] || fs->n_up[UP_FULL4])) kernels -= 1;  // rides along
-    r->kernels_per_frame = kernels;
     st = fs->fp16 ? set_smem_attrs<half4>() : set_smem_attrs<float4>();
+    if (st == STITCH_OK) st = fs->fp16 ? set_waves<half4>(r, fs) : set_waves<float4>(r, fs);
     if (st != STITCH_OK) return st;
-    return fs->fp16 ? set_waves<half4>(r, fs) : set_waves<float4>(r, fs);
+    // one launch for the canvas tiles with up to 4 cameras and the ZERO ones, two with up_four
+    kernels += fs->n_up[UP_FULL2] + fs->n_up[UP_FULL4] + fs->n_up[UP_SIMPLE] > 0;
+    kernels += fs->up_four && fs->n_up[UP_FULL4] > 0;
+    kernels += fs->n_up[UP_GENERAL] > 0;
+    r->kernels_per_frame = kernels;
+    return STITCH_OK;
 }
 
 stitch_status fused_frames(stitch_rig* r, const FramePtrs& fp, const OutDesc& od, cudaStream_t s) {

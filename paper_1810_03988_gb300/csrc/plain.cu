@@ -5,14 +5,14 @@
 //   bands (S4), their normalised blend on the canvas grid (S5), collapse and output (S6).
 // A launch covers all cameras; on the small rigs of stitch_frames_static the path is a chain of
 // sub-wave launches, so their number sets its time.  Two 640 x 360 cameras, 4 levels: 8 launches,
-// 128 us per call, against 22 launches (each camera, step and level its own) and 185 us.
+// 59 us per call, against 22 launches (each camera, step and level its own) and 185 us.
 #include "stitch_internal.cuh"
 
 namespace {
 
 constexpr int BX = 32, BY = 8;
 
-__device__ __forceinline__ float4 ld4(const float4* p) { return __ldg(p); }
+__device__ __forceinline__ float4 ld4(const float4* p) { return *p; }
 
 // The blocks of one launch over a rectangle per camera: camera i has blocks first[i] .. first[i + 1] - 1,
 // bx[i] to a row.
@@ -37,12 +37,19 @@ __device__ __forceinline__ int grid_cam(const CamGrid& cg, int ncam, int* bx, in
 // the first warp of every block, all on the same scheduler of an SM (38 us a camera, of which the pixels
 // take 2).  Here a map takes three lanes (the rows of A: u, v, w), which do the same operations side
 // by side, about 18 instructions, in a warp that changes from one wave of blocks to the next.
-__global__ void __launch_bounds__(BX* BY) k_plain_warp(const CamDev* __restrict__ cams, int ncam,
+//
+// CYL, SEAM: the cylindrical canvas and seam weights, which work in FP64 per pixel, are kernels of
+// their own: compiled as run-time choices, loop-invariant parts of their FP64 arithmetic ran for every
+// pixel of the planar feather path too (74 % of the FP64 pipe; 68 us for two 640 x 360 cameras, 19 us now).
+template <bool CYL, bool SEAM>
+__global__ void __launch_bounds__(BX* BY) k_plain_warp(const CamDev* cams, int ncam,
                                                         const __grid_constant__ CamGrid cg, const __grid_constant__ FramePtrs fp,
                                                         const __grid_constant__ RigGeom g, int sms) {
     __shared__ TileMap tm[MAXC];
     __shared__ int list[MAXC], s_n;
     __shared__ int ax[MAXC], ay[MAXC];
+    pdl_trigger();
+    pdl_wait();
     int bx, by;
     const int i = grid_cam(cg, ncam, &bx, &by);
     const CamDev& ci = cams[i];
@@ -62,7 +69,7 @@ __global__ void __launch_bounds__(BX* BY) k_plain_warp(const CamDev* __restrict_
         const int n = __popc(m);
         if (t == 0) s_n = n;
         __syncwarp();
-        for (int k0 = 0; k0 < n; k0 += 8) {
+        for (int k0 = 0; k0 < (CYL ? 0 : n); k0 += 8) {
             // lane 4 k + q: row q of the map of camera k (q = 2 serves w; lane 4 k + 3 repeats it)
             const int k = min(k0 + t / 4, n - 1), q = min(t % 4, 2);
             const CamDev& cj = cams[list[k]];
@@ -104,16 +111,16 @@ __global__ void __launch_bounds__(BX* BY) k_plain_warp(const CamDev* __restrict_
     float3 rgb = make_float3(0.f, 0.f, 0.f);
     float wi = 0.f, ws = 0.f;
     // seam weights: the pixel's owner among all cameras (FP64 decision)
-    const int own = g.seam ? seam_owner(g, ncam, [&](int k) -> const CamDev& { return cams[k]; }, x, y) : -1;
+    const int own = SEAM ? seam_owner(g, ncam, [&](int k) -> const CamDev& { return cams[k]; }, x, y) : -1;
     for (int k = 0; k < s_n; ++k) {
         const int j = list[k];
         const CamDev& cj = cams[j];
-        const SrcPos s = g.cyl ? map_point64(cj, g, x, y) : map_point(tm[k], (float)(x - ax[k]), (float)(y - ay[k]));
-        const float w = g.seam ? (own == j ? 1.f : 0.f) : (cj.V.contains(x, y) ? feather_weight(s, cj.W, cj.H) : 0.f);
+        const SrcPos s = CYL ? map_point64(cj, g, x, y) : map_point(tm[k], (float)(x - ax[k]), (float)(y - ay[k]));
+        const float w = SEAM ? (own == j ? 1.f : 0.f) : (cj.V.contains(x, y) ? feather_weight(s, cj.W, cj.H) : 0.f);
         ws += w;
         if (j == i) {
             wi = w;
-            rgb = bilinear_rgb(fp.p[i], fp.pitch[i], clamp_tap(s, cj.W, cj.H), cj.gain * (1.0f / 255.0f));
+            rgb = bilinear_rgb(fp.p[i], fp.pitch[i], cj.W, clamp_tap(s, cj.W, cj.H), cj.gain * (1.0f / 255.0f));
         }
     }
     const float what = ws > 0.f ? wi / ws : 0.f;
@@ -122,8 +129,10 @@ __global__ void __launch_bounds__(BX* BY) k_plain_warp(const CamDev* __restrict_
 
 // S3: G^{l+1} = REDUCE(G^l) on Om[l+1] (all four channels) of every camera, 25 taps read straight from
 // HBM/L2, all in flight.
-__global__ void __launch_bounds__(BX* BY) k_plain_reduce(const CamDev* __restrict__ cams, int ncam, int l,
+__global__ void __launch_bounds__(BX* BY) k_plain_reduce(const CamDev* cams, int ncam, int l,
                                                           const __grid_constant__ CamGrid cg, const __grid_constant__ RigGeom g) {
+    pdl_trigger();
+    pdl_wait();
     int bx, by;
     const CamDev& c = cams[grid_cam(cg, ncam, &bx, &by)];
     const Rect oc = c.Om[l + 1], of = c.Om[l];
@@ -159,7 +168,7 @@ __global__ void __launch_bounds__(BX* BY) k_plain_reduce(const CamDev* __restric
 // EXPAND of a coarse buffer (rect r of a level of size nxc x nyc) at fine (x, y), rgb only: taps
 // k - 1, k, k + 1 with weights 1/8, 3/4, 1/8 at even positions 2k and 0, 1/2, 1/2 at odd ones, so that
 // a warp's lanes take the same 9 loads (the tap of weight 0 adds nothing; it is kept inside the buffer).
-__device__ __forceinline__ float3 expand_rgb(const float4* __restrict__ buf, const Rect& r, int nxc, int nyc, int x,
+__device__ __forceinline__ float3 expand_rgb(const float4* buf, const Rect& r, int nxc, int nyc, int x,
                                              int y) {
     const bool ox = x & 1, oy = y & 1;
     const float wx[3] = {ox ? 0.f : 0.125f, ox ? 0.5f : 0.75f, ox ? 0.5f : 0.125f};
@@ -190,8 +199,10 @@ __device__ __forceinline__ float3 expand_rgb(const float4* __restrict__ buf, con
 
 // S4 - S6 on one level of the canvas: B^l = sum_i G^l(What_i) L^l_i / S^l with L^l_i = G^l_i -
 // EXPAND(G^{l+1}_i) (the top level: G^l_i), R^l = B^l + EXPAND(R^{l+1}); at level 0 mask, clamp, output.
-__global__ void __launch_bounds__(BX* BY) k_plain_level(const CamDev* __restrict__ cams, int l, const __grid_constant__ RigGeom g,
-                                                         float4* __restrict__ Bl, const float4* __restrict__ Rc, OutDesc od) {
+__global__ void __launch_bounds__(BX* BY) k_plain_level(const CamDev* cams, int l, const __grid_constant__ RigGeom g,
+                                                         float4* Bl, const float4* Rc, OutDesc od) {
+    pdl_trigger();
+    pdl_wait();
     const int x = blockIdx.x * BX + threadIdx.x, y = blockIdx.y * BY + threadIdx.y;
     if (x >= g.nx[l] || y >= g.ny[l]) return;
     const bool top = l == g.levels - 1;
@@ -295,13 +306,18 @@ stitch_status plain_frames(stitch_rig* r, const FramePtrs& fp, const OutDesc& od
         const CamGrid cg = cam_grid(r, l, &n);
         if (n == 0) continue;
         prof_mark(r, l == 0 ? "plain_warp" : "plain_reduce", s);
-        if (l == 0) k_plain_warp<<<n, blk, 0, s>>>(r->dcam, g.ncam, cg, fp, g, std::max(r->sms, 1));
-        else k_plain_reduce<<<n, blk, 0, s>>>(r->dcam, g.ncam, l - 1, cg, g);
+        if (l == 0) {
+            auto warp = g.cyl ? (g.seam ? k_plain_warp<true, true> : k_plain_warp<true, false>)
+                              : (g.seam ? k_plain_warp<false, true> : k_plain_warp<false, false>);
+            pdl_launch(warp, n, blk, 0, s, r->dcam, g.ncam, cg, fp, g, std::max(r->sms, 1));
+        } else {
+            pdl_launch(k_plain_reduce, n, blk, 0, s, r->dcam, g.ncam, l - 1, cg, g);
+        }
     }
     for (int l = g.levels - 1; l >= 0; --l) {
         prof_mark(r, "plain_level", s);
         const dim3 grid((g.nx[l] + BX - 1) / BX, (g.ny[l] + BY - 1) / BY);
-        k_plain_level<<<grid, blk, 0, s>>>(r->dcam, l, g, r->Bl[l], l + 1 < g.levels ? r->Bl[l + 1] : nullptr, od);
+        pdl_launch(k_plain_level, grid, blk, 0, s, r->dcam, l, g, r->Bl[l], l + 1 < g.levels ? r->Bl[l + 1] : nullptr, od);
     }
     return launch_status();
 }

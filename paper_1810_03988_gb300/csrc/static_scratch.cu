@@ -58,6 +58,8 @@ static_assert(sizeof(CamDev) % 8 == 0, "CamDev is copied in 8-byte words");
 static_assert(sizeof(CamPack) + sizeof(void*) + sizeof(int) <= 32764, "kernel parameter limit");
 
 __global__ void k_put_cams(const __grid_constant__ CamPack pk, int n, CamDev* __restrict__ dst) {
+    pdl_trigger();
+    pdl_wait();
     const uint2* src = reinterpret_cast<const uint2*>(pk.c);
     uint2* d = reinterpret_cast<uint2*>(dst);
     const int words = n * (int)(sizeof(CamDev) / 8);
@@ -159,7 +161,7 @@ extern "C" stitch_status stitch_frames_static(const stitch_rig_desc* desc, const
     // camera descriptors into the array, ordered on the stream before the path's kernels
     cudaStream_t s = (cudaStream_t)stream;
     static_assert(sizeof(r.hcam) == sizeof(CamPack), "descriptor pack layout");
-    k_put_cams<<<1, 256, 0, s>>>(*reinterpret_cast<const CamPack*>(r.hcam), g.ncam, r.dcam);
+    pdl_launch(k_put_cams, 1, 256, 0, s, *reinterpret_cast<const CamPack*>(r.hcam), g.ncam, r.dcam);
     if (cudaGetLastError() != cudaSuccess) return STITCH_ECUDA;
     int dev = -1;
     if (cudaGetDevice(&dev) != cudaSuccess ||

@@ -80,6 +80,34 @@ constexpr size_t kGuardBytes = 256;
 constexpr uint32_t kGuardWord = 0x7FC0DEADu;
 
 // ------------------------------------------------------------------------------------------------
+// Programmatic dependent launch: the kernels of a call's sequence are launched so that the next one
+// may start as soon as every block of the previous one has started (pdl_trigger), and each of their
+// blocks waits for the previous one's completion (pdl_wait) before its first access to anything but
+// the rig's constant tables, and before it returns.  As that kernel has waited for the one before
+// it, all earlier work of the stream is complete behind pdl_wait.  Without the launch attribute both
+// are no-ops.  Data that the previous kernels wrote is read by plain or __ldcg loads from pointers that
+// are not `const __restrict__`: loads of the read-only path are promised not to change while the kernel
+// runs, which begins before pdl_wait, and the compiler may move them above it.
+
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+template <typename... P, typename... A>
+inline void pdl_launch(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, const A&... args) {
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+}
+
+// ------------------------------------------------------------------------------------------------
 // small device helpers
 
 // reflect-101 border folding on a grid of n samples: ... 2 1 | 0 1 2 ... n-1 | n-2 n-3 ...
@@ -256,16 +284,78 @@ __device__ __forceinline__ Tap clamp_tap(const SrcPos& s, int W, int H) {
     return t;
 }
 
-// Bilinear RGB sample of an 8-bit frame, scaled by `scale` (= gain / 255).
-__device__ __forceinline__ float3 bilinear_rgb(const uint8_t* __restrict__ px, long long pitch, const Tap& t,
+// packed single-precision pairs (f32x2: two IEEE binary32 lanes, each rounded exactly as the
+// scalar operation), used where the path computes on pairs of channels
+
+__device__ __forceinline__ float2 f2fma(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
+__device__ __forceinline__ float2 f2add(float2 a, float2 b) { return __fadd2_rn(a, b); }
+// a - b as a + (-1) b: the product is exact, so this is the rounded difference, bit for bit
+__device__ __forceinline__ float2 f2sub(float2 a, float2 b) { return __ffma2_rn(b, make_float2(-1.0f, -1.0f), a); }
+__device__ __forceinline__ float2 f2mul(float2 a, float2 b) { return __fmul2_rn(a, b); }
+__device__ __forceinline__ float2 f2add_rm(float2 a, float2 b) { return __fadd2_rd(a, b); }  // toward -infinity
+
+__device__ __forceinline__ float2 f2(float v) { return make_float2(v, v); }
+
+// Byte j of w as a float, exactly: the bits 0x4B000000 | b encode 2^23 + b.
+__device__ __forceinline__ float byte_f(uint32_t w, uint32_t j) {
+    return __uint_as_float(__byte_perm(w, 0x4B000000u, 0x7440u | j)) - 8388608.0f;
+}
+
+// 2^23 + byte j of w, as a float (exact)
+__device__ __forceinline__ float byte_f23(uint32_t w, uint32_t j) {
+    return __uint_as_float(__byte_perm(w, 0x4B000000u, 0x7440u | j));
+}
+
+// The four texels of a bilinear sample (R, G, B in bytes 0 to 2 of a word), a and b the addresses of the
+// left one in both rows, i0 its column; the right ones repeat the left ones in the last column.  Two
+// neighbouring texels are 6 bytes at any offset: where base and pitch are multiples of 4 bytes (words)
+// and three words from the first one's on lie in the row, they are two or three aligned loads and a
+// funnel shift instead of six byte loads.
+struct Texels {
+    uint32_t t00, t01, t10, t11;
+};
+__device__ __forceinline__ Texels load_texels(const uint8_t* __restrict__ a, const uint8_t* __restrict__ b, int i0, int W,
+                                              bool words) {
+    Texels o;
+    const int off = (3 * i0) & 3;
+    if (words && 3 * i0 - off + 12 <= 3 * W) {
+        const uint32_t* wa = reinterpret_cast<const uint32_t*>(a - off);
+        const uint32_t* wb = reinterpret_cast<const uint32_t*>(b - off);
+        const uint32_t a0 = __ldg(wa), a1 = __ldg(wa + 1), b0 = __ldg(wb), b1 = __ldg(wb + 1);
+        uint32_t a2 = 0u, b2 = 0u;
+        if (off == 3) {
+            a2 = __ldg(wa + 2);
+            b2 = __ldg(wb + 2);
+        }
+        o.t00 = __funnelshift_r(a0, a1, 8 * off);
+        o.t01 = __byte_perm(o.t00, __funnelshift_r(a1, a2, 8 * off), 0x0543);
+        o.t10 = __funnelshift_r(b0, b1, 8 * off);
+        o.t11 = __byte_perm(o.t10, __funnelshift_r(b1, b2, 8 * off), 0x0543);
+    } else {
+        const int di = i0 + 1 < W ? 3 : 0;
+        auto texel = [](const uint8_t* p) {
+            return (uint32_t)__ldg(p) | (uint32_t)__ldg(p + 1) << 8 | (uint32_t)__ldg(p + 2) << 16;
+        };
+        o.t00 = texel(a);
+        o.t01 = texel(a + di);
+        o.t10 = texel(b);
+        o.t11 = texel(b + di);
+    }
+    return o;
+}
+__device__ __forceinline__ bool word_aligned(const uint8_t* px, long long pitch) {
+    return (((uint32_t)reinterpret_cast<uintptr_t>(px) | (uint32_t)pitch) & 3u) == 0u;
+}
+
+// Bilinear RGB sample of an 8-bit frame of width W, scaled by `scale` (= gain / 255).
+__device__ __forceinline__ float3 bilinear_rgb(const uint8_t* __restrict__ px, long long pitch, int W, const Tap& t,
                                                float scale) {
-    const uint8_t* r0 = px + (long long)t.j0 * pitch;
-    const uint8_t* r1 = px + (long long)t.j1 * pitch;
+    const Texels q = load_texels(px + (long long)t.j0 * pitch + 3 * t.i0, px + (long long)t.j1 * pitch + 3 * t.i0, t.i0, W,
+                                 word_aligned(px, pitch));
     float3 o;
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-        const float p00 = __ldg(r0 + 3 * t.i0 + c), p01 = __ldg(r0 + 3 * t.i1 + c);
-        const float p10 = __ldg(r1 + 3 * t.i0 + c), p11 = __ldg(r1 + 3 * t.i1 + c);
+        const float p00 = byte_f(q.t00, c), p01 = byte_f(q.t01, c), p10 = byte_f(q.t10, c), p11 = byte_f(q.t11, c);
         const float top = fmaf(t.fx, p01 - p00, p00);
         const float bot = fmaf(t.fx, p11 - p10, p10);
         const float v = fmaf(t.fy, bot - top, top) * scale;
