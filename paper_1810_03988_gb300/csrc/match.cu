@@ -61,19 +61,26 @@ struct MtState {
 
 constexpr float MT_EPS = 9.5367431640625e-7f;  // 2^-20, see FastInlier
 
-// Hash keys as words whose difference is tested at once: with k <= 16 two tables share a word (an
-// unused upper half differs in every bit), otherwise a table has a word of its own.
+// Hash keys as words whose difference is tested at once: with k <= 16 two tables share a word,
+// otherwise a table has a word of its own.  Words are padded to a power of two of at least 2; unused
+// words and halves differ in every bit.
 __host__ __device__ __forceinline__ bool mt_packed(const LshBits& lb) { return lb.k <= 16; }
-__host__ __device__ __forceinline__ int mt_words(const LshBits& lb) { return mt_packed(lb) ? (lb.L + 1) / 2 : lb.L; }
+inline int mt_words(const LshBits& lb) {
+    int w = 2;
+    while (w < (mt_packed(lb) ? (lb.L + 1) / 2 : lb.L)) w *= 2;
+    return w;
+}
 
 // One key word (blockIdx.y) of 128 descriptors of image A (blockIdx.z 0) or B; the first block also
 // sets up the call's state.  The bit positions are the same for the whole block, so they come from the
 // parameter space as uniform loads; the descriptors' words from shared memory.
-__global__ void __launch_bounds__(128) mt_keys(const unsigned* __restrict__ desc_a, const int* __restrict__ count_a,
-                                               const unsigned* __restrict__ desc_b, const int* __restrict__ count_b,
-                                               const __grid_constant__ LshBits lb, int cap, unsigned* __restrict__ keys_a,
-                                               unsigned* __restrict__ keys_b, MtState* __restrict__ st) {
+__global__ void __launch_bounds__(128) mt_keys(const unsigned* desc_a, const int* count_a,
+                                               const unsigned* desc_b, const int* count_b,
+                                               const __grid_constant__ LshBits lb, int cap, unsigned* keys_a,
+                                               unsigned* keys_b, MtState* st) {
     __shared__ unsigned d[8][128];
+    pdl_trigger();
+    pdl_wait();
     const int t = threadIdx.x, i = blockIdx.x * 128 + t, w = blockIdx.y;
     const bool isb = blockIdx.z != 0;
     if (blockIdx.x == 0 && w == 0 && !isb && t < 4) {
@@ -88,7 +95,7 @@ __global__ void __launch_bounds__(128) mt_keys(const unsigned* __restrict__ desc
     if (i >= n) return;
     const unsigned* src = (isb ? desc_b : desc_a) + 8 * (size_t)i;
 #pragma unroll
-    for (int k = 0; k < 8; ++k) d[k][t] = __ldg(src + k);
+    for (int k = 0; k < 8; ++k) d[k][t] = __ldcg(src + k);
     auto key_of = [&](int l) {
         unsigned key = 0;
 #pragma unroll 4
@@ -98,11 +105,11 @@ __global__ void __launch_bounds__(128) mt_keys(const unsigned* __restrict__ desc
         }
         return key;
     };
-    unsigned key;
+    unsigned key = isb ? 0u : 0xffffffffu;
     if (mt_packed(lb)) {
-        key = key_of(2 * w);
-        key |= 2 * w + 1 < lb.L ? key_of(2 * w + 1) << 16 : isb ? 0u : 0xffff0000u;
-    } else {
+        if (2 * w < lb.L) key = key_of(2 * w) | (key & 0xffff0000u);
+        if (2 * w + 1 < lb.L) key = key_of(2 * w + 1) << 16 | (key & 0xffffu);
+    } else if (w < lb.L) {
         key = key_of(w);
     }
     (isb ? keys_b : keys_a)[(size_t)w * cap + i] = key;
@@ -133,37 +140,28 @@ __device__ __forceinline__ void top2_add(Top2& t, int d, int b) {
     }
 }
 
-// Whether a query meets a descriptor of image B in some table: the keys differ in at most one bit.
-// x & (x - 1) clears the lowest bit of x; on packed halves a borrow leaves the lower half only when
-// that half is 0, that is, when it has already met.
-template <bool PACKED>
-__device__ __forceinline__ bool mt_meets(const unsigned* __restrict__ keys_b, const unsigned* __restrict__ ka, int nw, int cap,
-                                         int b) {
-    unsigned acc = 0xffffffffu;
-#pragma unroll 4
-    for (int w = 0; w < nw; ++w) {
-        const unsigned x = ka[w] ^ __ldg(keys_b + (size_t)w * cap + b);
-        const unsigned z = x & (x - (PACKED ? 0x00010001u : 1u));
-        acc = PACKED ? __vminu2(acc, z) : min(acc, z);
-    }
-    return PACKED ? (acc & 0xffffu) == 0u || (acc >> 16) == 0u : acc == 0u;
-}
-
 // A warp per query, its lanes over every descriptor of image B: those that the query meets in a table
-// are gathered and their distances taken 32 at a time.  Testing all pairs costs some 20 instructions
-// each, 38 us for 1000 x 1000 points and 8 tables, nearly all of it load latency; hashing into sorted buckets and probing them took
-// 32 us (a bitonic sort per table, then a chain of dependent loads per probe).
-template <bool PACKED>
-__global__ void __launch_bounds__(256) mt_match(const unsigned* __restrict__ desc_a, const int* __restrict__ count_a,
-                                                const unsigned* __restrict__ desc_b, const int* __restrict__ count_b,
-                                                const unsigned* __restrict__ keys_a, const unsigned* __restrict__ keys_b,
-                                                int nw, int cap, const int* __restrict__ xy_a, const int* __restrict__ xy_b,
-                                                int max_dist, int rnum, int rden, int2* __restrict__ best,
-                                                MtState* __restrict__ st) {
-    __shared__ unsigned s_ka[8][MT_MAX_WORDS];
+// (keys differing in at most one bit) are gathered and their distances taken 32 at a time.  Image B's
+// keys pass through shared memory in chunks, so that their loads are all in flight, the query's stay in
+// registers; a pair then costs some 30 instructions.  11 us for 1000 x 1000 points and 8 tables (38 us
+// with the keys read from global memory pair by pair); hashing into sorted buckets and probing them
+// took 32 us (a bitonic sort per table, then a chain of dependent loads per probe).
+constexpr int MT_CHUNK = 8192;  // key words of a chunk
+template <bool PACKED, int NW>
+__global__ void __launch_bounds__(256) mt_match(const unsigned* desc_a, const int* count_a,
+                                                const unsigned* desc_b, const int* count_b,
+                                                const unsigned* keys_a, const unsigned* keys_b,
+                                                int cap, const int* xy_a, const int* xy_b,
+                                                int max_dist, int rnum, int rden, int2* best,
+                                                MtState* st) {
+    constexpr int CB = MT_CHUNK / NW;  // descriptors of a chunk
+    __shared__ unsigned s_kb[NW][CB];
     __shared__ uint16_t s_hit[8][64];
     __shared__ int s_mn[4], s_mx[4], s_n;
     const int t = threadIdx.x, w = t >> 5, lane = t & 31, a = blockIdx.x * 8 + w;
+    const bool aligned_b = (reinterpret_cast<uintptr_t>(desc_b) & 15) == 0;
+    pdl_trigger();
+    pdl_wait();
     const int na = min(*count_a, cap), nb = min(*count_b, cap);
     if (blockIdx.x * 8 >= na) return;
     if (t < 4) {
@@ -171,28 +169,56 @@ __global__ void __launch_bounds__(256) mt_match(const unsigned* __restrict__ des
         s_mx[t] = INT_MIN;
         if (t == 0) s_n = 0;
     }
-    __syncthreads();
-    if (a < na) {
-        if (lane < nw) s_ka[w][lane] = keys_a[(size_t)lane * cap + a];
-        unsigned da[8];
+    unsigned da[8], ka[NW];
 #pragma unroll
-        for (int k = 0; k < 8; ++k) da[k] = desc_a[8 * (size_t)a + k];
-        __syncwarp();
-        constexpr int INF = 1 << 30;
-        Top2 best2{INF, -1, INF, -1};
-        int nh = 0;
-        auto take = [&](int n) {  // the first n gathered descriptors
-            if (lane < n) {
-                const int b = s_hit[w][lane];
-                top2_add(best2, hamming(da, desc_b + 8 * (size_t)b), b);
+    for (int k = 0; k < 8; ++k) da[k] = a < na ? desc_a[8 * (size_t)a + k] : 0u;
+#pragma unroll
+    for (int k = 0; k < NW; ++k) ka[k] = a < na ? keys_a[(size_t)k * cap + a] : 0u;
+    constexpr int INF = 1 << 30;
+    Top2 best2{INF, -1, INF, -1};
+    int nh = 0;
+    auto take = [&](int n) {  // the first n gathered descriptors
+        if (lane < n) {
+            const int b = s_hit[w][lane];
+            const uint4* q = reinterpret_cast<const uint4*>(desc_b) + 2 * (size_t)b;
+            unsigned db[8];
+            if (aligned_b) {
+                const uint4 q0 = __ldcg(q), q1 = __ldcg(q + 1);
+                db[0] = q0.x, db[1] = q0.y, db[2] = q0.z, db[3] = q0.w;
+                db[4] = q1.x, db[5] = q1.y, db[6] = q1.z, db[7] = q1.w;
+            } else {
+#pragma unroll
+                for (int k = 0; k < 8; ++k) db[k] = __ldcg(desc_b + 8 * (size_t)b + k);
             }
-            __syncwarp();
-        };
-        for (int b0 = 0; b0 < nb; b0 += 32) {
+            top2_add(best2, hamming(da, db), b);
+        }
+        __syncwarp();
+    };
+    for (int c0 = 0; c0 < nb; c0 += CB) {
+        const int cn = min(CB, nb - c0);
+        __syncthreads();
+#pragma unroll 8
+        for (int q = t; q < NW * CB; q += 256) {
+            const int i = q % CB;
+            if (i < cn) s_kb[q / CB][i] = __ldcg(keys_b + (size_t)(q / CB) * cap + c0 + i);
+        }
+        __syncthreads();
+        if (a >= na) continue;
+        for (int b0 = 0; b0 < cn; b0 += 32) {
             const int b = b0 + lane;
-            const bool hit = b < nb && mt_meets<PACKED>(keys_b, s_ka[w], nw, cap, b);
+            // x & (x - 1) clears the lowest bit of x; on packed halves a borrow leaves the lower half
+            // only when that half is 0, that is, when it has already met
+            unsigned acc = 0xffffffffu;
+#pragma unroll
+            for (int k = 0; k < NW; ++k) {
+                const unsigned x = ka[k] ^ s_kb[k][b];
+                const unsigned z = x & (x - (PACKED ? 0x00010001u : 1u));
+                acc = PACKED ? __vminu2(acc, z) : min(acc, z);
+            }
+            const bool hit = b < cn && (PACKED ? (acc & 0xffffu) == 0u || (acc >> 16) == 0u : acc == 0u);
             const unsigned m = __ballot_sync(0xffffffffu, hit);
-            if (hit) s_hit[w][nh + __popc(m & ((1u << lane) - 1u))] = (uint16_t)b;
+            if (m == 0u) continue;
+            if (hit) s_hit[w][nh + __popc(m & ((1u << lane) - 1u))] = (uint16_t)(c0 + b);
             nh += __popc(m);
             __syncwarp();
             if (nh >= 32) {
@@ -204,6 +230,8 @@ __global__ void __launch_bounds__(256) mt_match(const unsigned* __restrict__ des
                 __syncwarp();
             }
         }
+    }
+    if (a < na) {
         take(nh);
         // merge: the union's two nearest distinct indices are among the lanes' two nearest
         for (int off = 16; off > 0; off >>= 1) {
@@ -241,7 +269,7 @@ __global__ void __launch_bounds__(256) mt_match(const unsigned* __restrict__ des
 // The growth schedule by one block of 256 threads.  The top n grows to n + 1 at iteration E_j
 // (j = n - 4), E_0 = 1 and E_{j+1} = E_j + ceil(T_N m n (n-1) (n-2) / (N (N-1) (N-2) (N-3))) (m = 4,
 // T_N = 200000: the exact increment T_{n+1} - T_n of T_n = T_N C(n, m) / C(N, m)), up to n = N.
-__device__ __forceinline__ void mt_schedule(int N, long long* __restrict__ E) {
+__device__ __forceinline__ void mt_schedule(int N, long long* E) {
     __shared__ long long wsum[8];
     constexpr int PT = MT_MAX_POINTS / 256;
     const int t = threadIdx.x, lane = t & 31, w = t >> 5;
@@ -274,11 +302,13 @@ __device__ __forceinline__ void mt_schedule(int N, long long* __restrict__ E) {
 // A warp per query: an accepted match's place in quality order is the number of accepted matches
 // before it.  It writes the match and its normalised coordinates (x, y, u, v), the latter also in
 // single precision for mt_count.  The last block computes the growth schedule.
-__global__ void __launch_bounds__(256) mt_rank(const int2* __restrict__ best, const int* __restrict__ count_a, int cap,
-                                               const int* __restrict__ xy_a, const int* __restrict__ xy_b,
-                                               MtState* __restrict__ st, int* __restrict__ matches,
-                                               int* __restrict__ n_matches, double* __restrict__ xyuv,
-                                               float* __restrict__ xyuvf, long long* __restrict__ E, double inlier_px) {
+__global__ void __launch_bounds__(256) mt_rank(const int2* best, const int* count_a, int cap,
+                                               const int* xy_a, const int* xy_b,
+                                               MtState* st, int* matches,
+                                               int* n_matches, double* xyuv,
+                                               float* xyuvf, long long* E, double inlier_px) {
+    pdl_trigger();
+    pdl_wait();
     const int t = threadIdx.x, lane = t & 31, N = st->n;
     if (blockIdx.x == gridDim.x - 1) {
         mt_schedule(N, E);
@@ -349,6 +379,15 @@ __device__ __forceinline__ int nth_free(int j, const int* chosen, int c) {
     return j;
 }
 
+// a / b for finite b; a zero a, which half the entries of a DLT system are and which the division
+// leaves to its slow path, gets its signed zero directly.
+__device__ __forceinline__ double quotient(double a, double b) {
+    const unsigned long long x = (unsigned long long)__double_as_longlong(a), y = (unsigned long long)__double_as_longlong(b);
+    const bool zero = (x << 1) == 0ull;
+    const double q = dD(zero ? 1.0 : a, b);
+    return zero ? __longlong_as_double((long long)((x ^ y) & (1ull << 63))) : q;
+}
+
 // M h = r by 8 lanes (a lane per row of A = [M | r], four systems per warp): every entry receives the
 // operations of the sequential elimination with partial pivoting in the same order, so h is bit-identical.
 // Rows stay in their lanes; a lane keeps its row's place in the current order, and the pivot is the
@@ -376,7 +415,7 @@ __device__ bool solve8(double A[9], double h[8]) {
         ok &= v >= __double_as_longlong(1e-12) && v <= 0x7ff0000000000000ll;
         place = place == p ? c : place == c ? p : place;  // the pivot row and row c change places
         const int src = group + __ffs(__ballot_sync(FULL, place == c) >> group) - 1;
-        const double f = dD(A[c], __shfl_sync(FULL, A[c], src));
+        const double f = quotient(A[c], __shfl_sync(FULL, A[c], src));
 #pragma unroll
         for (int j = c + 1; j < 9; ++j) {
             const double x = __shfl_sync(FULL, A[j], src);
@@ -390,7 +429,7 @@ __device__ bool solve8(double A[9], double h[8]) {
 #pragma unroll
         for (int k = c + 1; k < 8; ++k) s = dS(s, prod[k]);
         const int src = group + __ffs(__ballot_sync(FULL, place == c) >> group) - 1;
-        h[c] = __shfl_sync(FULL, dD(s, A[c]), src);
+        h[c] = __shfl_sync(FULL, quotient(s, place == c ? A[c] : 1.0), src);
         prod[c] = dM(A[c], h[c]);
     }
     return ok;
@@ -428,9 +467,9 @@ struct FastInlier {
     }
 };
 
-__device__ __forceinline__ bool mt_inlier(const FastInlier& fast, const double* h, const double* __restrict__ xyuv,
-                                          const float* __restrict__ xyuvf, int i, double t2) {
-    const int d = fast(reinterpret_cast<const float4*>(xyuvf)[i]);
+__device__ __forceinline__ bool mt_inlier(const FastInlier& fast, const double* h, const double* xyuv,
+                                          float4 p, int i, double t2) {
+    const int d = fast(p);
     if (d >= 0) return d != 0;
     return inlier(h, xyuv[4 * i], xyuv[4 * i + 1], xyuv[4 * i + 2], xyuv[4 * i + 3], t2);
 }
@@ -439,17 +478,20 @@ __device__ __forceinline__ bool mt_inlier(const FastInlier& fast, const double* 
 // schedule c = #{j < N - 4 : E_j <= t}, n(t) = 4 + c, uniform sampling when E_c < t), one warp solves the
 // four 4-point systems, then each warp counts the inliers of one.  The solving warp is another one
 // from each wave of `sms` blocks to the next, so that the blocks of an SM solve on different
-// schedulers.  30 us for 1000 iterations on 374 matches, against 61 us for the two kernels with a
+// schedulers.  23 us for 1000 iterations on 374 matches, against 61 us for the two kernels with a
 // block per iteration (FP64 inlier tests alone: 30 us at two lanes per clock and SM).
-__global__ void __launch_bounds__(128) mt_hypotheses(int iters, const long long* __restrict__ E,
-                                                     const unsigned* __restrict__ rnd, const double* __restrict__ xyuv,
-                                                     const float* __restrict__ xyuvf, int sms,
-                                                     double* __restrict__ hyp, MtState* __restrict__ st) {
+__global__ void __launch_bounds__(128) mt_hypotheses(int iters, const long long* E,
+                                                     const unsigned* rnd, const double* xyuv,
+                                                     const float* xyuvf, int sms,
+                                                     double* hyp, MtState* st) {
     __shared__ int sidx[4][4];
     __shared__ double sh[4][8];
     __shared__ float shf[4][8];
     __shared__ int s_ok[4];
+    __shared__ float4 pts[MT_MAX_POINTS];  // the matches, brought in by the warps that do not solve
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, it = 4 * blockIdx.x + w;
+    pdl_trigger();
+    pdl_wait();
     const int N = st->n;
     if (N < 4) return;
     {
@@ -478,7 +520,12 @@ __global__ void __launch_bounds__(128) mt_hypotheses(int iters, const long long*
         }
     }
     __syncthreads();
-    if (w == (int)((blockIdx.x / (unsigned)sms) & 3u)) {
+    const int solver = (int)((blockIdx.x / (unsigned)sms) & 3u);
+    if (w != solver) {
+        const int k = (w - solver - 1) & 3;  // 0, 1, 2
+#pragma unroll 4
+        for (int i = 32 * k + lane; i < N; i += 96) pts[i] = __ldcg(reinterpret_cast<const float4*>(xyuvf) + i);
+    } else {
         // rows 2k, 2k+1 of pair k: (x, y, 1, 0, 0, 0, -ux, -uy | u), (0, 0, 0, x, y, 1, -vx, -vy | v)
         const int g = lane >> 3, r = lane & 7, m = sidx[g][r >> 1];
         const bool odd = r & 1;
@@ -500,7 +547,7 @@ __global__ void __launch_bounds__(128) mt_hypotheses(int iters, const long long*
     const double t2 = st->t2;
     const FastInlier fast(shf[w], st);
     int c = 0;
-    for (int i = lane; i < N; i += 32) c += mt_inlier(fast, sh[w], xyuv, xyuvf, i, t2);
+    for (int i = lane; i < N; i += 32) c += mt_inlier(fast, sh[w], xyuv, pts[i], i, t2);
     c = __reduce_add_sync(0xffffffffu, c);
     // most inliers, ties to the earlier iteration
     if (lane == 0) atomicMax(&st->best, (unsigned long long)(c + 1) << 32 | (unsigned long long)(0xffffffffu - (unsigned)it));
@@ -518,12 +565,12 @@ __global__ void __launch_bounds__(128) mt_hypotheses(int iters, const long long*
 // symmetric).  A sum is a chain of additions in order, 64 cycles each whether one lane adds or 32: warp 0
 // carries the 24 in its lanes, warp 1 the 5, on schedulers of their own, while the warps of the other
 // two schedulers form the products of the next 64 inliers.  The longest chain is two additions per
-// inlier (20 us for 333) and bounds the kernel; 51 us in all, against 61 us as three kernels.
+// inlier (20 us for 333) and bounds the kernel; 45 us in all, against 61 us as three kernels.
 constexpr int MF_THREADS = 512, MF_CHUNK = 64, MF_ONE = 24, MF_TWO = 5, MF_ROW = 35;
-__global__ void __launch_bounds__(MF_THREADS) mt_final(MtState* __restrict__ st, const double* __restrict__ hyp,
-                                                       const double* __restrict__ xyuv, const float* __restrict__ xyuvf,
-                                                       unsigned char* __restrict__ inl,
-                                                       double* __restrict__ H, int* __restrict__ n_inliers) {
+__global__ void __launch_bounds__(MF_THREADS, 1) mt_final(MtState* st, const double* hyp,
+                                                       const double* xyuv, const float* xyuvf,
+                                                       unsigned char* inl,
+                                                       double* H, int* n_inliers) {
     __shared__ double buf[2][MF_CHUNK * MF_ROW];  // products of a chunk's inliers: 24, then 5 pairs
     __shared__ uint16_t list[MT_MAX_POINTS];      // the inliers in quality order
     __shared__ double sums[MF_ONE + MF_TWO];
@@ -531,6 +578,8 @@ __global__ void __launch_bounds__(MF_THREADS) mt_final(MtState* __restrict__ st,
     __shared__ float hf[8];
     __shared__ int wcnt[MF_THREADS / 32], s_n;
     const int t = threadIdx.x, lane = t & 31, w = t >> 5;
+    pdl_trigger();
+    pdl_wait();
     const int N = st->n;
     const unsigned long long best = st->best;
     const int bc = (int)(best >> 32) - 1;
@@ -552,7 +601,7 @@ __global__ void __launch_bounds__(MF_THREADS) mt_final(MtState* __restrict__ st,
         const FastInlier fast(hf, st);
         for (int i0 = 0; i0 < N; i0 += MF_THREADS) {
             const int i = i0 + t;
-            const bool f = i < N && mt_inlier(fast, hb, xyuv, xyuvf, i, t2);
+            const bool f = i < N && mt_inlier(fast, hb, xyuv, reinterpret_cast<const float4*>(xyuvf)[i], i, t2);
             if (i < N) inl[i] = f;
             const unsigned m = __ballot_sync(0xffffffffu, f);
             if (lane == 0) wcnt[w] = __popc(m);
@@ -781,16 +830,20 @@ extern "C" stitch_status stitch_match_homography(stitch_matcher* c, const int32_
     const unsigned* db = reinterpret_cast<const unsigned*>(desc_b);
     const int nw = mt_words(lb), iters = prm->iters;
     unsigned *ka = c->keys, *kb = c->keys + (size_t)MT_MAX_WORDS * cap;
-    mt_keys<<<dim3((cap + 127) / 128, nw, 2), 128, 0, s>>>(da, count_a, db, count_b, lb, cap, ka, kb, c->st);
-    auto match = mt_packed(lb) ? mt_match<true> : mt_match<false>;
-    match<<<(cap + 7) / 8, 256, 0, s>>>(da, count_a, db, count_b, ka, kb, nw, cap, xy_a, xy_b, prm->max_dist,
-                                        prm->ratio_num, prm->ratio_den, c->best, c->st);
-    mt_rank<<<(cap + 7) / 8 + 1, 256, 0, s>>>(c->best, count_a, cap, xy_a, xy_b, c->st, matches, n_matches, c->xyuv,
-                                              c->xyuvf, c->E, prm->inlier_px);
+    pdl_launch(mt_keys, dim3((cap + 127) / 128, nw, 2), 128, 0, s, da, count_a, db, count_b, lb, cap, ka, kb, c->st);
+    const bool pk = mt_packed(lb);
+    auto match = nw <= 2   ? (pk ? mt_match<true, 2> : mt_match<false, 2>)
+                 : nw <= 4 ? (pk ? mt_match<true, 4> : mt_match<false, 4>)
+                 : nw <= 8 ? (pk ? mt_match<true, 8> : mt_match<false, 8>)
+                 : nw <= 16 ? (pk ? mt_match<true, 16> : mt_match<false, 16>)
+                            : mt_match<false, 32>;
+    pdl_launch(match, (cap + 7) / 8, 256, 0, s, da, count_a, db, count_b, ka, kb, cap, xy_a, xy_b, prm->max_dist,
+               prm->ratio_num, prm->ratio_den, c->best, c->st);
+    pdl_launch(mt_rank, (cap + 7) / 8 + 1, 256, 0, s, c->best, count_a, cap, xy_a, xy_b, c->st, matches, n_matches,
+               c->xyuv, c->xyuvf, c->E, prm->inlier_px);
     if (iters > 0)
-        mt_hypotheses<<<(iters + 3) / 4, 128, 0, s>>>(iters, c->E, rnd, c->xyuv, c->xyuvf, c->sms, c->hyp,
-                                                      c->st);
-    mt_final<<<1, MF_THREADS, 0, s>>>(c->st, c->hyp, c->xyuv, c->xyuvf, inlier, H, n_inliers);
+        pdl_launch(mt_hypotheses, (iters + 3) / 4, 128, 0, s, iters, c->E, rnd, c->xyuv, c->xyuvf, c->sms, c->hyp, c->st);
+    pdl_launch(mt_final, 1, MF_THREADS, 0, s, c->st, c->hyp, c->xyuv, c->xyuvf, inlier, H, n_inliers);
     stitch_status st = cudaGetLastError() == cudaSuccess ? STITCH_OK : STITCH_ECUDA;
     if (prev >= 0 && prev != c->device) cudaSetDevice(prev);
     return st;
