@@ -29,7 +29,7 @@ struct LorbAreas {
 };
 
 struct LorbPattern {
-    int8_t p[256][4];
+    char4 p[256];  // ax, ay, bx, by
 };
 
 struct Cand {
@@ -44,6 +44,14 @@ __device__ __forceinline__ bool in_areas(const LorbAreas& a, int x, int y) {
 }
 
 __device__ __forceinline__ unsigned gray_of(unsigned r, unsigned g, unsigned b) { return (77u * r + 150u * g + 29u * b + 128u) >> 8; }
+
+// gray of the four pixels in the bytes R G B R | G B R G | B R G B of a, b, c
+__device__ __forceinline__ void gray4(unsigned a, unsigned b, unsigned c, unsigned o[4]) {
+    o[0] = __dp4a(a, 0x001D964Du, 128u) >> 8;
+    o[1] = __dp4a(b, 0x00001D96u, __dp4a(a, 0x4D000000u, 128u)) >> 8;
+    o[2] = __dp4a(c, 0x0000001Du, __dp4a(b, 0x964D0000u, 128u)) >> 8;
+    o[3] = __dp4a(c, 0x1D964D00u, 128u) >> 8;
+}
 
 // Coarse, monotone (non-decreasing in R') bin of a response: the position of its leading bit and
 // the 4 bits below it; R' <= 0 in bin 0.  The N strongest candidates all lie in the bins at or above
@@ -61,6 +69,7 @@ __device__ __forceinline__ int lorb_bin(long long r) {
 struct LorbCount {
     int n, done, n2, pad;
     int hist[LORB_BINS];
+    char4 pat[256];  // the call's BRIEF pattern
 };
 
 // lorb_detect: gray, FAST, Harris response and non-maximum suppression of one tile, appending the
@@ -73,15 +82,15 @@ struct LorbCount {
 //  - the tile's gray is staged as words that hold a pixel and the one below it (16 bits each), so one
 //    32-bit load and one 16-bit-pair minimum or maximum serve two pixels, at any offset;
 //  - a pair is tested on its 4 compass pixels first (an arc of 9 of the 16 circle pixels holds two
-//    neighbouring ones).  The pairs that pass are gathered per warp, so the 16-pixel test and then
-//    the Harris response of the corners run with full warps instead of under a branch that nearly
-//    every warp takes for a few lanes.
-// One 3840 x 2160 view: 35 us against 134 us for gray and smoothed maps, response map (8 bytes per
+//    neighbouring ones).  The pairs that pass are gathered for the block, so the 16-pixel test and
+//    then the Harris response of the corners run with full warps instead of under a branch that nearly
+//    every warp takes for a few lanes, and spread over all warps however the corners lie.
+// One 3840 x 2160 view: 34 us (of which 18 us are issue slots; 35 us and a quarter more instructions with lists per warp) against 134 us for gray and smoothed maps, response map (8 bytes per
 // pixel written and read back) and suppression as three kernels.
 constexpr int DT_EX = 64, DT_EY = 32;   // evaluated pixels
 constexpr int DT_OX = 60, DT_OY = 30;   // owned pixels: columns 2 .. 61, rows 1 .. 30
 constexpr int DT_PX = 72, DT_PY = 39;   // gray words: 18 groups of 4 columns, 13 strips of 3 rows
-constexpr int DT_WARPS = 8;
+constexpr int DT_PAIRS = DT_EX * DT_EY / 2;
 
 // whether either of the two pixels p (16 bits each) has an arc value above it (mb: the largest of the
 // arcs' smallest values) or below it (md) by more than the threshold; lim = threshold + 256
@@ -89,16 +98,18 @@ __device__ __forceinline__ unsigned fast_excess(unsigned p, unsigned mb, unsigne
     return __vmaxu2((mb + 0x01000100u) - p, (p + 0x01000100u) - md);
 }
 
-__global__ void __launch_bounds__(256, 5) lorb_detect(const uint8_t* __restrict__ frame, long long pitch, int W, int H,
+__global__ void __launch_bounds__(256, 5) lorb_detect(const uint8_t* frame, long long pitch, int W, int H,
                                                       int ox, int oy, const __grid_constant__ LorbAreas areas, int lim,
-                                                      long long harris_t, Cand* __restrict__ cand, int* __restrict__ ncand,
-                                                      int cap, int* __restrict__ hist, int* __restrict__ n2) {
+                                                      long long harris_t, Cand* cand, int* ncand,
+                                                      int cap, int* hist, int* n2) {
     __shared__ __align__(16) unsigned P[DT_PX * DT_PY];
     __shared__ long long R[DT_EX * DT_EY];
     __shared__ unsigned mask[DT_EY][2];  // which pixels of a row have a response
-    __shared__ uint16_t pairs[DT_WARPS][128], corners[DT_WARPS][256];
-    __shared__ int s_n, s_base;
+    __shared__ uint16_t pairs[DT_PAIRS], corners[2 * DT_PAIRS];
+    __shared__ int s_np, s_nc, s_n, s_base;
     const int t = threadIdx.x, lane = t & 31, w = t >> 5;
+    pdl_trigger();
+    pdl_wait();
     // owned pixels start at (bx, by); bx is 1 modulo 4, so the staged columns start at a multiple of 4
     const int bx = ox + DT_OX * blockIdx.x, by = oy + DT_OY * blockIdx.y;
     if (blockIdx.x == 0 && blockIdx.y == 0 && t == 0) *n2 = 0;
@@ -107,7 +118,7 @@ __global__ void __launch_bounds__(256, 5) lorb_detect(const uint8_t* __restrict_
         any |= bx < areas.r[k][2] && bx + DT_OX > areas.r[k][0] && by < areas.r[k][3] && by + DT_OY > areas.r[k][1];
     if (!any) return;
     if (t < 2 * DT_EY) mask[t >> 1][t & 1] = 0u;
-    if (t == 0) s_n = 0;
+    if (t == 0) s_np = s_nc = s_n = 0;
     if (t < 18 * 13) {
         const int j = t % 18, st = t / 18, gx0 = bx - 5 + 4 * j;
         const bool words = ((reinterpret_cast<uintptr_t>(frame) | (uintptr_t)pitch) & 3) == 0 && gx0 + 3 < W;
@@ -123,14 +134,7 @@ __global__ void __launch_bounds__(256, 5) lorb_detect(const uint8_t* __restrict_
                 v[k][2] = __ldg(q + 2);
             }
 #pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                // bytes R G B R | G B R G | B R G B
-                const unsigned a = v[k][0], b = v[k][1], c = v[k][2];
-                g[k][0] = __dp4a(a, 0x001D964Du, 128u) >> 8;
-                g[k][1] = __dp4a(b, 0x00001D96u, __dp4a(a, 0x4D000000u, 128u)) >> 8;
-                g[k][2] = __dp4a(c, 0x0000001Du, __dp4a(b, 0x964D0000u, 128u)) >> 8;
-                g[k][3] = __dp4a(c, 0x1D964D00u, 128u) >> 8;
-            }
+            for (int k = 0; k < 4; ++k) gray4(v[k][0], v[k][1], v[k][2], g[k]);
         } else {
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
@@ -149,12 +153,19 @@ __global__ void __launch_bounds__(256, 5) lorb_detect(const uint8_t* __restrict_
                            g[k][3] | g[k + 1][3] << 16);
     }
     __syncthreads();
-    // evaluated pixel (ex, ey) is image pixel (bx - 2 + ex, by - 1 + ey), staged at P[ey + 3][ex + 3];
-    // warp w takes rows 4 w .. 4 w + 3 through all phases
+    // evaluated pixel (ex, ey) is image pixel (bx - 2 + ex, by - 1 + ey), staged at P[ey + 3][ex + 3]
     constexpr int fo[16] = {-3 * DT_PX,     -3 * DT_PX + 1, -2 * DT_PX + 2, -DT_PX + 3, 3,  DT_PX + 3,  2 * DT_PX + 2,  3 * DT_PX + 1,
                             3 * DT_PX,      3 * DT_PX - 1,  2 * DT_PX - 2,  DT_PX - 3,  -3, -DT_PX - 3, -2 * DT_PX - 2, -3 * DT_PX - 1};
     const unsigned below = (1u << lane) - 1u;
-    int np = 0;
+    // appends v of the lanes with `keep` to a list of the block
+    auto append = [&](bool keep, int v, uint16_t* list, int* n) {
+        const unsigned m = __ballot_sync(0xffffffffu, keep);
+        if (m == 0u) return;
+        int base = 0;
+        if (lane == 0) base = atomicAdd(n, __popc(m));
+        base = __shfl_sync(0xffffffffu, base, 0);
+        if (keep) list[base + __popc(m & below)] = (uint16_t)v;
+    };
 #pragma unroll
     for (int it = 0; it < 4; ++it) {
         const int ey = 4 * w + 2 * (it >> 1), ex = 32 * (it & 1) + lane;
@@ -162,17 +173,15 @@ __global__ void __launch_bounds__(256, 5) lorb_detect(const uint8_t* __restrict_
         const unsigned p = c[0], n = c[fo[0]], e = c[fo[4]], s = c[fo[8]], o = c[fo[12]];
         const unsigned x = fast_excess(p, __vminu2(__vmaxu2(n, s), __vmaxu2(e, o)), __vmaxu2(__vminu2(n, s), __vminu2(e, o)));
         const bool pass = ((int)(x & 0xffffu) > lim || (int)(x >> 16) > lim) && ex >= 1 && ex <= 62;
-        const unsigned m = __ballot_sync(0xffffffffu, pass);
-        if (pass) pairs[w][np + __popc(m & below)] = (uint16_t)(ey * DT_EX + ex);
-        np += __popc(m);
+        append(pass, ey * DT_EX + ex, pairs, &s_np);
     }
-    __syncwarp();
-    int nc = 0;
-    for (int i0 = 0; i0 < np; i0 += 32) {
+    __syncthreads();
+    const int np = s_np;
+    for (int i0 = 32 * w; i0 < np; i0 += 256) {
         bool lo = false, hi = false;
         int at = 0;
         if (i0 + lane < np) {
-            at = pairs[w][i0 + lane];
+            at = pairs[i0 + lane];
             const int ex = at & (DT_EX - 1), ey = at / DT_EX;
             const unsigned* c = P + (ey + 3) * DT_PX + ex + 3;
             unsigned v[16];
@@ -200,15 +209,13 @@ __global__ void __launch_bounds__(256, 5) lorb_detect(const uint8_t* __restrict_
             lo = (int)(x & 0xffffu) > lim && in_areas(areas, ix, iy);
             hi = (int)(x >> 16) > lim && in_areas(areas, ix, iy + 1);
         }
-        const unsigned ml = __ballot_sync(0xffffffffu, lo), mh = __ballot_sync(0xffffffffu, hi);
-        if (lo) corners[w][nc + __popc(ml & below)] = (uint16_t)at;
-        nc += __popc(ml);
-        if (hi) corners[w][nc + __popc(mh & below)] = (uint16_t)(at + DT_EX);
-        nc += __popc(mh);
+        append(lo, at, corners, &s_nc);
+        append(hi, at + DT_EX, corners, &s_nc);
     }
-    __syncwarp();
-    for (int i = lane; i < nc; i += 32) {
-        const int at = corners[w][i], ex = at & (DT_EX - 1), ey = at / DT_EX;
+    __syncthreads();
+    const int nc = s_nc;
+    for (int i = t; i < nc; i += 256) {
+        const int at = corners[i], ex = at & (DT_EX - 1), ey = at / DT_EX;
         const uint16_t* c = reinterpret_cast<const uint16_t*>(P + (ey + 3) * DT_PX + ex + 3);  // the pixel's own half
         const int b5[5] = {1, 4, 6, 4, 1};
         int A = 0, B = 0, C = 0;  // at most 256 * 255 * 255
@@ -236,13 +243,13 @@ __global__ void __launch_bounds__(256, 5) lorb_detect(const uint8_t* __restrict_
     __syncthreads();
     // non-maximum suppression (ties to the lower index), survivors into the pair list's memory: no two
     // are neighbours, so at most a quarter of the evaluated pixels
-    uint16_t* surv = &pairs[0][0];
-    static_assert(sizeof(pairs) / sizeof(uint16_t) >= (DT_OX / 2) * (DT_OY / 2), "room for the survivors");
-    for (int i0 = 0; i0 < nc; i0 += 32) {
+    uint16_t* surv = pairs;
+    static_assert(DT_PAIRS >= (DT_OX / 2) * (DT_OY / 2), "room for the survivors");
+    for (int i0 = 32 * w; i0 < nc; i0 += 256) {
         bool keep = false;
         int at = 0;
         if (i0 + lane < nc) {
-            at = corners[w][i0 + lane];
+            at = corners[i0 + lane];
             const int ex = at & (DT_EX - 1), ey = at / DT_EX;
             if (ex >= 2 && ex < 2 + DT_OX && ey >= 1 && ey < 1 + DT_OY && (mask[ey][ex >> 5] >> (ex & 31) & 1u)) {
                 const long long r = R[at];
@@ -261,11 +268,7 @@ __global__ void __launch_bounds__(256, 5) lorb_detect(const uint8_t* __restrict_
                 }
             }
         }
-        const unsigned m = __ballot_sync(0xffffffffu, keep);
-        int base = 0;
-        if (lane == 0 && m) base = atomicAdd(&s_n, __popc(m));
-        base = __shfl_sync(0xffffffffu, base, 0);
-        if (keep) surv[base + __popc(m & below)] = (uint16_t)at;
+        append(keep, at, surv, &s_n);
     }
     __syncthreads();
     if (t == 0) s_base = s_n ? atomicAdd(ncand, s_n) : 0;
@@ -333,8 +336,8 @@ struct SelectSmem {
     int need, nwin;
 };
 
-__device__ void lorb_select(const Cand* __restrict__ cand, int n, int npts, int W, int* __restrict__ out_xy,
-                            long long* __restrict__ out_resp, SelectSmem& sm) {
+__device__ void lorb_select(const Cand* cand, int n, int npts, int W, int* out_xy,
+                            long long* out_resp, SelectSmem& sm) {
     int* hist = sm.hist;
     Cand* win = sm.win;
     unsigned long long& s_prefix = sm.prefix;
@@ -442,15 +445,21 @@ __device__ void lorb_select(const Cand* __restrict__ cand, int n, int npts, int 
 // call, and selects the points itself when cand2 is too crowded to be ranked by counting.
 constexpr int PRUNE_THREADS = 1024, PRUNE_BLOCKS = 64;
 constexpr int RANK_MAX = 8192;  // candidates that lorb_rank_brief ranks by counting
-__global__ void __launch_bounds__(PRUNE_THREADS) lorb_prune(const Cand* __restrict__ cand, LorbCount* __restrict__ cnt, int cap,
-                                                            int npts, Cand* __restrict__ cand2, int W,
-                                                            int* __restrict__ out_xy, long long* __restrict__ out_resp,
-                                                            int* __restrict__ count) {
+__global__ void __launch_bounds__(PRUNE_THREADS) lorb_prune(const Cand* cand, LorbCount* cnt, int cap,
+                                                            int npts, Cand* cand2, int W,
+                                                            const __grid_constant__ LorbPattern pat,
+                                                            int* out_xy, long long* out_resp,
+                                                            int* count) {
     static_assert(PRUNE_THREADS == LORB_BINS && PRUNE_THREADS == SEL_THREADS, "one bin per thread; the block also selects");
     __shared__ SelectSmem sm;
     __shared__ int wsum[32];
     __shared__ int s_b, s_last;
     const int t = threadIdx.x, lane = t & 31, w = t >> 5;
+    pdl_trigger();
+    pdl_wait();
+    // the pattern to memory, where lorb_rank_brief's lanes read it side by side (lane-dependent reads of
+    // the parameter space are serialised)
+    if (blockIdx.x == 1 && t < 256) cnt->pat[t] = pat.p[t];
     const int n = min(cnt->n, cap), want = min(n, npts);
     const int* hist = cnt->hist;
     if (t == 0) s_b = LORB_BINS;  // want == 0: nothing
@@ -514,21 +523,22 @@ __global__ void __launch_bounds__(PRUNE_THREADS) lorb_prune(const Cand* __restri
 // point's BRIEF bits from a 35 x 35 patch of the frame: gray, the separable [1,4,6,4,1] sums (the
 // unnormalised S, at most 255 * 256), and one comparison per thread, packed by ballots.  A few
 // hundred points need 0.4 MB of patches, so no smoothed map of the image is ever formed; the kernel
-// is a chain of latencies (14 us for 500 points of a 4K view, against 19 us for a one-block selection
+// is a chain of latencies (9 us for 500 points of a 4K view, against 19 us for a one-block selection
 // and 11 us for BRIEF on the map, whose pattern was read from parameter space lane by lane).
-constexpr int RB_P = 35, RB_S = 31;  // patch, positions of S
-__global__ void __launch_bounds__(256) lorb_rank_brief(const uint8_t* __restrict__ frame, long long pitch, int W,
-                                                       const __grid_constant__ LorbPattern pat,
-                                                       const Cand* __restrict__ cand2, const LorbCount* __restrict__ cnt,
-                                                       const int* __restrict__ count, int* __restrict__ xy,
-                                                       long long* __restrict__ resp, unsigned* __restrict__ desc) {
-    __shared__ uint8_t g[RB_P * RB_P];
+constexpr int RB_P = 35, RB_W = 36, RB_S = 31;  // patch and its row pitch, positions of S
+__global__ void __launch_bounds__(256) lorb_rank_brief(const uint8_t* frame, long long pitch, int W,
+                                                       const Cand* cand2, const LorbCount* cnt,
+                                                       const int* count, int* xy,
+                                                       long long* resp, unsigned* desc) {
+    __shared__ __align__(4) uint8_t g[RB_P * RB_W];
     __shared__ uint16_t hs[RB_P][RB_S + 1], S[RB_S][RB_S + 1];
     __shared__ int s_w[8];
     const int t = threadIdx.x, lane = t & 31, w = t >> 5;
+    pdl_trigger();
+    pdl_wait();
     const int n2 = cnt->n2, want = *count;
     const bool selected = n2 > RANK_MAX;  // lorb_prune has written xy and resp
-    const char4 pr = make_char4(pat.p[t][0], pat.p[t][1], pat.p[t][2], pat.p[t][3]);
+    const bool words = word_aligned(frame, pitch);
     for (int i = blockIdx.x; i < (selected ? want : n2); i += gridDim.x) {
         int k = i, x, y;
         if (selected) {
@@ -556,20 +566,33 @@ __global__ void __launch_bounds__(256) lorb_rank_brief(const uint8_t* __restrict
             }
         }
         if (k < want) {  // the whole block
-            const uint8_t* p0 = frame + (long long)(y - 17) * pitch + 3LL * (x - 17);  // points keep 18 px from the border
-#pragma unroll
-            for (int q0 = 0; q0 < RB_P * RB_P; q0 += 256) {
-                const int q = q0 + t;
-                if (q < RB_P * RB_P) {
-                    const int r = q / RB_P;
-                    const uint8_t* p = p0 + (long long)r * pitch + 3 * (q - r * RB_P);
-                    g[q] = (uint8_t)gray_of(__ldg(p), __ldg(p + 1), __ldg(p + 2));
+            // points keep 18 px from the border, so the patch and a 36th column lie inside the image
+            const char4 pr = cnt->pat[t];
+            const uint8_t* p0 = frame + (long long)(y - 17) * pitch + 3LL * (x - 17);
+            if (words) {
+                // groups of 4 pixels (12 bytes at any offset): four aligned words, shifted
+                const int off = (3 * (x - 17)) & 3;
+                for (int q = t; q < RB_P * (RB_W / 4); q += 256) {
+                    const int r = q / (RB_W / 4), j = q - r * (RB_W / 4);
+                    const unsigned* p = reinterpret_cast<const unsigned*>(p0 - off + (long long)r * pitch + 12 * j);
+                    const unsigned v0 = __ldg(p), v1 = __ldg(p + 1), v2 = __ldg(p + 2), v3 = off ? __ldg(p + 3) : 0u;
+                    const unsigned a = __funnelshift_r(v0, v1, 8 * off), b = __funnelshift_r(v1, v2, 8 * off),
+                                   c = __funnelshift_r(v2, v3, 8 * off);
+                    unsigned o[4];
+                    gray4(a, b, c, o);
+                    *reinterpret_cast<unsigned*>(g + r * RB_W + 4 * j) = o[0] | o[1] << 8 | o[2] << 16 | o[3] << 24;
+                }
+            } else {
+                for (int q = t; q < RB_P * RB_P; q += 256) {
+                    const int r = q / RB_P, c = q - r * RB_P;
+                    const uint8_t* p = p0 + (long long)r * pitch + 3 * c;
+                    g[r * RB_W + c] = (uint8_t)gray_of(__ldg(p), __ldg(p + 1), __ldg(p + 2));
                 }
             }
             __syncthreads();
             for (int q = t; q < RB_P * RB_S; q += 256) {
                 const int r = q / RB_S, c = q - r * RB_S;
-                const uint8_t* p = g + r * RB_P + c;
+                const uint8_t* p = g + r * RB_W + c;
                 hs[r][c] = (uint16_t)(p[0] + 4 * p[1] + 6 * p[2] + 4 * p[3] + p[4]);
             }
             __syncthreads();
@@ -667,8 +690,8 @@ extern "C" stitch_status stitch_lorb_detect(stitch_lorb* c, const uint8_t* frame
     for (int k = 0; k < 256; ++k)
         for (int j = 0; j < 4; ++j) {
             if (pattern[4 * k + j] < -15 || pattern[4 * k + j] > 15) return STITCH_EINVAL;
-            pat.p[k][j] = pattern[4 * k + j];
         }
+    memcpy(pat.p, pattern, sizeof(pat.p));
     // areas clipped to the margin; bounding box of the candidates, and of what BRIEF reads
     LorbAreas ar{};
     int bx0 = width, by0 = height, bx1 = 0, by1 = 0;
@@ -697,18 +720,17 @@ extern "C" stitch_status stitch_lorb_detect(stitch_lorb* c, const uint8_t* frame
     if (ar.n > 0) {
         // tiles over the candidates' box, owned pixels starting at a column 1 modulo 4
         const int ox = 1 + ((bx0 - 1) & ~3), oy = by0;
-        lorb_detect<<<dim3((bx1 - ox + DT_OX - 1) / DT_OX, (by1 - oy + DT_OY - 1) / DT_OY), 256, 0, s>>>(
-            frame, pitch, width, height, ox, oy, ar, std::min(params->fast_t, 255) + 256, (long long)params->harris_t,
-            c->cand, &c->cnt->n, c->cap, c->cnt->hist, &c->cnt->n2);
+        pdl_launch(lorb_detect, dim3((bx1 - ox + DT_OX - 1) / DT_OX, (by1 - oy + DT_OY - 1) / DT_OY), 256, 0, s, frame, pitch,
+                   width, height, ox, oy, ar, std::min(params->fast_t, 255) + 256, (long long)params->harris_t, c->cand,
+                   &c->cnt->n, c->cap, c->cnt->hist, &c->cnt->n2);
     } else {
         ok(cudaMemsetAsync(&c->cnt->n2, 0, sizeof(int), s));
     }
-    lorb_prune<<<PRUNE_BLOCKS, PRUNE_THREADS, 0, s>>>(c->cand, c->cnt, c->cap, params->max_points, c->cand2, width, xy,
-                                                      reinterpret_cast<long long*>(resp), count);
+    pdl_launch(lorb_prune, PRUNE_BLOCKS, PRUNE_THREADS, 0, s, c->cand, c->cnt, c->cap, params->max_points, c->cand2, width,
+               pat, xy, reinterpret_cast<long long*>(resp), count);
     // the pruned candidates are a few more than the points: a block each, or a few passes
-    lorb_rank_brief<<<std::min(2 * params->max_points + 64, 1216), 256, 0, s>>>(
-        frame, pitch, width, pat, c->cand2, c->cnt, count, xy, reinterpret_cast<long long*>(resp),
-        reinterpret_cast<unsigned*>(desc));
+    pdl_launch(lorb_rank_brief, std::min(2 * params->max_points + 64, 1216), 256, 0, s, frame, pitch, width, c->cand2, c->cnt,
+               count, xy, reinterpret_cast<long long*>(resp), reinterpret_cast<unsigned*>(desc));
     ok(cudaGetLastError());
     if (prev >= 0 && prev != c->device) cudaSetDevice(prev);
     return st;
