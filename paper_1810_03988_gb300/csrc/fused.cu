@@ -179,7 +179,8 @@ constexpr int D1_XC = D1_SX - D1_THREADS;                    // the last 3 colum
 constexpr int D1_NSAMP = D1_SX * D1_SY;                      // level-0 samples of a tile's region
 // a FULL canvas tile's level-0 slot (64 x 32 samples per blended camera), written by the camera's
 // two down1 tiles over it (rows 0..15 and 16..31)
-constexpr int D1_SLOT = (2 * D1_TX) * (4 * D1_TY);
+constexpr int U0_TX = 2 * D1_TX, U0_TY = 4 * D1_TY;          // pixels of a canvas tile
+constexpr int D1_SLOT = U0_TX * U0_TY;
 // A slot element: the sample's R, G, B and normalised weight a as 16-bit codes, R | G << 16 and
 // B | a << 16.  Colours go in steps of 1/256 of an 8-bit level (a bilinear sample of 8-bit texels
 // rounds to within 1/512 of a level), the weight in steps of 1/65535; the blend divides by the sum
@@ -220,7 +221,7 @@ __device__ __forceinline__ int d1_vslot(int c) { return (c & 1) * D1_VODD + (c >
 __device__ __forceinline__ float2 d1_w(int n) { return f2(n == 0 || n == 4 ? 0.0625f : n == 2 ? 0.375f : 0.25f); }
 
 // Normalised feather weights of the level-0 samples of a down1 tile (S2: w_i / sum_j w_j over the
-// cameras whose validity box contains the sample), or -1 for samples outside the camera's pyramid
+// cameras whose validity box contains the sample), or 0 for samples outside the camera's pyramid
 // region Omega^0_i.  They depend on the geometry only, so the rig computes them once at creation
 // (the paper's pre-corrected parameters, Algorithm 4, and start-up preallocation, Sec. 4.3.2), one
 // block per tile; down1 then warps only its own camera.
@@ -239,7 +240,7 @@ __global__ void __launch_bounds__(D1W_THREADS) k_d1_weights(const CamDev* __rest
         const int r = q / D1_SX, c = q % D1_SX;
         const int x = fold101(vx0 + c, g.nx[0]), y = fold101(vy0 + r, g.ny[0]);
         if (!o0.contains(x, y)) {
-            out[q] = -1.f;
+            out[q] = 0.f;
             continue;
         }
         if (g.seam) {
@@ -298,40 +299,48 @@ __device__ __forceinline__ void stage_footprint(uint32_t* __restrict__ foot, con
         return;
     }
     constexpr int SG = D1Cap<CAP>::SG;
-    // q / gpr as (q m) >> 20: m is above 2^20 / gpr by less than 3, and 3 gpr q < 2^20
-    static_assert(3 * (CAP / 4) * (SG * D1_THREADS - 1) < 1 << 20, "exact quotients");
-    const int m = (int)__fdividef(1048576.0f, (float)gpr) + 2;
-    uint32_t w[SG][3];
+    // q / gpr as (q m) >> SH: m is above 2^SH / gpr by less than 3, and 3 gpr q < 2^SH
+    constexpr int SH = CAP > D1_FOOT ? 22 : 20;
+    static_assert(3 * (CAP / 4) * (SG * D1_THREADS - 1) < 1 << SH, "exact quotients");
+    static_assert((long long)SG * D1_THREADS * ((1 << SH) + 2) < 1LL << 32, "no overflow");
+    const unsigned m = (unsigned)(int)__fdividef((float)(1 << SH), (float)gpr) + 2u;
+    constexpr int RD = SG > D1Cap<D1_FOOT>::SG ? 6 : SG;  // groups in flight
+    static_assert(SG % RD == 0, "whole rounds");
 #pragma unroll
-    for (int k = 0; k < SG; ++k) {
-        const int q = t + k * D1_THREADS;
-        w[k][0] = w[k][1] = w[k][2] = 0u;
-        if (q < ng) {
-            const int rr = (q * m) >> 20, gx = q - rr * gpr;
-            const int u0 = fx0 + 4 * gx;
-            const uint8_t* src = px + (long long)(fy0 + rr) * pitch + 3 * u0;
-            if (u0 + 4 <= W) {
-                const uint32_t* s32 = reinterpret_cast<const uint32_t*>(src);
-                w[k][0] = __ldg(s32);
-                w[k][1] = __ldg(s32 + 1);
-                w[k][2] = __ldg(s32 + 2);
-            } else {
-                // the image's last texels: only the bytes of texels < W exist
-                const int nb = 3 * (W - u0);
+    for (int k0 = 0; k0 < SG; k0 += RD) {
+        if (k0 > 0 && k0 * D1_THREADS >= ng) break;
+        uint32_t w[RD][3];
 #pragma unroll
-                for (int j = 0; j < 12; ++j)
-                    if (j < nb) w[k][j >> 2] |= (uint32_t)__ldg(src + j) << (8 * (j & 3));
+        for (int k = 0; k < RD; ++k) {
+            const int q = t + (k0 + k) * D1_THREADS;
+            w[k][0] = w[k][1] = w[k][2] = 0u;
+            if (q < ng) {
+                const int rr = (int)(((unsigned)q * m) >> SH), gx = q - rr * gpr;
+                const int u0 = fx0 + 4 * gx;
+                const uint8_t* src = px + (long long)(fy0 + rr) * pitch + 3 * u0;
+                if (u0 + 4 <= W) {
+                    const uint32_t* s32 = reinterpret_cast<const uint32_t*>(src);
+                    w[k][0] = __ldg(s32);
+                    w[k][1] = __ldg(s32 + 1);
+                    w[k][2] = __ldg(s32 + 2);
+                } else {
+                    // the image's last texels: only the bytes of texels < W exist
+                    const int nb = 3 * (W - u0);
+#pragma unroll
+                    for (int j = 0; j < 12; ++j)
+                        if (j < nb) w[k][j >> 2] |= (uint32_t)__ldg(src + j) << (8 * (j & 3));
+                }
             }
         }
-    }
 #pragma unroll
-    for (int k = 0; k < SG; ++k) {
-        const int q = t + k * D1_THREADS;
-        if (q < ng) {
-            // bytes R0 G0 B0 R1 | G1 B1 R2 G2 | B2 R3 G3 B3 -> one word per texel
-            reinterpret_cast<uint4*>(foot)[q] =
-                make_uint4(__byte_perm(w[k][0], 0u, 0x0210), __byte_perm(w[k][0], w[k][1], 0x0543),
-                           __byte_perm(w[k][1], w[k][2], 0x0432), __byte_perm(w[k][2], 0u, 0x0321));
+        for (int k = 0; k < RD; ++k) {
+            const int q = t + (k0 + k) * D1_THREADS;
+            if (q < ng) {
+                // bytes R0 G0 B0 R1 | G1 B1 R2 G2 | B2 R3 G3 B3 -> one word per texel
+                reinterpret_cast<uint4*>(foot)[q] =
+                    make_uint4(__byte_perm(w[k][0], 0u, 0x0210), __byte_perm(w[k][0], w[k][1], 0x0543),
+                               __byte_perm(w[k][1], w[k][2], 0x0432), __byte_perm(w[k][2], 0u, 0x0321));
+            }
         }
     }
 }
@@ -349,9 +358,10 @@ __device__ __forceinline__ void d1_bilerp(uint32_t w00, uint32_t w01, uint32_t w
     const float2 top = f2fma(fxx, f2sub(a01, a00), f2sub(a00, f2(K23)));
     const float2 bot = f2fma(fxx, f2sub(a11, a10), f2sub(a10, f2(K23)));
     s.a = f2mul(f2fma(fyy, f2sub(bot, top), top), f2(scale));
-    const float b00 = byte_f23(w00, 2), b01 = byte_f23(w01, 2), b10 = byte_f23(w10, 2), b11 = byte_f23(w11, 2);
-    const float btop = fmaf(fx, b01 - b00, b00 - K23), bbot = fmaf(fx, b11 - b10, b10 - K23);
-    s.b.x = fmaf(fy, bbot - btop, btop) * scale;
+    // B of both rows as one pair
+    const float2 b0 = make_float2(byte_f23(w00, 2), byte_f23(w10, 2)), b1 = make_float2(byte_f23(w01, 2), byte_f23(w11, 2));
+    const float2 bb = f2fma(fxx, f2sub(b1, b0), f2sub(b0, f2(K23)));
+    s.b.x = fmaf(fy, bb.y - bb.x, bb.x) * scale;
 }
 
 // Per-tile constants of the sweep.
@@ -393,22 +403,29 @@ __device__ __forceinline__ void d1_frame_sample(const D1Ctx& x, const Pos& p, V4
     d1_bilerp(q.t00, q.t01, q.t10, q.t11, fx, fy, x.scale, s);
 }
 
-// Level-0 sample of virtual row r at the column whose anchored numerators and denominator at the
-// anchor row are (nuv, dqc): (r, g, b, normalised weight a), weight 0 outside Omega^0 (a < 0).
+// Level-0 sample at row offset dy (twice: canvas row minus the anchor row) of the column whose anchored
+// numerators and denominator at the anchor row are (nuv, dqc): (r, g, b, normalised weight a), weight 0 outside Omega^0.
 // The colour there is whatever the taps give: Omega^0 holds the 5 x 5 support of every stored G^1
 // sample, and a level-0 output of weight 0 adds nothing to a blend, so it is never read.
 // Position and taps are those of map_pos + sample_rgb, so the three modes give bit-identical
 // samples.  The floor of the offsets ru, rv (|ru|, |rv| < 2^22 on staged tiles, whose footprint
 // the planner bounds) comes from one addition rounded toward -infinity:
 // RD(ru + 1.5 2^23) = 1.5 2^23 + floor(ru), whose low bits hold the integer.
+//
+// rcp_normal(v): 1 / v of a normal float as __fdividef(1, v) gives it, without the scaling that division
+// needs for denormal operands (staged tiles: w > 0 by far on their whole region).
+__device__ __forceinline__ float rcp_normal(float v) {
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(v));
+    return r;
+}
 template <int MODE>
-__device__ __forceinline__ V4 d1_sample(const D1Ctx& x, float2 nuv, float dqc, int r, float a) {
-    const float2 dy = x.rowdy[r];
+__device__ __forceinline__ V4 d1_sample(const D1Ctx& x, float2 nuv, float dqc, float2 dy, float a) {
     const float den = fmaf(x.tm.q2, dy.x, dqc);
     const float2 n = f2fma(make_float2(x.tm.pu2, x.tm.pv2), dy, nuv);
-    const float rden = __fdividef(1.0f, den);
+    const float rden = MODE == D1M_FRAME ? __fdividef(1.0f, den) : rcp_normal(den);
     V4 s;
-    s.b.y = fmaxf(a, 0.0f);
+    s.b.y = a;
     if (MODE == D1M_FRAME) {
         float ru = n.x * rden, rv = n.y * rden;
         ru = fminf(fmaxf(ru, -1.0e7f), 1.0e7f);
@@ -430,14 +447,15 @@ __device__ __forceinline__ V4 d1_sample(const D1Ctx& x, float2 nuv, float dqc, i
         if (MODE == D1M_STAGED) {
             // top-left tap (V0 + floor(rv) - fy0) S + (U0 + floor(ru) - fx0), clamped into the footprint
             // (the planner's footprint holds every tap; the debug build records one that it misses)
-            const int raw = (int)(tv * (unsigned)x.S + tu + x.ibase);
-            (void)STITCH_DCHECK(raw >= 0 && raw <= x.maxidx, 1, raw);
-            const unsigned idx = min((unsigned)raw, (unsigned)x.maxidx);
-            const uint32_t* p = x.foot + idx;
-            w00 = p[0];
-            w01 = p[1];
-            w10 = p[x.S];
-            w11 = p[x.S + 1];
+            // in bytes
+            const unsigned raw = 4u * tu + (tv * (4u * (unsigned)x.S) + x.ibase);
+            (void)STITCH_DCHECK(raw <= 4u * (unsigned)x.maxidx, 1, (int)raw);
+            const char* p = reinterpret_cast<const char*>(x.foot) + min(raw, 4u * (unsigned)x.maxidx);
+            const char* p1 = p + 4 * x.S;
+            w00 = *reinterpret_cast<const uint32_t*>(p);
+            w01 = *reinterpret_cast<const uint32_t*>(p + 4);
+            w10 = *reinterpret_cast<const uint32_t*>(p1);
+            w11 = *reinterpret_cast<const uint32_t*>(p1 + 4);
         } else {
             // image clamp of S1: outside [0, W-1) x [0, H-1) the border texel, fraction 0
             const int lu = (int)(tu - D1_FLOOR_BITS) + (x.tm.U0 - x.fx0), lv = (int)(tv - D1_FLOOR_BITS) + (x.tm.V0 - x.fy0);
@@ -536,8 +554,8 @@ __device__ __forceinline__ void d1_sweep(const D1Ctx& x, float4* __restrict__ vc
             we = __ldg(wp);
             wo = __ldg(m < D1_TY ? wp + D1_SX : wp);
         }
-        const V4 se = d1_sample<MODE>(x, nuv, dqc, 2 * m, ae);
-        const V4 so = d1_sample<MODE>(x, nuv, dqc, 2 * m + 1, ao);
+        const V4 se = d1_sample<MODE>(x, nuv, dqc, x.rowdy[2 * m], ae);
+        const V4 so = d1_sample<MODE>(x, nuv, dqc, x.rowdy[2 * m + 1], ao);
         if (m >= 1) d1_put<T, OUTK>(oq, 0, se);
         if (m >= 2) *vp = f4_of(v4_fma(d1_w(4), se, C));
         C = v4_fma(d1_w(2), se, B);
@@ -551,7 +569,7 @@ __device__ __forceinline__ void d1_sweep(const D1Ctx& x, float4* __restrict__ vc
         oq.rows -= 2;
     }
 
-    const V4 se = d1_sample<MODE>(x, nuv, dqc, 2 * D1_TY + 2, we);
+    const V4 se = d1_sample<MODE>(x, nuv, dqc, x.rowdy[2 * D1_TY + 2], we);
     vcol[(D1_TY - 1) * D1_VROW] = f4_of(v4_fma(d1_w(4), se, C));
 }
 
@@ -620,8 +638,8 @@ __device__ __forceinline__ void down1_tile(const CamDev* __restrict__ cams, cons
     x.S = (x.fw + 3) & ~3;
     // footprint index of the top-left tap from the bit patterns tu, tv of the floor constants:
     // (tv - B + V0 - fy0) S + (tu - B + U0 - fx0), in arithmetic modulo 2^32
-    x.ibase = (unsigned)(ref.tm.V0 - x.fy0) * (unsigned)x.S + (unsigned)(ref.tm.U0 - x.fx0) -
-              D1_FLOOR_BITS * ((unsigned)x.S + 1u);
+    x.ibase = 4u * ((unsigned)(ref.tm.V0 - x.fy0) * (unsigned)x.S + (unsigned)(ref.tm.U0 - x.fx0) -
+                    D1_FLOOR_BITS * ((unsigned)x.S + 1u));
     x.maxidx = x.S * (x.fh - 1) - 2;
     if (staged && act) stage_footprint<CAP>(foot, px_i, pitch_i, x.W, x.fx0, x.fy0, x.fw, x.fh, t);
     if (t < D1_SY) {
@@ -696,9 +714,9 @@ __device__ __forceinline__ void down1_tile(const CamDev* __restrict__ cams, cons
             const float a = __ldg(x.wt + r * D1_SX + ce);
             V4 s;
             switch (mode) {
-                case D1M_STAGED: s = d1_sample<D1M_STAGED>(x, nuv, dqc, r, a); break;
-                case D1M_CLAMP: s = d1_sample<D1M_CLAMP>(x, nuv, dqc, r, a); break;
-                default: s = d1_sample<D1M_FRAME>(x, nuv, dqc, r, a); break;
+                case D1M_STAGED: s = d1_sample<D1M_STAGED>(x, nuv, dqc, x.rowdy[r], a); break;
+                case D1M_CLAMP: s = d1_sample<D1M_CLAMP>(x, nuv, dqc, x.rowdy[r], a); break;
+                default: s = d1_sample<D1M_FRAME>(x, nuv, dqc, x.rowdy[r], a); break;
             }
             ext[t] = f4_of(s);
         }
@@ -747,6 +765,104 @@ __global__ void __launch_bounds__(D1_THREADS, D1Cap<CAP>::BLOCKS) k_down1(const 
     const D1Tile tl = tiles[blockIdx.x];
     pdl_wait();
     down1_tile<T, CAP>(cams, g, fp, od, tl, refs, d1w, d1cols, g0buf, smem);
+}
+
+// ------------------------------------------------------------------------------------------------
+// solo: SOLO canvas tiles under which no pyramid level is read
+//
+// A 64 x 32 canvas tile whose two down1 tiles have no other output than its pixels (no needed G^1) is
+// warped by a kernel of its own: 32 rows per thread instead of 2 x 19, no weights, no REDUCE, the footprint
+// of both halves staged at once, and twice the resident warps (48 registers, 12 KB).  Each half keeps the
+// anchor of its down1 tile, so the samples are bit-identical to down1's.  Instruction issue bounds it
+// (78 per sample and warp, down1: 109).  8 x 4K: the 19 276 down1 tiles that it replaces took 93 us of
+// down1's 373, their 9638 canvas tiles take 70 us here.  Nothing depends on it, so it runs beside the
+// pyramid's launches, whose small levels leave most of the chip idle (launch_all): 815 -> 790 us per frame,
+// 803 when it follows down1 on the same stream; 4 x 1080p (1189 tiles) 210 -> 205.
+constexpr int SO_FOOT = 3072;  // footprint capacity in texels
+constexpr int SO_BLOCKS = 18;  // resident blocks per SM, bounds the registers (shared memory allows 17)
+// A rig uses it from this many tiles per SM on.  Below, the tiles stay with down1: 5 x 719p (325 tiles,
+// 2 per SM) takes 131 us either way, and a second stream only costs.
+constexpr int SO_MIN_PER_SM = 4;
+struct SoloTile {
+    int cam, x0, y0, fxy, fwh, ref0, ref1, coltab0, coltab1;
+};
+
+template <bool F32>
+__global__ void __launch_bounds__(D1_THREADS, SO_BLOCKS) k_solo(const CamDev* __restrict__ cams, const __grid_constant__ RigGeom g,
+                                                                const __grid_constant__ FramePtrs fp, OutDesc od,
+                                                                const SoloTile* __restrict__ tiles,
+                                                                const CamRef* __restrict__ refs,
+                                                                const float4* __restrict__ d1cols) {
+    __shared__ __align__(16) uint32_t foot[SO_FOOT];
+    const int t = threadIdx.x;
+    const int lane = t & 31;
+    const SoloTile tl = tiles[blockIdx.x];
+    const CamDev& c = cams[tl.cam];
+    D1Ctx x{};
+    x.scale = c.gain * (1.0f / 255.0f);
+    x.foot = foot;
+    x.fx0 = tl.fxy & 0xffff;
+    x.fy0 = (int)((unsigned)tl.fxy >> 16);
+    x.fw = tl.fwh & 0xffff;
+    x.fh = tl.fwh >> 16;
+    x.S = (x.fw + 3) & ~3;
+    x.maxidx = x.S * (x.fh - 1) - 2;
+    stage_footprint<SO_FOOT>(foot, fp.p[tl.cam], fp.pitch[tl.cam], c.W, x.fx0, x.fy0, x.fw, x.fh, t);
+    __syncthreads();
+    const int xo = tl.x0 + t, xc = min(xo, g.nx[0] - 1);
+    // 8-bit rows of whole words: a warp's 32 pixels are 24 words; word l holds bytes l % 3 .. of pixel
+    // l + l / 3 and the first of the next one
+    const bool words = !F32 && tl.x0 + U0_TX <= g.nx[0] && word_aligned((const uint8_t*)od.ptr, od.pitch);
+    const int wl = min(lane, 23), wp = wl + wl / 3;
+    const unsigned wsel = wl % 3 == 0 ? 0x4210u : wl % 3 == 1 ? 0x5421u : 0x6542u;
+#pragma unroll 1
+    for (int h = 0; h < 2; ++h) {
+        const CamRef& ref = refs[h ? tl.ref1 : tl.ref0];
+        x.tm = ref.tm;
+        x.ibase = 4u * ((unsigned)(x.tm.V0 - x.fy0) * (unsigned)x.S + (unsigned)(x.tm.U0 - x.fx0) -
+                        D1_FLOOR_BITS * ((unsigned)x.S + 1u));
+        float2 nuv;
+        float dqc;
+        if (g.cyl) {
+            const float4 cc = d1cols[(long long)(h ? tl.coltab1 : tl.coltab0) * D1_SX + (xc - tl.x0) + 2];
+            nuv = make_float2(cc.x, cc.y);
+            dqc = cc.z;
+        } else {
+            const float dx = (float)(xc - ref.ax);
+            nuv = make_float2(fmaf(x.tm.pu1, dx, x.tm.pu0), fmaf(x.tm.pv1, dx, x.tm.pv0));
+            dqc = fmaf(x.tm.q1, dx, x.tm.q0);
+        }
+        const int Y = tl.y0 + h * (U0_TY / 2);
+        const int rows = min(U0_TY / 2, g.ny[0] - Y);
+        float2 dy = f2((float)(Y - ref.ay));
+        char* q = (char*)od.ptr + (long long)Y * od.pitch +
+                  (words ? 3LL * (xo - lane) + 4 * lane : (F32 ? 12LL : 3LL) * xo);
+#pragma unroll 2
+        for (int r = 0; r < rows; ++r) {
+            const V4 s = d1_sample<D1M_STAGED>(x, nuv, dqc, dy, 1.0f);
+            dy = f2add(dy, f2(1.0f));
+            const float vr = __saturatef(s.a.x), vg = __saturatef(s.a.y), vb = __saturatef(s.b.x);
+            if (F32) {
+                if (xo < g.nx[0]) {
+                    float* f = reinterpret_cast<float*>(q);
+                    f[0] = vr;
+                    f[1] = vg;
+                    f[2] = vb;
+                }
+            } else {
+                const uint32_t px = __byte_perm(__byte_perm(quantize_bits(vr), quantize_bits(vg), 0x0040), quantize_bits(vb), 0x0410);
+                if (words) {
+                    const uint32_t lo = __shfl_sync(~0u, px, wp), hi = __shfl_sync(~0u, px, wp + 1);
+                    if (lane < 24) *reinterpret_cast<uint32_t*>(q) = __byte_perm(lo, hi, wsel);
+                } else if (xo < g.nx[0]) {
+                    q[0] = (char)px;
+                    q[1] = (char)(px >> 8);
+                    q[2] = (char)(px >> 16);
+                }
+            }
+            q += od.pitch;
+        }
+    }
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -1158,7 +1274,7 @@ __global__ void __launch_bounds__(256, 3) k_coarse_t(const CamDev* __restrict__ 
 // ------------------------------------------------------------------------------------------------
 // up: levels 1 and 0 of one canvas tile
 
-constexpr int U_TX = 64, U_TY = 32;                     // level-0 pixels per tile
+constexpr int U_TX = U0_TX, U_TY = U0_TY;               // level-0 pixels per tile (64 x 32)
 static_assert(D1_SLOT == U_TX * U_TY && 2 * D1_TX == U_TX && 4 * D1_TY == U_TY,
               "two down1 tiles over one canvas tile of up");
 constexpr int U_THREADS = 256;
@@ -1822,6 +1938,12 @@ enum UpKind { UP_SIMPLE = 0, UP_FULL2 = 1, UP_FULL4 = 2, UP_GENERAL = 3, UP_KIND
 struct FusedState {
     D1Tile* d1_tiles = nullptr;
     int n_d1 = 0;
+    int n_d1_pyr = 0;            // the first of them: those that the solo kernel does not take
+    SoloTile* solo_tiles = nullptr;
+    int n_solo_tiles = 0;
+    // the pyramid chain's stream while the solo kernel runs on the caller's (null: one after the other)
+    cudaStream_t chain = nullptr;
+    cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
     Tile* red_tiles[MAXL] = {};  // tiles producing level l (l >= 2), RSRig shape (the batched schedules)
     int n_red[MAXL] = {};
     Tile* rc_tiles[MAXL] = {};   // the same levels in the column-sweep kernel's 64 x 8 tiles (stitch_frames)
@@ -1982,7 +2104,7 @@ bool solidly_inside(const CamDev& c, const RigGeom& g, const Rect& q, double m =
 // and the footprint is at least 2 x 2 texels (grown inside the image where the rectangle maps
 // beyond an image border).  False when q is not entirely in front of the camera, maps beyond
 // |u|, |v| < 1e6, or the footprint (rows padded to 4 texels) exceeds the shared-memory capacity.
-bool d1_footprint(const CamDev& c, const RigGeom& g, const Rect& q, int& fx0, int& fy0, int& fw, int& fh) {
+bool d1_footprint(const CamDev& c, const RigGeom& g, const Rect& q, int cap, int& fx0, int& fy0, int& fw, int& fh) {
     if (c.W < 2 || c.H < 2) return false;
     double umin, umax, vmin, vmax;
     if (!source_range(c, g, q, &umin, &umax, &vmin, &vmax)) return false;
@@ -2000,7 +2122,7 @@ bool d1_footprint(const CamDev& c, const RigGeom& g, const Rect& q, int& fx0, in
         y1 = y0 + 2;
     }
     x0 &= ~3;
-    if (x1 - x0 < 2 || y1 - y0 < 2 || (long long)((x1 - x0 + 3) & ~3) * (y1 - y0) > D1_FOOT || y0 > 0xffff ||
+    if (x1 - x0 < 2 || y1 - y0 < 2 || (long long)((x1 - x0 + 3) & ~3) * (y1 - y0) > cap || y0 > 0xffff ||
         x0 > 0xffff)
         return false;
     fx0 = x0;
@@ -2074,19 +2196,21 @@ void plan_coarse_tiles(const stitch_rig* r, const std::vector<UpTile>* up, int t
     }
 }
 
-template <typename T>
-stitch_status launch_all(stitch_rig* r, FusedState* fs, const FramePtrs& fp, const OutDesc& od, cudaStream_t s) {
+// The launches of the pyramid: down1, REDUCE, coarse and canvas tiles.  solo() follows down1.  early: the
+// first launch may start while the stream's previous kernel drains (nothing but kernels lies between).
+template <typename T, typename Solo>
+void launch_chain(stitch_rig* r, FusedState* fs, const FramePtrs& fp, const OutDesc& od, cudaStream_t s, bool early,
+                  const Solo& solo) {
     const RigGeom& g = r->geom;
     const int L = g.levels;
-    if (L >= 2 && fs->n_d1 > 0) {
+    if (L >= 2 && fs->n_d1_pyr > 0) {
         prof_mark(r, "fused_down1", s);
-        if (fs->d1_small)
-            pdl_launch(k_down1<T, D1_FOOT_SMALL>, fs->n_d1, D1_THREADS, D1Cap<D1_FOOT_SMALL>::SMEM, s, r->dcam, g, fp, od,
-                       fs->d1_tiles, fs->refs, fs->d1w, fs->d1cols, (Slot*)fs->g0buf);
-        else
-            pdl_launch(k_down1<T, D1_FOOT>, fs->n_d1, D1_THREADS, D1_SMEM, s, r->dcam, g, fp, od, fs->d1_tiles, fs->refs,
-                       fs->d1w, fs->d1cols, (Slot*)fs->g0buf);
+        const auto k = fs->d1_small ? k_down1<T, D1_FOOT_SMALL> : k_down1<T, D1_FOOT>;
+        const size_t smem = fs->d1_small ? D1Cap<D1_FOOT_SMALL>::SMEM : D1_SMEM;
+        stream_launch(early, k, fs->n_d1_pyr, D1_THREADS, smem, s, r->dcam, g, fp, od, fs->d1_tiles, fs->refs, fs->d1w,
+                      fs->d1cols, (Slot*)fs->g0buf);
     }
+    solo();
     for (int l = 1; l + 1 < L; ++l) {
         if (fs->n_rc[l + 1] == 0) continue;
         prof_mark(r, "fused_reduce", s);
@@ -2127,7 +2251,31 @@ stitch_status launch_all(stitch_rig* r, FusedState* fs, const FramePtrs& fp, con
         pdl_launch(k_up_general<T>, fs->n_up[UP_GENERAL], U_THREADS, 0, s, r->dcam, g, fp, od, R2, fs->up_tiles[UP_GENERAL],
                    fs->refs);
     }
-    return launch_status();
+}
+
+// With a solo kernel, the pyramid's chain runs on the rig's own stream of the highest priority and the solo
+// kernel on the caller's: it is launched once down1 is, and its blocks take the room that the chain leaves.
+// Both begin after all earlier work of the caller's stream and are joined to it.  Under the profiler's marks
+// everything runs on the caller's stream.
+template <typename T>
+stitch_status launch_all(stitch_rig* r, FusedState* fs, const FramePtrs& fp, const OutDesc& od, cudaStream_t s) {
+    const auto solo = [&] {
+        if (fs->n_solo_tiles == 0) return;
+        prof_mark(r, "fused_solo", s);
+        const auto k = od.is_float ? k_solo<true> : k_solo<false>;
+        k<<<fs->n_solo_tiles, D1_THREADS, 0, s>>>(r->dcam, r->geom, fp, od, fs->solo_tiles, fs->refs, fs->d1cols);
+    };
+    if (!fs->chain || r->prof) {
+        launch_chain<T>(r, fs, fp, od, s, true, solo);
+        return launch_status();
+    }
+    STITCH_CUDA_TRY(cudaEventRecord(fs->ev_fork, s));
+    STITCH_CUDA_TRY(cudaStreamWaitEvent(fs->chain, fs->ev_fork, 0));
+    launch_chain<T>(r, fs, fp, od, fs->chain, false, solo);
+    const stitch_status st = launch_status();
+    STITCH_CUDA_TRY(cudaEventRecord(fs->ev_join, fs->chain));
+    STITCH_CUDA_TRY(cudaStreamWaitEvent(s, fs->ev_join, 0));
+    return st;
 }
 
 template <typename T>
@@ -2224,7 +2372,7 @@ stitch_status fused_plan(stitch_rig* r) {
                     t.wtab = (t.flags & D1_INTERIOR) ? -1 : fs->n_wtab++;
                     t.wsel = t.wtab;
                     int fx0, fy0, fw, fh;
-                    if (d1_footprint(c, g, Rect{bx0, bx1, by0, by1}, fx0, fy0, fw, fh)) {
+                    if (d1_footprint(c, g, Rect{bx0, bx1, by0, by1}, D1_FOOT, fx0, fy0, fw, fh)) {
                         t.fxy = fx0 | (fy0 << 16);
                         t.fwh = fw | (fh << 16);
                         ++fs->n_staged;
@@ -2478,6 +2626,53 @@ stitch_status fused_plan(stitch_rig* r) {
         d1.swap(kd);
         d1c.swap(kc);
     }
+    // canvas tiles that the solo kernel takes: both of their down1 tiles write its pixels and nothing else,
+    // sample the staged footprint without clamping, and the footprint of both fits.  Their down1 tiles go
+    // to the end of the list (the batched schedules launch all of it).
+    std::vector<SoloTile> solo;
+    {
+        std::vector<char> in_solo(d1.size(), 0);
+        std::unordered_map<long long, size_t> at;  // (camera, level-1 origin) -> down1 tile
+        const auto key = [](int cam, int k0, int j0) { return ((long long)cam << 42) | ((long long)k0 << 21) | j0; };
+        for (size_t k = 0; k < d1.size(); ++k) at[key(d1[k].cam, d1[k].k0, d1[k].j0)] = k;
+        const auto warp_only = [](const D1Tile& t) {
+            return (t.flags & (D1_SOLO_OUT | D1_NOCLAMP | D1_G0_OUT | D1_G1_OUT)) == (D1_SOLO_OUT | D1_NOCLAMP) && t.fwh != 0;
+        };
+        for (size_t k = 0; k < d1.size(); ++k) {
+            const D1Tile& a = d1[k];
+            if ((a.j0 / D1_TY) & 1 || !warp_only(a)) continue;
+            const auto it = at.find(key(a.cam, a.k0, a.j0 + D1_TY));
+            if (it == at.end() || !warp_only(d1[it->second])) continue;
+            const D1Tile& b = d1[it->second];
+            const int x0 = 2 * a.k0, y0 = 2 * a.j0;
+            const Rect q{x0, std::min(x0 + U0_TX, g.nx[0]), y0, std::min(y0 + U0_TY, g.ny[0])};
+            int fx0, fy0, fw, fh;
+            if (!d1_footprint(r->hcam[a.cam], g, q, SO_FOOT, fx0, fy0, fw, fh)) continue;
+            solo.push_back({a.cam, x0, y0, fx0 | (fy0 << 16), fw | (fh << 16), a.ref, b.ref, a.coltab, b.coltab});
+            in_solo[k] = in_solo[it->second] = 1;
+        }
+        int sms = 0;
+        if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, r->device) != cudaSuccess || sms < 1)
+            return STITCH_ECUDA;
+        if ((int)solo.size() < SO_MIN_PER_SM * sms) solo.clear();
+        if (!solo.empty()) {
+            std::vector<D1Tile> kd;
+            std::vector<D1Cams> kc;
+            for (char pass = 0; pass < 2; ++pass) {
+                for (size_t k = 0; k < d1.size(); ++k)
+                    if (in_solo[k] == pass) {
+                        kd.push_back(d1[k]);
+                        kc.push_back(d1c[k]);
+                    }
+                if (pass == 0) fs->n_d1_pyr = (int)kd.size();
+            }
+            d1.swap(kd);
+            d1c.swap(kc);
+        } else {
+            fs->n_d1_pyr = (int)d1.size();
+        }
+        fs->n_solo_tiles = (int)solo.size();
+    }
     // footprint capacity: the smaller one when at most 2 % of the staged tiles need more
     {
         int staged = 0, over = 0;
@@ -2504,7 +2699,7 @@ stitch_status fused_plan(stitch_rig* r) {
                          : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bpsm, k_down1<float4, D1_FOOT>, D1_THREADS, D1_SMEM);
         if (oe != cudaSuccess) return STITCH_ECUDA;
         const size_t K = (size_t)std::max(bpsm, 1) * sms;
-        for (size_t k = 0; k + K < d1.size(); ++k) {
+        for (size_t k = 0; k + K < (size_t)fs->n_d1_pyr; ++k) {
             const D1Tile& nx = d1[k + K];
             if (nx.fwh == 0) continue;
             d1[k].pf_fxy = nx.fxy;
@@ -2531,6 +2726,8 @@ stitch_status fused_plan(stitch_rig* r) {
     st = upload(r, d1c, &fs->d1_cams);
     if (st != STITCH_OK) return st;
     st = upload(r, cols, &fs->d1cols);
+    if (st != STITCH_OK) return st;
+    st = upload(r, solo, &fs->solo_tiles);
     if (st != STITCH_OK) return st;
     fs->n_d1 = (int)d1.size();
     if (fs->n_d1 > 0) {
@@ -2561,8 +2758,15 @@ stitch_status fused_plan(stitch_rig* r) {
         if (st != STITCH_OK) return st;
         fs->n_up[k] = (int)up[k].size();
     }
+    if (fs->n_solo_tiles > 0) {
+        int lo = 0, hi = 0;
+        STITCH_CUDA_TRY(cudaDeviceGetStreamPriorityRange(&lo, &hi));
+        STITCH_CUDA_TRY(cudaStreamCreateWithPriority(&fs->chain, cudaStreamNonBlocking, hi));
+        STITCH_CUDA_TRY(cudaEventCreateWithFlags(&fs->ev_fork, cudaEventDisableTiming));
+        STITCH_CUDA_TRY(cudaEventCreateWithFlags(&fs->ev_join, cudaEventDisableTiming));
+    }
     int kernels = 0;
-    if (L >= 2 && fs->n_d1 > 0) kernels += 1;
+    if (L >= 2) kernels += (fs->n_d1_pyr > 0) + (fs->n_solo_tiles > 0);
     for (int l = 2; l < L; ++l) kernels += (fs->n_rc[l] > 0) + (fs->n_co[l] > 0);
     st = fs->fp16 ? set_smem_attrs<half4>() : set_smem_attrs<float4>();
     if (st == STITCH_OK) st = fs->fp16 ? set_waves<half4>(r, fs) : set_waves<float4>(r, fs);
@@ -2596,6 +2800,11 @@ stitch_status fused_precompute(stitch_rig* r) {
 }
 
 void fused_release(stitch_rig* r) {
+    if (FusedState* fs = (FusedState*)r->fused) {
+        if (fs->chain) cudaStreamDestroy(fs->chain);
+        if (fs->ev_fork) cudaEventDestroy(fs->ev_fork);
+        if (fs->ev_join) cudaEventDestroy(fs->ev_join);
+    }
     delete (FusedState*)r->fused;
     r->fused = nullptr;
 }

@@ -92,8 +92,10 @@ constexpr uint32_t kGuardWord = 0x7FC0DEADu;
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
+// stream_launch: with the attribute (early) or without it
 template <typename... P, typename... A>
-inline void pdl_launch(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, const A&... args) {
+inline void stream_launch(bool early, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
+                          const A&... args) {
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = grid;
     cfg.blockDim = block;
@@ -103,8 +105,12 @@ inline void pdl_launch(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem,
     at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at.val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = &at;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = early ? 1 : 0;
     cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+}
+template <typename... P, typename... A>
+inline void pdl_launch(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, const A&... args) {
+    stream_launch(true, kernel, grid, block, smem, s, args...);
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -501,11 +507,10 @@ __device__ __forceinline__ float3 sample_rgb_inside(const uint8_t* __restrict__ 
     return o;
 }
 
-__device__ __forceinline__ unsigned char quantize_u8(float v) {
-    // v already clamped to [0, 1]: 2^23 + 255 v rounded once to nearest even in the addition of one
-    // fused multiply-add, whose low byte is round-half-even(255 v)
-    return (unsigned char)(__float_as_uint(fmaf(v, 255.0f, 8388608.0f)) & 0xffu);
-}
+// v already clamped to [0, 1]: 2^23 + 255 v rounded once to nearest even in the addition of one
+// fused multiply-add, whose low byte is round-half-even(255 v)
+__device__ __forceinline__ uint32_t quantize_bits(float v) { return __float_as_uint(fmaf(v, 255.0f, 8388608.0f)); }
+__device__ __forceinline__ unsigned char quantize_u8(float v) { return (unsigned char)(quantize_bits(v) & 0xffu); }
 
 // ------------------------------------------------------------------------------------------------
 // index-range planning on one axis (host)
