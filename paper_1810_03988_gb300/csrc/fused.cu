@@ -42,7 +42,7 @@
 #include <cstdio>
 #include <cstring>
 #include <string>
-#include <unordered_map>
+#include <tuple>
 
 #include "stitch_internal.cuh"
 
@@ -131,6 +131,17 @@ struct D1Tile {
     int pf_fxy, pf_fwh, pf_cw;
     int wsel;  // weight table the samples take: wtab, or the table of ones for INTERIOR tiles
 };
+
+// A down1 tile with what its camera adds, in one record: a block knows its staging loads after one round
+// trip to memory instead of three (tile, reference, camera).  8 x 4K 742 -> 738 us per frame.
+struct __align__(16) D1Rec {
+    D1Tile tl;
+    TileMap tm;
+    int ax, ay, W, H;
+    float scale;
+    int pad[2];
+};
+static_assert(sizeof(D1Rec) == 128, "one line");
 
 // Cameras (CamRef range, in camera order) whose validity box meets a down1 tile's level-0 inputs,
 // and the position of the tile's own camera among them: the weight normalisation of the tile.
@@ -483,15 +494,14 @@ __device__ __forceinline__ Slot slot_encode(V4 s, float enc) {
                       __byte_perm(__float_as_uint(ba.x), __float_as_uint(ba.y), 0x5410));
 }
 
-// (R, G, B) of a slot element in scaled units (dsc = scale / SLOT_RGB) and its weight code.
-__device__ __forceinline__ float4 slot_decode(Slot w, float dsc) {
-    constexpr float K23 = 8388608.0f;
-    const float2 c = make_float2(__uint_as_float(__byte_perm(w.x, 0x4B000000u, 0x7610)),
-                                 __uint_as_float(__byte_perm(w.x, 0x4B000000u, 0x7632)));
-    const float2 rg = f2mul(f2sub(c, f2(K23)), f2(dsc));
-    const float b = (__uint_as_float(__byte_perm(w.y, 0x4B000000u, 0x7610)) - K23) * dsc;
-    const float a = __uint_as_float(__byte_perm(w.y, 0x4B000000u, 0x7632)) - K23;
-    return make_float4(rg.x, rg.y, b, a);
+// The codes (R, G, B, weight) of a slot element as floats.
+__device__ __forceinline__ float4 slot_codes(Slot w) {
+    const float2 k23 = f2(8388608.0f);
+    const float2 rg = f2sub(make_float2(__uint_as_float(__byte_perm(w.x, 0x4B000000u, 0x7610)),
+                                        __uint_as_float(__byte_perm(w.x, 0x4B000000u, 0x7632))), k23);
+    const float2 ba = f2sub(make_float2(__uint_as_float(__byte_perm(w.y, 0x4B000000u, 0x7610)),
+                                        __uint_as_float(__byte_perm(w.y, 0x4B000000u, 0x7632))), k23);
+    return make_float4(rg.x, rg.y, ba.x, ba.y);
 }
 
 // Where a tile's level-0 samples go besides the pyramid: nowhere, the FULL canvas tile's level-0
@@ -583,8 +593,8 @@ __device__ __forceinline__ void d1_bar(int id) {
 // One down1 tile, worked on by the D1_THREADS threads t = 0 .. 63 that share barrier `bar`.
 template <typename T, int CAP = D1_FOOT>
 __device__ __forceinline__ void down1_tile(const CamDev* __restrict__ cams, const RigGeom& g, const FramePtrs& fp,
-                                           const OutDesc& od, const D1Tile& tl, const CamRef* __restrict__ refs,
-                                           const float* __restrict__ d1w, const float4* __restrict__ d1cols,
+                                           const OutDesc& od, const D1Rec& rec, const float* __restrict__ d1w,
+                                           const float4* __restrict__ d1cols,
                                            Slot* __restrict__ g0buf, float4* smem, int t = threadIdx.x, int bar = 0) {
     uint32_t* foot = reinterpret_cast<uint32_t*>(smem);
     constexpr int SM_FOOT = D1Cap<CAP>::SM_FOOT;
@@ -592,13 +602,11 @@ __device__ __forceinline__ void down1_tile(const CamDev* __restrict__ cams, cons
     float4* ext = reinterpret_cast<float4*>(reinterpret_cast<char*>(smem) + SM_FOOT + D1_SM_V);  // [19][3]
     float2* rowdy = reinterpret_cast<float2*>(reinterpret_cast<char*>(smem) + SM_FOOT + D1_SM_V + D1_SM_X);
 
+    const D1Tile& tl = rec.tl;
     const int i = tl.cam;
-    const CamDev& ci = cams[i];
-    const Rect o1 = ci.Om[1];
     const int k0 = tl.k0, j0 = tl.j0;              // level-1 tile origin
     const int vx0 = 2 * k0 - 2, vy0 = 2 * j0 - 2;  // level-0 virtual origin
     const bool act = t < D1_THREADS;
-    const CamRef ref = refs[tl.ref];
     const uint8_t* px_i = fp.p[i];
     const long long pitch_i = fp.pitch[i];
 
@@ -621,14 +629,14 @@ __device__ __forceinline__ void down1_tile(const CamDev* __restrict__ cams, cons
     }
 
     D1Ctx x;
-    x.tm = ref.tm;
+    x.tm = rec.tm;
     x.rowdy = rowdy;
     x.wt = d1w + (long long)tl.wsel * D1_NSAMP;
     x.px = px_i;
     x.pitch = pitch_i;
-    x.W = ci.W;
-    x.H = ci.H;
-    x.scale = ci.gain * (1.0f / 255.0f);
+    x.W = rec.W;
+    x.H = rec.H;
+    x.scale = rec.scale;
     x.foot = foot;
     const bool staged = tl.fwh != 0;
     x.fx0 = tl.fxy & 0xffff;
@@ -638,12 +646,12 @@ __device__ __forceinline__ void down1_tile(const CamDev* __restrict__ cams, cons
     x.S = (x.fw + 3) & ~3;
     // footprint index of the top-left tap from the bit patterns tu, tv of the floor constants:
     // (tv - B + V0 - fy0) S + (tu - B + U0 - fx0), in arithmetic modulo 2^32
-    x.ibase = 4u * ((unsigned)(ref.tm.V0 - x.fy0) * (unsigned)x.S + (unsigned)(ref.tm.U0 - x.fx0) -
+    x.ibase = 4u * ((unsigned)(x.tm.V0 - x.fy0) * (unsigned)x.S + (unsigned)(x.tm.U0 - x.fx0) -
                     D1_FLOOR_BITS * ((unsigned)x.S + 1u));
     x.maxidx = x.S * (x.fh - 1) - 2;
     if (staged && act) stage_footprint<CAP>(foot, px_i, pitch_i, x.W, x.fx0, x.fy0, x.fw, x.fh, t);
     if (t < D1_SY) {
-        const float dy = (float)(fold101(vy0 + t, g.ny[0]) - ref.ay);
+        const float dy = (float)(fold101(vy0 + t, g.ny[0]) - rec.ay);
         rowdy[t] = make_float2(dy, dy);
     }
     // column terms: the anchored homography on the planar canvas, the column table on the
@@ -655,7 +663,7 @@ __device__ __forceinline__ void down1_tile(const CamDev* __restrict__ cams, cons
             nuv = make_float2(cc.x, cc.y);
             dqc = cc.z;
         } else {
-            const float dx = (float)(fold101(vx0 + c, g.nx[0]) - ref.ax);
+            const float dx = (float)(fold101(vx0 + c, g.nx[0]) - rec.ax);
             nuv = make_float2(fmaf(x.tm.pu1, dx, x.tm.pu0), fmaf(x.tm.pv1, dx, x.tm.pv0));
             dqc = fmaf(x.tm.q1, dx, x.tm.q0);
         }
@@ -734,6 +742,8 @@ __device__ __forceinline__ void down1_tile(const CamDev* __restrict__ cams, cons
     d1_bar(bar);
     // S3 horizontal pass and store of G^1: output (p, jj) takes columns 2p .. 2p+4
     if (act) {
+        const CamDev& ci = cams[i];
+        const Rect o1 = ci.Om[1];
         T* dst = reinterpret_cast<T*>(ci.FG[1]);
         const int p = t & 31, kk = k0 + p;
 #pragma unroll
@@ -752,19 +762,36 @@ __device__ __forceinline__ void down1_tile(const CamDev* __restrict__ cams, cons
     }
 }
 
+// A record in 16-byte loads, all in flight at once.
+template <typename R>
+__device__ __forceinline__ R load_record(const R* __restrict__ p) {
+    static_assert(sizeof(R) % 16 == 0, "16-byte words");
+    union U {
+        uint4 w[sizeof(R) / 16];
+        R r;
+        __device__ U() {}
+    } u;
+#pragma unroll
+    for (int k = 0; k < (int)(sizeof(R) / 16); ++k) u.w[k] = __ldg(reinterpret_cast<const uint4*>(p) + k);
+    return u.r;
+}
+__host__ __device__ inline D1Rec d1_record(const D1Tile& tl, const CamDev& c, const CamRef& ref) {
+    return D1Rec{tl, ref.tm, ref.ax, ref.ay, c.W, c.H, c.gain * (1.0f / 255.0f), {0, 0}};
+}
+
 template <typename T, int CAP>
 __global__ void __launch_bounds__(D1_THREADS, D1Cap<CAP>::BLOCKS) k_down1(const CamDev* __restrict__ cams, RigGeom g,
                                                                         FramePtrs fp, OutDesc od,
-                                                                        const D1Tile* __restrict__ tiles,
-                                                                        const CamRef* __restrict__ refs,
+                                                                        const D1Rec* __restrict__ recs, int n, int wave,
                                                                         const float* __restrict__ d1w,
                                                                         const float4* __restrict__ d1cols,
                                                                         Slot* __restrict__ g0buf) {
     extern __shared__ float4 smem[];
     pdl_trigger();
-    const D1Tile tl = tiles[blockIdx.x];
+    const D1Rec rec = load_record(recs + blockIdx.x);
+    if (threadIdx.x == 0 && blockIdx.x + wave < n) prefetch_l2(recs + blockIdx.x + wave);
     pdl_wait();
-    down1_tile<T, CAP>(cams, g, fp, od, tl, refs, d1w, d1cols, g0buf, smem);
+    down1_tile<T, CAP>(cams, g, fp, od, rec, d1w, d1cols, g0buf, smem);
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -783,23 +810,26 @@ constexpr int SO_BLOCKS = 18;  // resident blocks per SM, bounds the registers (
 // A rig uses it from this many tiles per SM on.  Below, the tiles stay with down1: 5 x 719p (325 tiles,
 // 2 per SM) takes 131 us either way, and a second stream only costs.
 constexpr int SO_MIN_PER_SM = 4;
-struct SoloTile {
-    int cam, x0, y0, fxy, fwh, ref0, ref1, coltab0, coltab1;
+struct __align__(16) SoloTile {
+    int cam, x0, y0, fxy, fwh, W;
+    float scale;
+    int coltab[2], ax[2], ay[2];
+    TileMap tm[2];  // of the upper and the lower half
+    int pad;
 };
+static_assert(sizeof(SoloTile) == 144, "nine 16-byte words");
 
 template <bool F32>
-__global__ void __launch_bounds__(D1_THREADS, SO_BLOCKS) k_solo(const CamDev* __restrict__ cams, const __grid_constant__ RigGeom g,
+__global__ void __launch_bounds__(D1_THREADS, SO_BLOCKS) k_solo(const __grid_constant__ RigGeom g,
                                                                 const __grid_constant__ FramePtrs fp, OutDesc od,
                                                                 const SoloTile* __restrict__ tiles,
-                                                                const CamRef* __restrict__ refs,
                                                                 const float4* __restrict__ d1cols) {
     __shared__ __align__(16) uint32_t foot[SO_FOOT];
     const int t = threadIdx.x;
     const int lane = t & 31;
-    const SoloTile tl = tiles[blockIdx.x];
-    const CamDev& c = cams[tl.cam];
+    const SoloTile tl = load_record(tiles + blockIdx.x);
     D1Ctx x{};
-    x.scale = c.gain * (1.0f / 255.0f);
+    x.scale = tl.scale;
     x.foot = foot;
     x.fx0 = tl.fxy & 0xffff;
     x.fy0 = (int)((unsigned)tl.fxy >> 16);
@@ -807,7 +837,7 @@ __global__ void __launch_bounds__(D1_THREADS, SO_BLOCKS) k_solo(const CamDev* __
     x.fh = tl.fwh >> 16;
     x.S = (x.fw + 3) & ~3;
     x.maxidx = x.S * (x.fh - 1) - 2;
-    stage_footprint<SO_FOOT>(foot, fp.p[tl.cam], fp.pitch[tl.cam], c.W, x.fx0, x.fy0, x.fw, x.fh, t);
+    stage_footprint<SO_FOOT>(foot, fp.p[tl.cam], fp.pitch[tl.cam], tl.W, x.fx0, x.fy0, x.fw, x.fh, t);
     __syncthreads();
     const int xo = tl.x0 + t, xc = min(xo, g.nx[0] - 1);
     // 8-bit rows of whole words: a warp's 32 pixels are 24 words; word l holds bytes l % 3 .. of pixel
@@ -817,24 +847,24 @@ __global__ void __launch_bounds__(D1_THREADS, SO_BLOCKS) k_solo(const CamDev* __
     const unsigned wsel = wl % 3 == 0 ? 0x4210u : wl % 3 == 1 ? 0x5421u : 0x6542u;
 #pragma unroll 1
     for (int h = 0; h < 2; ++h) {
-        const CamRef& ref = refs[h ? tl.ref1 : tl.ref0];
-        x.tm = ref.tm;
+        x.tm = h ? tl.tm[1] : tl.tm[0];
+        const int ax = h ? tl.ax[1] : tl.ax[0], ay = h ? tl.ay[1] : tl.ay[0];
         x.ibase = 4u * ((unsigned)(x.tm.V0 - x.fy0) * (unsigned)x.S + (unsigned)(x.tm.U0 - x.fx0) -
                         D1_FLOOR_BITS * ((unsigned)x.S + 1u));
         float2 nuv;
         float dqc;
         if (g.cyl) {
-            const float4 cc = d1cols[(long long)(h ? tl.coltab1 : tl.coltab0) * D1_SX + (xc - tl.x0) + 2];
+            const float4 cc = d1cols[(long long)(h ? tl.coltab[1] : tl.coltab[0]) * D1_SX + (xc - tl.x0) + 2];
             nuv = make_float2(cc.x, cc.y);
             dqc = cc.z;
         } else {
-            const float dx = (float)(xc - ref.ax);
+            const float dx = (float)(xc - ax);
             nuv = make_float2(fmaf(x.tm.pu1, dx, x.tm.pu0), fmaf(x.tm.pv1, dx, x.tm.pv0));
             dqc = fmaf(x.tm.q1, dx, x.tm.q0);
         }
         const int Y = tl.y0 + h * (U0_TY / 2);
         const int rows = min(U0_TY / 2, g.ny[0] - Y);
-        float2 dy = f2((float)(Y - ref.ay));
+        float2 dy = f2((float)(Y - ay));
         char* q = (char*)od.ptr + (long long)Y * od.pitch +
                   (words ? 3LL * (xo - lane) + 4 * lane : (F32 ? 12LL : 3LL) * xo);
 #pragma unroll 2
@@ -1002,9 +1032,11 @@ __device__ __forceinline__ void reduce_col_tile(const CamDev* __restrict__ cams,
     const Rect oc = c.Om[l + 1], of = c.Om[l];
     const int vx0 = 2 * tl.x0 - 2, vy0 = 2 * tl.y0 - 2;
     const T* src = reinterpret_cast<const T*>(c.FG[l]);
+    T* dst = reinterpret_cast<T*>(c.FG[l + 1]);
     const int nxl = g.nx[l], nyl = g.ny[l];
     const long long w = of.w();
     const int t = threadIdx.x;
+    pdl_wait();  // only constant tables above: read while the previous kernel drains
     // a tile whose inputs lie inside Omega^l (so inside the level: nothing folds) reads them straight
     const bool inside = vx0 >= of.x0 && vx0 + SX <= of.x1 && vy0 >= of.y0 && vy0 + SY <= of.y1;
     auto elem = [&](int r, int x, bool xin) -> float4 {
@@ -1060,7 +1092,6 @@ __device__ __forceinline__ void reduce_col_tile(const CamDev* __restrict__ cams,
         vres[jj * RC_VROW + (cc & 1) * RC_VODD + (cc >> 1)] = f4_of(acc);
     }
     __syncthreads();
-    T* dst = reinterpret_cast<T*>(c.FG[l + 1]);
     const int p = t % TX, k = tl.x0 + p;
 #pragma unroll
     for (int q = 0; q < TY * TX / RC_THREADS; ++q) {
@@ -1085,7 +1116,6 @@ __global__ void __launch_bounds__(RC_THREADS, 8) k_reduce_t(const CamDev* __rest
     const int nb = blockIdx.x + wave;
     pdl_trigger();
     const Tile tl = tiles[blockIdx.x];
-    pdl_wait();
     reduce_col_tile<T>(cams, g, l, tl, smem, nb < n ? tiles + nb : nullptr);
 }
 
@@ -1124,17 +1154,26 @@ __device__ __forceinline__ void expand_quad(const float4* __restrict__ a, int ld
 }
 
 // Tiled coarse level: R^l on a tile of level l (l >= 2), one 2 x 2 quad per thread, cameras in
-// chunks of 2.  Virtual level-(l+1) region: origin (X0/2 - 2, Y0/2 - 2), TX/2 + 4 by TY/2 + 4.
+// chunks of 2.  Latency bounds it (at most a few waves): the tables are read before the wait for the
+// previous kernel, and every load of the first chunk (R^{l+1}, two cameras' G^{l+1}, the first one's G^l)
+// is in flight at once, one barrier before the blend.  With a round trip and a barrier for each of
+// those: level 2 of 8 x 4K 36 us, now 29; levels 3 to 5 17 + 11 + 6.4, now 13.9 + 9.2 + 7.1.  Virtual level-(l+1) region: origin (X0/2 - 2, Y0/2 - 2), TX/2 + 4 by TY/2 + 4.
 // The tile shape is a template parameter (the batched schedule's tuner picks one per batch); the
 // single-rig path uses 32 x 32.
 constexpr int CT_NC = 2;
+// A camera's regions and buffers of the levels a coarse tile reads (l and l + 1), in shared memory.
+struct CoCam {
+    Rect z, o, oc;
+    const void *fg, *fgc;
+};
+static_assert(sizeof(CoCam) % 16 == 0, "16-byte units");
 template <int X, int Y>
 struct CShape {
     static constexpr int TX = X, TY = Y;                   // level-l outputs
     static constexpr int CX = X / 2 + 4, CY = Y / 2 + 4;   // level-(l+1) virtual region
     static constexpr int CN = CX * CY, TN = X * Y;
     static constexpr int QUADS = (X / 2) * (Y / 2);
-    static constexpr int SMEM_F4 = CN + CT_NC * CN;  // shared memory in float4 units
+    static constexpr int SMEM_F4 = CN + CT_NC * CN + CT_NC * (int)sizeof(CoCam) / 16;  // shared memory in float4 units
     static_assert(QUADS == 256, "one 2 x 2 quad per thread of a 256-thread block");
 };
 using CS32x32 = CShape<32, 32>;
@@ -1153,17 +1192,36 @@ __device__ __forceinline__ void coarse_tile(const CamDev* __restrict__ cams, con
                                             T* __restrict__ Rl, const T* __restrict__ Rc, const LevelTile& tl,
                                             const int* __restrict__ camlist, float4* smem) {
     float4* rc = smem;                                                   // [CS::CN] R^{l+1}
-    float4 (*gc)[CS::CN] = reinterpret_cast<float4 (*)[CS::CN]>(rc + CS::CN);  // [CT_NC][CS::CN] G^{l+1}, then R - G
+    float4 (*gc)[CS::CN] = reinterpret_cast<float4 (*)[CS::CN]>(rc + CS::CN);  // [CT_NC][CS::CN] R^{l+1} - G^{l+1}
+    CoCam* cc = reinterpret_cast<CoCam*>(rc + CS::CN + CT_NC * CS::CN);        // the chunk's cameras
     const bool top = l == g.levels - 1;
     const int X0 = tl.x0, Y0 = tl.y0;
     const int ax = X0 / 2 - 2, ay = Y0 / 2 - 2;
     const int nxl = g.nx[l], nyl = g.ny[l];
     const int t = threadIdx.x;
-    if (!top) {
-        for (int q = t; q < CS::CN; q += 256) {
-            const int r = q / CS::CX, c = q - r * CS::CX;
-            const int x = fold101(ax + c, g.nx[l + 1]), y = fold101(ay + r, g.ny[l + 1]);
-            rc[q] = ld(Rc + (long long)y * g.nx[l + 1] + x);
+    const auto cameras = [&](int c0) {
+        if (t < min(CT_NC, tl.count - c0)) {
+            const CamDev& c = cams[camlist[tl.first + c0 + t]];
+            const int lc = top ? l : l + 1;
+            cc[t] = CoCam{c.Z[l], c.Om[l], c.Om[lc], c.FG[l], c.FG[lc]};
+        }
+    };
+    cameras(0);  // constant tables: read while the previous kernel drains
+    pdl_wait();
+    // A thread takes the same positions of the level l + 1 region for R and for every camera's G, so it forms
+    // the differences in registers, and all loads of the first chunk are in flight at once.
+    constexpr int NK = (CS::CN + 255) / 256;
+    int px[NK], py[NK];
+    float4 rv[NK];
+#pragma unroll
+    for (int k = 0; k < NK; ++k) {
+        const int q = t + 256 * k, r = q / CS::CX, c = q - r * CS::CX;
+        rv[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+        px[k] = py[k] = 0;
+        if (!top && q < CS::CN) {
+            px[k] = fold101(ax + c, g.nx[l + 1]);
+            py[k] = fold101(ay + r, g.ny[l + 1]);
+            rv[k] = ld(Rc + (long long)py[k] * g.nx[l + 1] + px[k]);
         }
     }
     const int qx = t % (CS::TX / 2), qy = t / (CS::TX / 2);
@@ -1175,66 +1233,69 @@ __device__ __forceinline__ void coarse_tile(const CamDev* __restrict__ cams, con
         nrg[k] = make_float2(0.f, 0.f);
         nb[k] = den[k] = 0.f;
     }
-    for (int c0 = 0; c0 < tl.count; c0 += CT_NC) {
-        const int nc = min(CT_NC, tl.count - c0);
-        __syncthreads();
-        // the chunk's G^{l+1} regions into shared memory, all loads in flight before the stores
-        {
-            constexpr int NC2 = (CT_NC * CS::CN + 255) / 256;
-            float4 w[NC2];
+    // the quad's G^l of a camera: each value is read by this thread only, so it goes straight into
+    // registers (only inside Z^l, where it enters the blend)
+    const auto quad = [&](int ci, float4 gq[4]) {
+        const Rect z = cc[ci].z, o = cc[ci].o;
+        const T* fg = reinterpret_cast<const T*>(cc[ci].fg);
 #pragma unroll
-            for (int k = 0; k < NC2; ++k) {
-                const int q = t + 256 * k;
-                w[k] = make_float4(0.f, 0.f, 0.f, 0.f);
-                if (!top && q < nc * CS::CN) {
-                    const int ci = q / CS::CN, qq = q - ci * CS::CN;
-                    const CamDev& c = cams[camlist[tl.first + c0 + ci]];
-                    const int r = qq / CS::CX, cc = qq - r * CS::CX;
-                    const int x = fold101(ax + cc, g.nx[l + 1]), y = fold101(ay + r, g.ny[l + 1]);
-                    const Rect o = c.Om[l + 1];
-                    if (o.contains(x, y))
-                        w[k] = ld(reinterpret_cast<const T*>(c.FG[l + 1]) + (long long)(y - o.y0) * o.w() + (x - o.x0));
-                }
-            }
-#pragma unroll
-            for (int k = 0; k < NC2; ++k) {
-                const int q = t + 256 * k;
-                if (!top && q < nc * CS::CN) gc[q / CS::CN][q % CS::CN] = w[k];
-            }
+        for (int k = 0; k < 4; ++k) {
+            const int x = X0 + 2 * qx + (k & 1), y = Y0 + 2 * qy + (k >> 1);
+            gq[k] = has_quad && z.contains(x, y) ? ld(fg + (long long)(y - o.y0) * o.w() + (x - o.x0))
+                                                 : make_float4(0.f, 0.f, 0.f, 0.f);
         }
-        __syncthreads();
-        if (!top) {
-            for (int q = t; q < nc * CS::CN; q += 256) {
-                const int ci = q / CS::CN, qq = q - ci * CS::CN;
-                const float4 a = rc[qq], b = gc[ci][qq];
-                gc[ci][qq] = make_float4(a.x - b.x, a.y - b.y, a.z - b.z, 0.f);
-            }
+    };
+    __syncthreads();
+    for (int c0 = 0; c0 == 0 || c0 < tl.count; c0 += CT_NC) {
+        const int nc = min(CT_NC, tl.count - c0);
+        if (c0 > 0) {
+            __syncthreads();
+            cameras(c0);
             __syncthreads();
         }
-        if (has_quad) {
-            for (int ci = 0; ci < nc; ++ci) {
-                // the quad's G^l of the camera: each value is read by this thread only, so it goes
-                // straight into registers (only inside Z^l, where it enters the blend)
-                const CamDev& c = cams[camlist[tl.first + c0 + ci]];
-                const Rect z = c.Z[l], o = c.Om[l];
-                const T* fg = reinterpret_cast<const T*>(c.FG[l]);
-                float4 gq[4];
+        float4 gq[4];
+        {
+            float4 w[CT_NC][NK];
 #pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    const int x = X0 + 2 * qx + (k & 1), y = Y0 + 2 * qy + (k >> 1);
-                    gq[k] = z.contains(x, y) ? ld(fg + (long long)(y - o.y0) * o.w() + (x - o.x0)) : make_float4(0.f, 0.f, 0.f, 0.f);
-                }
-                V3 e[4] = {v3_zero(), v3_zero(), v3_zero(), v3_zero()};
-                if (!top) expand_quad(gc[ci], CS::CX, qx + 1, qy + 1, e);
+            for (int ci = 0; ci < CT_NC; ++ci)
 #pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    const int x = X0 + 2 * qx + (k & 1), y = Y0 + 2 * qy + (k >> 1);
-                    if (!z.contains(x, y)) continue;
-                    const float4 gv = gq[k];
-                    nrg[k] = f2fma(f2(gv.w), f2add(make_float2(gv.x, gv.y), e[k].rg), nrg[k]);
-                    nb[k] = fmaf(gv.w, gv.z + e[k].b, nb[k]);
-                    den[k] += gv.w;
+                for (int k = 0; k < NK; ++k) {
+                    w[ci][k] = make_float4(0.f, 0.f, 0.f, 0.f);
+                    if (!top && ci < nc && t + 256 * k < CS::CN) {
+                        const Rect o = cc[ci].oc;
+                        if (o.contains(px[k], py[k]))
+                            w[ci][k] = ld(reinterpret_cast<const T*>(cc[ci].fgc) + (long long)(py[k] - o.y0) * o.w() + (px[k] - o.x0));
+                    }
                 }
+            if (nc > 0) quad(0, gq);
+            if (!top) {
+#pragma unroll
+                for (int k = 0; k < NK; ++k) {
+                    const int q = t + 256 * k;
+                    if (q >= CS::CN) continue;
+                    if (c0 == 0) rc[q] = rv[k];
+                    else rv[k] = rc[q];
+#pragma unroll
+                    for (int ci = 0; ci < CT_NC; ++ci)
+                        gc[ci][q] = make_float4(rv[k].x - w[ci][k].x, rv[k].y - w[ci][k].y, rv[k].z - w[ci][k].z, 0.f);
+                }
+            }
+        }
+        __syncthreads();
+        for (int ci = 0; ci < nc; ++ci) {
+            if (ci > 0) quad(ci, gq);
+            if (!has_quad) continue;
+            const Rect z = cc[ci].z;
+            V3 e[4] = {v3_zero(), v3_zero(), v3_zero(), v3_zero()};
+            if (!top) expand_quad(gc[ci], CS::CX, qx + 1, qy + 1, e);
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const int x = X0 + 2 * qx + (k & 1), y = Y0 + 2 * qy + (k >> 1);
+                if (!z.contains(x, y)) continue;
+                const float4 gv = gq[k];
+                nrg[k] = f2fma(f2(gv.w), f2add(make_float2(gv.x, gv.y), e[k].rg), nrg[k]);
+                nb[k] = fmaf(gv.w, gv.z + e[k].b, nb[k]);
+                den[k] += gv.w;
             }
         }
     }
@@ -1267,7 +1328,6 @@ __global__ void __launch_bounds__(256, 3) k_coarse_t(const CamDev* __restrict__ 
     extern __shared__ float4 smem[];
     pdl_trigger();
     const LevelTile tl = tiles[blockIdx.x];
-    pdl_wait();
     coarse_tile<T, CSRig>(cams, g, l, Rl, Rc, tl, camlist, smem);
 }
 
@@ -1434,123 +1494,109 @@ __device__ __forceinline__ void up_full_tile(const CamDev* __restrict__ cams, co
     }
     pdl_wait();
     __syncthreads();
-    // loads of level 1 and 2 data, all of a thread's loads in flight before the stores
-    if (L >= 2) {
-        constexpr int NL = (NC * U1_N + U_THREADS - 1) / U_THREADS;
-        float4 v[NL];
+    // Level 1 and 2 data.  A thread takes the same positions for every camera (and for R^2), so it forms
+    // Delta^2_i = R^2 - G^2_i in registers; the loads of level 2 and of the first two cameras' level 1 are
+    // in flight before the first store, and the level-1 blend follows after one barrier.  With this, the
+    // blend's R and G in pairs, 16-byte slot loads and 16-bit stores of the staged bytes, the 8 x 4K launch
+    // takes 214 us (250 with a round trip and a barrier for level 1, level 2 and its differences each).
+    constexpr int N1 = (U1_N + U_THREADS - 1) / U_THREADS;
+    static_assert(U2_N <= U_THREADS, "one level-2 position per thread");
+    int x1[N1], y1[N1];
 #pragma unroll
-        for (int k = 0; k < NL; ++k) {
-            const int q = t + k * U_THREADS;
-            v[k] = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (q < nc * U1_N) {
-                const int ci = q / U1_N, qq = q - ci * U1_N;
-                const int r = qq / U1_X, cc = qq - r * U1_X;
-                const int x = fold101(a1x + cc, g.nx[1]), y = fold101(a1y + r, g.ny[1]);
-                const Rect o1 = ucs.om1[ci];
-                if (o1.contains(x, y))
-                    v[k] = ld(reinterpret_cast<const T*>(ucs.fg1[ci]) + (long long)(y - o1.y0) * o1.w() + (x - o1.x0));
-            }
-        }
+    for (int k = 0; k < N1; ++k) {
+        const int q = t + k * U_THREADS, r = q / U1_X, cc = q - r * U1_X;
+        x1[k] = fold101(a1x + cc, g.nx[1]);
+        y1[k] = q < U1_N ? fold101(a1y + r, g.ny[1]) : -1;  // no Omega^1 holds row -1
+    }
+    float4 rv = make_float4(0.f, 0.f, 0.f, 0.f), g2[NC];
+    if (L >= 3 && t < U2_N) {
+        const int r = t / U2_X, cc = t - r * U2_X;
+        const int x = fold101(a2x + cc, g.nx[2]), y = fold101(a2y + r, g.ny[2]);
+        rv = ld(R2 + (long long)y * g.nx[2] + x);
 #pragma unroll
-        for (int k = 0; k < NL; ++k) {
-            const int q = t + k * U_THREADS;
-            if (q < nc * U1_N) d1[q] = v[k];
+        for (int ci = 0; ci < NC; ++ci) {
+            g2[ci] = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (ci >= nc) continue;
+            const Rect o2 = ucs.om2[ci];
+            if (o2.contains(x, y))
+                g2[ci] = ld(reinterpret_cast<const T*>(ucs.fg2[ci]) + (long long)(y - o2.y0) * o2.w() + (x - o2.x0));
         }
     }
-    if (L >= 3) {
-        constexpr int NL = ((NC + 1) * U2_N + U_THREADS - 1) / U_THREADS;
-        float4 v[NL];
+    if (L >= 2) {
 #pragma unroll
-        for (int k = 0; k < NL; ++k) {
-            const int q = t + k * U_THREADS;
-            v[k] = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (q < (nc + 1) * U2_N) {
-                const int ci = q / U2_N, qq = q - ci * U2_N;
-                const int r = qq / U2_X, cc = qq - r * U2_X;
-                const int x = fold101(a2x + cc, g.nx[2]), y = fold101(a2y + r, g.ny[2]);
-                if (ci == nc) {
-                    v[k] = ld(R2 + (long long)y * g.nx[2] + x);
-                } else {
-                    const Rect o2 = ucs.om2[ci];
-                    if (o2.contains(x, y))
-                        v[k] = ld(reinterpret_cast<const T*>(ucs.fg2[ci]) + (long long)(y - o2.y0) * o2.w() + (x - o2.x0));
-                }
+        for (int c0 = 0; c0 < NC; c0 += 2) {
+            if (c0 >= nc) break;
+            float4 v[2][N1];
+#pragma unroll
+            for (int b = 0; b < 2; ++b) {
+                if (c0 + b >= nc) break;
+                const Rect o1 = ucs.om1[c0 + b];
+                const T* fg = reinterpret_cast<const T*>(ucs.fg1[c0 + b]);
+#pragma unroll
+                for (int k = 0; k < N1; ++k)
+                    v[b][k] = o1.contains(x1[k], y1[k]) ? ld(fg + (long long)(y1[k] - o1.y0) * o1.w() + (x1[k] - o1.x0))
+                                                        : make_float4(0.f, 0.f, 0.f, 0.f);
             }
-        }
+            if (c0 == 0 && L >= 3 && t < U2_N) {
+                r2s[t] = rv;
 #pragma unroll
-        for (int k = 0; k < NL; ++k) {
-            const int q = t + k * U_THREADS;
-            if (q < (nc + 1) * U2_N) {
-                const int ci = q / U2_N, qq = q - ci * U2_N;
-                if (ci == nc) r2s[qq] = v[k];
-                else d2[q] = v[k];
+                for (int ci = 0; ci < NC; ++ci)
+                    if (ci < nc) d2[ci * U2_N + t] = make_float4(rv.x - g2[ci].x, rv.y - g2[ci].y, rv.z - g2[ci].z, 0.f);
+            }
+#pragma unroll
+            for (int b = 0; b < 2; ++b) {
+                if (c0 + b >= nc) break;
+#pragma unroll
+                for (int k = 0; k < N1; ++k)
+                    if (t + k * U_THREADS < U1_N) d1[(c0 + b) * U1_N + t + k * U_THREADS] = v[b][k];
             }
         }
     }
     if (pf) up_prefetch<T, NC>(cams, *pf, refs, g0buf);  // the tile one resident wave later
     __syncthreads();
-    if (L >= 3) {
-        // Delta^2_i = R^2 - G^2_i
-        for (int q = t; q < nc * U2_N; q += U_THREADS) {
-            const float4 rv = r2s[q % U2_N], gv = d2[q];
-            d2[q] = make_float4(rv.x - gv.x, rv.y - gv.y, rv.z - gv.z, 0.f);
-        }
-        __syncthreads();
-    }
     if (L >= 2 && t < U_QUADS1) {
         // level 1: R^1 = sum_i a_i (G^1_i + EXPAND(Delta^2_i)), then Delta^1_i = R^1 - G^1_i in place
         const int qx = t % (U1_X / 2), qy = t / (U1_X / 2);
-        float3 num[4];
-        float den[4];
+        float2 nrg[4];
+        float nb[4], den[4];
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
-            num[k] = make_float3(0.f, 0.f, 0.f);
-            den[k] = 0.f;
+            nrg[k] = make_float2(0.f, 0.f);
+            nb[k] = den[k] = 0.f;
         }
         for (int c = 0; c < nc; ++c) {
-            float3 e[4] = {make_float3(0.f, 0.f, 0.f), make_float3(0.f, 0.f, 0.f), make_float3(0.f, 0.f, 0.f),
-                           make_float3(0.f, 0.f, 0.f)};
-            if (L >= 3) {
-                V3 e2[4];
-                expand_quad(d2 + c * U2_N, U2_X, qx, qy, e2);
-#pragma unroll
-                for (int k = 0; k < 4; ++k) e[k] = make_float3(e2[k].rg.x, e2[k].rg.y, e2[k].b);
-            }
-
+            V3 e[4] = {v3_zero(), v3_zero(), v3_zero(), v3_zero()};
+            if (L >= 3) expand_quad(d2 + c * U2_N, U2_X, qx, qy, e);
             // outside the camera's Z^1 its weight pyramid is exactly 0, so those terms add nothing
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
                 const float4 gv = d1[c * U1_N + (2 * qy + (k >> 1)) * U1_X + 2 * qx + (k & 1)];
-                num[k].x = fmaf(gv.w, gv.x + e[k].x, num[k].x);
-                num[k].y = fmaf(gv.w, gv.y + e[k].y, num[k].y);
-                num[k].z = fmaf(gv.w, gv.z + e[k].z, num[k].z);
+                nrg[k] = f2fma(f2(gv.w), f2add(make_float2(gv.x, gv.y), e[k].rg), nrg[k]);
+                nb[k] = fmaf(gv.w, gv.z + e[k].b, nb[k]);
                 den[k] += gv.w;
             }
         }
-        float3 r1[4];
         bool need_plain = false;
+        float rd[4];
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
-            if (den[k] > 1e-12f) {
-                const float rd = __frcp_rn(den[k]);
-                r1[k] = make_float3(num[k].x * rd, num[k].y * rd, num[k].z * rd);
-            } else {
-                r1[k] = make_float3(0.f, 0.f, 0.f);
-                need_plain = true;
-            }
+            rd[k] = __frcp_rn(den[k]);
+            need_plain |= !(den[k] > 1e-12f);
         }
-        if (need_plain && L >= 3) {
-            V3 e[4];
-            expand_quad(r2s, U2_X, qx, qy, e);
-#pragma unroll
-            for (int k = 0; k < 4; ++k)
-                if (!(den[k] > 1e-12f)) r1[k] = make_float3(e[k].rg.x, e[k].rg.y, e[k].b);
-        }
+        V3 e[4] = {v3_zero(), v3_zero(), v3_zero(), v3_zero()};
+        if (need_plain && L >= 3) expand_quad(r2s, U2_X, qx, qy, e);
         for (int c = 0; c < nc; ++c) {
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
                 float4& dv = d1[c * U1_N + (2 * qy + (k >> 1)) * U1_X + 2 * qx + (k & 1)];
-                dv = make_float4(r1[k].x - dv.x, r1[k].y - dv.y, r1[k].z - dv.z, 0.f);
+                const float4 gv = dv;
+                if (den[k] > 1e-12f) {
+                    // R^1 rounded before the difference, as every other reader of a collapsed level sees it
+                    dv = make_float4(__fmul_rn(nrg[k].x, rd[k]) - gv.x, __fmul_rn(nrg[k].y, rd[k]) - gv.y,
+                                     __fmul_rn(nb[k], rd[k]) - gv.z, 0.f);
+                } else {
+                    dv = make_float4(e[k].rg.x - gv.x, e[k].rg.y - gv.y, e[k].b - gv.z, 0.f);
+                }
             }
         }
     }
@@ -1574,57 +1620,78 @@ __device__ __forceinline__ void up_full_tile(const CamDev* __restrict__ cams, co
     // tile (slot g0)
     for (int qd = t; qd < U_QUADS0; qd += U_THREADS) {
         const int qx = qd % (U_TX / 2), qy = qd / (U_TX / 2);
-        float3 num[4];
-        float den[4];
+        float2 nrg[4];
+        float nb[4], den[4];
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
-            num[k] = make_float3(0.f, 0.f, 0.f);
-            den[k] = 0.f;
+            nrg[k] = make_float2(0.f, 0.f);
+            nb[k] = den[k] = 0.f;
         }
         // the level-0 samples of every blended camera, NB cameras at a time (all their loads in
-        // flight at once); the weights enter as their slot codes
-
+        // flight at once; two neighbouring samples are one 16-byte load); the weights enter as their
+        // slot codes
         for (int c0 = 0; c0 < nc; c0 += NB) {
-            Slot gw[NB][4];
+            uint4 gw[NB][2];
 #pragma unroll
             for (int b = 0; b < NB; ++b) {
                 const int slot = c0 + b < nc ? cr[c0 + b].g0 : -1;
                 const Slot* gq = g0buf + (long long)max(slot, 0) * (U_TX * U_TY) + (2 * qy) * U_TX + 2 * qx;
 #pragma unroll
-                for (int k = 0; k < 4; ++k)
-                    gw[b][k] = slot >= 0 ? __ldcg(gq + (k >> 1) * U_TX + (k & 1)) : make_uint2(0u, 0u);
+                for (int k = 0; k < 2; ++k)
+                    gw[b][k] = slot >= 0 ? __ldcg(reinterpret_cast<const uint4*>(gq + k * U_TX)) : make_uint4(0u, 0u, 0u, 0u);
             }
 #pragma unroll
             for (int b = 0; b < NB; ++b) {
                 const int c = c0 + b;
                 if (c >= nc || cr[c].g0 < 0) continue;
+                const float dsc = ucs.dsc[c];
                 V3 e[4];
                 expand_quad(d1 + c * U1_N, U1_X, qx + 1, qy + 1, e);
                 // a camera's weight is 0 (and its sample 0) where it does not cover the pixel: the
                 // terms add nothing there, so no test is needed
 #pragma unroll
                 for (int k = 0; k < 4; ++k) {
-                    const float4 gv = slot_decode(gw[b][k], ucs.dsc[c]);
-                    num[k].x = fmaf(gv.w, gv.x + e[k].rg.x, num[k].x);
-                    num[k].y = fmaf(gv.w, gv.y + e[k].rg.y, num[k].y);
-                    num[k].z = fmaf(gv.w, gv.z + e[k].b, num[k].z);
+                    const uint4 w = gw[b][k >> 1];
+                    const float4 gv = slot_codes(k & 1 ? make_uint2(w.z, w.w) : make_uint2(w.x, w.y));
+                    // R and G are rounded before the addition, B is not: additions of a packed product
+                    // are fused with it, those of its two halves are not
+                    const float2 rg = f2mul(make_float2(gv.x, gv.y), f2(dsc));
+                    const float2 sum = make_float2(__fadd_rn(rg.x, e[k].rg.x), __fadd_rn(rg.y, e[k].rg.y));
+                    nrg[k] = f2fma(f2(gv.w), sum, nrg[k]);
+                    nb[k] = fmaf(gv.w, fmaf(gv.z, dsc, e[k].b), nb[k]);
                     den[k] += gv.w;
                 }
             }
         }
+        float3 v[4];
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
-            const int dx = 2 * qx + (k & 1), dy = 2 * qy + (k >> 1);
-            const int x = X0 + dx, y = Y0 + dy;
-            if (x >= X1 || y >= Y1) continue;
-            float rr = 0.f, gg = 0.f, bb = 0.f;
+            v[k] = make_float3(0.f, 0.f, 0.f);
             if (den[k] > 0.f) {
                 const float rd = __frcp_rn(den[k]);
-                rr = __saturatef(num[k].x * rd);
-                gg = __saturatef(num[k].y * rd);
-                bb = __saturatef(num[k].z * rd);
+                v[k] = make_float3(__saturatef(nrg[k].x * rd), __saturatef(nrg[k].y * rd), __saturatef(nb[k] * rd));
             }
-            put_pixel(stage, od, dx, dy, x, y, rr, gg, bb);
+        }
+        if (od.is_float) {
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const int x = X0 + 2 * qx + (k & 1), y = Y0 + 2 * qy + (k >> 1);
+                if (x >= X1 || y >= Y1) continue;
+                float* o = (float*)((char*)od.ptr + (long long)y * od.pitch) + 3 * x;
+                o[0] = v[k].x;
+                o[1] = v[k].y;
+                o[2] = v[k].z;
+            }
+        } else {
+            // two neighbouring pixels are three 16-bit words of the staged tile (what lies past the canvas
+            // is staged too, and not copied out)
+#pragma unroll
+            for (int k = 0; k < 4; k += 2) {
+                unsigned short* o = reinterpret_cast<unsigned short*>(stage + (2 * qy + (k >> 1)) * 3 * U_TX + 6 * qx);
+                o[0] = (unsigned short)__byte_perm(quantize_bits(v[k].x), quantize_bits(v[k].y), 0x0040);
+                o[1] = (unsigned short)__byte_perm(quantize_bits(v[k].z), quantize_bits(v[k + 1].x), 0x0040);
+                o[2] = (unsigned short)__byte_perm(quantize_bits(v[k + 1].y), quantize_bits(v[k + 1].z), 0x0040);
+            }
         }
     }
     if (!od.is_float) {
@@ -1938,6 +2005,7 @@ enum UpKind { UP_SIMPLE = 0, UP_FULL2 = 1, UP_FULL4 = 2, UP_GENERAL = 3, UP_KIND
 struct FusedState {
     D1Tile* d1_tiles = nullptr;
     int n_d1 = 0;
+    D1Rec* d1_recs = nullptr;
     int n_d1_pyr = 0;            // the first of them: those that the solo kernel does not take
     SoloTile* solo_tiles = nullptr;
     int n_solo_tiles = 0;
@@ -1960,7 +2028,7 @@ struct FusedState {
     int n_staged = 0;            // down1 tiles with a staged source footprint
     bool d1_small = false;       // down1 with the smaller footprint capacity (13 blocks per SM)
     bool up_four = false;        // up_full with four resident blocks per SM
-    int wave_red = 0, wave_up = 0;  // resident blocks on the device (L2 prefetch distance)
+    int wave_d1 = 0, wave_red = 0, wave_up = 0;  // resident blocks on the device (L2 prefetch distance)
     void* R[MAXL] = {};          // R^l on the canvas grid, l >= 2
     CamRef* refs = nullptr;
     UpTile* up_tiles[UP_KINDS] = {};
@@ -2207,8 +2275,8 @@ void launch_chain(stitch_rig* r, FusedState* fs, const FramePtrs& fp, const OutD
         prof_mark(r, "fused_down1", s);
         const auto k = fs->d1_small ? k_down1<T, D1_FOOT_SMALL> : k_down1<T, D1_FOOT>;
         const size_t smem = fs->d1_small ? D1Cap<D1_FOOT_SMALL>::SMEM : D1_SMEM;
-        stream_launch(early, k, fs->n_d1_pyr, D1_THREADS, smem, s, r->dcam, g, fp, od, fs->d1_tiles, fs->refs, fs->d1w,
-                      fs->d1cols, (Slot*)fs->g0buf);
+        stream_launch(early, k, fs->n_d1_pyr, D1_THREADS, smem, s, r->dcam, g, fp, od, fs->d1_recs, fs->n_d1_pyr, fs->wave_d1,
+                      fs->d1w, fs->d1cols, (Slot*)fs->g0buf);
     }
     solo();
     for (int l = 1; l + 1 < L; ++l) {
@@ -2263,7 +2331,7 @@ stitch_status launch_all(stitch_rig* r, FusedState* fs, const FramePtrs& fp, con
         if (fs->n_solo_tiles == 0) return;
         prof_mark(r, "fused_solo", s);
         const auto k = od.is_float ? k_solo<true> : k_solo<false>;
-        k<<<fs->n_solo_tiles, D1_THREADS, 0, s>>>(r->dcam, r->geom, fp, od, fs->solo_tiles, fs->refs, fs->d1cols);
+        k<<<fs->n_solo_tiles, D1_THREADS, 0, s>>>(r->geom, fp, od, fs->solo_tiles, fs->d1cols);
     };
     if (!fs->chain || r->prof) {
         launch_chain<T>(r, fs, fp, od, s, true, solo);
@@ -2387,9 +2455,13 @@ stitch_status fused_plan(stitch_rig* r) {
     plan_reduce_tiles(r, RSCol::TX, RSCol::TY, redc);
     // classify the canvas tiles of `up`
     std::vector<UpTile> up[UP_KINDS];
-    std::unordered_map<long long, size_t> d1_index;  // (camera, level-1 origin) -> down1 tile
-    for (size_t k = 0; k < d1.size(); ++k)
-        d1_index[((long long)d1[k].cam << 42) | ((long long)d1[k].k0 << 21) | d1[k].j0] = k;
+    // down1 tile of a camera at a level-1 origin (the list is in the order of camera, row, column)
+    const auto find_d1 = [&](int cam, int k0, int j0) -> size_t {
+        const auto key = [](const D1Tile& t) { return std::make_tuple(t.cam, t.j0, t.k0); };
+        const auto want = std::make_tuple(cam, j0, k0);
+        const auto it = std::lower_bound(d1.begin(), d1.end(), want, [&](const D1Tile& t, const auto& w) { return key(t) < w; });
+        return it != d1.end() && key(*it) == want ? (size_t)(it - d1.begin()) : SIZE_MAX;
+    };
     for (int Y0 = 0; Y0 < g.ny[0]; Y0 += U_TY)
         for (int X0 = 0; X0 < g.nx[0]; X0 += U_TX) {
             const int X1 = std::min(X0 + U_TX, g.nx[0]), Y1 = std::min(Y0 + U_TY, g.ny[0]);
@@ -2439,11 +2511,10 @@ stitch_status fused_plan(stitch_rig* r) {
                     // with a level-1 pass, the camera's down1 tile over this canvas tile writes the
                     // output (its level-0 samples are the output here)
                     if (L >= 2) {
-                        auto it = d1_index.find(((long long)last_v << 42) | ((long long)(X0 / 2) << 21) | (Y0 / 2));
-                        auto it2 = d1_index.find(((long long)last_v << 42) | ((long long)(X0 / 2) << 21) | (Y0 / 2 + D1_TY));
-                        if (it != d1_index.end() && it2 != d1_index.end()) {
-                            d1[it->second].flags |= D1_SOLO_OUT;
-                            d1[it2->second].flags |= D1_SOLO_OUT;
+                        const size_t a = find_d1(last_v, X0 / 2, Y0 / 2), b = find_d1(last_v, X0 / 2, Y0 / 2 + D1_TY);
+                        if (a != SIZE_MAX && b != SIZE_MAX) {
+                            d1[a].flags |= D1_SOLO_OUT;
+                            d1[b].flags |= D1_SOLO_OUT;
                             kind = -1;
                         }
                     }
@@ -2457,9 +2528,9 @@ stitch_status fused_plan(stitch_rig* r) {
                         d1k[k][0] = d1k[k][1] = SIZE_MAX;
                         if (!rects_meet(r->hcam[rk.cam].V, X0, X1, Y0, Y1)) continue;
                         for (int h = 0; h < 2; ++h) {
-                            auto it = d1_index.find(((long long)rk.cam << 42) | ((long long)(X0 / 2) << 21) | (Y0 / 2 + h * D1_TY));
-                            if (it == d1_index.end()) kind = UP_GENERAL;
-                            else d1k[k][h] = it->second;
+                            const size_t a = find_d1(rk.cam, X0 / 2, Y0 / 2 + h * D1_TY);
+                            if (a == SIZE_MAX) kind = UP_GENERAL;
+                            else d1k[k][h] = a;
                         }
                     }
                     if (kind != UP_GENERAL)
@@ -2632,24 +2703,24 @@ stitch_status fused_plan(stitch_rig* r) {
     std::vector<SoloTile> solo;
     {
         std::vector<char> in_solo(d1.size(), 0);
-        std::unordered_map<long long, size_t> at;  // (camera, level-1 origin) -> down1 tile
-        const auto key = [](int cam, int k0, int j0) { return ((long long)cam << 42) | ((long long)k0 << 21) | j0; };
-        for (size_t k = 0; k < d1.size(); ++k) at[key(d1[k].cam, d1[k].k0, d1[k].j0)] = k;
         const auto warp_only = [](const D1Tile& t) {
             return (t.flags & (D1_SOLO_OUT | D1_NOCLAMP | D1_G0_OUT | D1_G1_OUT)) == (D1_SOLO_OUT | D1_NOCLAMP) && t.fwh != 0;
         };
         for (size_t k = 0; k < d1.size(); ++k) {
             const D1Tile& a = d1[k];
             if ((a.j0 / D1_TY) & 1 || !warp_only(a)) continue;
-            const auto it = at.find(key(a.cam, a.k0, a.j0 + D1_TY));
-            if (it == at.end() || !warp_only(d1[it->second])) continue;
-            const D1Tile& b = d1[it->second];
+            const size_t below = find_d1(a.cam, a.k0, a.j0 + D1_TY);
+            if (below == SIZE_MAX || !warp_only(d1[below])) continue;
+            const D1Tile& b = d1[below];
             const int x0 = 2 * a.k0, y0 = 2 * a.j0;
             const Rect q{x0, std::min(x0 + U0_TX, g.nx[0]), y0, std::min(y0 + U0_TY, g.ny[0])};
             int fx0, fy0, fw, fh;
             if (!d1_footprint(r->hcam[a.cam], g, q, SO_FOOT, fx0, fy0, fw, fh)) continue;
-            solo.push_back({a.cam, x0, y0, fx0 | (fy0 << 16), fw | (fh << 16), a.ref, b.ref, a.coltab, b.coltab});
-            in_solo[k] = in_solo[it->second] = 1;
+            const CamRef &ra = refs[a.ref], &rb = refs[b.ref];
+            const CamDev& c = r->hcam[a.cam];
+            solo.push_back({a.cam, x0, y0, fx0 | (fy0 << 16), fw | (fh << 16), c.W, c.gain * (1.0f / 255.0f),
+                            {a.coltab, b.coltab}, {ra.ax, rb.ax}, {ra.ay, rb.ay}, {ra.tm, rb.tm}, 0});
+            in_solo[k] = in_solo[below] = 1;
         }
         int sms = 0;
         if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, r->device) != cudaSuccess || sms < 1)
@@ -2699,6 +2770,7 @@ stitch_status fused_plan(stitch_rig* r) {
                          : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bpsm, k_down1<float4, D1_FOOT>, D1_THREADS, D1_SMEM);
         if (oe != cudaSuccess) return STITCH_ECUDA;
         const size_t K = (size_t)std::max(bpsm, 1) * sms;
+        fs->wave_d1 = (int)K;
         for (size_t k = 0; k + K < (size_t)fs->n_d1_pyr; ++k) {
             const D1Tile& nx = d1[k + K];
             if (nx.fwh == 0) continue;
@@ -2726,6 +2798,10 @@ stitch_status fused_plan(stitch_rig* r) {
     st = upload(r, d1c, &fs->d1_cams);
     if (st != STITCH_OK) return st;
     st = upload(r, cols, &fs->d1cols);
+    if (st != STITCH_OK) return st;
+    std::vector<D1Rec> recs(fs->n_d1_pyr);
+    for (int k = 0; k < fs->n_d1_pyr; ++k) recs[k] = d1_record(d1[k], r->hcam[d1[k].cam], refs[d1[k].ref]);
+    st = upload(r, recs, &fs->d1_recs);
     if (st != STITCH_OK) return st;
     st = upload(r, solo, &fs->solo_tiles);
     if (st != STITCH_OK) return st;
@@ -2959,10 +3035,13 @@ __global__ void __launch_bounds__(B_THREADS, MINB) k_batch(const BatchRigDev* __
                 case BT_D1: {
                     // up to four consecutive down1 tiles of the rig, one per group of 64 threads
                     const int grp = t / D1_THREADS;
-                    if (grp < tk.pad0)
-                        down1_tile<T>(rg.cams, rg.g, rg.fp, rg.od, rg.d1[tk.idx + grp], rg.refs, rg.d1w, rg.d1cols,
-                                      (Slot*)rg.g0buf, reinterpret_cast<float4*>(reinterpret_cast<char*>(smem) + grp * D1_SMEM),
+                    if (grp < tk.pad0) {
+                        const D1Tile& tl = rg.d1[tk.idx + grp];
+                        down1_tile<T>(rg.cams, rg.g, rg.fp, rg.od, d1_record(tl, rg.cams[tl.cam], rg.refs[tl.ref]), rg.d1w,
+                                      rg.d1cols, (Slot*)rg.g0buf,
+                                      reinterpret_cast<float4*>(reinterpret_cast<char*>(smem) + grp * D1_SMEM),
                                       t % D1_THREADS, 1 + grp);
+                    }
                     break;
                 }
                 case BT_RED:
@@ -3025,7 +3104,9 @@ __global__ void __launch_bounds__(D1_THREADS, D1Cap<CAP>::BLOCKS) k_mr_down1(con
     extern __shared__ float4 smem[];
     const BTask tk = tasks[blockIdx.x];
     const BatchRigDev& rg = rigs[tk.rig];
-    down1_tile<T, CAP>(rg.cams, rg.g, rg.fp, rg.od, task_tile<D1Tile>(tk), rg.refs, rg.d1w, rg.d1cols, (Slot*)rg.g0buf, smem);
+    const D1Tile& tl = task_tile<D1Tile>(tk);
+    down1_tile<T, CAP>(rg.cams, rg.g, rg.fp, rg.od, d1_record(tl, rg.cams[tl.cam], rg.refs[tl.ref]), rg.d1w, rg.d1cols,
+                       (Slot*)rg.g0buf, smem);
 }
 
 template <typename T, typename RS>
