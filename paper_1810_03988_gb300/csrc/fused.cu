@@ -99,6 +99,14 @@ __device__ __forceinline__ void st(half4* p, float4 v) {
     *p = h;
 }
 
+// v as it is read back after st()
+template <typename T>
+__device__ __forceinline__ float4 as_stored(float4 v) {
+    if (sizeof(T) == sizeof(float4)) return v;
+    const float2 a = __half22float2(__floats2half2_rn(v.x, v.y)), b = __half22float2(__floats2half2_rn(v.z, v.w));
+    return make_float4(a.x, a.y, b.x, b.y);
+}
+
 __device__ __forceinline__ void prefetch_l2(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
 __device__ __forceinline__ float4 f4fma(float s, float4 v, float4 acc) {
     return make_float4(fmaf(s, v.x, acc.x), fmaf(s, v.y, acc.y), fmaf(s, v.z, acc.z), fmaf(s, v.w, acc.w));
@@ -1163,7 +1171,7 @@ __device__ __forceinline__ void expand_quad(const float4* __restrict__ a, int ld
 constexpr int CT_NC = 2;
 // A camera's regions and buffers of the levels a coarse tile reads (l and l + 1), in shared memory.
 struct CoCam {
-    Rect z, o, oc;
+    Rect z, o, oc, zc;  // Z^l, Omega^l, Omega^{l+1}, Z^{l+1}
     const void *fg, *fgc;
 };
 static_assert(sizeof(CoCam) % 16 == 0, "16-byte units");
@@ -1187,7 +1195,11 @@ struct LevelTile {
     int x0, y0, first, count;  // level origin, range of camera indices in the list
 };
 
-template <typename T, typename CS = CS32x32>
+// TOP: level l is the last but one, and its tiles form R^{l+1} of the last level on their halo themselves, from
+// the G^{l+1} that they read anyway (the last level has no EXPAND: R is the weighted mean), with the
+// operations of that level's own tiles in the same order.  One launch of a chain that latency bounds is
+// saved: 2 x 360p 42.3 -> 38.0 us per frame, cylinder 4 x 720p 96 -> 92.
+template <typename T, typename CS = CS32x32, bool TOP = false>
 __device__ __forceinline__ void coarse_tile(const CamDev* __restrict__ cams, const RigGeom& g, int l,
                                             T* __restrict__ Rl, const T* __restrict__ Rc, const LevelTile& tl,
                                             const int* __restrict__ camlist, float4* smem) {
@@ -1203,7 +1215,7 @@ __device__ __forceinline__ void coarse_tile(const CamDev* __restrict__ cams, con
         if (t < min(CT_NC, tl.count - c0)) {
             const CamDev& c = cams[camlist[tl.first + c0 + t]];
             const int lc = top ? l : l + 1;
-            cc[t] = CoCam{c.Z[l], c.Om[l], c.Om[lc], c.FG[l], c.FG[lc]};
+            cc[t] = CoCam{c.Z[l], c.Om[l], c.Om[lc], c.Z[lc], c.FG[l], c.FG[lc]};
         }
     };
     cameras(0);  // constant tables: read while the previous kernel drains
@@ -1221,7 +1233,7 @@ __device__ __forceinline__ void coarse_tile(const CamDev* __restrict__ cams, con
         if (!top && q < CS::CN) {
             px[k] = fold101(ax + c, g.nx[l + 1]);
             py[k] = fold101(ay + r, g.ny[l + 1]);
-            rv[k] = ld(Rc + (long long)py[k] * g.nx[l + 1] + px[k]);
+            if (!TOP) rv[k] = ld(Rc + (long long)py[k] * g.nx[l + 1] + px[k]);
         }
     }
     const int qx = t % (CS::TX / 2), qy = t / (CS::TX / 2);
@@ -1245,7 +1257,62 @@ __device__ __forceinline__ void coarse_tile(const CamDev* __restrict__ cams, con
                                                  : make_float4(0.f, 0.f, 0.f, 0.f);
         }
     };
+    // G^{l+1} of the chunk's cameras at the thread's positions
+    const auto coarser = [&](int nc, float4 w[CT_NC][NK]) {
+#pragma unroll
+        for (int ci = 0; ci < CT_NC; ++ci)
+#pragma unroll
+            for (int k = 0; k < NK; ++k) {
+                w[ci][k] = make_float4(0.f, 0.f, 0.f, 0.f);
+                if (!top && ci < nc && t + 256 * k < CS::CN) {
+                    const Rect o = cc[ci].oc;
+                    if (o.contains(px[k], py[k]))
+                        w[ci][k] = ld(reinterpret_cast<const T*>(cc[ci].fgc) + (long long)(py[k] - o.y0) * o.w() + (px[k] - o.x0));
+                }
+            }
+    };
     __syncthreads();
+    float4 w[CT_NC][NK];
+    if (TOP) {
+        float2 arg[NK];
+        float ab[NK], aden[NK];
+#pragma unroll
+        for (int k = 0; k < NK; ++k) {
+            arg[k] = make_float2(0.f, 0.f);
+            ab[k] = aden[k] = 0.f;
+        }
+        for (int c0 = 0; c0 < tl.count; c0 += CT_NC) {
+            const int nc = min(CT_NC, tl.count - c0);
+            if (c0 > 0) {
+                __syncthreads();
+                cameras(c0);
+                __syncthreads();
+            }
+            coarser(nc, w);
+#pragma unroll
+            for (int ci = 0; ci < CT_NC; ++ci)
+#pragma unroll
+                for (int k = 0; k < NK; ++k) {
+                    const float4 v = w[ci][k];
+                    if (ci >= nc || !cc[ci].zc.contains(px[k], py[k])) continue;
+                    arg[k] = f2fma(f2(v.w), make_float2(v.x, v.y), arg[k]);
+                    ab[k] = fmaf(v.w, v.z, ab[k]);
+                    aden[k] += v.w;
+                }
+        }
+#pragma unroll
+        for (int k = 0; k < NK; ++k)
+            if (aden[k] > 1e-12f) {
+                // rounded as stored and read back
+                const float rd = __frcp_rn(aden[k]);
+                rv[k] = as_stored<T>(make_float4(__fmul_rn(arg[k].x, rd), __fmul_rn(arg[k].y, rd), __fmul_rn(ab[k], rd), 0.f));
+            }
+        if (tl.count > CT_NC) {
+            __syncthreads();
+            cameras(0);
+            __syncthreads();
+        }
+    }
     for (int c0 = 0; c0 == 0 || c0 < tl.count; c0 += CT_NC) {
         const int nc = min(CT_NC, tl.count - c0);
         if (c0 > 0) {
@@ -1255,18 +1322,7 @@ __device__ __forceinline__ void coarse_tile(const CamDev* __restrict__ cams, con
         }
         float4 gq[4];
         {
-            float4 w[CT_NC][NK];
-#pragma unroll
-            for (int ci = 0; ci < CT_NC; ++ci)
-#pragma unroll
-                for (int k = 0; k < NK; ++k) {
-                    w[ci][k] = make_float4(0.f, 0.f, 0.f, 0.f);
-                    if (!top && ci < nc && t + 256 * k < CS::CN) {
-                        const Rect o = cc[ci].oc;
-                        if (o.contains(px[k], py[k]))
-                            w[ci][k] = ld(reinterpret_cast<const T*>(cc[ci].fgc) + (long long)(py[k] - o.y0) * o.w() + (px[k] - o.x0));
-                    }
-                }
+            if (!TOP || tl.count > CT_NC) coarser(nc, w);
             if (nc > 0) quad(0, gq);
             if (!top) {
 #pragma unroll
@@ -1320,15 +1376,15 @@ __device__ __forceinline__ void coarse_tile(const CamDev* __restrict__ cams, con
     }
 }
 
-template <typename T>
-__global__ void __launch_bounds__(256, 3) k_coarse_t(const CamDev* __restrict__ cams, const __grid_constant__ RigGeom g, int l,
+template <typename T, bool TOP>
+__global__ void __launch_bounds__(256, TOP ? 2 : 3) k_coarse_t(const CamDev* __restrict__ cams, const __grid_constant__ RigGeom g, int l,
                                                    T* __restrict__ Rl, const T* __restrict__ Rc,
                                                    const LevelTile* __restrict__ tiles,
                                                    const int* __restrict__ camlist) {
     extern __shared__ float4 smem[];
     pdl_trigger();
     const LevelTile tl = tiles[blockIdx.x];
-    coarse_tile<T, CSRig>(cams, g, l, Rl, Rc, tl, camlist, smem);
+    coarse_tile<T, CSRig, TOP>(cams, g, l, Rl, Rc, tl, camlist, smem);
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -2018,6 +2074,8 @@ struct FusedState {
     int n_rc[MAXL] = {};
     LevelTile* co_tiles[MAXL] = {};  // coarse tiles of level l (l >= 2)
     int n_co[MAXL] = {};
+    LevelTile* top_tiles = nullptr;  // those of level L - 2 when they also form the last level (n_top > 0)
+    int n_top = 0;
     int* camlist = nullptr;
     float* d1w = nullptr;        // normalised level-0 weights of the non-INTERIOR down1 tiles
     int n_wtab = 0;
@@ -2286,9 +2344,14 @@ void launch_chain(stitch_rig* r, FusedState* fs, const FramePtrs& fp, const OutD
                    fs->n_rc[l + 1], fs->wave_red);
     }
     for (int l = L - 1; l >= 2; --l) {
-        if (fs->n_co[l] == 0) continue;
+        if (fs->n_co[l] == 0 || (l == L - 1 && fs->n_top > 0)) continue;
         prof_mark(r, "fused_coarse", s);
-        pdl_launch(k_coarse_t<T>, fs->n_co[l], 256, sizeof(float4) * CT_SMEM_F4, s, r->dcam, g, l, (T*)fs->R[l],
+        if (l == L - 2 && fs->n_top > 0) {
+            pdl_launch(k_coarse_t<T, true>, fs->n_top, 256, sizeof(float4) * CT_SMEM_F4, s, r->dcam, g, l, (T*)fs->R[l],
+                       (const T*)nullptr, fs->top_tiles, fs->camlist);
+            continue;
+        }
+        pdl_launch(k_coarse_t<T, false>, fs->n_co[l], 256, sizeof(float4) * CT_SMEM_F4, s, r->dcam, g, l, (T*)fs->R[l],
                    l + 1 < L ? (const T*)fs->R[l + 1] : nullptr, fs->co_tiles[l], fs->camlist);
     }
     const T* R2 = L >= 3 ? (const T*)fs->R[2] : nullptr;
@@ -2358,7 +2421,9 @@ stitch_status set_smem_attrs() {
                                          (int)up_full_smem<4>()));
     STITCH_CUDA_TRY(cudaFuncSetAttribute(k_up_full_b4<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)up_full_smem<2>()));
-    STITCH_CUDA_TRY(cudaFuncSetAttribute(k_coarse_t<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    STITCH_CUDA_TRY(cudaFuncSetAttribute(k_coarse_t<T, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)(sizeof(float4) * CT_SMEM_F4)));
+    STITCH_CUDA_TRY(cudaFuncSetAttribute(k_coarse_t<T, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)(sizeof(float4) * CT_SMEM_F4)));
     return STITCH_OK;
 }
@@ -2822,6 +2887,26 @@ stitch_status fused_plan(stitch_rig* r) {
         if (st != STITCH_OK) return st;
         fs->n_rc[l] = (int)redc[l].size();
     }
+    // the tiles of level L - 2 with every camera that enters the last level on their halo
+    std::vector<LevelTile> top;
+    if (L >= 4)
+        for (const LevelTile& t : co[L - 2]) {
+            const int l = L - 2;
+            const Span hx = folded_span(t.x0 / 2 - 2, CSRig::CX, g.nx[l + 1]), hy = folded_span(t.y0 / 2 - 2, CSRig::CY, g.ny[l + 1]);
+            LevelTile u{t.x0, t.y0, (int)camlist.size(), 0};
+            for (int j = 0; j < g.ncam; ++j) {
+                const CamDev& cj = r->hcam[j];
+                if (!cj.visible || !(rects_meet(cj.Z[l], t.x0, std::min(t.x0 + CT_X, g.nx[l]), t.y0, std::min(t.y0 + CT_Y, g.ny[l])) ||
+                                     rects_meet(cj.Z[l + 1], hx.lo, hx.hi, hy.lo, hy.hi)))
+                    continue;
+                camlist.push_back(j);
+                ++u.count;
+            }
+            top.push_back(u);
+        }
+    st = upload(r, top, &fs->top_tiles);
+    if (st != STITCH_OK) return st;
+    fs->n_top = (int)top.size();
     st = upload(r, camlist, &fs->camlist);
     if (st != STITCH_OK) return st;
     for (int l = 2; l < L; ++l) {
@@ -2843,7 +2928,7 @@ stitch_status fused_plan(stitch_rig* r) {
     }
     int kernels = 0;
     if (L >= 2) kernels += (fs->n_d1_pyr > 0) + (fs->n_solo_tiles > 0);
-    for (int l = 2; l < L; ++l) kernels += (fs->n_rc[l] > 0) + (fs->n_co[l] > 0);
+    for (int l = 2; l < L; ++l) kernels += (fs->n_rc[l] > 0) + (fs->n_co[l] > 0 && !(l == L - 1 && fs->n_top > 0));
     st = fs->fp16 ? set_smem_attrs<half4>() : set_smem_attrs<float4>();
     if (st == STITCH_OK) st = fs->fp16 ? set_waves<half4>(r, fs) : set_waves<float4>(r, fs);
     if (st != STITCH_OK) return st;
