@@ -141,13 +141,15 @@ struct D1Tile {
 };
 
 // A down1 tile with what its camera adds, in one record: a block knows its staging loads after one round
-// trip to memory instead of three (tile, reference, camera).  8 x 4K 742 -> 738 us per frame.
+// trip to memory instead of three (tile, reference, camera).  With the first weights under way before the barrier: 8 x 4K 742 -> 725 us per frame.
 struct __align__(16) D1Rec {
-    D1Tile tl;
+    int cam, k0, j0, flags, fxy, fwh, g0, coltab, pf_fxy, pf_fwh, pf_cw, wsel;  // of the D1Tile
     TileMap tm;
     int ax, ay, W, H;
     float scale;
-    int pad[2];
+    int g1_w;     // G^1 row length
+    int clip;     // outputs inside Omega^1: columns [b0, b1), rows [b2, b3) of the tile, one byte each
+    void* g1;     // where the tile's first G^1 output lies (used only for those inside Omega^1)
 };
 static_assert(sizeof(D1Rec) == 128, "one line");
 
@@ -553,13 +555,13 @@ __device__ __forceinline__ void d1_put(const D1Out<T>& o, int dy, V4 s) {
 // go in pairs (2m, 2m + 1), m = 0 .. 8, with two running sums: on entry to pair m, C holds output
 // row m - 2 (taps 0..3 applied) and B row m - 1 (taps 0, 1); row 2m completes C (stored from m = 2
 // on), moves B on by tap 2 into C and starts row m in B; row 2m + 1 adds tap 3 to C and tap 1 to B.
-// Row 18 completes output row 7.
+// Row 18 completes output row 7.  w01: the weights of rows 0 and 1.
 template <typename T, int MODE, int OUTK, bool ONES>
 __device__ __forceinline__ void d1_sweep(const D1Ctx& x, float4* __restrict__ vcol, const float* __restrict__ wcol,
-                                         float2 nuv, float dqc, const D1Out<T>& o) {
+                                         float2 w01, float2 nuv, float dqc, const D1Out<T>& o) {
     V4 B = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)}, C = B;
     // weights of INTERIOR tiles are all 1; the others are loaded one row pair ahead
-    float we = ONES ? 1.0f : __ldg(wcol), wo = ONES ? 1.0f : __ldg(wcol + D1_SX);
+    float we = ONES ? 1.0f : w01.x, wo = ONES ? 1.0f : w01.y;
     const float* wp = wcol + 2 * D1_SX;        // weights of row 2m + 2
     float4* vp = vcol - 2 * D1_VROW;           // vres row of output m - 2
     D1Out<T> oq = o;
@@ -600,8 +602,7 @@ __device__ __forceinline__ void d1_bar(int id) {
 
 // One down1 tile, worked on by the D1_THREADS threads t = 0 .. 63 that share barrier `bar`.
 template <typename T, int CAP = D1_FOOT>
-__device__ __forceinline__ void down1_tile(const CamDev* __restrict__ cams, const RigGeom& g, const FramePtrs& fp,
-                                           const OutDesc& od, const D1Rec& rec, const float* __restrict__ d1w,
+__device__ __forceinline__ void down1_tile(const RigGeom& g, const FramePtrs& fp, const OutDesc& od, const D1Rec& rec, const float* __restrict__ d1w,
                                            const float4* __restrict__ d1cols,
                                            Slot* __restrict__ g0buf, float4* smem, int t = threadIdx.x, int bar = 0) {
     uint32_t* foot = reinterpret_cast<uint32_t*>(smem);
@@ -610,7 +611,7 @@ __device__ __forceinline__ void down1_tile(const CamDev* __restrict__ cams, cons
     float4* ext = reinterpret_cast<float4*>(reinterpret_cast<char*>(smem) + SM_FOOT + D1_SM_V);  // [19][3]
     float2* rowdy = reinterpret_cast<float2*>(reinterpret_cast<char*>(smem) + SM_FOOT + D1_SM_V + D1_SM_X);
 
-    const D1Tile& tl = rec.tl;
+    const D1Rec& tl = rec;
     const int i = tl.cam;
     const int k0 = tl.k0, j0 = tl.j0;              // level-1 tile origin
     const int vx0 = 2 * k0 - 2, vy0 = 2 * j0 - 2;  // level-0 virtual origin
@@ -679,6 +680,9 @@ __device__ __forceinline__ void down1_tile(const CamDev* __restrict__ cams, cons
     const int mode = staged ? (tl.flags & D1_NOCLAMP ? D1M_STAGED : D1M_CLAMP) : D1M_FRAME;
     const int flags = tl.flags;
     const int X0 = 2 * k0, Y0 = 2 * j0;
+    // the sweep's first weights are on their way before the barrier
+    const float* wcol = x.wt + t + 2;
+    const float2 w01 = act ? make_float2(__ldg(wcol), __ldg(wcol + D1_SX)) : make_float2(0.f, 0.f);
     d1_bar(bar);
     if (act) {
         // sweep thread t takes virtual column t + 2 (the 64 columns of the canvas tile's pixels);
@@ -702,27 +706,26 @@ __device__ __forceinline__ void down1_tile(const CamDev* __restrict__ cams, cons
             o.rows = xo < g.nx[0] ? max(0, min(2 * D1_TY, g.ny[0] - Y0)) : 0;
         }
         float4* vcol = vres + d1_vslot(c);
-        const float* wcol = x.wt + c;
         // the staged mode (nearly every tile) has a sweep per output kind; the rare clamping and
         // frame-reading modes take the kind at run time
         if (mode == D1M_STAGED && (flags & D1_INTERIOR)) {
             switch (o.kind) {
-                case D1O_SLOT: d1_sweep<T, D1M_STAGED, D1O_SLOT, true>(x, vcol, wcol, nuv, dqc, o); break;
-                case D1O_U8: d1_sweep<T, D1M_STAGED, D1O_U8, true>(x, vcol, wcol, nuv, dqc, o); break;
-                case D1O_F32: d1_sweep<T, D1M_STAGED, D1O_F32, true>(x, vcol, wcol, nuv, dqc, o); break;
-                default: d1_sweep<T, D1M_STAGED, D1O_NONE, true>(x, vcol, wcol, nuv, dqc, o); break;
+                case D1O_SLOT: d1_sweep<T, D1M_STAGED, D1O_SLOT, true>(x, vcol, wcol, w01, nuv, dqc, o); break;
+                case D1O_U8: d1_sweep<T, D1M_STAGED, D1O_U8, true>(x, vcol, wcol, w01, nuv, dqc, o); break;
+                case D1O_F32: d1_sweep<T, D1M_STAGED, D1O_F32, true>(x, vcol, wcol, w01, nuv, dqc, o); break;
+                default: d1_sweep<T, D1M_STAGED, D1O_NONE, true>(x, vcol, wcol, w01, nuv, dqc, o); break;
             }
         } else if (mode == D1M_STAGED) {
             switch (o.kind) {
-                case D1O_SLOT: d1_sweep<T, D1M_STAGED, D1O_SLOT, false>(x, vcol, wcol, nuv, dqc, o); break;
-                case D1O_U8: d1_sweep<T, D1M_STAGED, D1O_U8, false>(x, vcol, wcol, nuv, dqc, o); break;
-                case D1O_F32: d1_sweep<T, D1M_STAGED, D1O_F32, false>(x, vcol, wcol, nuv, dqc, o); break;
-                default: d1_sweep<T, D1M_STAGED, D1O_NONE, false>(x, vcol, wcol, nuv, dqc, o); break;
+                case D1O_SLOT: d1_sweep<T, D1M_STAGED, D1O_SLOT, false>(x, vcol, wcol, w01, nuv, dqc, o); break;
+                case D1O_U8: d1_sweep<T, D1M_STAGED, D1O_U8, false>(x, vcol, wcol, w01, nuv, dqc, o); break;
+                case D1O_F32: d1_sweep<T, D1M_STAGED, D1O_F32, false>(x, vcol, wcol, w01, nuv, dqc, o); break;
+                default: d1_sweep<T, D1M_STAGED, D1O_NONE, false>(x, vcol, wcol, w01, nuv, dqc, o); break;
             }
         } else if (mode == D1M_CLAMP) {
-            d1_sweep<T, D1M_CLAMP, D1O_ANY, false>(x, vcol, wcol, nuv, dqc, o);
+            d1_sweep<T, D1M_CLAMP, D1O_ANY, false>(x, vcol, wcol, w01, nuv, dqc, o);
         } else {
-            d1_sweep<T, D1M_FRAME, D1O_ANY, false>(x, vcol, wcol, nuv, dqc, o);
+            d1_sweep<T, D1M_FRAME, D1O_ANY, false>(x, vcol, wcol, w01, nuv, dqc, o);
         }
         if (t < D1_XC * D1_SY && (flags & D1_G1_OUT)) {
             const int r = t / D1_XC, k = t - r * D1_XC, ce = k < 2 ? k : D1_SX - 1;
@@ -750,13 +753,13 @@ __device__ __forceinline__ void down1_tile(const CamDev* __restrict__ cams, cons
     d1_bar(bar);
     // S3 horizontal pass and store of G^1: output (p, jj) takes columns 2p .. 2p+4
     if (act) {
-        const CamDev& ci = cams[i];
-        const Rect o1 = ci.Om[1];
-        T* dst = reinterpret_cast<T*>(ci.FG[1]);
-        const int p = t & 31, kk = k0 + p;
+        T* dst = reinterpret_cast<T*>(rec.g1);
+        const int p = t & 31;
+        const bool in_x = p >= (rec.clip & 0xff) && p < (rec.clip >> 8 & 0xff);
+        const int y0 = rec.clip >> 16 & 0xff, y1 = rec.clip >> 24 & 0xff;
 #pragma unroll
         for (int q = 0; q < D1_TY / 2; ++q) {
-            const int jj = (t >> 5) + 2 * q, j = j0 + jj;
+            const int jj = (t >> 5) + 2 * q;
             const float4* ev = vres + jj * D1_VROW + p;  // columns 2p, 2p+2, 2p+4
             const float4* odp = ev + D1_VODD;           // columns 2p+1, 2p+3
             V4 acc = v4_mul(d1_w(0), v4_of(ev[0]));
@@ -765,7 +768,7 @@ __device__ __forceinline__ void down1_tile(const CamDev* __restrict__ cams, cons
             acc = v4_fma(d1_w(3), v4_of(odp[1]), acc);
             acc = v4_fma(d1_w(4), v4_of(ev[2]), acc);
             // tiles lie on the global grid, so they may start before and end after Omega^1
-            if (o1.contains(kk, j)) st(dst + (long long)(j - o1.y0) * o1.w() + (kk - o1.x0), f4_of(acc));
+            if (in_x && jj >= y0 && jj < y1) st(dst + (long long)jj * rec.g1_w + p, f4_of(acc));
         }
     }
 }
@@ -783,12 +786,19 @@ __device__ __forceinline__ R load_record(const R* __restrict__ p) {
     for (int k = 0; k < (int)(sizeof(R) / 16); ++k) u.w[k] = __ldg(reinterpret_cast<const uint4*>(p) + k);
     return u.r;
 }
-__host__ __device__ inline D1Rec d1_record(const D1Tile& tl, const CamDev& c, const CamRef& ref) {
-    return D1Rec{tl, ref.tm, ref.ax, ref.ay, c.W, c.H, c.gain * (1.0f / 255.0f), {0, 0}};
+// elem: bytes of a G^1 element
+__host__ __device__ inline D1Rec d1_record(const D1Tile& tl, const CamDev& c, const CamRef& ref, size_t elem) {
+    const Rect o = c.Om[1];
+    const auto cut = [](int v, int n) { return (unsigned)(v < 0 ? 0 : v > n ? n : v); };
+    const unsigned clip = cut(o.x0 - tl.k0, D1_TX) | cut(o.x1 - tl.k0, D1_TX) << 8 | cut(o.y0 - tl.j0, D1_TY) << 16 |
+                          cut(o.y1 - tl.j0, D1_TY) << 24;
+    char* g1 = (char*)c.FG[1] + ((long long)(tl.j0 - o.y0) * o.w() + (tl.k0 - o.x0)) * (long long)elem;
+    return D1Rec{tl.cam, tl.k0, tl.j0, tl.flags, tl.fxy, tl.fwh, tl.g0, tl.coltab, tl.pf_fxy, tl.pf_fwh, tl.pf_cw, tl.wsel,
+                 ref.tm, ref.ax, ref.ay, c.W, c.H, c.gain * (1.0f / 255.0f), o.w(), (int)clip, g1};
 }
 
 template <typename T, int CAP>
-__global__ void __launch_bounds__(D1_THREADS, D1Cap<CAP>::BLOCKS) k_down1(const CamDev* __restrict__ cams, RigGeom g,
+__global__ void __launch_bounds__(D1_THREADS, D1Cap<CAP>::BLOCKS) k_down1(RigGeom g,
                                                                         FramePtrs fp, OutDesc od,
                                                                         const D1Rec* __restrict__ recs, int n, int wave,
                                                                         const float* __restrict__ d1w,
@@ -799,7 +809,7 @@ __global__ void __launch_bounds__(D1_THREADS, D1Cap<CAP>::BLOCKS) k_down1(const 
     const D1Rec rec = load_record(recs + blockIdx.x);
     if (threadIdx.x == 0 && blockIdx.x + wave < n) prefetch_l2(recs + blockIdx.x + wave);
     pdl_wait();
-    down1_tile<T, CAP>(cams, g, fp, od, rec, d1w, d1cols, g0buf, smem);
+    down1_tile<T, CAP>(g, fp, od, rec, d1w, d1cols, g0buf, smem);
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -2333,7 +2343,7 @@ void launch_chain(stitch_rig* r, FusedState* fs, const FramePtrs& fp, const OutD
         prof_mark(r, "fused_down1", s);
         const auto k = fs->d1_small ? k_down1<T, D1_FOOT_SMALL> : k_down1<T, D1_FOOT>;
         const size_t smem = fs->d1_small ? D1Cap<D1_FOOT_SMALL>::SMEM : D1_SMEM;
-        stream_launch(early, k, fs->n_d1_pyr, D1_THREADS, smem, s, r->dcam, g, fp, od, fs->d1_recs, fs->n_d1_pyr, fs->wave_d1,
+        stream_launch(early, k, fs->n_d1_pyr, D1_THREADS, smem, s, g, fp, od, fs->d1_recs, fs->n_d1_pyr, fs->wave_d1,
                       fs->d1w, fs->d1cols, (Slot*)fs->g0buf);
     }
     solo();
@@ -2865,7 +2875,7 @@ stitch_status fused_plan(stitch_rig* r) {
     st = upload(r, cols, &fs->d1cols);
     if (st != STITCH_OK) return st;
     std::vector<D1Rec> recs(fs->n_d1_pyr);
-    for (int k = 0; k < fs->n_d1_pyr; ++k) recs[k] = d1_record(d1[k], r->hcam[d1[k].cam], refs[d1[k].ref]);
+    for (int k = 0; k < fs->n_d1_pyr; ++k) recs[k] = d1_record(d1[k], r->hcam[d1[k].cam], refs[d1[k].ref], elem);
     st = upload(r, recs, &fs->d1_recs);
     if (st != STITCH_OK) return st;
     st = upload(r, solo, &fs->solo_tiles);
@@ -3122,7 +3132,7 @@ __global__ void __launch_bounds__(B_THREADS, MINB) k_batch(const BatchRigDev* __
                     const int grp = t / D1_THREADS;
                     if (grp < tk.pad0) {
                         const D1Tile& tl = rg.d1[tk.idx + grp];
-                        down1_tile<T>(rg.cams, rg.g, rg.fp, rg.od, d1_record(tl, rg.cams[tl.cam], rg.refs[tl.ref]), rg.d1w,
+                        down1_tile<T>(rg.g, rg.fp, rg.od, d1_record(tl, rg.cams[tl.cam], rg.refs[tl.ref], sizeof(T)), rg.d1w,
                                       rg.d1cols, (Slot*)rg.g0buf,
                                       reinterpret_cast<float4*>(reinterpret_cast<char*>(smem) + grp * D1_SMEM),
                                       t % D1_THREADS, 1 + grp);
@@ -3190,7 +3200,7 @@ __global__ void __launch_bounds__(D1_THREADS, D1Cap<CAP>::BLOCKS) k_mr_down1(con
     const BTask tk = tasks[blockIdx.x];
     const BatchRigDev& rg = rigs[tk.rig];
     const D1Tile& tl = task_tile<D1Tile>(tk);
-    down1_tile<T, CAP>(rg.cams, rg.g, rg.fp, rg.od, d1_record(tl, rg.cams[tl.cam], rg.refs[tl.ref]), rg.d1w, rg.d1cols,
+    down1_tile<T, CAP>(rg.g, rg.fp, rg.od, d1_record(tl, rg.cams[tl.cam], rg.refs[tl.ref], sizeof(T)), rg.d1w, rg.d1cols,
                        (Slot*)rg.g0buf, smem);
 }
 
