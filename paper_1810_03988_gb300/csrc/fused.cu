@@ -822,7 +822,9 @@ __global__ void __launch_bounds__(D1_THREADS, D1Cap<CAP>::BLOCKS) k_down1(RigGeo
 // (78 per sample and warp, down1: 109).  8 x 4K: the 19 276 down1 tiles that it replaces took 93 us of
 // down1's 373, their 9638 canvas tiles take 70 us here.  Nothing depends on it, so it runs beside the
 // pyramid's launches, whose small levels leave most of the chip idle (launch_all): 815 -> 790 us per frame,
-// 803 when it follows down1 on the same stream; 4 x 1080p (1189 tiles) 210 -> 205.
+// 803 when it follows down1 on the same stream; 4 x 1080p (1189 tiles) 210 -> 205.  Two waves of resident
+// blocks share the tiles (8 x 4K 725 -> 714; 716 with 2.4 waves, 720 with one, 722 with a block per tile): a
+// block that goes on to its next tile does not give its place up to a launch of the chain in between.
 constexpr int SO_FOOT = 3072;  // footprint capacity in texels
 constexpr int SO_BLOCKS = 18;  // resident blocks per SM, bounds the registers (shared memory allows 17)
 // A rig uses it from this many tiles per SM on.  Below, the tiles stay with down1: 5 x 719p (325 tiles,
@@ -840,75 +842,79 @@ static_assert(sizeof(SoloTile) == 144, "nine 16-byte words");
 template <bool F32>
 __global__ void __launch_bounds__(D1_THREADS, SO_BLOCKS) k_solo(const __grid_constant__ RigGeom g,
                                                                 const __grid_constant__ FramePtrs fp, OutDesc od,
-                                                                const SoloTile* __restrict__ tiles,
+                                                                const SoloTile* __restrict__ tiles, int ntiles,
                                                                 const float4* __restrict__ d1cols) {
     __shared__ __align__(16) uint32_t foot[SO_FOOT];
     const int t = threadIdx.x;
     const int lane = t & 31;
-    const SoloTile tl = load_record(tiles + blockIdx.x);
-    D1Ctx x{};
-    x.scale = tl.scale;
-    x.foot = foot;
-    x.fx0 = tl.fxy & 0xffff;
-    x.fy0 = (int)((unsigned)tl.fxy >> 16);
-    x.fw = tl.fwh & 0xffff;
-    x.fh = tl.fwh >> 16;
-    x.S = (x.fw + 3) & ~3;
-    x.maxidx = x.S * (x.fh - 1) - 2;
-    stage_footprint<SO_FOOT>(foot, fp.p[tl.cam], fp.pitch[tl.cam], tl.W, x.fx0, x.fy0, x.fw, x.fh, t);
-    __syncthreads();
-    const int xo = tl.x0 + t, xc = min(xo, g.nx[0] - 1);
-    // 8-bit rows of whole words: a warp's 32 pixels are 24 words; word l holds bytes l % 3 .. of pixel
-    // l + l / 3 and the first of the next one
-    const bool words = !F32 && tl.x0 + U0_TX <= g.nx[0] && word_aligned((const uint8_t*)od.ptr, od.pitch);
-    const int wl = min(lane, 23), wp = wl + wl / 3;
-    const unsigned wsel = wl % 3 == 0 ? 0x4210u : wl % 3 == 1 ? 0x5421u : 0x6542u;
 #pragma unroll 1
-    for (int h = 0; h < 2; ++h) {
-        x.tm = h ? tl.tm[1] : tl.tm[0];
-        const int ax = h ? tl.ax[1] : tl.ax[0], ay = h ? tl.ay[1] : tl.ay[0];
-        x.ibase = 4u * ((unsigned)(x.tm.V0 - x.fy0) * (unsigned)x.S + (unsigned)(x.tm.U0 - x.fx0) -
-                        D1_FLOOR_BITS * ((unsigned)x.S + 1u));
-        float2 nuv;
-        float dqc;
-        if (g.cyl) {
-            const float4 cc = d1cols[(long long)(h ? tl.coltab[1] : tl.coltab[0]) * D1_SX + (xc - tl.x0) + 2];
-            nuv = make_float2(cc.x, cc.y);
-            dqc = cc.z;
-        } else {
-            const float dx = (float)(xc - ax);
-            nuv = make_float2(fmaf(x.tm.pu1, dx, x.tm.pu0), fmaf(x.tm.pv1, dx, x.tm.pv0));
-            dqc = fmaf(x.tm.q1, dx, x.tm.q0);
-        }
-        const int Y = tl.y0 + h * (U0_TY / 2);
-        const int rows = min(U0_TY / 2, g.ny[0] - Y);
-        float2 dy = f2((float)(Y - ay));
-        char* q = (char*)od.ptr + (long long)Y * od.pitch +
-                  (words ? 3LL * (xo - lane) + 4 * lane : (F32 ? 12LL : 3LL) * xo);
-#pragma unroll 2
-        for (int r = 0; r < rows; ++r) {
-            const V4 s = d1_sample<D1M_STAGED>(x, nuv, dqc, dy, 1.0f);
-            dy = f2add(dy, f2(1.0f));
-            const float vr = __saturatef(s.a.x), vg = __saturatef(s.a.y), vb = __saturatef(s.b.x);
-            if (F32) {
-                if (xo < g.nx[0]) {
-                    float* f = reinterpret_cast<float*>(q);
-                    f[0] = vr;
-                    f[1] = vg;
-                    f[2] = vb;
-                }
+    for (int bi = blockIdx.x; bi < ntiles; bi += gridDim.x) {
+        const SoloTile tl = load_record(tiles + bi);
+        D1Ctx x{};
+        x.scale = tl.scale;
+        x.foot = foot;
+        x.fx0 = tl.fxy & 0xffff;
+        x.fy0 = (int)((unsigned)tl.fxy >> 16);
+        x.fw = tl.fwh & 0xffff;
+        x.fh = tl.fwh >> 16;
+        x.S = (x.fw + 3) & ~3;
+        x.maxidx = x.S * (x.fh - 1) - 2;
+        if (bi != blockIdx.x) __syncthreads();
+        stage_footprint<SO_FOOT>(foot, fp.p[tl.cam], fp.pitch[tl.cam], tl.W, x.fx0, x.fy0, x.fw, x.fh, t);
+        __syncthreads();
+        const int xo = tl.x0 + t, xc = min(xo, g.nx[0] - 1);
+        // 8-bit rows of whole words: a warp's 32 pixels are 24 words; word l holds bytes l % 3 .. of pixel
+        // l + l / 3 and the first of the next one
+        const bool words = !F32 && tl.x0 + U0_TX <= g.nx[0] && word_aligned((const uint8_t*)od.ptr, od.pitch);
+        const int wl = min(lane, 23), wp = wl + wl / 3;
+        const unsigned wsel = wl % 3 == 0 ? 0x4210u : wl % 3 == 1 ? 0x5421u : 0x6542u;
+#pragma unroll 1
+        for (int h = 0; h < 2; ++h) {
+            x.tm = h ? tl.tm[1] : tl.tm[0];
+            const int ax = h ? tl.ax[1] : tl.ax[0], ay = h ? tl.ay[1] : tl.ay[0];
+            x.ibase = 4u * ((unsigned)(x.tm.V0 - x.fy0) * (unsigned)x.S + (unsigned)(x.tm.U0 - x.fx0) -
+                            D1_FLOOR_BITS * ((unsigned)x.S + 1u));
+            float2 nuv;
+            float dqc;
+            if (g.cyl) {
+                const float4 cc = d1cols[(long long)(h ? tl.coltab[1] : tl.coltab[0]) * D1_SX + (xc - tl.x0) + 2];
+                nuv = make_float2(cc.x, cc.y);
+                dqc = cc.z;
             } else {
-                const uint32_t px = __byte_perm(__byte_perm(quantize_bits(vr), quantize_bits(vg), 0x0040), quantize_bits(vb), 0x0410);
-                if (words) {
-                    const uint32_t lo = __shfl_sync(~0u, px, wp), hi = __shfl_sync(~0u, px, wp + 1);
-                    if (lane < 24) *reinterpret_cast<uint32_t*>(q) = __byte_perm(lo, hi, wsel);
-                } else if (xo < g.nx[0]) {
-                    q[0] = (char)px;
-                    q[1] = (char)(px >> 8);
-                    q[2] = (char)(px >> 16);
-                }
+                const float dx = (float)(xc - ax);
+                nuv = make_float2(fmaf(x.tm.pu1, dx, x.tm.pu0), fmaf(x.tm.pv1, dx, x.tm.pv0));
+                dqc = fmaf(x.tm.q1, dx, x.tm.q0);
             }
-            q += od.pitch;
+            const int Y = tl.y0 + h * (U0_TY / 2);
+            const int rows = min(U0_TY / 2, g.ny[0] - Y);
+            float2 dy = f2((float)(Y - ay));
+            char* q = (char*)od.ptr + (long long)Y * od.pitch +
+                      (words ? 3LL * (xo - lane) + 4 * lane : (F32 ? 12LL : 3LL) * xo);
+#pragma unroll 2
+            for (int r = 0; r < rows; ++r) {
+                const V4 s = d1_sample<D1M_STAGED>(x, nuv, dqc, dy, 1.0f);
+                dy = f2add(dy, f2(1.0f));
+                const float vr = __saturatef(s.a.x), vg = __saturatef(s.a.y), vb = __saturatef(s.b.x);
+                if (F32) {
+                    if (xo < g.nx[0]) {
+                        float* f = reinterpret_cast<float*>(q);
+                        f[0] = vr;
+                        f[1] = vg;
+                        f[2] = vb;
+                    }
+                } else {
+                    const uint32_t px = __byte_perm(__byte_perm(quantize_bits(vr), quantize_bits(vg), 0x0040), quantize_bits(vb), 0x0410);
+                    if (words) {
+                        const uint32_t lo = __shfl_sync(~0u, px, wp), hi = __shfl_sync(~0u, px, wp + 1);
+                        if (lane < 24) *reinterpret_cast<uint32_t*>(q) = __byte_perm(lo, hi, wsel);
+                    } else if (xo < g.nx[0]) {
+                        q[0] = (char)px;
+                        q[1] = (char)(px >> 8);
+                        q[2] = (char)(px >> 16);
+                    }
+                }
+                q += od.pitch;
+            }
         }
     }
 }
@@ -2074,7 +2080,7 @@ struct FusedState {
     D1Rec* d1_recs = nullptr;
     int n_d1_pyr = 0;            // the first of them: those that the solo kernel does not take
     SoloTile* solo_tiles = nullptr;
-    int n_solo_tiles = 0;
+    int n_solo_tiles = 0, solo_grid = 0;
     // the pyramid chain's stream while the solo kernel runs on the caller's (null: one after the other)
     cudaStream_t chain = nullptr;
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
@@ -2404,7 +2410,7 @@ stitch_status launch_all(stitch_rig* r, FusedState* fs, const FramePtrs& fp, con
         if (fs->n_solo_tiles == 0) return;
         prof_mark(r, "fused_solo", s);
         const auto k = od.is_float ? k_solo<true> : k_solo<false>;
-        k<<<fs->n_solo_tiles, D1_THREADS, 0, s>>>(r->geom, fp, od, fs->solo_tiles, fs->d1cols);
+        k<<<fs->solo_grid, D1_THREADS, 0, s>>>(r->geom, fp, od, fs->solo_tiles, fs->n_solo_tiles, fs->d1cols);
     };
     if (!fs->chain || r->prof) {
         launch_chain<T>(r, fs, fp, od, s, true, solo);
@@ -2930,7 +2936,11 @@ stitch_status fused_plan(stitch_rig* r) {
         fs->n_up[k] = (int)up[k].size();
     }
     if (fs->n_solo_tiles > 0) {
-        int lo = 0, hi = 0;
+        int sms = 0, per = 0, lo = 0, hi = 0;
+        STITCH_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, r->device));
+        STITCH_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, r->desc.out_float ? k_solo<true> : k_solo<false>,
+                                                                      D1_THREADS, 0));
+        fs->solo_grid = std::min(fs->n_solo_tiles, 2 * std::max(per, 1) * std::max(sms, 1));
         STITCH_CUDA_TRY(cudaDeviceGetStreamPriorityRange(&lo, &hi));
         STITCH_CUDA_TRY(cudaStreamCreateWithPriority(&fs->chain, cudaStreamNonBlocking, hi));
         STITCH_CUDA_TRY(cudaEventCreateWithFlags(&fs->ev_fork, cudaEventDisableTiming));
