@@ -301,7 +301,7 @@ __device__ __forceinline__ void mt_schedule(int N, long long* E) {
 
 // A warp per query: an accepted match's place in quality order is the number of accepted matches
 // before it.  It writes the match and its normalised coordinates (x, y, u, v), the latter also in
-// single precision for mt_count.  The last block computes the growth schedule.
+// single precision for the inlier tests.  The last block computes the growth schedule.
 __global__ void __launch_bounds__(256) mt_rank(const int2* best, const int* count_a, int cap,
                                                const int* xy_a, const int* xy_b,
                                                MtState* st, int* matches,
