@@ -1177,6 +1177,34 @@ __device__ __forceinline__ void expand_quad(const float4* __restrict__ a, int ld
     e[3] = odd(ho[1], ho[2]);
 }
 
+// Polyphase EXPAND of four fine samples of one column, rows 4 m .. 4 m + 3, odd: whether the column is.  a
+// points at the coarse sample (row 2 m - 1, the column's own or left one); the row stride is ld.  The
+// operations are expand_quad's, in its order.  A warp's lanes take neighbouring columns, so a 128-bit load
+// of the coarse row covers 17 samples (two to three wavefronts; the quads' lanes take 32 of them, four), and
+// the fine samples of a row are read and written without the quads' two-way bank conflicts.
+__device__ __forceinline__ void expand_col4(const float4* __restrict__ a, int ld, bool odd, V3 e[4]) {
+    const float2 k75 = f2(0.75f), k125 = f2(0.125f), k5 = f2(0.5f);
+    const float ws = odd ? 0.5f : 0.125f;
+    const float4* left = a - (odd ? 0 : 1);
+    V3 h[4];
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+        const V3 c0 = v3_of(left[r * ld]), c1 = v3_of(a[r * ld]), c2 = v3_of(a[r * ld + 1]);
+        h[r].rg = f2mul(f2(ws), f2add(c0.rg, c2.rg));
+        h[r].b = ws * (c0.b + c2.b);
+        if (!odd) {
+            h[r].rg = f2fma(k75, c1.rg, h[r].rg);
+            h[r].b = fmaf(0.75f, c1.b, h[r].b);
+        }
+    }
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+        e[2 * q] = {f2fma(k75, h[q + 1].rg, f2mul(k125, f2add(h[q].rg, h[q + 2].rg))),
+                    fmaf(0.75f, h[q + 1].b, 0.125f * (h[q].b + h[q + 2].b))};
+        e[2 * q + 1] = {f2mul(k5, f2add(h[q + 1].rg, h[q + 2].rg)), 0.5f * (h[q + 1].b + h[q + 2].b)};
+    }
+}
+
 // Tiled coarse level: R^l on a tile of level l (l >= 2), one 2 x 2 quad per thread, cameras in
 // chunks of 2.  Latency bounds it (at most a few waves): the tables are read before the wait for the
 // previous kernel, and every load of the first chunk (R^{l+1}, two cameras' G^{l+1}, the first one's G^l)
@@ -1415,7 +1443,6 @@ constexpr int U1_X = U_TX / 2 + 4, U1_Y = U_TY / 2 + 4;  // 36 x 20
 constexpr int U2_X = U_TX / 4 + 4, U2_Y = U_TY / 4 + 4;  // 20 x 12
 constexpr int U1_N = U1_X * U1_Y, U2_N = U2_X * U2_Y;
 constexpr int U_QUADS0 = (U_TX / 2) * (U_TY / 2);        // 512 level-0 quads
-constexpr int U_QUADS1 = (U1_X / 2) * (U1_Y / 2);        // 180 level-1 quads
 
 // Write a tile's uint8 output staged in shared memory (rows of 3*U_TX bytes): 32-bit stores when
 // the destination rows are 4-byte aligned and the tile is full width, bytes otherwise.
@@ -1535,8 +1562,9 @@ __device__ __forceinline__ void up_prefetch(const CamDev* __restrict__ cams, con
     }
 }
 
-// NB: blended cameras whose level-0 slot loads are in flight at once (1 or 2)
-template <typename T, int NC, int NB = (NC < 2 ? NC : 2)>
+// NB: blended cameras whose level-0 slot loads are in flight at once (1 or 2); COLS: the shape of a thread's
+// level-1 work, see there
+template <typename T, int NC, int NB = (NC < 2 ? NC : 2), bool COLS = false>
 __device__ __forceinline__ void up_full_tile(const CamDev* __restrict__ cams, const RigGeom& g, const FramePtrs& fp,
                                              const OutDesc& od, const T* __restrict__ R2, const UpTile& tl,
                                              const CamRef* __restrict__ refs, const Slot* __restrict__ g0buf,
@@ -1626,9 +1654,21 @@ __device__ __forceinline__ void up_full_tile(const CamDev* __restrict__ cams, co
     }
     if (pf) up_prefetch<T, NC>(cams, *pf, refs, g0buf);  // the tile one resident wave later
     __syncthreads();
-    if (L >= 2 && t < U_QUADS1) {
-        // level 1: R^1 = sum_i a_i (G^1_i + EXPAND(Delta^2_i)), then Delta^1_i = R^1 - G^1_i in place
-        const int qx = t % (U1_X / 2), qy = t / (U1_X / 2);
+    if (L >= 2 && t < U1_N / 4) {
+        // level 1: R^1 = sum_i a_i (G^1_i + EXPAND(Delta^2_i)), then Delta^1_i = R^1 - G^1_i in place; four
+        // rows of a column per thread, or a 2 x 2 quad.  Columns take half the shared-memory wavefronts, but
+        // more registers: 4 x 1080p 187 -> 183 us per frame, cylinder 4 x 720p 91 -> 89.5 with them; at four blocks
+        // per SM (64 registers) they spill, 8 x 4K 714 -> 727, and the batched kernels lose a block.
+        static_assert(U1_N / 4 == (U1_X / 2) * (U1_Y / 2), "as many columns of four as quads");
+        const int tx = t % (COLS ? U1_X : U1_X / 2), ty = t / (COLS ? U1_X : U1_X / 2);
+        const bool odd = tx & 1;
+        const auto at1 = [&](int k) {
+            return COLS ? (4 * ty + k) * U1_X + tx : (2 * ty + (k >> 1)) * U1_X + 2 * tx + (k & 1);
+        };
+        const auto expand = [&](const float4* a, V3 e[4]) {
+            if (COLS) expand_col4(a + 2 * ty * U2_X + (tx >> 1) + 1, U2_X, odd, e);
+            else expand_quad(a, U2_X, tx, ty, e);
+        };
         float2 nrg[4];
         float nb[4], den[4];
 #pragma unroll
@@ -1638,11 +1678,11 @@ __device__ __forceinline__ void up_full_tile(const CamDev* __restrict__ cams, co
         }
         for (int c = 0; c < nc; ++c) {
             V3 e[4] = {v3_zero(), v3_zero(), v3_zero(), v3_zero()};
-            if (L >= 3) expand_quad(d2 + c * U2_N, U2_X, qx, qy, e);
+            if (L >= 3) expand(d2 + c * U2_N, e);
             // outside the camera's Z^1 its weight pyramid is exactly 0, so those terms add nothing
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
-                const float4 gv = d1[c * U1_N + (2 * qy + (k >> 1)) * U1_X + 2 * qx + (k & 1)];
+                const float4 gv = d1[c * U1_N + at1(k)];
                 nrg[k] = f2fma(f2(gv.w), f2add(make_float2(gv.x, gv.y), e[k].rg), nrg[k]);
                 nb[k] = fmaf(gv.w, gv.z + e[k].b, nb[k]);
                 den[k] += gv.w;
@@ -1656,11 +1696,11 @@ __device__ __forceinline__ void up_full_tile(const CamDev* __restrict__ cams, co
             need_plain |= !(den[k] > 1e-12f);
         }
         V3 e[4] = {v3_zero(), v3_zero(), v3_zero(), v3_zero()};
-        if (need_plain && L >= 3) expand_quad(r2s, U2_X, qx, qy, e);
+        if (need_plain && L >= 3) expand(r2s, e);
         for (int c = 0; c < nc; ++c) {
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
-                float4& dv = d1[c * U1_N + (2 * qy + (k >> 1)) * U1_X + 2 * qx + (k & 1)];
+                float4& dv = d1[c * U1_N + at1(k)];
                 const float4 gv = dv;
                 if (den[k] > 1e-12f) {
                     // R^1 rounded before the difference, as every other reader of a collapsed level sees it
@@ -1790,14 +1830,14 @@ __device__ __forceinline__ void up_full_block(const CamDev* __restrict__ cams, c
     if (NCMAX > 2) {
         if (b < ul.n4) {
             const int nb = b + ul.wave;
-            up_full_tile<T, NCMAX, NB>(cams, g, fp, od, R2, ul.t4[b], refs, g0buf, usm, nb < ul.n4 ? ul.t4 + nb : nullptr);
+            up_full_tile<T, NCMAX, NB, (NB > 1)>(cams, g, fp, od, R2, ul.t4[b], refs, g0buf, usm, nb < ul.n4 ? ul.t4 + nb : nullptr);
             return;
         }
         b -= ul.n4;
     }
     if (b < ul.n2) {
         const int nb = b + ul.wave;
-        up_full_tile<T, 2, NB>(cams, g, fp, od, R2, ul.t2[b], refs, g0buf, usm, nb < ul.n2 ? ul.t2 + nb : nullptr);
+        up_full_tile<T, 2, NB, (NB > 1)>(cams, g, fp, od, R2, ul.t2[b], refs, g0buf, usm, nb < ul.n2 ? ul.t2 + nb : nullptr);
         return;
     }
     pdl_wait();
