@@ -556,7 +556,12 @@ __device__ __forceinline__ void d1_put(const D1Out<T>& o, int dy, V4 s) {
 // row m - 2 (taps 0..3 applied) and B row m - 1 (taps 0, 1); row 2m completes C (stored from m = 2
 // on), moves B on by tap 2 into C and starts row m in B; row 2m + 1 adds tap 3 to C and tap 1 to B.
 // Row 18 completes output row 7.  w01: the weights of rows 0 and 1.
-template <typename T, int MODE, int OUTK, bool ONES>
+//
+// ROLLED: row 18 is a last, half pass of the loop instead of a third copy of the sample's code.  With many
+// waves of tiles, warps of different variants share the instruction cache and fetching is the largest
+// stall (2.1 cycles per issue): 8 x 4K 715 -> 692 us per frame, 8 rigs batched 1433 -> 1404.  With few it only takes the overlap of the last
+// two samples: cylinder 4 x 720p 89.5 -> 90.6, so the larger capacity keeps the copy.
+template <typename T, int MODE, int OUTK, bool ONES, bool ROLLED>
 __device__ __forceinline__ void d1_sweep(const D1Ctx& x, float4* __restrict__ vcol, const float* __restrict__ wcol,
                                          float2 w01, float2 nuv, float dqc, const D1Out<T>& o) {
     V4 B = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)}, C = B;
@@ -568,16 +573,20 @@ __device__ __forceinline__ void d1_sweep(const D1Ctx& x, float4* __restrict__ vc
     oq.p -= 2 * o.step;                        // output row 2m - 2
     oq.rows += 2;
 #pragma unroll 1
-    for (int m = 0; m <= D1_TY; ++m) {
+    for (int m = 0; ROLLED || m <= D1_TY; ++m) {
         const float ae = we, ao = wo;
-        if (!ONES) {
+        if (!ONES && m <= D1_TY) {
             we = __ldg(wp);
             wo = __ldg(m < D1_TY ? wp + D1_SX : wp);
         }
         const V4 se = d1_sample<MODE>(x, nuv, dqc, x.rowdy[2 * m], ae);
+        if (ROLLED) {
+            if (m >= 2) *vp = f4_of(v4_fma(d1_w(4), se, C));
+            if (m > D1_TY) return;
+        }
         const V4 so = d1_sample<MODE>(x, nuv, dqc, x.rowdy[2 * m + 1], ao);
         if (m >= 1) d1_put<T, OUTK>(oq, 0, se);
-        if (m >= 2) *vp = f4_of(v4_fma(d1_w(4), se, C));
+        if (!ROLLED && m >= 2) *vp = f4_of(v4_fma(d1_w(4), se, C));
         C = v4_fma(d1_w(2), se, B);
         B = v4_mul(d1_w(0), se);
         if (m >= 1) d1_put<T, OUTK>(oq, 1, so);
@@ -588,7 +597,6 @@ __device__ __forceinline__ void d1_sweep(const D1Ctx& x, float4* __restrict__ vc
         oq.p += 2 * o.step;
         oq.rows -= 2;
     }
-
     const V4 se = d1_sample<MODE>(x, nuv, dqc, x.rowdy[2 * D1_TY + 2], we);
     vcol[(D1_TY - 1) * D1_VROW] = f4_of(v4_fma(d1_w(4), se, C));
 }
@@ -706,26 +714,27 @@ __device__ __forceinline__ void down1_tile(const RigGeom& g, const FramePtrs& fp
             o.rows = xo < g.nx[0] ? max(0, min(2 * D1_TY, g.ny[0] - Y0)) : 0;
         }
         float4* vcol = vres + d1_vslot(c);
+        constexpr bool ROLLED = CAP <= D1_FOOT_SMALL;
         // the staged mode (nearly every tile) has a sweep per output kind; the rare clamping and
         // frame-reading modes take the kind at run time
         if (mode == D1M_STAGED && (flags & D1_INTERIOR)) {
             switch (o.kind) {
-                case D1O_SLOT: d1_sweep<T, D1M_STAGED, D1O_SLOT, true>(x, vcol, wcol, w01, nuv, dqc, o); break;
-                case D1O_U8: d1_sweep<T, D1M_STAGED, D1O_U8, true>(x, vcol, wcol, w01, nuv, dqc, o); break;
-                case D1O_F32: d1_sweep<T, D1M_STAGED, D1O_F32, true>(x, vcol, wcol, w01, nuv, dqc, o); break;
-                default: d1_sweep<T, D1M_STAGED, D1O_NONE, true>(x, vcol, wcol, w01, nuv, dqc, o); break;
+                case D1O_SLOT: d1_sweep<T, D1M_STAGED, D1O_SLOT, true, ROLLED>(x, vcol, wcol, w01, nuv, dqc, o); break;
+                case D1O_U8: d1_sweep<T, D1M_STAGED, D1O_U8, true, ROLLED>(x, vcol, wcol, w01, nuv, dqc, o); break;
+                case D1O_F32: d1_sweep<T, D1M_STAGED, D1O_F32, true, ROLLED>(x, vcol, wcol, w01, nuv, dqc, o); break;
+                default: d1_sweep<T, D1M_STAGED, D1O_NONE, true, ROLLED>(x, vcol, wcol, w01, nuv, dqc, o); break;
             }
         } else if (mode == D1M_STAGED) {
             switch (o.kind) {
-                case D1O_SLOT: d1_sweep<T, D1M_STAGED, D1O_SLOT, false>(x, vcol, wcol, w01, nuv, dqc, o); break;
-                case D1O_U8: d1_sweep<T, D1M_STAGED, D1O_U8, false>(x, vcol, wcol, w01, nuv, dqc, o); break;
-                case D1O_F32: d1_sweep<T, D1M_STAGED, D1O_F32, false>(x, vcol, wcol, w01, nuv, dqc, o); break;
-                default: d1_sweep<T, D1M_STAGED, D1O_NONE, false>(x, vcol, wcol, w01, nuv, dqc, o); break;
+                case D1O_SLOT: d1_sweep<T, D1M_STAGED, D1O_SLOT, false, ROLLED>(x, vcol, wcol, w01, nuv, dqc, o); break;
+                case D1O_U8: d1_sweep<T, D1M_STAGED, D1O_U8, false, ROLLED>(x, vcol, wcol, w01, nuv, dqc, o); break;
+                case D1O_F32: d1_sweep<T, D1M_STAGED, D1O_F32, false, ROLLED>(x, vcol, wcol, w01, nuv, dqc, o); break;
+                default: d1_sweep<T, D1M_STAGED, D1O_NONE, false, ROLLED>(x, vcol, wcol, w01, nuv, dqc, o); break;
             }
         } else if (mode == D1M_CLAMP) {
-            d1_sweep<T, D1M_CLAMP, D1O_ANY, false>(x, vcol, wcol, w01, nuv, dqc, o);
+            d1_sweep<T, D1M_CLAMP, D1O_ANY, false, ROLLED>(x, vcol, wcol, w01, nuv, dqc, o);
         } else {
-            d1_sweep<T, D1M_FRAME, D1O_ANY, false>(x, vcol, wcol, w01, nuv, dqc, o);
+            d1_sweep<T, D1M_FRAME, D1O_ANY, false, ROLLED>(x, vcol, wcol, w01, nuv, dqc, o);
         }
         if (t < D1_XC * D1_SY && (flags & D1_G1_OUT)) {
             const int r = t / D1_XC, k = t - r * D1_XC, ce = k < 2 ? k : D1_SX - 1;
