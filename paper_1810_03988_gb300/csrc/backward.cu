@@ -64,7 +64,7 @@ __device__ __forceinline__ bool gvalid(const Pos& p, const BwMap& m) {
 
 // The sample at p.  The texel values enter as 2^23 + byte, whose differences are those of the bytes,
 // R and G as one pair.
-__device__ __forceinline__ void gsample(const uint8_t* __restrict__ px, long long pitch, const BwMap& m, const Pos& p,
+__device__ __forceinline__ void gsample(const uint8_t* px, long long pitch, const BwMap& m, const Pos& p,
                                         GSample& s) {
     int i0, j0;
     float fx, fy;

@@ -303,7 +303,7 @@ __global__ void __launch_bounds__(D1W_THREADS) k_d1_weights(const CamDev* __rest
 // 16-byte store.  Frames whose base or pitch is not a multiple of 4 bytes are read byte by byte.
 
 template <int CAP>
-__device__ __forceinline__ void stage_footprint(uint32_t* __restrict__ foot, const uint8_t* __restrict__ px,
+__device__ __forceinline__ void stage_footprint(uint32_t* __restrict__ foot, const uint8_t* px,
                                                 long long pitch, int W, int fx0, int fy0, int fw, int fh, int t) {
     const int gpr = (fw + 3) >> 2, ng = gpr * fh;  // groups per row = S / 4
     if (!STITCH_DCHECK(ng <= CAP / 4, 2, ng)) return;
@@ -313,7 +313,7 @@ __device__ __forceinline__ void stage_footprint(uint32_t* __restrict__ foot, con
             uint32_t w = 0u;
             if (u < fw) {
                 const uint8_t* src = px + (long long)(fy0 + rr) * pitch + 3 * (fx0 + u);
-                w = (uint32_t)__ldg(src) | ((uint32_t)__ldg(src + 1) << 8) | ((uint32_t)__ldg(src + 2) << 16);
+                w = (uint32_t)__ldca(src) | ((uint32_t)__ldca(src + 1) << 8) | ((uint32_t)__ldca(src + 2) << 16);
             }
             foot[q] = w;
         }
@@ -341,15 +341,15 @@ __device__ __forceinline__ void stage_footprint(uint32_t* __restrict__ foot, con
                 const uint8_t* src = px + (long long)(fy0 + rr) * pitch + 3 * u0;
                 if (u0 + 4 <= W) {
                     const uint32_t* s32 = reinterpret_cast<const uint32_t*>(src);
-                    w[k][0] = __ldg(s32);
-                    w[k][1] = __ldg(s32 + 1);
-                    w[k][2] = __ldg(s32 + 2);
+                    w[k][0] = __ldca(s32);
+                    w[k][1] = __ldca(s32 + 1);
+                    w[k][2] = __ldca(s32 + 2);
                 } else {
                     // the image's last texels: only the bytes of texels < W exist
                     const int nb = 3 * (W - u0);
 #pragma unroll
                     for (int j = 0; j < 12; ++j)
-                        if (j < nb) w[k][j >> 2] |= (uint32_t)__ldg(src + j) << (8 * (j & 3));
+                        if (j < nb) w[k][j >> 2] |= (uint32_t)__ldca(src + j) << (8 * (j & 3));
                 }
             }
         }
@@ -1254,7 +1254,7 @@ struct LevelTile {
 // saved: 2 x 360p 42.3 -> 38.0 us per frame, cylinder 4 x 720p 96 -> 92.
 template <typename T, typename CS = CS32x32, bool TOP = false>
 __device__ __forceinline__ void coarse_tile(const CamDev* __restrict__ cams, const RigGeom& g, int l,
-                                            T* __restrict__ Rl, const T* __restrict__ Rc, const LevelTile& tl,
+                                            T* __restrict__ Rl, const T* Rc, const LevelTile& tl,
                                             const int* __restrict__ camlist, float4* smem) {
     float4* rc = smem;                                                   // [CS::CN] R^{l+1}
     float4 (*gc)[CS::CN] = reinterpret_cast<float4 (*)[CS::CN]>(rc + CS::CN);  // [CT_NC][CS::CN] R^{l+1} - G^{l+1}
@@ -1431,7 +1431,7 @@ __device__ __forceinline__ void coarse_tile(const CamDev* __restrict__ cams, con
 
 template <typename T, bool TOP>
 __global__ void __launch_bounds__(256, TOP ? 2 : 3) k_coarse_t(const CamDev* __restrict__ cams, const __grid_constant__ RigGeom g, int l,
-                                                   T* __restrict__ Rl, const T* __restrict__ Rc,
+                                                   T* __restrict__ Rl, const T* Rc,
                                                    const LevelTile* __restrict__ tiles,
                                                    const int* __restrict__ camlist) {
     extern __shared__ float4 smem[];
@@ -1548,7 +1548,7 @@ struct UpCams {
 // (one 128-byte line per thread and pass) and their G^1 rows inside Omega^1.
 template <typename T, int NC>
 __device__ __forceinline__ void up_prefetch(const CamDev* __restrict__ cams, const UpTile& tn,
-                                            const CamRef* __restrict__ refs, const Slot* __restrict__ g0buf) {
+                                            const CamRef* __restrict__ refs, const Slot* g0buf) {
     const int nc = min(tn.count, NC);
     const int a1x = tn.x0 / 2 - 2, a1y = tn.y0 / 2 - 2;
     for (int c = 0; c < nc; ++c) {
@@ -1575,8 +1575,8 @@ __device__ __forceinline__ void up_prefetch(const CamDev* __restrict__ cams, con
 // level-1 work, see there
 template <typename T, int NC, int NB = (NC < 2 ? NC : 2), bool COLS = false>
 __device__ __forceinline__ void up_full_tile(const CamDev* __restrict__ cams, const RigGeom& g, const FramePtrs& fp,
-                                             const OutDesc& od, const T* __restrict__ R2, const UpTile& tl,
-                                             const CamRef* __restrict__ refs, const Slot* __restrict__ g0buf,
+                                             const OutDesc& od, const T* R2, const UpTile& tl,
+                                             const CamRef* __restrict__ refs, const Slot* g0buf,
                                              float4* usm, const UpTile* pf = nullptr) {
     float4* d1 = usm;                // [NC][U1_N]: G^1 of each camera, then R^1 - G^1
     float4* d2 = d1 + NC * U1_N;     // [NC][U2_N]: G^2 of each camera, then R^2 - G^2
@@ -1832,8 +1832,8 @@ struct UpLaunch {
 // NCMAX: the most cameras a tile of this launch has (2 or 4)
 template <typename T, int NCMAX, int NB>
 __device__ __forceinline__ void up_full_block(const CamDev* __restrict__ cams, const RigGeom& g, const FramePtrs& fp,
-                                              const OutDesc& od, const T* __restrict__ R2, const UpLaunch& ul,
-                                              const CamRef* __restrict__ refs, const Slot* __restrict__ g0buf, float4* usm) {
+                                              const OutDesc& od, const T* R2, const UpLaunch& ul,
+                                              const CamRef* __restrict__ refs, const Slot* g0buf, float4* usm) {
     int b = blockIdx.x;
     pdl_trigger();
     if (NCMAX > 2) {
@@ -1859,16 +1859,16 @@ __device__ __forceinline__ void up_full_block(const CamDev* __restrict__ cams, c
 template <typename T, int NCMAX>
 __global__ void __launch_bounds__(U_THREADS, 3) k_up_full(const CamDev* __restrict__ cams, const __grid_constant__ RigGeom g,
                                                            const __grid_constant__ FramePtrs fp, OutDesc od,
-                                                           const T* __restrict__ R2, const __grid_constant__ UpLaunch ul,
-                                                           const CamRef* __restrict__ refs, const Slot* __restrict__ g0buf) {
+                                                           const T* R2, const __grid_constant__ UpLaunch ul,
+                                                           const CamRef* __restrict__ refs, const Slot* g0buf) {
     extern __shared__ float4 usm[];
     up_full_block<T, NCMAX, 2>(cams, g, fp, od, R2, ul, refs, g0buf, usm);
 }
 template <typename T>
 __global__ void __launch_bounds__(U_THREADS, 4) k_up_full_b4(const CamDev* __restrict__ cams, const __grid_constant__ RigGeom g,
                                                               const __grid_constant__ FramePtrs fp, OutDesc od,
-                                                              const T* __restrict__ R2, const __grid_constant__ UpLaunch ul,
-                                                              const CamRef* __restrict__ refs, const Slot* __restrict__ g0buf) {
+                                                              const T* R2, const __grid_constant__ UpLaunch ul,
+                                                              const CamRef* __restrict__ refs, const Slot* g0buf) {
     extern __shared__ float4 usm[];
     up_full_block<T, 2, 1>(cams, g, fp, od, R2, ul, refs, g0buf, usm);
 }
@@ -1913,7 +1913,7 @@ __device__ __forceinline__ float3 expand_smem(const float4* __restrict__ a, int 
 
 template <typename T>
 __device__ __forceinline__ void up_general_tile(const CamDev* __restrict__ cams, const RigGeom& g, const FramePtrs& fp,
-                                                const OutDesc& od, const T* __restrict__ R2, const UpTile& tl,
+                                                const OutDesc& od, const T* R2, const UpTile& tl,
                                                 const CamRef* __restrict__ refs, float4* smem) {
     float4* g1 = smem;                   // [UG1_N]
     float4* g2 = g1 + UG1_N;             // [UG2_X * UG2_Y]
@@ -2109,7 +2109,7 @@ constexpr int UG_SMEM_F4 = 2 * UG1_N + 2 * UG2_X * UG2_Y;
 
 template <typename T>
 __global__ void __launch_bounds__(U_THREADS) k_up_general(const CamDev* __restrict__ cams, RigGeom g, FramePtrs fp,
-                                                           OutDesc od, const T* __restrict__ R2,
+                                                           OutDesc od, const T* R2,
                                                            const UpTile* __restrict__ tiles,
                                                            const CamRef* __restrict__ refs) {
     __shared__ float4 smem[UG_SMEM_F4];

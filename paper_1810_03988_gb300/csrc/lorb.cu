@@ -129,9 +129,9 @@ __global__ void __launch_bounds__(256, 5) lorb_detect(const uint8_t* frame, long
             for (int k = 0; k < 4; ++k) {
                 const int y = min(by - 4 + 3 * st + k, H - 1);
                 const unsigned* q = reinterpret_cast<const unsigned*>(frame + (long long)y * pitch + 3LL * gx0);
-                v[k][0] = __ldg(q);
-                v[k][1] = __ldg(q + 1);
-                v[k][2] = __ldg(q + 2);
+                v[k][0] = __ldca(q);
+                v[k][1] = __ldca(q + 1);
+                v[k][2] = __ldca(q + 2);
             }
 #pragma unroll
             for (int k = 0; k < 4; ++k) gray4(v[k][0], v[k][1], v[k][2], g[k]);
@@ -142,7 +142,7 @@ __global__ void __launch_bounds__(256, 5) lorb_detect(const uint8_t* frame, long
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
                     const uint8_t* q = row + 3LL * min(gx0 + i, W - 1);
-                    g[k][i] = gray_of(__ldg(q), __ldg(q + 1), __ldg(q + 2));
+                    g[k][i] = gray_of(__ldca(q), __ldca(q + 1), __ldca(q + 2));
                 }
             }
         }
@@ -575,7 +575,7 @@ __global__ void __launch_bounds__(256) lorb_rank_brief(const uint8_t* frame, lon
                 for (int q = t; q < RB_P * (RB_W / 4); q += 256) {
                     const int r = q / (RB_W / 4), j = q - r * (RB_W / 4);
                     const unsigned* p = reinterpret_cast<const unsigned*>(p0 - off + (long long)r * pitch + 12 * j);
-                    const unsigned v0 = __ldg(p), v1 = __ldg(p + 1), v2 = __ldg(p + 2), v3 = off ? __ldg(p + 3) : 0u;
+                    const unsigned v0 = __ldca(p), v1 = __ldca(p + 1), v2 = __ldca(p + 2), v3 = off ? __ldca(p + 3) : 0u;
                     const unsigned a = __funnelshift_r(v0, v1, 8 * off), b = __funnelshift_r(v1, v2, 8 * off),
                                    c = __funnelshift_r(v2, v3, 8 * off);
                     unsigned o[4];
@@ -586,7 +586,7 @@ __global__ void __launch_bounds__(256) lorb_rank_brief(const uint8_t* frame, lon
                 for (int q = t; q < RB_P * RB_P; q += 256) {
                     const int r = q / RB_P, c = q - r * RB_P;
                     const uint8_t* p = p0 + (long long)r * pitch + 3 * c;
-                    g[r * RB_W + c] = (uint8_t)gray_of(__ldg(p), __ldg(p + 1), __ldg(p + 2));
+                    g[r * RB_W + c] = (uint8_t)gray_of(__ldca(p), __ldca(p + 1), __ldca(p + 2));
                 }
             }
             __syncthreads();

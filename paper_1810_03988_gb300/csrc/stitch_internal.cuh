@@ -85,9 +85,11 @@ constexpr uint32_t kGuardWord = 0x7FC0DEADu;
 // blocks waits for the previous one's completion (pdl_wait) before its first access to anything but
 // the rig's constant tables, and before it returns.  As that kernel has waited for the one before
 // it, all earlier work of the stream is complete behind pdl_wait.  Without the launch attribute both
-// are no-ops.  Data that the previous kernels wrote is read by plain or __ldcg loads from pointers that
-// are not `const __restrict__`: loads of the read-only path are promised not to change while the kernel
-// runs, which begins before pdl_wait, and the compiler may move them above it.
+// are no-ops.  The read-only path (__ldg, and loads through `const __restrict__` pointers, which the
+// compiler may turn into it) is for the rig's constant tables: its loads are promised not to change while
+// the kernel runs, which begins before pdl_wait, and the compiler may move them above it.  What earlier
+// work wrote is read by plain loads, __ldca or __ldcg, through pointers without `__restrict__`: the
+// previous kernels' results, and the frames, whose producer may be a kernel that triggers early itself.
 
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
@@ -320,18 +322,18 @@ __device__ __forceinline__ float byte_f23(uint32_t w, uint32_t j) {
 struct Texels {
     uint32_t t00, t01, t10, t11;
 };
-__device__ __forceinline__ Texels load_texels(const uint8_t* __restrict__ a, const uint8_t* __restrict__ b, int i0, int W,
+__device__ __forceinline__ Texels load_texels(const uint8_t* a, const uint8_t* b, int i0, int W,
                                               bool words) {
     Texels o;
     const int off = (3 * i0) & 3;
     if (words && 3 * i0 - off + 12 <= 3 * W) {
         const uint32_t* wa = reinterpret_cast<const uint32_t*>(a - off);
         const uint32_t* wb = reinterpret_cast<const uint32_t*>(b - off);
-        const uint32_t a0 = __ldg(wa), a1 = __ldg(wa + 1), b0 = __ldg(wb), b1 = __ldg(wb + 1);
+        const uint32_t a0 = __ldca(wa), a1 = __ldca(wa + 1), b0 = __ldca(wb), b1 = __ldca(wb + 1);
         uint32_t a2 = 0u, b2 = 0u;
         if (off == 3) {
-            a2 = __ldg(wa + 2);
-            b2 = __ldg(wb + 2);
+            a2 = __ldca(wa + 2);
+            b2 = __ldca(wb + 2);
         }
         o.t00 = __funnelshift_r(a0, a1, 8 * off);
         o.t01 = __byte_perm(o.t00, __funnelshift_r(a1, a2, 8 * off), 0x0543);
@@ -340,7 +342,7 @@ __device__ __forceinline__ Texels load_texels(const uint8_t* __restrict__ a, con
     } else {
         const int di = i0 + 1 < W ? 3 : 0;
         auto texel = [](const uint8_t* p) {
-            return (uint32_t)__ldg(p) | (uint32_t)__ldg(p + 1) << 8 | (uint32_t)__ldg(p + 2) << 16;
+            return (uint32_t)__ldca(p) | (uint32_t)__ldca(p + 1) << 8 | (uint32_t)__ldca(p + 2) << 16;
         };
         o.t00 = texel(a);
         o.t01 = texel(a + di);
@@ -354,7 +356,7 @@ __device__ __forceinline__ bool word_aligned(const uint8_t* px, long long pitch)
 }
 
 // Bilinear RGB sample of an 8-bit frame of width W, scaled by `scale` (= gain / 255).
-__device__ __forceinline__ float3 bilinear_rgb(const uint8_t* __restrict__ px, long long pitch, int W, const Tap& t,
+__device__ __forceinline__ float3 bilinear_rgb(const uint8_t* px, long long pitch, int W, const Tap& t,
                                                float scale) {
     const Texels q = load_texels(px + (long long)t.j0 * pitch + 3 * t.i0, px + (long long)t.j1 * pitch + 3 * t.i0, t.i0, W,
                                  word_aligned(px, pitch));
@@ -462,7 +464,7 @@ __device__ __forceinline__ float weight_of(const Pos& p, float Wm, float Hm) {
 }
 
 // Bilinear RGB sample with clamped coordinates, scaled by `scale` (= gain / 255).
-__device__ __forceinline__ float3 sample_rgb(const uint8_t* __restrict__ px, long long pitch, const Pos& p, int W,
+__device__ __forceinline__ float3 sample_rgb(const uint8_t* px, long long pitch, const Pos& p, int W,
                                              int H, float scale) {
     int i0, j0;
     float fx, fy;
@@ -479,8 +481,8 @@ __device__ __forceinline__ float3 sample_rgb(const uint8_t* __restrict__ px, lon
     float3 o;
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-        const float p00 = u8_to_f(__ldg(a + c)), p01 = u8_to_f(__ldg(a + di + c));
-        const float p10 = u8_to_f(__ldg(b + c)), p11 = u8_to_f(__ldg(b + di + c));
+        const float p00 = u8_to_f(__ldca(a + c)), p01 = u8_to_f(__ldca(a + di + c));
+        const float p10 = u8_to_f(__ldca(b + c)), p11 = u8_to_f(__ldca(b + di + c));
         const float top = fmaf(fx, p01 - p00, p00);
         const float bot = fmaf(fx, p11 - p10, p10);
         const float v = fmaf(fy, bot - top, top) * scale;
@@ -490,15 +492,15 @@ __device__ __forceinline__ float3 sample_rgb(const uint8_t* __restrict__ px, lon
 }
 
 // Bilinear RGB sample of a position known to lie in [0, W-1) x [0, H-1) (no clamping needed).
-__device__ __forceinline__ float3 sample_rgb_inside(const uint8_t* __restrict__ px, long long pitch, const Pos& p,
+__device__ __forceinline__ float3 sample_rgb_inside(const uint8_t* px, long long pitch, const Pos& p,
                                                     float scale) {
     const uint8_t* a = px + (long long)p.iv * pitch + 3 * p.iu;
     const uint8_t* b = a + pitch;
     float3 o;
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-        const float p00 = u8_to_f(__ldg(a + c)), p01 = u8_to_f(__ldg(a + 3 + c));
-        const float p10 = u8_to_f(__ldg(b + c)), p11 = u8_to_f(__ldg(b + 3 + c));
+        const float p00 = u8_to_f(__ldca(a + c)), p01 = u8_to_f(__ldca(a + 3 + c));
+        const float p10 = u8_to_f(__ldca(b + c)), p11 = u8_to_f(__ldca(b + 3 + c));
         const float top = fmaf(p.fu, p01 - p00, p00);
         const float bot = fmaf(p.fu, p11 - p10, p10);
         const float v = fmaf(p.fv, bot - top, top) * scale;
