@@ -2387,37 +2387,41 @@ void plan_coarse_tiles(const stitch_rig* r, const std::vector<UpTile>* up, int t
     }
 }
 
-// The launches of the pyramid: down1, REDUCE, coarse and canvas tiles.  solo() follows down1.  early: the
-// first launch may start while the stream's previous kernel drains (nothing but kernels lies between).
+// The launches of the pyramid: down1, REDUCE, coarse and canvas tiles.  solo() follows down1.  early: whether
+// the first of them, whichever that is, may start while the stream's previous kernel drains.
 template <typename T, typename Solo>
 void launch_chain(stitch_rig* r, FusedState* fs, const FramePtrs& fp, const OutDesc& od, cudaStream_t s, bool early,
                   const Solo& solo) {
     const RigGeom& g = r->geom;
     const int L = g.levels;
+    const auto put = [&](auto kernel, dim3 grid, int block, size_t smem, const auto&... args) {
+        stream_launch(early, kernel, grid, block, smem, s, args...);
+        early = true;
+    };
     if (L >= 2 && fs->n_d1_pyr > 0) {
         prof_mark(r, "fused_down1", s);
         const auto k = fs->d1_small ? k_down1<T, D1_FOOT_SMALL> : k_down1<T, D1_FOOT>;
         const size_t smem = fs->d1_small ? D1Cap<D1_FOOT_SMALL>::SMEM : D1_SMEM;
-        stream_launch(early, k, fs->n_d1_pyr, D1_THREADS, smem, s, g, fp, od, fs->d1_recs, fs->n_d1_pyr, fs->wave_d1,
-                      fs->d1w, fs->d1cols, (Slot*)fs->g0buf);
+        put(k, fs->n_d1_pyr, D1_THREADS, smem, g, fp, od, fs->d1_recs, fs->n_d1_pyr, fs->wave_d1, fs->d1w, fs->d1cols,
+            (Slot*)fs->g0buf);
     }
     solo();
     for (int l = 1; l + 1 < L; ++l) {
         if (fs->n_rc[l + 1] == 0) continue;
         prof_mark(r, "fused_reduce", s);
-        pdl_launch(k_reduce_t<T>, fs->n_rc[l + 1], RC_THREADS, RC_SMEM, s, r->dcam, g, l, fs->rc_tiles[l + 1],
-                   fs->n_rc[l + 1], fs->wave_red);
+        put(k_reduce_t<T>, fs->n_rc[l + 1], RC_THREADS, RC_SMEM, r->dcam, g, l, fs->rc_tiles[l + 1], fs->n_rc[l + 1],
+            fs->wave_red);
     }
     for (int l = L - 1; l >= 2; --l) {
         if (fs->n_co[l] == 0 || (l == L - 1 && fs->n_top > 0)) continue;
         prof_mark(r, "fused_coarse", s);
         if (l == L - 2 && fs->n_top > 0) {
-            pdl_launch(k_coarse_t<T, true>, fs->n_top, 256, sizeof(float4) * CT_SMEM_F4, s, r->dcam, g, l, (T*)fs->R[l],
-                       (const T*)nullptr, fs->top_tiles, fs->camlist);
+            put(k_coarse_t<T, true>, fs->n_top, 256, sizeof(float4) * CT_SMEM_F4, r->dcam, g, l, (T*)fs->R[l],
+                (const T*)nullptr, fs->top_tiles, fs->camlist);
             continue;
         }
-        pdl_launch(k_coarse_t<T, false>, fs->n_co[l], 256, sizeof(float4) * CT_SMEM_F4, s, r->dcam, g, l, (T*)fs->R[l],
-                   l + 1 < L ? (const T*)fs->R[l + 1] : nullptr, fs->co_tiles[l], fs->camlist);
+        put(k_coarse_t<T, false>, fs->n_co[l], 256, sizeof(float4) * CT_SMEM_F4, r->dcam, g, l, (T*)fs->R[l],
+            l + 1 < L ? (const T*)fs->R[l + 1] : nullptr, fs->co_tiles[l], fs->camlist);
     }
     const T* R2 = L >= 3 ? (const T*)fs->R[2] : nullptr;
     const Slot* g0 = (const Slot*)fs->g0buf;
@@ -2427,25 +2431,24 @@ void launch_chain(stitch_rig* r, FusedState* fs, const FramePtrs& fp, const OutD
         // many waves of tiles with at most 2 cameras, four blocks per SM; the others three
         prof_mark(r, "fused_up_full", s);
         ul.n4 = 0;
-        pdl_launch(k_up_full_b4<T>, n2 + ns, U_THREADS, up_full_smem<2>(), s, r->dcam, g, fp, od, R2, ul, fs->refs, g0);
+        put(k_up_full_b4<T>, n2 + ns, U_THREADS, up_full_smem<2>(), r->dcam, g, fp, od, R2, ul, fs->refs, g0);
         if (n4) {
             prof_mark(r, "fused_up_full4", s);
             ul.n4 = n4;
             ul.n2 = 0;
-            pdl_launch(k_up_full<T, 4>, n4, U_THREADS, up_full_smem<4>(), s, r->dcam, g, fp, od, R2, ul, fs->refs, g0);
+            put(k_up_full<T, 4>, n4, U_THREADS, up_full_smem<4>(), r->dcam, g, fp, od, R2, ul, fs->refs, g0);
         }
     } else if (n2 + n4) {
         prof_mark(r, "fused_up_full", s);
-        if (n4) pdl_launch(k_up_full<T, 4>, n4 + n2 + ns, U_THREADS, up_full_smem<4>(), s, r->dcam, g, fp, od, R2, ul, fs->refs, g0);
-        else pdl_launch(k_up_full<T, 2>, n2 + ns, U_THREADS, up_full_smem<2>(), s, r->dcam, g, fp, od, R2, ul, fs->refs, g0);
+        if (n4) put(k_up_full<T, 4>, n4 + n2 + ns, U_THREADS, up_full_smem<4>(), r->dcam, g, fp, od, R2, ul, fs->refs, g0);
+        else put(k_up_full<T, 2>, n2 + ns, U_THREADS, up_full_smem<2>(), r->dcam, g, fp, od, R2, ul, fs->refs, g0);
     } else if (ns) {
         prof_mark(r, "fused_up_simple", s);
-        pdl_launch(k_up_simple, ns, U_THREADS, 0, s, r->dcam, g, fp, od, fs->up_tiles[UP_SIMPLE], fs->refs);
+        put(k_up_simple, ns, U_THREADS, 0, r->dcam, g, fp, od, fs->up_tiles[UP_SIMPLE], fs->refs);
     }
     if (fs->n_up[UP_GENERAL]) {
         prof_mark(r, "fused_up_general", s);
-        pdl_launch(k_up_general<T>, fs->n_up[UP_GENERAL], U_THREADS, 0, s, r->dcam, g, fp, od, R2, fs->up_tiles[UP_GENERAL],
-                   fs->refs);
+        put(k_up_general<T>, fs->n_up[UP_GENERAL], U_THREADS, 0, r->dcam, g, fp, od, R2, fs->up_tiles[UP_GENERAL], fs->refs);
     }
 }
 
@@ -2454,7 +2457,7 @@ void launch_chain(stitch_rig* r, FusedState* fs, const FramePtrs& fp, const OutD
 // Both begin after all earlier work of the caller's stream and are joined to it.  Under the profiler's marks
 // everything runs on the caller's stream.
 template <typename T>
-stitch_status launch_all(stitch_rig* r, FusedState* fs, const FramePtrs& fp, const OutDesc& od, cudaStream_t s) {
+stitch_status launch_all(stitch_rig* r, FusedState* fs, const FramePtrs& fp, const OutDesc& od, cudaStream_t s, bool early) {
     const auto solo = [&] {
         if (fs->n_solo_tiles == 0) return;
         prof_mark(r, "fused_solo", s);
@@ -2462,7 +2465,7 @@ stitch_status launch_all(stitch_rig* r, FusedState* fs, const FramePtrs& fp, con
         k<<<fs->solo_grid, D1_THREADS, 0, s>>>(r->geom, fp, od, fs->solo_tiles, fs->n_solo_tiles, fs->d1cols);
     };
     if (!fs->chain || r->prof) {
-        launch_chain<T>(r, fs, fp, od, s, true, solo);
+        launch_chain<T>(r, fs, fp, od, s, early, solo);
         return launch_status();
     }
     STITCH_CUDA_TRY(cudaEventRecord(fs->ev_fork, s));
@@ -3009,10 +3012,10 @@ stitch_status fused_plan(stitch_rig* r) {
     return STITCH_OK;
 }
 
-stitch_status fused_frames(stitch_rig* r, const FramePtrs& fp, const OutDesc& od, cudaStream_t s) {
+stitch_status fused_frames(stitch_rig* r, const FramePtrs& fp, const OutDesc& od, cudaStream_t s, bool early) {
     FusedState* fs = (FusedState*)r->fused;
     if (!fs) return STITCH_EINVAL;
-    return fs->fp16 ? launch_all<half4>(r, fs, fp, od, s) : launch_all<float4>(r, fs, fp, od, s);
+    return fs->fp16 ? launch_all<half4>(r, fs, fp, od, s, early) : launch_all<float4>(r, fs, fp, od, s, early);
 }
 
 stitch_status fused_precompute(stitch_rig* r) {
@@ -3600,7 +3603,7 @@ stitch_status b_launch_streams(BatchState* b, cudaStream_t s) {
     for (int k = 0; k < b->n; ++k) {
         stitch_rig* r = b->rigs[k];
         STITCH_CUDA_TRY(cudaStreamWaitEvent(b->rs[k], b->fork, 0));
-        const stitch_status st = launch_all<T>(r, (FusedState*)r->fused, b->h_rigs[k].fp, b->h_rigs[k].od, b->rs[k]);
+        const stitch_status st = launch_all<T>(r, (FusedState*)r->fused, b->h_rigs[k].fp, b->h_rigs[k].od, b->rs[k], false);
         if (st != STITCH_OK) return st;
         STITCH_CUDA_TRY(cudaEventRecord(b->rdone[k], b->rs[k]));
         STITCH_CUDA_TRY(cudaStreamWaitEvent(s, b->rdone[k], 0));

@@ -120,7 +120,7 @@ extern "C" stitch_status stitch_frames_host_async(stitch_rig* r, const uint8_t* 
         // stitch: after the upload and after call k-2's download read this slot's canvas
         ok(cudaStreamWaitEvent(p->s_comp, sl.in_done, 0));
         ok(cudaStreamWaitEvent(p->s_comp, sl.out_done, 0));
-        if (st == STITCH_OK) st = stitch_frames(r, dframes, dpitch, sl.out, (int64_t)row, p->s_comp);
+        if (st == STITCH_OK) st = rig_frames(r, dframes, dpitch, sl.out, (int64_t)row, p->s_comp, false);
         ok(cudaEventRecord(sl.comp_done, p->s_comp));
         // download, and the caller's stream waits for it
         ok(cudaStreamWaitEvent(p->s_out, sl.comp_done, 0));

@@ -298,9 +298,13 @@ stitch_status plain_plan(stitch_rig* r) {
     return STITCH_OK;
 }
 
-stitch_status plain_frames(stitch_rig* r, const FramePtrs& fp, const OutDesc& od, cudaStream_t s) {
+stitch_status plain_frames(stitch_rig* r, const FramePtrs& fp, const OutDesc& od, cudaStream_t s, bool early) {
     const RigGeom& g = r->geom;
     const dim3 blk(BX, BY);
+    const auto put = [&](auto kernel, dim3 grid, const auto&... args) {
+        stream_launch(early, kernel, grid, blk, 0, s, args...);
+        early = true;
+    };
     for (int l = 0; l < g.levels; ++l) {
         int n;
         const CamGrid cg = cam_grid(r, l, &n);
@@ -309,15 +313,15 @@ stitch_status plain_frames(stitch_rig* r, const FramePtrs& fp, const OutDesc& od
         if (l == 0) {
             auto warp = g.cyl ? (g.seam ? k_plain_warp<true, true> : k_plain_warp<true, false>)
                               : (g.seam ? k_plain_warp<false, true> : k_plain_warp<false, false>);
-            pdl_launch(warp, n, blk, 0, s, r->dcam, g.ncam, cg, fp, g, std::max(r->sms, 1));
+            put(warp, n, r->dcam, g.ncam, cg, fp, g, std::max(r->sms, 1));
         } else {
-            pdl_launch(k_plain_reduce, n, blk, 0, s, r->dcam, g.ncam, l - 1, cg, g);
+            put(k_plain_reduce, n, r->dcam, g.ncam, l - 1, cg, g);
         }
     }
     for (int l = g.levels - 1; l >= 0; --l) {
         prof_mark(r, "plain_level", s);
         const dim3 grid((g.nx[l] + BX - 1) / BX, (g.ny[l] + BY - 1) / BY);
-        pdl_launch(k_plain_level, grid, blk, 0, s, r->dcam, l, g, r->Bl[l], l + 1 < g.levels ? r->Bl[l + 1] : nullptr, od);
+        put(k_plain_level, grid, r->dcam, l, g, r->Bl[l], l + 1 < g.levels ? r->Bl[l + 1] : nullptr, od);
     }
     return launch_status();
 }

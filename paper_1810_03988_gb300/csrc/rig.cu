@@ -427,6 +427,13 @@ stitch_status stitch_rig_get_camera(const stitch_rig* r, int32_t index, double* 
 
 stitch_status stitch_frames(stitch_rig* r, const uint8_t* const* frames, const int64_t* pitches, void* out,
                             int64_t out_pitch, void* stream) {
+    return rig_frames(r, frames, pitches, out, out_pitch, (cudaStream_t)stream, true);
+}
+
+}  // extern "C"
+
+stitch_status rig_frames(stitch_rig* r, const uint8_t* const* frames, const int64_t* pitches, void* out, int64_t out_pitch,
+                         cudaStream_t s, bool early) {
     if (!r || !out) return STITCH_EINVAL;
     const long long row = (long long)r->geom.nx[0] * (r->desc.out_float ? 12 : 3);
     if (out_pitch < row) return STITCH_EINVAL;
@@ -435,11 +442,12 @@ stitch_status stitch_frames(stitch_rig* r, const uint8_t* const* frames, const i
     DeviceGuard dg(r->device);
     if (!dg.ok) return STITCH_ECUDA;
     OutDesc od{out, out_pitch, r->desc.out_float};
-    cudaStream_t s = (cudaStream_t)stream;
-    stitch_status st = r->desc.path == STITCH_PATH_PLAIN ? plain_frames(r, fp, od, s) : fused_frames(r, fp, od, s);
+    const stitch_status st = r->desc.path == STITCH_PATH_PLAIN ? plain_frames(r, fp, od, s, early) : fused_frames(r, fp, od, s, early);
     prof_mark(r, nullptr, s);
     return st;
 }
+
+extern "C" {
 
 stitch_status stitch_frames_host(stitch_rig* r, const uint8_t* const* host_frames, const int64_t* pitches,
                                  void* host_out, int64_t out_pitch, void* stream) {
@@ -472,7 +480,7 @@ stitch_status stitch_frames_host(stitch_rig* r, const uint8_t* const* host_frame
         r->stage_out = nullptr;
         return STITCH_ENOMEM;
     }
-    stitch_status st = stitch_frames(r, dframes, dpitch, r->stage_out, row, stream);
+    stitch_status st = rig_frames(r, dframes, dpitch, r->stage_out, row, s, false);
     if (st != STITCH_OK) return st;
     STITCH_CUDA_TRY(cudaMemcpy2DAsync(host_out, (size_t)out_pitch, r->stage_out, (size_t)row, (size_t)row,
                                       r->geom.ny[0], cudaMemcpyDeviceToHost, s));

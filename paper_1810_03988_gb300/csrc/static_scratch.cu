@@ -168,5 +168,5 @@ extern "C" stitch_status stitch_frames_static(const stitch_rig_desc* desc, const
         cudaDeviceGetAttribute(&r.sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
         return STITCH_ECUDA;
     OutDesc od{out, out_pitch, desc->out_float};
-    return plain_frames(&r, fp, od, s);
+    return plain_frames(&r, fp, od, s, true);
 }

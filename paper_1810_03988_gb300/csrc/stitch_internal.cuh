@@ -94,7 +94,10 @@ constexpr uint32_t kGuardWord = 0x7FC0DEADu;
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
-// stream_launch: with the attribute (early) or without it
+// stream_launch: with the attribute (early) or without it.  The attribute relaxes a launch's dependency on
+// the stream's previous kernel only, so a call on the caller's stream begins with it whatever the caller
+// queued before.  Where the library itself has just queued an event wait or a copy, the first launch goes
+// without: there is no kernel for it to overlap with.
 template <typename... P, typename... A>
 inline void stream_launch(bool early, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
                           const A&... args) {
@@ -640,9 +643,12 @@ void* rig_alloc(stitch_rig* r, size_t bytes);
 
 // Path entry points (one translation unit each).
 stitch_status plain_plan(stitch_rig* r);
-stitch_status plain_frames(stitch_rig* r, const FramePtrs& fp, const OutDesc& od, cudaStream_t s);
+stitch_status plain_frames(stitch_rig* r, const FramePtrs& fp, const OutDesc& od, cudaStream_t s, bool early);
 stitch_status fused_plan(stitch_rig* r);
-stitch_status fused_frames(stitch_rig* r, const FramePtrs& fp, const OutDesc& od, cudaStream_t s);
+stitch_status fused_frames(stitch_rig* r, const FramePtrs& fp, const OutDesc& od, cudaStream_t s, bool early);
+// stitch_frames with the choice whether its first launch carries the programmatic attribute (stream_launch)
+stitch_status rig_frames(stitch_rig* r, const uint8_t* const* frames, const int64_t* pitches, void* out, int64_t out_pitch,
+                         cudaStream_t s, bool early);
 void fused_release(stitch_rig* r);
 void fused_tile_counts(const stitch_rig* r, int counts[8]);
 stitch_status backward_plan(stitch_rig* r);

@@ -1,0 +1,88 @@
+"""What the library's host side hands the GPU, call by call, on a CUDA runtime that only takes notes."""
+import ctypes
+
+import numpy as np
+import pytest
+
+import synth
+from tests.fake_lib import FakeLib, Launch
+
+
+class _Camera:
+    def __init__(self, width, height, H, gain=1.0):
+        self.width, self.height, self.H, self.gain = width, height, H, gain
+
+
+@pytest.fixture(scope="module")
+def fake(tmp_path_factory):
+    return FakeLib(tmp_path_factory.mktemp("fake"))
+
+
+def _shift(x, y):
+    return np.array([[1.0, 0.0, x], [0.0, 1.0, y], [0.0, 0.0, 1.0]])
+
+
+def _apart():
+    """Two cameras far apart: solo canvas tiles (more than 4 per SM) and empty ones between, nothing blended."""
+    return [_Camera(1600, 1400, _shift(-20.0, -20.0)), _Camera(1600, 1400, _shift(2200.0, -20.0))], 3776, 1344
+
+
+def _two():
+    cfg = synth.config_2cam(scale=0.25)
+    return cfg.cameras, cfg.canvas_w, cfg.canvas_h
+
+
+def _stitch(fake, rig, cams, cw, ch, entry="stitch_frames", stream=None, elem=3):
+    fp, pt = fake.frame_args(cams)
+    out = ctypes.create_string_buffer(cw * ch * elem)
+    fake.log()
+    assert getattr(fake.lib, entry)(rig, fp, pt, out, cw * elem, stream) == 0
+    return fake.log()
+
+
+def _first_after_waits(log):
+    """Per stream, the launches whose predecessor on the stream is an event wait."""
+    last, out = {}, []
+    for e in log:
+        if isinstance(e, Launch):
+            if last.get(e.stream) == "wait":
+                out.append(e)
+            last[e.stream] = "launch"
+        elif e[0] == "wait":
+            last[int(e[1])] = "wait"
+    return out
+
+
+@pytest.mark.parametrize("entry", ["stitch_frames", "stitch_frames_host_async", "batch"])
+@pytest.mark.parametrize("path", ["fused", "plain"])
+@pytest.mark.parametrize("scene", [_apart, _two])
+def test_no_launch_that_follows_an_event_wait_is_programmatic(fake, entry, path, scene, monkeypatch):
+    if path == "plain" and entry == "batch":
+        pytest.skip("a batch takes fused rigs")
+    cams, cw, ch = scene()
+    rig = fake.rig(cams, cw, ch, 3, path=path)
+    if entry == "batch":
+        monkeypatch.setenv("STITCH_TUNE", "streams")
+        batch = ctypes.c_void_p()
+        assert fake.lib.stitch_batch_create((ctypes.c_void_p * 1)(rig), 1, ctypes.byref(batch)) == 0
+        fp, pt = fake.frame_args(cams)
+        out = ctypes.create_string_buffer(cw * ch * 3)
+        args = ((ctypes.c_void_p * 1)(ctypes.addressof(fp)), (ctypes.c_void_p * 1)(ctypes.addressof(pt)),
+                (ctypes.c_void_p * 1)(ctypes.addressof(out)), (ctypes.c_int64 * 1)(3 * cw))
+        for _ in range(2):  # the first call times the schedules
+            fake.log()
+            assert fake.lib.stitch_batch_frames(batch, *args, None) == 0
+        log = fake.log()
+        fake.lib.stitch_batch_destroy(batch)
+    else:
+        log = _stitch(fake, rig, cams, cw, ch, entry)
+    launches = [e for e in log if isinstance(e, Launch)]
+    forked = any("k_solo" in e.kernel for e in launches)
+    assert forked == (scene is _apart and path == "fused")
+    after = _first_after_waits(log)
+    assert (len(after) > 0) == (forked or entry != "stitch_frames")
+    assert not [e for e in after if e.early], after
+    # the launches behind them overlap, and so does the first one on the caller's stream
+    chain = [e for e in launches if "k_solo" not in e.kernel and e not in after]
+    assert all(e.early for e in chain), chain
+    fake.lib.stitch_rig_destroy(rig)
