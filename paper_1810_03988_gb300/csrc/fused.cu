@@ -829,15 +829,18 @@ __global__ void __launch_bounds__(D1_THREADS, D1Cap<CAP>::BLOCKS) k_down1(RigGeo
 // of both halves staged at once, and twice the resident warps (48 registers, 12 KB).  Each half keeps the
 // anchor of its down1 tile, so the samples are bit-identical to down1's.  Instruction issue bounds it
 // (78 per sample and warp, down1: 109).  8 x 4K: the 19 276 down1 tiles that it replaces took 93 us of
-// down1's 373, their 9638 canvas tiles take 70 us here.  Nothing depends on it, so it runs beside the
-// pyramid's launches, whose small levels leave most of the chip idle (launch_all): 815 -> 790 us per frame,
-// 803 when it follows down1 on the same stream; 4 x 1080p (1189 tiles) 210 -> 205.  Two waves of resident
-// blocks share the tiles (8 x 4K 725 -> 714; 716 with 2.4 waves, 720 with one, 722 with a block per tile): a
-// block that goes on to its next tile does not give its place up to a launch of the chain in between.
+// down1's 373, their 9638 canvas tiles take 69 us here: 667 us per frame, 714 without this kernel; 4 x 1080p
+// (1189 tiles) 180 and 183.  Two waves of resident blocks share the tiles: a block per tile takes 74 us.
+//
+// It is launched behind down1 on the caller's stream, without the programmatic attribute, and does not
+// trigger: with pdl_trigger at its start the whole 8 x 4K frame takes 716 us (4 x 1080p 192), its own time
+// being the same, and with the attribute and pdl_wait alone 4 x 1080p takes 184.  Beside the pyramid's
+// launches, which then ran on a second stream of the highest priority, 8 x 4K took 695 us (4 x 1080p 184, 8
+// rigs batched 1405 against 1350), as the fork and the join cost more than the overlap gave.
 constexpr int SO_FOOT = 3072;  // footprint capacity in texels
 constexpr int SO_BLOCKS = 18;  // resident blocks per SM, bounds the registers (shared memory allows 17)
 // A rig uses it from this many tiles per SM on.  Below, the tiles stay with down1: 5 x 719p (325 tiles,
-// 2 per SM) takes 131 us either way, and a second stream only costs.
+// 2 per SM) takes 117 us with down1 and 137 with this kernel, 4 x 1080p (8 per SM) 183 and 180.
 constexpr int SO_MIN_PER_SM = 4;
 struct __align__(16) SoloTile {
     int cam, x0, y0, fxy, fwh, W;
@@ -2130,9 +2133,6 @@ struct FusedState {
     int n_d1_pyr = 0;            // the first of them: those that the solo kernel does not take
     SoloTile* solo_tiles = nullptr;
     int n_solo_tiles = 0, solo_grid = 0;
-    // the pyramid chain's stream while the solo kernel runs on the caller's (null: one after the other)
-    cudaStream_t chain = nullptr;
-    cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
     Tile* red_tiles[MAXL] = {};  // tiles producing level l (l >= 2), RSRig shape (the batched schedules)
     int n_red[MAXL] = {};
     Tile* rc_tiles[MAXL] = {};   // the same levels in the column-sweep kernel's 64 x 8 tiles (stitch_frames)
@@ -2387,11 +2387,10 @@ void plan_coarse_tiles(const stitch_rig* r, const std::vector<UpTile>* up, int t
     }
 }
 
-// The launches of the pyramid: down1, REDUCE, coarse and canvas tiles.  solo() follows down1.  early: whether
-// the first of them, whichever that is, may start while the stream's previous kernel drains.
-template <typename T, typename Solo>
-void launch_chain(stitch_rig* r, FusedState* fs, const FramePtrs& fp, const OutDesc& od, cudaStream_t s, bool early,
-                  const Solo& solo) {
+// The launches of a call: down1, solo, REDUCE, coarse and canvas tiles.  early: whether the first of them,
+// whichever that is, may start while the stream's previous kernel drains.
+template <typename T>
+stitch_status launch_all(stitch_rig* r, FusedState* fs, const FramePtrs& fp, const OutDesc& od, cudaStream_t s, bool early) {
     const RigGeom& g = r->geom;
     const int L = g.levels;
     const auto put = [&](auto kernel, dim3 grid, int block, size_t smem, const auto&... args) {
@@ -2405,7 +2404,12 @@ void launch_chain(stitch_rig* r, FusedState* fs, const FramePtrs& fp, const OutD
         put(k, fs->n_d1_pyr, D1_THREADS, smem, g, fp, od, fs->d1_recs, fs->n_d1_pyr, fs->wave_d1, fs->d1w, fs->d1cols,
             (Slot*)fs->g0buf);
     }
-    solo();
+    if (fs->n_solo_tiles > 0) {
+        prof_mark(r, "fused_solo", s);
+        stream_launch(false, od.is_float ? k_solo<true> : k_solo<false>, fs->solo_grid, D1_THREADS, 0, s, g, fp, od,
+                      fs->solo_tiles, fs->n_solo_tiles, fs->d1cols);
+        early = true;
+    }
     for (int l = 1; l + 1 < L; ++l) {
         if (fs->n_rc[l + 1] == 0) continue;
         prof_mark(r, "fused_reduce", s);
@@ -2450,31 +2454,7 @@ void launch_chain(stitch_rig* r, FusedState* fs, const FramePtrs& fp, const OutD
         prof_mark(r, "fused_up_general", s);
         put(k_up_general<T>, fs->n_up[UP_GENERAL], U_THREADS, 0, r->dcam, g, fp, od, R2, fs->up_tiles[UP_GENERAL], fs->refs);
     }
-}
-
-// With a solo kernel, the pyramid's chain runs on the rig's own stream of the highest priority and the solo
-// kernel on the caller's: it is launched once down1 is, and its blocks take the room that the chain leaves.
-// Both begin after all earlier work of the caller's stream and are joined to it.  Under the profiler's marks
-// everything runs on the caller's stream.
-template <typename T>
-stitch_status launch_all(stitch_rig* r, FusedState* fs, const FramePtrs& fp, const OutDesc& od, cudaStream_t s, bool early) {
-    const auto solo = [&] {
-        if (fs->n_solo_tiles == 0) return;
-        prof_mark(r, "fused_solo", s);
-        const auto k = od.is_float ? k_solo<true> : k_solo<false>;
-        k<<<fs->solo_grid, D1_THREADS, 0, s>>>(r->geom, fp, od, fs->solo_tiles, fs->n_solo_tiles, fs->d1cols);
-    };
-    if (!fs->chain || r->prof) {
-        launch_chain<T>(r, fs, fp, od, s, early, solo);
-        return launch_status();
-    }
-    STITCH_CUDA_TRY(cudaEventRecord(fs->ev_fork, s));
-    STITCH_CUDA_TRY(cudaStreamWaitEvent(fs->chain, fs->ev_fork, 0));
-    launch_chain<T>(r, fs, fp, od, fs->chain, false, solo);
-    const stitch_status st = launch_status();
-    STITCH_CUDA_TRY(cudaEventRecord(fs->ev_join, fs->chain));
-    STITCH_CUDA_TRY(cudaStreamWaitEvent(s, fs->ev_join, 0));
-    return st;
+    return launch_status();
 }
 
 template <typename T>
@@ -2988,15 +2968,11 @@ stitch_status fused_plan(stitch_rig* r) {
         fs->n_up[k] = (int)up[k].size();
     }
     if (fs->n_solo_tiles > 0) {
-        int sms = 0, per = 0, lo = 0, hi = 0;
+        int sms = 0, per = 0;
         STITCH_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, r->device));
         STITCH_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, r->desc.out_float ? k_solo<true> : k_solo<false>,
                                                                       D1_THREADS, 0));
         fs->solo_grid = std::min(fs->n_solo_tiles, 2 * std::max(per, 1) * std::max(sms, 1));
-        STITCH_CUDA_TRY(cudaDeviceGetStreamPriorityRange(&lo, &hi));
-        STITCH_CUDA_TRY(cudaStreamCreateWithPriority(&fs->chain, cudaStreamNonBlocking, hi));
-        STITCH_CUDA_TRY(cudaEventCreateWithFlags(&fs->ev_fork, cudaEventDisableTiming));
-        STITCH_CUDA_TRY(cudaEventCreateWithFlags(&fs->ev_join, cudaEventDisableTiming));
     }
     int kernels = 0;
     if (L >= 2) kernels += (fs->n_d1_pyr > 0) + (fs->n_solo_tiles > 0);
@@ -3033,11 +3009,6 @@ stitch_status fused_precompute(stitch_rig* r) {
 }
 
 void fused_release(stitch_rig* r) {
-    if (FusedState* fs = (FusedState*)r->fused) {
-        if (fs->chain) cudaStreamDestroy(fs->chain);
-        if (fs->ev_fork) cudaEventDestroy(fs->ev_fork);
-        if (fs->ev_join) cudaEventDestroy(fs->ev_join);
-    }
     delete (FusedState*)r->fused;
     r->fused = nullptr;
 }

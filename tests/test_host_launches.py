@@ -77,12 +77,25 @@ def test_no_launch_that_follows_an_event_wait_is_programmatic(fake, entry, path,
     else:
         log = _stitch(fake, rig, cams, cw, ch, entry)
     launches = [e for e in log if isinstance(e, Launch)]
-    forked = any("k_solo" in e.kernel for e in launches)
-    assert forked == (scene is _apart and path == "fused")
+    assert any("k_solo" in e.kernel for e in launches) == (scene is _apart and path == "fused")
     after = _first_after_waits(log)
-    assert (len(after) > 0) == (forked or entry != "stitch_frames")
+    assert (len(after) > 0) == (entry != "stitch_frames")
     assert not [e for e in after if e.early], after
     # the launches behind them overlap, and so does the first one on the caller's stream
     chain = [e for e in launches if "k_solo" not in e.kernel and e not in after]
     assert all(e.early for e in chain), chain
+    fake.lib.stitch_rig_destroy(rig)
+
+
+@pytest.mark.parametrize("priority", [0, -3])
+@pytest.mark.parametrize("scene", [_apart, _two])
+def test_a_call_runs_on_the_caller_s_stream_at_its_priority(fake, scene, priority):
+    cams, cw, ch = scene()
+    streams = fake.lib.fake_streams()
+    rig = fake.rig(cams, cw, ch, 3)
+    assert fake.lib.fake_streams() == streams, "a rig has no stream of its own"
+    stream = fake.lib.fake_stream(priority)
+    launches = [e for e in _stitch(fake, rig, cams, cw, ch, stream=stream) if isinstance(e, Launch)]
+    assert len(launches) > 3
+    assert len({e.stream for e in launches}) == 1 and {e.priority for e in launches} == {priority}, launches
     fake.lib.stitch_rig_destroy(rig)
