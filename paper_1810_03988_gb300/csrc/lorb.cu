@@ -64,8 +64,9 @@ __device__ __forceinline__ int lorb_bin(long long r) {
     return 16 * e + m;
 }
 
-// Counters of a call, zero between calls but for n2 (lorb_prune's last block clears them): survivors,
-// finished lorb_prune blocks, pruned candidates, survivors per response bin.
+// Counters of a call, zero between calls but for n2 (lorb_prune's last block clears them; after a sequence
+// that a refused launch cut short, the next call does): survivors, finished lorb_prune blocks, pruned
+// candidates, survivors per response bin.
 struct LorbCount {
     int n, done, n2, pad;
     int hist[LORB_BINS];
@@ -616,6 +617,7 @@ struct stitch_lorb {
     Cand* cand = nullptr;
     Cand* cand2 = nullptr;  // the pruned candidates
     LorbCount* cnt = nullptr;
+    bool stale = false;  // a refused launch left counts behind: the next call clears them
 };
 
 static void lorb_free(stitch_lorb* c) {
@@ -717,6 +719,14 @@ extern "C" stitch_status stitch_lorb_detect(stitch_lorb* c, const uint8_t* frame
     auto ok = [&](cudaError_t e) {
         if (e != cudaSuccess && st == STITCH_OK) st = STITCH_ECUDA;
     };
+    bool keep = false;
+    if (c->stale) {
+        // while the stream is captured the clearing is part of the graph: the next call clears too
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        ok(cudaStreamIsCapturing(s, &cap));
+        keep = cap != cudaStreamCaptureStatusNone;
+        ok(cudaMemsetAsync(c->cnt, 0, offsetof(LorbCount, pat), s));
+    }
     if (ar.n > 0) {
         // tiles over the candidates' box, owned pixels starting at a column 1 modulo 4
         const int ox = 1 + ((bx0 - 1) & ~3), oy = by0;
@@ -732,6 +742,7 @@ extern "C" stitch_status stitch_lorb_detect(stitch_lorb* c, const uint8_t* frame
     pdl_launch(lorb_rank_brief, std::min(2 * params->max_points + 64, 1216), 256, 0, s, frame, pitch, width, c->cand2, c->cnt,
                count, xy, reinterpret_cast<long long*>(resp), reinterpret_cast<unsigned*>(desc));
     ok(cudaGetLastError());
+    c->stale = keep || st != STITCH_OK;
     if (prev >= 0 && prev != c->device) cudaSetDevice(prev);
     return st;
 }

@@ -99,3 +99,34 @@ def test_a_call_runs_on_the_caller_s_stream_at_its_priority(fake, scene, priorit
     assert len(launches) > 3
     assert len({e.stream for e in launches}) == 1 and {e.priority for e in launches} == {priority}, launches
     fake.lib.stitch_rig_destroy(rig)
+
+
+def test_lorb_counts_are_cleared_after_a_refused_launch(fake):
+    """The counters of a detection are cleared by its own kernels; a sequence that a refused launch cuts
+    short leaves that to the next call."""
+    from paper_1810_03988_gb300 import stitch
+    W, H, N = 64, 64, 8
+    ctx = ctypes.c_void_p()
+    assert fake.lib.stitch_lorb_create(W, H, N, 0, ctypes.byref(ctx)) == 0
+    frame, out = ctypes.create_string_buffer(3 * W * H), [ctypes.create_string_buffer(64 * N) for _ in range(4)]
+    areas, pattern = (ctypes.c_int32 * 4)(0, 0, W, H), (ctypes.c_int8 * 1024)()
+
+    def detect():
+        fake.log()
+        st = fake.lib.stitch_lorb_detect(ctx, frame, W, H, 3 * W, areas, 1, ctypes.byref(stitch.stitch_lorb_params(20, 0, N)),
+                                         pattern, *out, None)
+        log = fake.log()
+        return st, [e[2] for e in log if e[0] == "memset"], [e.kernel for e in log if isinstance(e, Launch)]
+
+    st, cleared, kernels = detect()
+    assert st == 0 and not cleared and len(kernels) == 3
+    for refused in (1, 2):  # behind lorb_detect, behind lorb_prune
+        fake.lib.fake_refuse(refused)
+        st, cleared, kernels = detect()
+        assert st == stitch.STITCH_ECUDA and not cleared and len(kernels) == 2
+        st, cleared, kernels = detect()
+        assert st == 0 and len(kernels) == 3
+        assert len(cleared) == 1 and int(cleared[0]) >= 4 * (4 + 1024), "the counters and the histogram"
+        st, cleared, _ = detect()
+        assert st == 0 and not cleared
+    fake.lib.stitch_lorb_destroy(ctx)
