@@ -3597,7 +3597,7 @@ std::string b_cache_key(const BatchState* b) {
     cudaDeviceProp prop;
     if (cudaGetDeviceProperties(&prop, b->device) != cudaSuccess) return std::string();
     uint64_t h = 1469598103934665603ull;
-    const char tag[] = "libstitch batch schedule 2";
+    const char tag[] = "libstitch batch schedule 3";  // another number whenever a timed kernel or launch changes
     h = fnv1a(h, tag, sizeof(tag));
     h = fnv1a(h, &b->n, sizeof(b->n));
     for (const stitch_rig* r : b->rigs) {

@@ -1,5 +1,6 @@
 """What the library's host side hands the GPU, call by call, on a CUDA runtime that only takes notes."""
 import ctypes
+import struct
 
 import numpy as np
 import pytest
@@ -130,3 +131,45 @@ def test_lorb_counts_are_cleared_after_a_refused_launch(fake):
         st, cleared, _ = detect()
         assert st == 0 and not cleared
     fake.lib.stitch_lorb_destroy(ctx)
+
+
+def test_schedules_timed_with_earlier_kernels_are_timed_again(fake, monkeypatch, tmp_path):
+    """The tuning cache's key changes with the kernels that the tuner times: a line stored by a library with
+    earlier ones (key version 2) is not taken, a line stored by this one is."""
+    cams, cw, ch = _two()
+    rig = fake.rig(cams, cw, ch, 3)
+    blob = b"libstitch batch schedule %d\0" + struct.pack("<i", 1)
+    blob += struct.pack("<9i", len(cams), cw, ch, 3, 0, 0, 0, 0, 0) + struct.pack("<3d", 0.0, 0.0, 0.0)
+    for c in cams:
+        blob += struct.pack("<ii", c.width, c.height) + np.asarray(c.H, np.float64).tobytes() + struct.pack("<f", c.gain)
+
+    def line(version, mode):
+        h = 1469598103934665603
+        for byte in blob % version:
+            h = (h ^ byte) * 1099511628211 % 2 ** 64
+        return '{"key": "fake|152|%016x", "mode": "%s", "order": 1, "variant": 1, "chunk": 4, "shape": 0, "ms": 1.0}\n' % (h, mode)
+
+    cache = tmp_path / "tune"
+    monkeypatch.setenv("STITCH_TUNE_CACHE", str(cache))
+    monkeypatch.delenv("STITCH_TUNE", raising=False)
+
+    def from_cache():
+        batch = ctypes.c_void_p()
+        assert fake.lib.stitch_batch_create((ctypes.c_void_p * 1)(rig), 1, ctypes.byref(batch)) == 0
+        fp, pt = fake.frame_args(cams)
+        out = ctypes.create_string_buffer(cw * ch * 3)
+        args = ((ctypes.c_void_p * 1)(ctypes.addressof(fp)), (ctypes.c_void_p * 1)(ctypes.addressof(pt)),
+                (ctypes.c_void_p * 1)(ctypes.addressof(out)), (ctypes.c_int64 * 1)(3 * cw))
+        assert fake.lib.stitch_batch_frames(batch, *args, None) == 0
+        order = ctypes.c_int32()
+        assert fake.lib.stitch_batch_get_schedule(batch, ctypes.byref(order), None, None) == 0
+        fake.lib.stitch_batch_destroy(batch)
+        return bool(order.value >> 24 & 1)
+
+    cache.write_text(line(2, "streams"))
+    assert not from_cache()          # timed, and stored behind the old line
+    assert len(cache.read_text().splitlines()) == 2
+    assert from_cache()
+    cache.write_text(line(3, "streams"))
+    assert from_cache()              # the key is formed as this test forms it
+    fake.lib.stitch_rig_destroy(rig)
