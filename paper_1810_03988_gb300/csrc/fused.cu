@@ -557,10 +557,10 @@ __device__ __forceinline__ void d1_put(const D1Out<T>& o, int dy, V4 s) {
 // on), moves B on by tap 2 into C and starts row m in B; row 2m + 1 adds tap 3 to C and tap 1 to B.
 // Row 18 completes output row 7.  w01: the weights of rows 0 and 1.
 //
-// ROLLED: row 18 is a last, half pass of the loop instead of a third copy of the sample's code.  With many
-// waves of tiles, warps of different variants share the instruction cache and fetching is the largest
-// stall (2.1 cycles per issue): 8 x 4K 715 -> 692 us per frame, 8 rigs batched 1433 -> 1404.  With few it only takes the overlap of the last
-// two samples: cylinder 4 x 720p 89.5 -> 90.6, so the larger capacity keeps the copy.
+// ROLLED: row 18 is a last, half pass of the loop instead of a third copy of the sample's code.  Over many
+// waves of tiles, warps of different variants share the instruction cache and fetching is the largest stall
+// (2.1 cycles per issue before); over few, the copy's overlap of the last two samples counts more
+// (d1_rolled).
 template <typename T, int MODE, int OUTK, bool ONES, bool ROLLED>
 __device__ __forceinline__ void d1_sweep(const D1Ctx& x, float4* __restrict__ vcol, const float* __restrict__ wcol,
                                          float2 w01, float2 nuv, float dqc, const D1Out<T>& o) {
@@ -609,7 +609,7 @@ __device__ __forceinline__ void d1_bar(int id) {
 }
 
 // One down1 tile, worked on by the D1_THREADS threads t = 0 .. 63 that share barrier `bar`.
-template <typename T, int CAP = D1_FOOT>
+template <typename T, int CAP = D1_FOOT, bool ROLLED = false>
 __device__ __forceinline__ void down1_tile(const RigGeom& g, const FramePtrs& fp, const OutDesc& od, const D1Rec& rec, const float* __restrict__ d1w,
                                            const float4* __restrict__ d1cols,
                                            Slot* __restrict__ g0buf, float4* smem, int t = threadIdx.x, int bar = 0) {
@@ -714,7 +714,6 @@ __device__ __forceinline__ void down1_tile(const RigGeom& g, const FramePtrs& fp
             o.rows = xo < g.nx[0] ? max(0, min(2 * D1_TY, g.ny[0] - Y0)) : 0;
         }
         float4* vcol = vres + d1_vslot(c);
-        constexpr bool ROLLED = CAP <= D1_FOOT_SMALL;
         // the staged mode (nearly every tile) has a sweep per output kind; the rare clamping and
         // frame-reading modes take the kind at run time
         if (mode == D1M_STAGED && (flags & D1_INTERIOR)) {
@@ -806,7 +805,7 @@ __host__ __device__ inline D1Rec d1_record(const D1Tile& tl, const CamDev& c, co
                  ref.tm, ref.ax, ref.ay, c.W, c.H, c.gain * (1.0f / 255.0f), o.w(), (int)clip, g1};
 }
 
-template <typename T, int CAP>
+template <typename T, int CAP, bool ROLLED>
 __global__ void __launch_bounds__(D1_THREADS, D1Cap<CAP>::BLOCKS) k_down1(RigGeom g,
                                                                         FramePtrs fp, OutDesc od,
                                                                         const D1Rec* __restrict__ recs, int n, int wave,
@@ -818,8 +817,13 @@ __global__ void __launch_bounds__(D1_THREADS, D1Cap<CAP>::BLOCKS) k_down1(RigGeo
     const D1Rec rec = load_record(recs + blockIdx.x);
     if (threadIdx.x == 0 && blockIdx.x + wave < n) prefetch_l2(recs + blockIdx.x + wave);
     pdl_wait();
-    down1_tile<T, CAP>(g, fp, od, rec, d1w, d1cols, g0buf, smem);
+    down1_tile<T, CAP, ROLLED>(g, fp, od, rec, d1w, d1cols, g0buf, smem);
 }
+
+// Whether n tiles over `resident` blocks take the rolled sweep (d1_sweep): from 2.5 waves on.  Rolled and
+// copied, us per call: 0.3 waves (2 x 360p) 36.9 and 36.8, 2.1 (cylinder 4 x 720p) 89.9 and 89.6, 2.9 (5 x 719p)
+// 116.1 and 116.5, 5.5 (4 x 1080p) 181.2 and 182.8, 29 (8 x 4K) 694 and 717, 8 rigs batched 1405 and 1433.
+inline bool d1_rolled(long long n, long long resident) { return 2 * n >= 5 * resident; }
 
 // ------------------------------------------------------------------------------------------------
 // solo: SOLO canvas tiles under which no pyramid level is read
@@ -2150,6 +2154,7 @@ struct FusedState {
     int n_g0 = 0;
     int n_staged = 0;            // down1 tiles with a staged source footprint
     bool d1_small = false;       // down1 with the smaller footprint capacity (13 blocks per SM)
+    bool d1_rolled = false;      // and with the rolled sweep
     bool up_four = false;        // up_full with four resident blocks per SM
     int wave_d1 = 0, wave_red = 0, wave_up = 0;  // resident blocks on the device (L2 prefetch distance)
     void* R[MAXL] = {};          // R^l on the canvas grid, l >= 2
@@ -2399,7 +2404,8 @@ stitch_status launch_all(stitch_rig* r, FusedState* fs, const FramePtrs& fp, con
     };
     if (L >= 2 && fs->n_d1_pyr > 0) {
         prof_mark(r, "fused_down1", s);
-        const auto k = fs->d1_small ? k_down1<T, D1_FOOT_SMALL> : k_down1<T, D1_FOOT>;
+        const auto k = fs->d1_small ? (fs->d1_rolled ? k_down1<T, D1_FOOT_SMALL, true> : k_down1<T, D1_FOOT_SMALL, false>)
+                                    : (fs->d1_rolled ? k_down1<T, D1_FOOT, true> : k_down1<T, D1_FOOT, false>);
         const size_t smem = fs->d1_small ? D1Cap<D1_FOOT_SMALL>::SMEM : D1_SMEM;
         put(k, fs->n_d1_pyr, D1_THREADS, smem, g, fp, od, fs->d1_recs, fs->n_d1_pyr, fs->wave_d1, fs->d1w, fs->d1cols,
             (Slot*)fs->g0buf);
@@ -2459,9 +2465,10 @@ stitch_status launch_all(stitch_rig* r, FusedState* fs, const FramePtrs& fp, con
 
 template <typename T>
 stitch_status set_smem_attrs() {
-    STITCH_CUDA_TRY(cudaFuncSetAttribute(k_down1<T, D1_FOOT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)D1_SMEM));
-    STITCH_CUDA_TRY(cudaFuncSetAttribute(k_down1<T, D1_FOOT_SMALL>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)D1Cap<D1_FOOT_SMALL>::SMEM));
+    for (const auto k : {k_down1<T, D1_FOOT, false>, k_down1<T, D1_FOOT, true>})
+        STITCH_CUDA_TRY(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)D1_SMEM));
+    for (const auto k : {k_down1<T, D1_FOOT_SMALL, false>, k_down1<T, D1_FOOT_SMALL, true>})
+        STITCH_CUDA_TRY(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)D1Cap<D1_FOOT_SMALL>::SMEM));
     STITCH_CUDA_TRY(cudaFuncSetAttribute(k_reduce_t<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)RC_SMEM));
     STITCH_CUDA_TRY(cudaFuncSetAttribute(k_up_full<T, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)up_full_smem<2>()));
@@ -2878,12 +2885,13 @@ stitch_status fused_plan(stitch_rig* r) {
             return STITCH_ECUDA;
         int bpsm = 0;
         const cudaError_t oe =
-            fs->d1_small ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bpsm, k_down1<float4, D1_FOOT_SMALL>, D1_THREADS,
+            fs->d1_small ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bpsm, k_down1<float4, D1_FOOT_SMALL, false>, D1_THREADS,
                                                                          D1Cap<D1_FOOT_SMALL>::SMEM)
-                         : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bpsm, k_down1<float4, D1_FOOT>, D1_THREADS, D1_SMEM);
+                         : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bpsm, k_down1<float4, D1_FOOT, false>, D1_THREADS, D1_SMEM);
         if (oe != cudaSuccess) return STITCH_ECUDA;
         const size_t K = (size_t)std::max(bpsm, 1) * sms;
         fs->wave_d1 = (int)K;
+        fs->d1_rolled = d1_rolled(fs->n_d1_pyr, (long long)K);
         for (size_t k = 0; k + K < (size_t)fs->n_d1_pyr; ++k) {
             const D1Tile& nx = d1[k + K];
             if (nx.fwh == 0) continue;
@@ -3226,14 +3234,14 @@ __global__ void __launch_bounds__(U_THREADS) k_batch_general(const BatchRigDev* 
 
 // Multi-rig stage kernels (the alternative batched schedule): one block per task of one task type,
 // tasks of every rig in one launch, each kernel with its own register and shared-memory budget.
-template <typename T, int CAP>
+template <typename T, int CAP, bool ROLLED>
 __global__ void __launch_bounds__(D1_THREADS, D1Cap<CAP>::BLOCKS) k_mr_down1(const BatchRigDev* __restrict__ rigs,
                                                              const BTask* __restrict__ tasks) {
     extern __shared__ float4 smem[];
     const BTask tk = tasks[blockIdx.x];
     const BatchRigDev& rg = rigs[tk.rig];
     const D1Tile& tl = task_tile<D1Tile>(tk);
-    down1_tile<T, CAP>(rg.g, rg.fp, rg.od, d1_record(tl, rg.cams[tl.cam], rg.refs[tl.ref], sizeof(T)), rg.d1w, rg.d1cols,
+    down1_tile<T, CAP, ROLLED>(rg.g, rg.fp, rg.od, d1_record(tl, rg.cams[tl.cam], rg.refs[tl.ref], sizeof(T)), rg.d1w, rg.d1cols,
                        (Slot*)rg.g0buf, smem);
 }
 
@@ -3414,12 +3422,14 @@ stitch_status b_launch_staged(BatchState* b, int shape, cudaStream_t s) {
     for (const StageGroup& gr : b->groups[shape]) {
         if (!gr.count) continue;
         switch (gr.type) {
-            case BT_D1:
-                if (b->d1_small)
-                    k_mr_down1<T, D1_FOOT_SMALL><<<gr.count, D1_THREADS, D1Cap<D1_FOOT_SMALL>::SMEM, s>>>(b->d_rigs, gr.d_tasks);
-                else
-                    k_mr_down1<T, D1_FOOT><<<gr.count, D1_THREADS, D1_SMEM, s>>>(b->d_rigs, gr.d_tasks);
+            case BT_D1: {
+                const int blocks = b->d1_small ? D1Cap<D1_FOOT_SMALL>::BLOCKS : D1Cap<D1_FOOT>::BLOCKS;
+                const bool rolled = d1_rolled(gr.count, (long long)blocks * b->sms);
+                const auto k = b->d1_small ? (rolled ? k_mr_down1<T, D1_FOOT_SMALL, true> : k_mr_down1<T, D1_FOOT_SMALL, false>)
+                                           : (rolled ? k_mr_down1<T, D1_FOOT, true> : k_mr_down1<T, D1_FOOT, false>);
+                k<<<gr.count, D1_THREADS, b->d1_small ? D1Cap<D1_FOOT_SMALL>::SMEM : D1_SMEM, s>>>(b->d_rigs, gr.d_tasks);
                 break;
+            }
             case BT_RED:
                 if (b_rs(shape)) k_mr_reduce_col<T><<<gr.count, RC_THREADS, RC_SMEM, s>>>(b->d_rigs, gr.d_tasks);
                 else k_mr_reduce<T, RSRig><<<gr.count, 256, RSRig::SMEM, s>>>(b->d_rigs, gr.d_tasks);
@@ -3448,9 +3458,10 @@ stitch_status b_launch_staged(BatchState* b, int shape, cudaStream_t s) {
 
 template <typename T>
 stitch_status b_staged_attrs() {
-    STITCH_CUDA_TRY(cudaFuncSetAttribute(k_mr_down1<T, D1_FOOT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)D1_SMEM));
-    STITCH_CUDA_TRY(cudaFuncSetAttribute(k_mr_down1<T, D1_FOOT_SMALL>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)D1Cap<D1_FOOT_SMALL>::SMEM));
+    for (const auto k : {k_mr_down1<T, D1_FOOT, false>, k_mr_down1<T, D1_FOOT, true>})
+        STITCH_CUDA_TRY(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)D1_SMEM));
+    for (const auto k : {k_mr_down1<T, D1_FOOT_SMALL, false>, k_mr_down1<T, D1_FOOT_SMALL, true>})
+        STITCH_CUDA_TRY(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)D1Cap<D1_FOOT_SMALL>::SMEM));
     STITCH_CUDA_TRY(cudaFuncSetAttribute(k_mr_up_full_b4<T, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)up_full_smem<2>()));
     STITCH_CUDA_TRY(cudaFuncSetAttribute(k_mr_up_full_b4<T, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize,

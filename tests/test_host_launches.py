@@ -1,5 +1,6 @@
 """What the library's host side hands the GPU, call by call, on a CUDA runtime that only takes notes."""
 import ctypes
+import re
 import struct
 
 import numpy as np
@@ -172,4 +173,19 @@ def test_schedules_timed_with_earlier_kernels_are_timed_again(fake, monkeypatch,
     assert from_cache()
     cache.write_text(line(3, "streams"))
     assert from_cache()              # the key is formed as this test forms it
+    fake.lib.stitch_rig_destroy(rig)
+
+
+@pytest.mark.parametrize("spread", [1.0, 1.6])  # source pixels per canvas pixel: footprints of either capacity
+@pytest.mark.parametrize("cw,ch", [(1200, 400), (4000, 1200)])  # about one wave of down1 tiles, and many
+def test_the_sweep_of_down1_goes_by_the_number_of_waves(fake, spread, cw, ch):
+    w, h = int(0.6 * cw * spread), int(0.9 * ch * spread)
+    cams = [_Camera(w, h, np.diag([1 / spread, 1 / spread, 1.0]) + _shift(x, 0.05 * ch) - np.eye(3)) for x in (0.0, 0.4 * cw)]
+    rig = fake.rig(cams, cw, ch, 3)
+    log = _stitch(fake, rig, cams, cw, ch)
+    down1 = [e.kernel for e in log if isinstance(e, Launch) and "k_down1" in e.kernel]
+    assert len(down1) == 1
+    capacity, rolled = re.search(r"k_down1I6float4Li(\d+)ELb([01])E", down1[0]).groups()
+    assert int(capacity) == (1536 if spread == 1.0 else 2048)
+    assert rolled == ("1" if cw == 4000 else "0")
     fake.lib.stitch_rig_destroy(rig)
