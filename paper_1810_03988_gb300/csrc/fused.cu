@@ -233,6 +233,7 @@ struct D1Cap {
     static_assert(CAP % 16 == 0, "whole groups of 4 texels, 16-byte aligned parts");
 };
 constexpr size_t D1_SMEM = D1Cap<D1_FOOT>::SMEM;  // the larger capacity's
+static_assert(D1_SMEM <= 48 * 1024, "within what a kernel may take without being asked");
 static_assert(D1_SX == 67 && D1_THREADS == 64 && D1_XC == 3, "column-per-thread sweep of a 67-column region");
 static_assert(D1_SM_V % 16 == 0 && D1_SM_X % 16 == 0, "16-byte aligned parts");
 
@@ -820,10 +821,19 @@ __global__ void __launch_bounds__(D1_THREADS, D1Cap<CAP>::BLOCKS) k_down1(RigGeo
     down1_tile<T, CAP, ROLLED>(g, fp, od, rec, d1w, d1cols, g0buf, smem);
 }
 
-// Whether n tiles over `resident` blocks take the rolled sweep (d1_sweep): from 2.5 waves on.  Rolled and
-// copied, us per call: 0.3 waves (2 x 360p) 36.9 and 36.8, 2.1 (cylinder 4 x 720p) 89.9 and 89.6, 2.9 (5 x 719p)
-// 116.1 and 116.5, 5.5 (4 x 1080p) 181.2 and 182.8, 29 (8 x 4K) 694 and 717, 8 rigs batched 1405 and 1433.
-inline bool d1_rolled(long long n, long long resident) { return 2 * n >= 5 * resident; }
+// Whether n tiles in one launch, or in launches side by side, take the rolled sweep (d1_sweep): from 2.5
+// waves of resident blocks on.  Rolled and copied, us per call: 0.3 waves (2 x 360p) 36.9 and 36.8, 2.1 (cylinder
+// 4 x 720p) 89.9 and 89.6, 2.9 (5 x 719p) 116.1 and 116.5, 5.5 (4 x 1080p) 181.2 and 182.8, 29 (8 x 4K) 694 and
+// 717, 8 rigs batched 1405 and 1433 (rigs on streams by their own waves: 1345 to 1351, by all rigs' 1340).
+inline bool d1_rolled(long long n, bool small, int sms) {
+    return 2 * n >= 5LL * (small ? D1Cap<D1_FOOT_SMALL>::BLOCKS : D1Cap<D1_FOOT>::BLOCKS) * sms;
+}
+
+template <typename T>
+auto d1_kernel(bool small, bool rolled) {
+    return small ? (rolled ? k_down1<T, D1_FOOT_SMALL, true> : k_down1<T, D1_FOOT_SMALL, false>)
+                 : (rolled ? k_down1<T, D1_FOOT, true> : k_down1<T, D1_FOOT, false>);
+}
 
 // ------------------------------------------------------------------------------------------------
 // solo: SOLO canvas tiles under which no pyramid level is read
@@ -2393,9 +2403,10 @@ void plan_coarse_tiles(const stitch_rig* r, const std::vector<UpTile>* up, int t
 }
 
 // The launches of a call: down1, solo, REDUCE, coarse and canvas tiles.  early: whether the first of them,
-// whichever that is, may start while the stream's previous kernel drains.
+// whichever that is, may start while the stream's previous kernel drains.  rolled: the form of down1's sweep.
 template <typename T>
-stitch_status launch_all(stitch_rig* r, FusedState* fs, const FramePtrs& fp, const OutDesc& od, cudaStream_t s, bool early) {
+stitch_status launch_all(stitch_rig* r, FusedState* fs, const FramePtrs& fp, const OutDesc& od, cudaStream_t s, bool early,
+                         bool rolled) {
     const RigGeom& g = r->geom;
     const int L = g.levels;
     const auto put = [&](auto kernel, dim3 grid, int block, size_t smem, const auto&... args) {
@@ -2404,10 +2415,8 @@ stitch_status launch_all(stitch_rig* r, FusedState* fs, const FramePtrs& fp, con
     };
     if (L >= 2 && fs->n_d1_pyr > 0) {
         prof_mark(r, "fused_down1", s);
-        const auto k = fs->d1_small ? (fs->d1_rolled ? k_down1<T, D1_FOOT_SMALL, true> : k_down1<T, D1_FOOT_SMALL, false>)
-                                    : (fs->d1_rolled ? k_down1<T, D1_FOOT, true> : k_down1<T, D1_FOOT, false>);
         const size_t smem = fs->d1_small ? D1Cap<D1_FOOT_SMALL>::SMEM : D1_SMEM;
-        put(k, fs->n_d1_pyr, D1_THREADS, smem, g, fp, od, fs->d1_recs, fs->n_d1_pyr, fs->wave_d1, fs->d1w, fs->d1cols,
+        put(d1_kernel<T>(fs->d1_small, rolled), fs->n_d1_pyr, D1_THREADS, smem, g, fp, od, fs->d1_recs, fs->n_d1_pyr, fs->wave_d1, fs->d1w, fs->d1cols,
             (Slot*)fs->g0buf);
     }
     if (fs->n_solo_tiles > 0) {
@@ -2465,10 +2474,6 @@ stitch_status launch_all(stitch_rig* r, FusedState* fs, const FramePtrs& fp, con
 
 template <typename T>
 stitch_status set_smem_attrs() {
-    for (const auto k : {k_down1<T, D1_FOOT, false>, k_down1<T, D1_FOOT, true>})
-        STITCH_CUDA_TRY(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)D1_SMEM));
-    for (const auto k : {k_down1<T, D1_FOOT_SMALL, false>, k_down1<T, D1_FOOT_SMALL, true>})
-        STITCH_CUDA_TRY(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)D1Cap<D1_FOOT_SMALL>::SMEM));
     STITCH_CUDA_TRY(cudaFuncSetAttribute(k_reduce_t<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)RC_SMEM));
     STITCH_CUDA_TRY(cudaFuncSetAttribute(k_up_full<T, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)up_full_smem<2>()));
@@ -2884,14 +2889,12 @@ stitch_status fused_plan(stitch_rig* r) {
         if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, r->device) != cudaSuccess || sms < 1)
             return STITCH_ECUDA;
         int bpsm = 0;
-        const cudaError_t oe =
-            fs->d1_small ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bpsm, k_down1<float4, D1_FOOT_SMALL, false>, D1_THREADS,
-                                                                         D1Cap<D1_FOOT_SMALL>::SMEM)
-                         : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bpsm, k_down1<float4, D1_FOOT, false>, D1_THREADS, D1_SMEM);
-        if (oe != cudaSuccess) return STITCH_ECUDA;
+        fs->d1_rolled = d1_rolled(fs->n_d1_pyr, fs->d1_small, sms);
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bpsm, d1_kernel<float4>(fs->d1_small, fs->d1_rolled), D1_THREADS,
+                                                          fs->d1_small ? D1Cap<D1_FOOT_SMALL>::SMEM : D1_SMEM) != cudaSuccess)
+            return STITCH_ECUDA;
         const size_t K = (size_t)std::max(bpsm, 1) * sms;
         fs->wave_d1 = (int)K;
-        fs->d1_rolled = d1_rolled(fs->n_d1_pyr, (long long)K);
         for (size_t k = 0; k + K < (size_t)fs->n_d1_pyr; ++k) {
             const D1Tile& nx = d1[k + K];
             if (nx.fwh == 0) continue;
@@ -2999,7 +3002,8 @@ stitch_status fused_plan(stitch_rig* r) {
 stitch_status fused_frames(stitch_rig* r, const FramePtrs& fp, const OutDesc& od, cudaStream_t s, bool early) {
     FusedState* fs = (FusedState*)r->fused;
     if (!fs) return STITCH_EINVAL;
-    return fs->fp16 ? launch_all<half4>(r, fs, fp, od, s, early) : launch_all<float4>(r, fs, fp, od, s, early);
+    return fs->fp16 ? launch_all<half4>(r, fs, fp, od, s, early, fs->d1_rolled)
+                    : launch_all<float4>(r, fs, fp, od, s, early, fs->d1_rolled);
 }
 
 stitch_status fused_precompute(stitch_rig* r) {
@@ -3350,6 +3354,7 @@ struct BatchState {
     int shape = 0;                             // the combination chosen
     bool staged = false;             // schedule chosen by the tuner: staged launches or persistent
     bool d1_small = false;           // staged down1 launches with the smaller footprint capacity (every rig's)
+    bool d1_rolled = false;          // the form of down1's sweep, by all rigs' tiles (staged, streams)
     bool up_four = false;            // staged up_full launches at four blocks per SM
     bool streams = false;            // ... or every rig's own launch sequence on its own stream
     cudaStream_t rs[B_MAXRIGS] = {};
@@ -3423,10 +3428,8 @@ stitch_status b_launch_staged(BatchState* b, int shape, cudaStream_t s) {
         if (!gr.count) continue;
         switch (gr.type) {
             case BT_D1: {
-                const int blocks = b->d1_small ? D1Cap<D1_FOOT_SMALL>::BLOCKS : D1Cap<D1_FOOT>::BLOCKS;
-                const bool rolled = d1_rolled(gr.count, (long long)blocks * b->sms);
-                const auto k = b->d1_small ? (rolled ? k_mr_down1<T, D1_FOOT_SMALL, true> : k_mr_down1<T, D1_FOOT_SMALL, false>)
-                                           : (rolled ? k_mr_down1<T, D1_FOOT, true> : k_mr_down1<T, D1_FOOT, false>);
+                const auto k = b->d1_small ? (b->d1_rolled ? k_mr_down1<T, D1_FOOT_SMALL, true> : k_mr_down1<T, D1_FOOT_SMALL, false>)
+                                           : (b->d1_rolled ? k_mr_down1<T, D1_FOOT, true> : k_mr_down1<T, D1_FOOT, false>);
                 k<<<gr.count, D1_THREADS, b->d1_small ? D1Cap<D1_FOOT_SMALL>::SMEM : D1_SMEM, s>>>(b->d_rigs, gr.d_tasks);
                 break;
             }
@@ -3458,10 +3461,6 @@ stitch_status b_launch_staged(BatchState* b, int shape, cudaStream_t s) {
 
 template <typename T>
 stitch_status b_staged_attrs() {
-    for (const auto k : {k_mr_down1<T, D1_FOOT, false>, k_mr_down1<T, D1_FOOT, true>})
-        STITCH_CUDA_TRY(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)D1_SMEM));
-    for (const auto k : {k_mr_down1<T, D1_FOOT_SMALL, false>, k_mr_down1<T, D1_FOOT_SMALL, true>})
-        STITCH_CUDA_TRY(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)D1Cap<D1_FOOT_SMALL>::SMEM));
     STITCH_CUDA_TRY(cudaFuncSetAttribute(k_mr_up_full_b4<T, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)up_full_smem<2>()));
     STITCH_CUDA_TRY(cudaFuncSetAttribute(k_mr_up_full_b4<T, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -3585,7 +3584,8 @@ stitch_status b_launch_streams(BatchState* b, cudaStream_t s) {
     for (int k = 0; k < b->n; ++k) {
         stitch_rig* r = b->rigs[k];
         STITCH_CUDA_TRY(cudaStreamWaitEvent(b->rs[k], b->fork, 0));
-        const stitch_status st = launch_all<T>(r, (FusedState*)r->fused, b->h_rigs[k].fp, b->h_rigs[k].od, b->rs[k], false);
+        const stitch_status st = launch_all<T>(r, (FusedState*)r->fused, b->h_rigs[k].fp, b->h_rigs[k].od, b->rs[k], false,
+                                               b->d1_rolled);
         if (st != STITCH_OK) return st;
         STITCH_CUDA_TRY(cudaEventRecord(b->rdone[k], b->rs[k]));
         STITCH_CUDA_TRY(cudaStreamWaitEvent(s, b->rdone[k], 0));
@@ -3918,12 +3918,13 @@ stitch_status fused_batch_create(stitch_rig* const* rigs, int n, void** out) {
         // the occupancy variants the rigs' own launches take (down1: the smaller footprint capacity
         // when every rig takes it; up_full: four blocks per SM for many waves of blended tiles)
         {
-            long long nfull = 0;
+            long long nfull = 0, nd1 = 0;
             b->d1_small = true;
             for (int k = 0; k < n; ++k) {
                 const FusedState* fs = (const FusedState*)rigs[k]->fused;
                 b->d1_small = b->d1_small && fs->d1_small;
                 nfull += fs->n_up[UP_FULL2] + fs->n_up[UP_FULL4];
+                nd1 += fs->n_d1;
             }
             int sms = 0;
             if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, rigs[0]->device) != cudaSuccess) {
@@ -3931,6 +3932,7 @@ stitch_status fused_batch_create(stitch_rig* const* rigs, int n, void** out) {
                 sms = 1;
             }
             b->up_four = nfull >= 8LL * 4 * std::max(sms, 1);
+            b->d1_rolled = d1_rolled(nd1, b->d1_small, std::max(sms, 1));
         }
         std::vector<BTask> wred[MAXL], wco[MAXL];
         for (int k = 0; k < n; ++k) {

@@ -176,8 +176,8 @@ def test_schedules_timed_with_earlier_kernels_are_timed_again(fake, monkeypatch,
     fake.lib.stitch_rig_destroy(rig)
 
 
-@pytest.mark.parametrize("spread", [1.0, 1.6])  # source pixels per canvas pixel: footprints of either capacity
-@pytest.mark.parametrize("cw,ch", [(1200, 400), (4000, 1200)])  # about one wave of down1 tiles, and many
+@pytest.mark.parametrize("spread", [1.0, 1.12])  # source pixels per canvas pixel: footprints of either capacity
+@pytest.mark.parametrize("cw,ch", [(1200, 400), (7000, 2000)])  # about one wave of down1 tiles, and many
 def test_the_sweep_of_down1_goes_by_the_number_of_waves(fake, spread, cw, ch):
     w, h = int(0.6 * cw * spread), int(0.9 * ch * spread)
     cams = [_Camera(w, h, np.diag([1 / spread, 1 / spread, 1.0]) + _shift(x, 0.05 * ch) - np.eye(3)) for x in (0.0, 0.4 * cw)]
@@ -187,5 +187,5 @@ def test_the_sweep_of_down1_goes_by_the_number_of_waves(fake, spread, cw, ch):
     assert len(down1) == 1
     capacity, rolled = re.search(r"k_down1I6float4Li(\d+)ELb([01])E", down1[0]).groups()
     assert int(capacity) == (1536 if spread == 1.0 else 2048)
-    assert rolled == ("1" if cw == 4000 else "0")
+    assert rolled == ("1" if cw == 7000 else "0")
     fake.lib.stitch_rig_destroy(rig)
