@@ -166,8 +166,9 @@ __global__ void __launch_bounds__(BX* BY) k_plain_reduce(const CamDev* cams, int
 }
 
 // EXPAND of a coarse buffer (rect r of a level of size nxc x nyc) at fine (x, y), rgb only: taps
-// k - 1, k, k + 1 with weights 1/8, 3/4, 1/8 at even positions 2k and 0, 1/2, 1/2 at odd ones, so that
-// a warp's lanes take the same 9 loads (the tap of weight 0 adds nothing; it is kept inside the buffer).
+// k - 1, k, k + 1 with weights 1/8, 3/4, 1/8 at even positions 2k and k, k + 1 with 1/2, 1/2 at odd ones.  A
+// warp's lanes take the same 9 loads (those an odd position has no use for are kept inside the buffer); the
+// taps that it does not have are left out, not multiplied by 0, which a value out of range would survive.
 __device__ __forceinline__ float3 expand_rgb(const float4* buf, const Rect& r, int nxc, int nyc, int x,
                                              int y) {
     const bool ox = x & 1, oy = y & 1;
@@ -179,17 +180,23 @@ __device__ __forceinline__ float3 expand_rgb(const float4* buf, const Rect& r, i
         xo[a] = min(max(fold101((x >> 1) + a - 1, nxc) - r.x0, 0), r.w() - 1);
         yo[a] = min(max(fold101((y >> 1) + a - 1, nyc) - r.y0, 0), r.h() - 1);
     }
+    float4 v[3][3];
+#pragma unroll
+    for (int a = 0; a < 3; ++a)
+#pragma unroll
+        for (int b = 0; b < 3; ++b) v[a][b] = ld4(buf + (long long)yo[a] * r.w() + xo[b]);
     float3 acc = make_float3(0.f, 0.f, 0.f);
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
         float3 row = make_float3(0.f, 0.f, 0.f);
 #pragma unroll
         for (int b = 0; b < 3; ++b) {
-            const float4 v = ld4(buf + (long long)yo[a] * r.w() + xo[b]);
-            row.x = fmaf(wx[b], v.x, row.x);
-            row.y = fmaf(wx[b], v.y, row.y);
-            row.z = fmaf(wx[b], v.z, row.z);
+            if (b == 0 && ox) continue;
+            row.x = fmaf(wx[b], v[a][b].x, row.x);
+            row.y = fmaf(wx[b], v[a][b].y, row.y);
+            row.z = fmaf(wx[b], v[a][b].z, row.z);
         }
+        if (a == 0 && oy) continue;
         acc.x = fmaf(wy[a], row.x, acc.x);
         acc.y = fmaf(wy[a], row.y, acc.y);
         acc.z = fmaf(wy[a], row.z, acc.z);
