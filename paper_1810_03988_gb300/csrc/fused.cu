@@ -2039,7 +2039,7 @@ __device__ __forceinline__ void up_general_tile(const CamDev* __restrict__ cams,
             const float w = g.seam ? (own[k] == a ? 1.f : 0.f) : feather_weight(sp, c.W, c.H);
             if (!(w > 0.f)) continue;
             const float what = w / ws[k];
-            float3 v = bilinear_rgb(fp.p[i], fp.pitch[i], c.W, clamp_tap(sp, c.W, c.H), scale);
+            float3 v = bilinear_rgb<false>(fp.p[i], fp.pitch[i], c.W, clamp_tap(sp, c.W, c.H), scale);
             if (L >= 2) {
                 const float3 e = expand_smem(g1, UG1_X, dx, dy);
                 v.x -= e.x;

@@ -358,15 +358,25 @@ __device__ __forceinline__ bool word_aligned(const uint8_t* px, long long pitch)
     return (((uint32_t)reinterpret_cast<uintptr_t>(px) | (uint32_t)pitch) & 3u) == 0u;
 }
 
-// Bilinear RGB sample of an 8-bit frame of width W, scaled by `scale` (= gain / 255).
+// Exact float of an 8-bit value with one integer OR and one add: the bits 0x4B000000 | b encode
+// 2^23 + b, so subtracting 2^23 leaves b (IEEE-754 single precision, no rounding).
+__device__ __forceinline__ float u8_to_f(uint32_t b) { return __int_as_float(0x4B000000u | b) - 8388608.0f; }
+
+// Bilinear RGB sample of an 8-bit frame of width W, scaled by `scale` (= gain / 255).  WORDS: taps from word
+// loads (load_texels) where they are possible, otherwise byte by byte.
+template <bool WORDS = true>
 __device__ __forceinline__ float3 bilinear_rgb(const uint8_t* px, long long pitch, int W, const Tap& t,
                                                float scale) {
-    const Texels q = load_texels(px + (long long)t.j0 * pitch + 3 * t.i0, px + (long long)t.j1 * pitch + 3 * t.i0, t.i0, W,
-                                 word_aligned(px, pitch));
+    const uint8_t *r0 = px + (long long)t.j0 * pitch, *r1 = px + (long long)t.j1 * pitch;
+    Texels q{};
+    if (WORDS) q = load_texels(r0 + 3 * t.i0, r1 + 3 * t.i0, t.i0, W, word_aligned(px, pitch));
     float3 o;
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-        const float p00 = byte_f(q.t00, c), p01 = byte_f(q.t01, c), p10 = byte_f(q.t10, c), p11 = byte_f(q.t11, c);
+        const float p00 = WORDS ? byte_f(q.t00, c) : u8_to_f(__ldca(r0 + 3 * t.i0 + c));
+        const float p01 = WORDS ? byte_f(q.t01, c) : u8_to_f(__ldca(r0 + 3 * t.i1 + c));
+        const float p10 = WORDS ? byte_f(q.t10, c) : u8_to_f(__ldca(r1 + 3 * t.i0 + c));
+        const float p11 = WORDS ? byte_f(q.t11, c) : u8_to_f(__ldca(r1 + 3 * t.i1 + c));
         const float top = fmaf(t.fx, p01 - p00, p00);
         const float bot = fmaf(t.fx, p11 - p10, p10);
         const float v = fmaf(t.fy, bot - top, top) * scale;
@@ -385,9 +395,6 @@ __host__ __device__ __forceinline__ void tile_anchor(const Rect& V, int X, int Y
 // ------------------------------------------------------------------------------------------------
 // lean per-sample helpers used by the fused kernels
 
-// Exact float of an 8-bit value with one integer OR and one add: the bits 0x4B000000 | b encode
-// 2^23 + b, so subtracting 2^23 leaves b (IEEE-754 single precision, no rounding).
-__device__ __forceinline__ float u8_to_f(uint32_t b) { return __int_as_float(0x4B000000u | b) - 8388608.0f; }
 
 // One camera's mapping of canvas point anchor + (dx, dy): fraction-exact source position,
 // float source coordinates for the weight, and the sign of w.
