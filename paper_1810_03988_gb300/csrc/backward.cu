@@ -196,7 +196,7 @@ __device__ __forceinline__ void grad_terms(const GSample& s, const Pos& p, const
 // of the values and gets its partner's sums of them for its own of the other half.  Every sum adds
 // the same pairs as warp_sum (the lanes 16, 8, 4, 2, 1 apart), so the results are bit-identical, with
 // about M instead of 5 M shuffles.  Value index(i) of lane l's results v[0 .. left) is sum index(i).
-template <int M, int K, int BASE = 0>
+template <int M, int K>
 struct WarpSums {
     static constexpr int HALF = (M + 1) / 2;
     static constexpr int LEFT = WarpSums<HALF, K / 2>::LEFT;
@@ -218,8 +218,8 @@ struct WarpSums {
         return r < M ? r : -1;
     }
 };
-template <int M, int BASE>
-struct WarpSums<M, 0, BASE> {
+template <int M>
+struct WarpSums<M, 0> {
     static constexpr int LEFT = M;
     __device__ __forceinline__ static void run(float*, int) {}
     __device__ __forceinline__ static int index(int i, int) { return i; }

@@ -141,7 +141,8 @@ struct D1Tile {
 };
 
 // A down1 tile with what its camera adds, in one record: a block knows its staging loads after one round
-// trip to memory instead of three (tile, reference, camera).  With the first weights under way before the barrier: 8 x 4K 742 -> 725 us per frame.
+// trip to memory instead of three (tile, reference, camera).  With the first weights under way before the
+// barrier too, 8 x 4K went from 742 to 725 us per frame.
 struct __align__(16) D1Rec {
     int cam, k0, j0, flags, fxy, fwh, g0, coltab, pf_fxy, pf_fwh, pf_cw, wsel;  // of the D1Tile
     TileMap tm;
@@ -611,8 +612,8 @@ __device__ __forceinline__ void d1_bar(int id) {
 
 // One down1 tile, worked on by the D1_THREADS threads t = 0 .. 63 that share barrier `bar`.
 template <typename T, int CAP = D1_FOOT, bool ROLLED = false>
-__device__ __forceinline__ void down1_tile(const RigGeom& g, const FramePtrs& fp, const OutDesc& od, const D1Rec& rec, const float* __restrict__ d1w,
-                                           const float4* __restrict__ d1cols,
+__device__ __forceinline__ void down1_tile(const RigGeom& g, const FramePtrs& fp, const OutDesc& od, const D1Rec& rec,
+                                           const float* __restrict__ d1w, const float4* __restrict__ d1cols,
                                            Slot* __restrict__ g0buf, float4* smem, int t = threadIdx.x, int bar = 0) {
     uint32_t* foot = reinterpret_cast<uint32_t*>(smem);
     constexpr int SM_FOOT = D1Cap<CAP>::SM_FOOT;
@@ -1056,8 +1057,6 @@ __device__ __forceinline__ void reduce_tile(const CamDev* __restrict__ cams, con
     }
 }
 
-// Blocks start in index order as resident ones finish, so block b prefetches into L2 the input of
-// tile b + wave (wave = resident blocks on the device), which starts about when b ends.
 // Column-sweep REDUCE of the single-rig path: 64 x 8 outputs of level l+1 from the 131 x 19 region
 // of level l.  Thread t takes virtual column t + 2 and runs the vertical pass down its 19 rows in
 // registers, with its loads straight from G^l a few rows ahead; the columns 0, 1 and 130 are one
@@ -1159,6 +1158,8 @@ __device__ __forceinline__ void reduce_col_tile(const CamDev* __restrict__ cams,
     }
 }
 
+// Blocks start in index order as resident ones finish, so block b prefetches into L2 the input of
+// tile b + wave (wave = resident blocks on the device), which starts about when b ends.
 template <typename T>
 __global__ void __launch_bounds__(RC_THREADS, 8) k_reduce_t(const CamDev* __restrict__ cams, const __grid_constant__ RigGeom g,
                                                            int l, const Tile* __restrict__ tiles, int n, int wave) {
@@ -1235,7 +1236,8 @@ __device__ __forceinline__ void expand_col4(const float4* __restrict__ a, int ld
 // chunks of 2.  Latency bounds it (at most a few waves): the tables are read before the wait for the
 // previous kernel, and every load of the first chunk (R^{l+1}, two cameras' G^{l+1}, the first one's G^l)
 // is in flight at once, one barrier before the blend.  With a round trip and a barrier for each of
-// those: level 2 of 8 x 4K 36 us, now 29; levels 3 to 5 17 + 11 + 6.4, now 13.9 + 9.2 + 7.1.  Virtual level-(l+1) region: origin (X0/2 - 2, Y0/2 - 2), TX/2 + 4 by TY/2 + 4.
+// those, level 2 of 8 x 4K took 36 us, then 29, and levels 3 and 4 17 + 11, then 13.9 + 9.2.
+// Virtual level-(l+1) region: origin (X0/2 - 2, Y0/2 - 2), TX/2 + 4 by TY/2 + 4.
 // The tile shape is a template parameter (the batched schedule's tuner picks one per batch); the
 // single-rig path uses 32 x 32.
 constexpr int CT_NC = 2;
@@ -1839,8 +1841,8 @@ __device__ __forceinline__ void up_full_tile(const CamDev* __restrict__ cams, co
 }
 
 // The tiles of an up launch: n4 tiles with 3 or 4 cameras, then n2 with at most 2, then the ZERO (and
-// fallback SOLO) tiles, so that none of them needs a launch (and a tail) of its own; wave2, wave4:
-// resident blocks on the device (the distance of the L2 prefetch, see k_reduce_t).
+// fallback SOLO) tiles, so that none of them needs a launch (and a tail) of its own; wave: resident
+// blocks on the device (the distance of the L2 prefetch, see k_reduce_t).
 struct UpLaunch {
     const UpTile *t4, *t2, *simple;
     int n4, n2, wave;

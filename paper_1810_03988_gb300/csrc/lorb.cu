@@ -86,8 +86,9 @@ struct LorbCount {
 //    neighbouring ones).  The pairs that pass are gathered for the block, so the 16-pixel test and
 //    then the Harris response of the corners run with full warps instead of under a branch that nearly
 //    every warp takes for a few lanes, and spread over all warps however the corners lie.
-// One 3840 x 2160 view: 34 us (of which 18 us are issue slots; 35 us and a quarter more instructions with lists per warp) against 134 us for gray and smoothed maps, response map (8 bytes per
-// pixel written and read back) and suppression as three kernels.
+// One 3840 x 2160 view: 34 us (of which 18 us are issue slots; 35 us and a quarter more instructions with
+// lists per warp) against 134 us for gray and smoothed maps, response map (8 bytes per pixel written and
+// read back) and suppression as three kernels.
 constexpr int DT_EX = 64, DT_EY = 32;   // evaluated pixels
 constexpr int DT_OX = 60, DT_OY = 30;   // owned pixels: columns 2 .. 61, rows 1 .. 30
 constexpr int DT_PX = 72, DT_PY = 39;   // gray words: 18 groups of 4 columns, 13 strips of 3 rows

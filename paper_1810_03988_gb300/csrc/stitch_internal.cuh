@@ -501,24 +501,6 @@ __device__ __forceinline__ float3 sample_rgb(const uint8_t* px, long long pitch,
     return o;
 }
 
-// Bilinear RGB sample of a position known to lie in [0, W-1) x [0, H-1) (no clamping needed).
-__device__ __forceinline__ float3 sample_rgb_inside(const uint8_t* px, long long pitch, const Pos& p,
-                                                    float scale) {
-    const uint8_t* a = px + (long long)p.iv * pitch + 3 * p.iu;
-    const uint8_t* b = a + pitch;
-    float3 o;
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-        const float p00 = u8_to_f(__ldca(a + c)), p01 = u8_to_f(__ldca(a + 3 + c));
-        const float p10 = u8_to_f(__ldca(b + c)), p11 = u8_to_f(__ldca(b + 3 + c));
-        const float top = fmaf(p.fu, p01 - p00, p00);
-        const float bot = fmaf(p.fu, p11 - p10, p10);
-        const float v = fmaf(p.fv, bot - top, top) * scale;
-        if (c == 0) o.x = v; else if (c == 1) o.y = v; else o.z = v;
-    }
-    return o;
-}
-
 // v already clamped to [0, 1]: 2^23 + 255 v rounded once to nearest even in the addition of one
 // fused multiply-add, whose low byte is round-half-even(255 v)
 __device__ __forceinline__ uint32_t quantize_bits(float v) { return __float_as_uint(fmaf(v, 255.0f, 8388608.0f)); }
